@@ -98,6 +98,7 @@ gsi_status gsi_graph_create(const int32_t *vlab, int32_t n, const int32_t *src, 
         if (g->off) cudaFree(g->off);
         if (g->ci) cudaFree(g->ci);
         if (g->cl) cudaFree(g->cl);
+        if (g->dir) cudaFree(g->dir);
         if (g->sig) cudaFree(g->sig);
         if (g->gperm) cudaFree(g->gperm);
         if (g->gsig) cudaFree(g->gsig);
@@ -117,6 +118,7 @@ void gsi_graph_destroy(gsi_graph *g) {
     cudaFree(g->off);
     cudaFree(g->ci);
     cudaFree(g->cl);
+    cudaFree(g->dir);
     cudaFree(g->sig);
     cudaFree(g->gperm);
     cudaFree(g->gsig);

@@ -108,6 +108,33 @@ __global__ void k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int lb
     }
 }
 
+// Label directories of the lists of at least dir_min entries (gsi_graph::dir):
+// each lane looks at one segment, and the warp fills the directories of the
+// long ones together, one binary search of cl per label rank.  Most segments
+// are short, so this is one read of off plus the few directories.
+__global__ void k_label_dir(const uint32_t *__restrict__ off, const uint16_t *__restrict__ cl, uint64_t nseg, int32_t LV,
+                            uint32_t dir_min, uint32_t *__restrict__ dir) {
+    const int lane = threadIdx.x & 31;
+    const uint64_t step = (uint64_t)gridDim.x * blockDim.x;
+    for (uint64_t s0 = (uint64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); s0 < nseg; s0 += step) {
+        const uint64_t s = s0 + (uint64_t)lane;
+        const uint32_t a = s < nseg ? off[s] : 0u, b = s < nseg ? off[s + 1] : 0u;
+        for (unsigned m = __ballot_sync(FULL_MASK, b - a >= dir_min); m; m &= m - 1) {
+            const int j = __ffs(m) - 1;
+            const uint32_t x = __shfl_sync(FULL_MASK, a, j), y = __shfl_sync(FULL_MASK, b, j);
+            for (int32_t r = lane; r <= LV; r += 32) {
+                uint32_t lo = x, hi = y;
+                while (lo < hi) {
+                    const uint32_t mid = lo + ((hi - lo) >> 1);
+                    if ((int32_t)cl[mid] < r) lo = mid + 1;
+                    else hi = mid;
+                }
+                dir[((x + 1) >> 1) + (uint32_t)r] = lo;
+            }
+        }
+    }
+}
+
 __global__ void k_fill_u32(uint32_t *a, uint64_t n, uint32_t v) {
     for (uint64_t i = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (uint64_t)gridDim.x * blockDim.x)
         a[i] = v;
@@ -297,6 +324,8 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_CUDA_TRY(cudaMallocAsync(&g->off, sizeof(uint32_t) * (size_t)(nseg + 1), st));
     GSI_CUDA_TRY(cudaMallocAsync(&g->ci, sizeof(int32_t) * (size_t)(2 * m + 1), st));
     GSI_CUDA_TRY(cudaMallocAsync(&g->cl, sizeof(uint16_t) * (size_t)(2 * m + 1), st));
+    GSI_CUDA_TRY(cudaMallocAsync(&g->dir, sizeof(uint32_t) * (size_t)(m + 1), st));
+    g->dir_min = 2u * ((uint32_t)LV + 1u);
     GSI_CUDA_TRY(cudaMallocAsync(&g->sig, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
     if (m > 0) {
         int32_t *d_uniq = nullptr;
@@ -308,6 +337,7 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
         k_csr_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, d_vrank, m, L, lb, nb, keys);
         GSI_TRY(radix_sort_u64(keys, tmp, 2 * m, sb + lb + nb, st));
         k_csr_fill<<<grid_for(2 * m), NT, 0, st>>>(keys, 2 * m, lb, nb, nseg, g->off, g->ci, g->cl);
+        k_label_dir<<<grid_for((int64_t)nseg), NT, 0, st>>>(g->off, g->cl, nseg, LV, g->dir_min, g->dir);
         cudaFreeAsync(d_uniq, st);
         cudaFreeAsync(d_vrank, st);
     } else {
@@ -350,7 +380,8 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     cudaEventDestroy(e1);
     g->build_ms = ms;
     g->device_bytes = sizeof(uint32_t) * (nseg + 1) + sizeof(int32_t) * (uint64_t)(2 * m + 1) +
-                      sizeof(uint16_t) * (uint64_t)(2 * m + 1) + sizeof(uint32_t) * GSI_SIG_WORDS * (uint64_t)n +
+                      sizeof(uint16_t) * (uint64_t)(2 * m + 1) + sizeof(uint32_t) * (uint64_t)(m + 1) +
+                      sizeof(uint32_t) * GSI_SIG_WORDS * (uint64_t)n +
                       sizeof(uint32_t) * GSI_SIG_WORDS * (uint64_t)g->np;
     return GSI_OK;
 }

@@ -19,6 +19,12 @@ struct gsi_graph {
     uint32_t *off = nullptr;    // [n*L + 1]
     int32_t *ci = nullptr;      // [2m], each N(v,l) sorted by (label rank of neighbour, id)
     uint16_t *cl = nullptr;     // [2m], label rank of ci[p]
+    // label directory of the long lists: for N(v,l) = ci[a..b) with
+    // b - a >= dir_min, dir[(a+1)/2 + r] is the position of its first
+    // neighbour of label rank >= r, r in [0, LV].  dir_min = 2 (LV + 1), so
+    // the lists' entries never overlap; the other entries are unset
+    uint32_t *dir = nullptr;    // [m + 1]
+    uint32_t dir_min = 0;
     uint32_t *sig = nullptr;    // [16 * n], column-first
     // the same signatures grouped by vertex label: gperm holds the vertex ids
     // of each label rank in ascending order, every group padded with -1 to a

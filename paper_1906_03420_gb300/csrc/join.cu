@@ -62,7 +62,7 @@ namespace {
 struct CapStoreProducer {
     const int32_t *M;
     const uint32_t *off;
-    const uint16_t *cl;
+    LabelIndex cl;
     uint32_t *caps;
     uint64_t W;
     StepDev s;
@@ -366,7 +366,7 @@ gsi_status launch_join_scan(const gsi_graph *g, const int32_t *M, uint64_t R, co
                             uint64_t *scratch, cudaStream_t st) {
     // scratch: [scan block sums][per-row bounds as uint32]
     uint32_t *caps = reinterpret_cast<uint32_t *>(scratch + scan_blocks((int64_t)R) + 1);
-    CapStoreProducer p1{M, g->off, g->cl, caps, (uint64_t)JOIN_ROW_WEIGHT, step_dev(g, s)};
+    CapStoreProducer p1{M, g->off, LabelIndex{g->cl, g->dir, g->dir_min}, caps, (uint64_t)JOIN_ROW_WEIGHT, step_dev(g, s)};
     CapLoadProducer p2{caps, (uint64_t)JOIN_ROW_WEIGHT};
     GSI_CUDA_TRY(two_producer_scan(p1, p2, (int64_t)R, StoreWriter<uint64_t>{F}, scratch, st));
     return GSI_OK;
@@ -400,7 +400,7 @@ gsi_status launch_join(const gsi_graph *g, const int32_t *M, uint64_t R, const J
     }
     JoinArgs a;
     a.M = M; a.R = (int64_t)R; a.F = F; a.total = total; a.part = part;
-    a.off = g->off; a.ci = g->ci; a.cl = g->cl; a.cand = cand;
+    a.off = g->off; a.ci = g->ci; a.cl = LabelIndex{g->cl, g->dir, g->dir_min}; a.cand = cand;
     a.out = out; a.out_cap = out_cap; a.out_count = out_count; a.stats = stats;
     a.W = JOIN_ROW_WEIGHT;
     a.rmax = JOIN_NV / JOIN_ROW_WEIGHT + 2;
@@ -432,7 +432,7 @@ JoinArgs make_join_args(const gsi_graph *g, const JoinStep &s, const uint32_t *c
                         unsigned long long *stats) {
     JoinArgs a;
     std::memset(&a, 0, sizeof a);
-    a.off = g->off; a.ci = g->ci; a.cl = g->cl; a.cand = cand;
+    a.off = g->off; a.ci = g->ci; a.cl = LabelIndex{g->cl, g->dir, g->dir_min}; a.cand = cand;
     a.stats = stats;
     a.W = JOIN_ROW_WEIGHT;
     a.rmax = JOIN_NV / JOIN_ROW_WEIGHT + 2;

@@ -283,7 +283,7 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
                 const uint32_t x0 = __ldg(a.off + seg), x1 = __ldg(a.off + seg + 1);
                 for (uint32_t m = mask; m; m &= m - 1) {
                     const int p = __ffs(m) - 1;
-                    if (!ranked_contains(a.ci, a.cl, x0, x1, (uint32_t)a.s.ulab, __ldg(a.ci + lob + (uint32_t)p)))
+                    if (!ranked_contains(a.ci, a.cl.cl, x0, x1, (uint32_t)a.s.ulab, __ldg(a.ci + lob + (uint32_t)p)))
                         mask &= ~(1u << p);
                 }
             }

@@ -7,9 +7,28 @@
 
 namespace gsi {
 
-// [lo, hi) of the entries with label rank `r` inside the (rank, id)-sorted list cl[a..b)
-__device__ inline void label_range(const uint16_t *__restrict__ cl, uint32_t a, uint32_t b, uint32_t r,
-                                   uint32_t *lo, uint32_t *hi) {
+// The label ranks of the lists with the directory of the long ones (see gsi_graph).
+struct LabelIndex {
+    const uint16_t *cl;
+    const uint32_t *dir;
+    uint32_t dir_min;
+};
+
+// [lo, hi) of the entries with label rank `r` inside the (rank, id)-sorted
+// list cl[a..b).  A list of at least dir_min entries is looked up in its
+// directory: two adjacent words instead of log2(b - a) dependent probes, the
+// first of which are misses (a 10^4-entry hub list cost about 5 us that way).
+// Below dir_min the list's label ranks span a few cache lines and the search
+// stays in L1.
+__device__ inline void label_range(const LabelIndex &x, uint32_t a, uint32_t b, uint32_t r, uint32_t *lo,
+                                   uint32_t *hi) {
+    if (b - a >= x.dir_min) {
+        const uint32_t *p = x.dir + ((a + 1) >> 1) + r;
+        *lo = __ldg(p);
+        *hi = __ldg(p + 1);
+        return;
+    }
+    const uint16_t *__restrict__ cl = x.cl;
     // the two bounds searched in lockstep: each round issues both probes,
     // so the chain of dependent loads is as long as one search
     uint32_t l1 = a, h1 = b, l2 = a, h2 = b;
@@ -44,7 +63,7 @@ struct StepDev {
 // one-launch-per-query and batched kernels reuse their table regions), so it
 // is read through L2 (ld.global.cg), never through the read-only path.
 __device__ inline uint32_t row_bound(const StepDev &s, const int32_t *row, const uint32_t *__restrict__ off,
-                                     const uint16_t *__restrict__ cl) {
+                                     const LabelIndex &cl) {
     uint32_t best = 0xffffffffu;
     for (int j = 0; j < s.d; ++j) {
         uint64_t seg = (uint64_t)(uint32_t)__ldcg(row + s.col[j]) * (uint64_t)s.L + (uint64_t)s.lab[j];
@@ -60,32 +79,6 @@ __device__ inline uint32_t row_bound(const StepDev &s, const int32_t *row, const
 // 27 bits, the index of its linking edge above (lists stay below 2^27).
 constexpr uint32_t BOUND_LEN_BITS = 27;
 constexpr uint32_t BOUND_LEN_MASK = (1u << BOUND_LEN_BITS) - 1;
-
-// row_bound plus where the shortest sub-list starts and which linking edge
-// gives it (the join tile then stages the row without searching again), and
-// the summed length of all sub-lists.
-__device__ inline uint32_t row_bound_full(const StepDev &s, const int32_t *row, const uint32_t *__restrict__ off,
-                                          const uint16_t *__restrict__ cl, uint32_t *lo_best, int *jb,
-                                          uint64_t *lsum) {
-    uint32_t best = 0xffffffffu, bl = 0;
-    int bj = 0;
-    uint64_t sum = 0;
-    for (int j = 0; j < s.d; ++j) {
-        uint64_t seg = (uint64_t)(uint32_t)__ldcg(row + s.col[j]) * (uint64_t)s.L + (uint64_t)s.lab[j];
-        uint32_t a = __ldg(off + seg), b = __ldg(off + seg + 1), lo, hi;
-        label_range(cl, a, b, (uint32_t)s.ulab, &lo, &hi);
-        if (hi - lo < best) {
-            best = hi - lo;
-            bl = lo;
-            bj = j;
-        }
-        sum += hi - lo;
-    }
-    *lo_best = bl;
-    *jb = bj;
-    *lsum = sum;
-    return best;
-}
 
 // Membership of x (label rank r) in a whole list ci[a..b), sorted by
 // (label rank, id): binary search on the pair.
@@ -127,7 +120,7 @@ struct JoinArgs {
     const int64_t *part;
     const uint32_t *off;
     const int32_t *ci;
-    const uint16_t *cl;
+    LabelIndex cl;
     const uint32_t *cand;
     int32_t *out;
     uint64_t out_cap;
