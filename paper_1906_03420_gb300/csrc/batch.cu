@@ -5,7 +5,7 @@
 // seeds its table with the set bits of its word range and runs the query's
 // join steps on those rows depth-first inside its own slice of the batch
 // arena (a scratch region and two table regions used in turn), with CTA-local
-// scans and survivor counters.  When a step leaves more than split_rows rows
+// long-row tables and survivor counters.  When a step leaves more than split_rows rows
 // and steps remain, the CTA keeps the first split_rows rows and moves the
 // rest, in pieces of split_rows rows, to a spill area and a spill queue; any
 // CTA continues such a piece from the next step.  Idle CTAs take spill units
@@ -31,7 +31,6 @@
 namespace gsi {
 namespace {
 
-constexpr int BVT = JOIN_VT;
 constexpr uint64_t SPILL_SLOTS = 1ull << 18;                  // spill queue capacity (units)
 constexpr unsigned long long WAIT_SPIN_LIMIT = 1ull << 26;    // x ~100 ns sleeps: several seconds
 constexpr long long UNIT_DONE = -(1ll << 62);
@@ -152,11 +151,11 @@ __device__ __forceinline__ void discard_l2(const void *p, uint64_t bytes) {
 // the row pass (the batched autotuner picks one).
 template <int NT, int RPT>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__ BatchArgs b) {
-    constexpr int BNT = NT, BNV = NT * BVT;
+    constexpr int BNT = NT;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wt[BNT / 32];
     __shared__ long long unit_s;
-    __shared__ unsigned long long cnt_s, lcnt_s, off_s, slot_s;
+    __shared__ unsigned long long cnt_s, lctr_s, off_s, slot_s;
     __shared__ unsigned rfail_s;
     __shared__ int fail_s, skip_s;
     __shared__ __align__(16) JoinArgs a_s;
@@ -165,7 +164,6 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
     int32_t *reg[2] = {reinterpret_cast<int32_t *>(slice + b.s_bytes),
                        reinterpret_cast<int32_t *>(slice + b.s_bytes + b.t_bytes)};
     const uint64_t S_words = b.s_bytes / 8;
-    const uint64_t W = (uint64_t)JOIN_ROW_WEIGHT;
     BatchCtl *c = b.ctl;
     int32_t *const result = c->result;
     const unsigned long long result_cap = c->result_cap;
@@ -230,24 +228,17 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             const bool last = t == k - 1;
             cap = b.t_bytes / (4ull * (uint64_t)(t + 1));
             if (last && bq->count_only) cap = 0;
-            // long rows (bound above SHORT_MAX) and their slot offsets in the scratch region
-            const LongLayout ll = long_layout(S_words, t);
-            LongTable lt;
-            lt.rows = reinterpret_cast<int32_t *>(S);
-            lt.bnd = reinterpret_cast<uint32_t *>(lt.rows + ll.cap * (uint64_t)t);
-            lt.blo = lt.bnd + ll.cap;
-            lt.cap = ll.cap;
-            lt.count = &lcnt_s;
-            uint64_t *F = S + ll.f_off;
+            // long rows (bound above SHORT_MAX) in the scratch region
+            const LongTable lt = long_table(S, S_words, t, R, &lctr_s);
             if (threadIdx.x == 0) {
                 cnt_s = 0;
-                lcnt_s = 0;
+                lctr_s = 0;
                 rfail_s = 0;
             }
             __syncthreads();
             // short rows joined inline, long rows set aside
             unsigned long long abytes = 0, items = 0, lbytes = 0;
-            row_pass<BNT, true, RPT, false>(a, M, R, 0, (uint64_t)BNT * RPT, out, cap, &cnt_s, lt, &rfail_s, smem,
+            row_pass<BNT, true, RPT, false>(a, M, R, 0, (uint64_t)BNT * RPT, BNT * RPT, out, cap, &cnt_s, lt, &rfail_s, smem,
                                             &abytes, &items, &lbytes);
             if (a.stats) {                       // one add per step of a unit
                 abytes = block_sum<BNT, unsigned long long>(abytes, wt);
@@ -261,37 +252,11 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             }
             __syncthreads();
             if (rfail_s) { failed = true; break; }     // long-row table full: the plain path
-            const uint64_t L = lcnt_s;
+            const uint64_t L = lctr_s & ((1ull << lt.rbits) - 1ull), total = lctr_s >> lt.rbits;
             if (L > 0) {
-                // the long rows through the candidate-slot tiles, CTA-local
-                unsigned long long run = 0;
-                for (uint64_t base = 0; base < L; base += BNT) {
-                    const uint64_t i = base + threadIdx.x;
-                    const unsigned long long v =
-                        i < L ? (unsigned long long)(lt.bnd[i] & BOUND_LEN_MASK) + W : 0ull;
-                    unsigned long long tot;
-                    const unsigned long long ex = block_exclusive_scan<BNT, unsigned long long>(v, wt, &tot) + run;
-                    if (i < L) F[i] = ex;
-                    run += tot;
-                }
-                const uint64_t total = run;
-                if (threadIdx.x == 0) F[L] = total;
-                __syncthreads();
-                // tiles in order; each tile spans at most BNV/W + 1 rows past its first
-                const uint64_t ntiles = (total + BNV - 1) / BNV;
-                int64_t r_lo = 0;
-                const uint64_t span = BNV / W + 1;
-                for (uint64_t tile = 0; tile < ntiles; ++tile) {
-                    const uint64_t s_next = min((tile + 1) * (uint64_t)BNV, total);
-                    const uint64_t lim = min(L - (uint64_t)r_lo, span);
-                    unsigned long long cn = 0;
-                    for (uint64_t j = threadIdx.x; j <= lim; j += BNT) cn += F[r_lo + j] <= s_next;
-                    cn = block_sum<BNT, unsigned long long>(cn, wt);
-                    const int64_t r_next = r_lo + (int64_t)cn - 1;
-                    join_tile<BNT, BVT, false, true>(a, lt.rows, (int64_t)L, F, total, r_lo, r_next, out, cap, &cnt_s,
-                                                     tile, lt.bnd, lt.blo);
-                    r_lo = r_next;
-                }
+                // the long rows' slot tiles, CTA-local
+                const unsigned warp = threadIdx.x >> 5;
+                long_rows_join(a, lt, L, total, warp, BNT / 32, out, cap, &cnt_s, smem + warp * long_warp_smem(t, a.s.d));
             }
             __syncthreads();
             discard_l2<BNT>(M, R * (uint64_t)t * 4);    // this step's input is dead
@@ -443,12 +408,12 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     if (stats) {
         GSI_CUDA_TRY(cudaMallocAsync(&L.dstats, 24, st));
     }
-    size_t sm = join_smem(LONG_RMAX, 1, 1);
+    size_t sm = long_warp_smem(1, 1) * (size_t)(L.nt / 32);
     for (int i = 0; i < nq; ++i) {
         BatchPlan &p = plans[i];
         if (!p.active) continue;
         for (int t = 1; t < p.k; ++t) {
-            sm = std::max(sm, join_smem(LONG_RMAX, p.steps[t].t, p.steps[t].d));
+            sm = std::max(sm, long_warp_smem(p.steps[t].t, p.steps[t].d) * (size_t)(L.nt / 32));
             sm = std::max(sm, rows_smem(L.nt, p.steps[t].t, L.rpt));
         }
     }
@@ -506,7 +471,6 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
             cfg[(size_t)bqs[i].cfg0 + t] =
                 make_join_args(g, p.steps[t], p.bitmaps + (uint64_t)p.order[t] * (uint64_t)g->nwords, co, L.dstats);
             cfg[(size_t)bqs[i].cfg0 + t].isect = o.isect;
-            cfg[(size_t)bqs[i].cfg0 + t].rmax = LONG_RMAX;     // its tiles see long rows only
         }
         // word ranges of the seed bitmap holding about seeds_per_item seeds each
         const uint64_t nw = (uint64_t)g->nwords;

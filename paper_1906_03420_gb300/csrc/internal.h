@@ -123,21 +123,21 @@ inline uint64_t join_tiles(uint64_t total) { return (total + JOIN_NV - 1) / JOIN
 
 // One join step of a cooperative query launch (see join.cu): the host sets
 // the regions, the device the sizes.
-struct DStep {
-    // set by the host
+struct DStepIn {                       // set by the host
     const int32_t *M;                  // input table (t columns)
     int32_t *out;                      // output table region
     uint64_t out_bytes;                // bytes of the output region
     uint64_t row_cap;                  // output rows allowed (0 = no limit)
-    uint64_t *S;                       // scratch region: the long-row table (rows, bound
-                                       // records), its slot offsets F and tile partition
+    uint64_t *S;                       // scratch region: the long-row table
     uint64_t S_words;
     int32_t t, count_only;
+};
+struct DStep {
+    DStepIn in;
     // set on the device
     unsigned long long count;          // survivors (exact even past out_cap); [0]: seed size
-    unsigned long long next_tile;
-    unsigned long long nlong;          // rows set aside for the slot tiles (bound above SHORT_MAX)
-    uint64_t R, total, ntiles, out_cap;
+    unsigned long long nlong;          // rows set aside for the slot tiles and their slots (LongTable::ctr)
+    uint64_t out_cap;
 };
 
 // Grid-barrier and status words of one cooperative query launch.
@@ -159,8 +159,7 @@ gsi_status selftest_barrier_timeout(int dev, unsigned long long spin_limit, doub
 // (join_args_size() * k bytes) to cfg_host and returns the dynamic shared
 // memory the launch needs; the caller uploads them to cfg_dev together with
 // the k step records (host-initialised static fields) and the zeroed control
-// words.  launch_query_coop then launches; bsum: QUERY_MAX_CTAS words.
-// steps[0].count receives |seed|.
+// words.  launch_query_coop then launches; steps[0].count receives |seed|.
 // memo: query_memo_tables(steps, k) tables of n 8-byte entries, zeroed before
 // the launch (per-vertex label sub-list locations, see join_rows.cuh), or null.
 int query_memo_tables(const std::vector<JoinStep> &steps, int k);
@@ -171,7 +170,7 @@ gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &s
 // warp groups, no memo).  listwise (launch): the kernel variant that also
 // counts whole-list bytes (stats[2]).
 gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bitmap, size_t smem, void *cfg_dev,
-                             DStep *dsteps, QueryCtl *ctl, unsigned long long *bsum, int *grid_out, bool listwise,
+                             DStep *dsteps, QueryCtl *ctl, int *grid_out, bool listwise,
                              cudaStream_t stream);
 
 }  // namespace gsi

@@ -9,10 +9,9 @@
 //   3. join   the fused kernel: one CTA per tile of NV slots.
 //
 // Device-driven (k_query): the seed and every iteration of one query in one
-// cooperative launch, the same three phases separated by bounded grid
-// barriers, tiles taken from a counter.  Its bound scan also keeps each row's
-// shortest sub-list (start, length, linking edge), so the join tiles stage
-// rows without searching again.
+// cooperative launch: per step the row pass (join_rows.cuh), which joins short
+// rows and sets long ones aside with their slot offsets, and the long rows'
+// slot tiles, with a bounded grid barrier after each.
 //
 // Output bound.  Every neighbour list N(v,l) is stored sorted by (label rank
 // of the neighbour, neighbour id), so the neighbours of v via l that carry
@@ -115,8 +114,8 @@ __global__ void __launch_bounds__(NT) k_join(const __grid_constant__ JoinArgs a)
 
 // ------------------------------------------------- one launch per query
 // The whole join of one query in a single cooperative launch: the seed, then
-// for every step the bound scan, the tile partition and the join tiles, with
-// a grid barrier between phases.  All CTAs are co-resident (cooperative
+// for every step the row pass and, when it set rows aside, the long rows'
+// tiles, with a grid barrier after each.  All CTAs are co-resident (cooperative
 // launch), so the barrier is a counter and a generation word; every wait is
 // bounded, and a CTA that gives up sets an error bit and returns, as does
 // every CTA that later sees the bit, so the kernel always terminates.
@@ -157,158 +156,74 @@ __device__ __forceinline__ bool grid_barrier(QueryCtl *ctl, unsigned nblocks) {
     return ok_s != 0;
 }
 
-// Sum of v over this CTA's predecessors (j < blockIdx.x) and over all CTAs.
-__device__ __forceinline__ void cta_prefix(const unsigned long long *bsum, unsigned nblocks, unsigned long long *wt,
-                                           unsigned long long *pre, unsigned long long *tot) {
-    unsigned long long p = 0, q = 0;
-    for (unsigned j = threadIdx.x; j < nblocks; j += blockDim.x) {
-        const unsigned long long v = __ldcg(bsum + j);
-        q += v;
-        if (j < blockIdx.x) p += v;
-    }
-    *pre = block_sum<JOIN_NT, unsigned long long>(p, wt);
-    *tot = block_sum<JOIN_NT, unsigned long long>(q, wt);
+// Copies a struct of 4-byte words with the whole CTA.
+template <int NT, typename T>
+__device__ __forceinline__ void copy_words(T *dst, const T *src) {
+    static_assert(sizeof(T) % 4 == 0, "whole words");
+    for (int i = threadIdx.x; i < (int)(sizeof(T) / 4); i += NT)
+        reinterpret_cast<uint32_t *>(dst)[i] = reinterpret_cast<const uint32_t *>(src)[i];
 }
 
-// The long rows of a step (bound above SHORT_MAX) through the candidate-slot
-// tiles: per-CTA slot sums, slot offsets F, the first row of every tile, then
-// the tiles dealt round-robin over the CTAs, with a grid barrier after each
-// phase.  Survivors
-// join those of the row pass in st->out.  False when a barrier wait gave up
-// or the partition does not fit (fail bit 1).
-template <int NT, int VT>
-__device__ __forceinline__ bool long_rows_join(const JoinArgs &a, DStep *st, QueryCtl *ctl, const LongTable &lt,
-                                               uint64_t L, uint64_t *F, int64_t *part, uint64_t part_cap,
-                                               uint64_t cap, unsigned long long *bsum, unsigned long long *wt) {
-    constexpr int NV = NT * VT;
-    const unsigned G = gridDim.x;
-    const uint64_t W = (uint64_t)JOIN_ROW_WEIGHT;
-    unsigned long long pre, tot;
-    // slots of each long row: its bound plus W staging slots; per-CTA sums
-    const uint64_t per = (L + G - 1) / G;
-    const uint64_t chunk = (per + SCAN_NV - 1) / SCAN_NV * SCAN_NV;
-    const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = min(L, lo + chunk);
-    unsigned long long sum = 0;
-    for (uint64_t i = lo + threadIdx.x; i < hi; i += NT) sum += (unsigned long long)(__ldcg(lt.bnd + i) & BOUND_LEN_MASK) + W;
-    sum = block_sum<NT, unsigned long long>(sum, wt);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = sum;
-    if (!grid_barrier(ctl, G)) return false;
-    // slot offsets F over the long rows
-    cta_prefix(bsum, G, wt, &pre, &tot);
-    const uint64_t total = tot;
-    const uint64_t ntiles = (total + NV - 1) / NV;
-    if (ntiles + 1 > part_cap) {
-        if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->fail, 1u);
-        return false;
-    }
-    {
-        unsigned long long run = pre;
-        for (uint64_t base = lo; base < hi; base += NT) {
-            const uint64_t i = base + threadIdx.x;
-            const unsigned long long v = i < hi ? (unsigned long long)(__ldcg(lt.bnd + i) & BOUND_LEN_MASK) + W : 0ull;
-            unsigned long long t2;
-            const unsigned long long ex = block_exclusive_scan<NT, unsigned long long>(v, wt, &t2) + run;
-            if (i < hi) F[i] = ex;
-            run += t2;
-        }
-    }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        F[L] = total;
-        st->total = total;
-        st->ntiles = ntiles;
-    }
-    if (!grid_barrier(ctl, G)) return false;
-    // first long row of every tile
-    for (uint64_t b = (uint64_t)blockIdx.x * NT + threadIdx.x; b <= ntiles; b += (uint64_t)G * NT) {
-        const uint64_t sl = min(b * (uint64_t)NV, total);
-        int64_t l2 = 0, h2 = (int64_t)L;
-        while (l2 < h2) {
-            int64_t mid = (l2 + h2 + 1) >> 1;
-            if (__ldcg(F + mid) <= sl) l2 = mid;
-            else h2 = mid - 1;
-        }
-        part[b] = l2;
-    }
-    if (!grid_barrier(ctl, G)) return false;
-    // the join tiles, dealt round-robin: every tile holds the same number of
-    // candidate slots, so no counter is needed to balance them
-    for (uint64_t tile = blockIdx.x; tile < ntiles; tile += G) {
-        __syncthreads();                  // the previous tile's readers of shared memory are done
-        join_tile<NT, VT, false, true>(a, lt.rows, (int64_t)L, F, total, __ldcg(part + tile), __ldcg(part + tile + 1),
-                                       st->out, cap, &st->count, tile, lt.bnd, lt.blo);
-    }
-    return grid_barrier(ctl, G);
-}
-
-template <int NT, int VT, bool LW>
+template <int NT, bool LW>
 __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cfgs, DStep *steps, int k, QueryCtl *ctl,
-                                              const uint32_t *__restrict__ seed_bitmap, int64_t nwords,
-                                              unsigned long long *bsum) {
+                                              const uint32_t *__restrict__ seed_bitmap, int64_t nwords) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wt[NT / 32];
-    __shared__ __align__(16) JoinArgs a_s;
+    __shared__ unsigned long long at_s;
+    __shared__ __align__(16) JoinArgs args_s[2];      // this step's configuration and the next one's
+    __shared__ __align__(16) DStepIn ins_s[2];
     const unsigned G = gridDim.x;
-    unsigned long long pre, tot;
+    copy_words<NT>(&args_s[1], cfgs + 1);
+    copy_words<NT>(&ins_s[1], &steps[1].in);
 
-    // ---- seed: C(u_first) as the one-column table in the first region (Alg. 2)
-    int32_t *seed_out = const_cast<int32_t *>(steps[1].M);
+    // ---- seed: C(u_first) as the one-column table in the first region (Alg.
+    // 2).  Each CTA lists the set bits of an equal share of the words, at a
+    // place that one atomic reserves (the order of rows is free): one read of
+    // the bitmap and one grid barrier.
     {
-        const uint64_t per = ((uint64_t)nwords + G - 1) / G;
-        const uint64_t chunk = (per + SCAN_NV - 1) / SCAN_NV * SCAN_NV;
+        int32_t *seed_out = const_cast<int32_t *>(steps[1].in.M);
+        const uint64_t chunk = (((uint64_t)nwords + G - 1) / G + 31) & ~31ull;
         const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = min((uint64_t)nwords, lo + chunk);
-        unsigned long long c = 0;
-        for (uint64_t i = lo + threadIdx.x; i < hi; i += NT) c += __popc(seed_bitmap[i]);
-        c = block_sum<NT, unsigned long long>(c, wt);
-        if (threadIdx.x == 0) bsum[blockIdx.x] = c;
-        if (!grid_barrier(ctl, G)) return;
-        cta_prefix(bsum, G, wt, &pre, &tot);
-        unsigned long long run = pre;
         for (uint64_t base = lo; base < hi; base += NT) {
             const uint64_t i = base + threadIdx.x;
-            const uint32_t b = i < hi ? seed_bitmap[i] : 0u;
-            unsigned long long t2;
-            unsigned long long pos = block_exclusive_scan<NT, unsigned long long>(__popc(b), wt, &t2) + run;
-            uint32_t x = b;
-            while (x) {
-                seed_out[pos++] = (int32_t)(i * 32 + (uint64_t)(__ffs(x) - 1));
-                x &= x - 1;
-            }
-            run += t2;
+            uint32_t x = i < hi ? seed_bitmap[i] : 0u;
+            unsigned long long tot;
+            unsigned long long pos = block_exclusive_scan<NT, unsigned long long>(__popc(x), wt, &tot);
+            if (tot == 0) continue;
+            if (threadIdx.x == 0) at_s = atomicAdd(&steps[0].count, tot);
+            __syncthreads();
+            for (pos += at_s; x; x &= x - 1) seed_out[pos++] = (int32_t)(i * 32 + (uint64_t)(__ffs(x) - 1));
+            __syncthreads();
         }
-        if (blockIdx.x == 0 && threadIdx.x == 0) steps[0].count = tot;
         if (!grid_barrier(ctl, G)) return;
     }
 
     for (int t = 1; t < k; ++t) {
         DStep *st = steps + t;
-        {   // this step's configuration, once per CTA, in shared memory
-            const uint32_t *src = reinterpret_cast<const uint32_t *>(cfgs + t);
-            uint32_t *dst = reinterpret_cast<uint32_t *>(&a_s);
-            for (int i = threadIdx.x; i < (int)(sizeof(JoinArgs) / 4); i += NT) dst[i] = src[i];
-        }
-        const JoinArgs &a = a_s;
+        const JoinArgs &a = args_s[t & 1];
+        const DStepIn &in_s = ins_s[t & 1];
         const uint64_t R = __ldcg(&steps[t - 1].count);
         // the previous table must have fit its region
         if (t > 1 && R > __ldcg(&steps[t - 1].out_cap)) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->fail, 2u);
             return;
         }
-        const LongLayout ll = long_layout(st->S_words, t);
-        LongTable lt;
-        lt.rows = reinterpret_cast<int32_t *>(st->S);
-        lt.bnd = reinterpret_cast<uint32_t *>(lt.rows + ll.cap * (uint64_t)t);
-        lt.blo = lt.bnd + ll.cap;
-        lt.cap = ll.cap;
-        lt.count = &st->nlong;
-        uint64_t cap = st->out_bytes / (4ull * (uint64_t)(t + 1));
-        if (st->row_cap && st->row_cap < cap) cap = st->row_cap;
-        if (st->count_only) cap = 0;
+        if (R == 0) return;                                   // no embeddings: the counts stay zero
+        if (t + 1 < k) {                                      // read behind this step's barriers
+            copy_words<NT>(&args_s[(t + 1) & 1], cfgs + t + 1);
+            copy_words<NT>(&ins_s[(t + 1) & 1], &steps[t + 1].in);
+        }
+        const LongTable lt = long_table(in_s.S, in_s.S_words, t, R, &st->nlong);
+        int32_t *const out = in_s.out;
+        uint64_t cap = in_s.out_bytes / (4ull * (uint64_t)(t + 1));
+        if (in_s.row_cap && in_s.row_cap < cap) cap = in_s.row_cap;
+        if (in_s.count_only) cap = 0;
         if (blockIdx.x == 0 && threadIdx.x == 0) st->out_cap = cap;
-        __syncthreads();
         // ---- short rows joined inline, long rows set aside (one pass over M)
         unsigned long long abytes = 0, items = 0, lbytes = 0;
-        row_pass<NT, true, ROW_RPT, LW>(a, st->M, R, (uint64_t)blockIdx.x * NT * ROW_RPT, (uint64_t)G * NT * ROW_RPT,
-                                        st->out, cap, &st->count, lt, &ctl->fail, smem, &abytes, &items, &lbytes);
+        const int nb = batch_rows(R, G, NT * ROW_RPT);
+        row_pass<NT, true, ROW_RPT, LW>(a, in_s.M, R, (uint64_t)blockIdx.x * nb, (uint64_t)G * nb, nb, out, cap,
+                                        &st->count, lt, &ctl->fail, smem, &abytes, &items, &lbytes);
         if (a.stats) {                       // one add per CTA and step
             abytes = block_sum<NT, unsigned long long>(abytes, wt);
             items = block_sum<NT, unsigned long long>(items, wt);
@@ -322,11 +237,14 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         if (!grid_barrier(ctl, G)) return;
         if (__ldcg(&ctl->fail) & 1u) return;                  // long-row table full: a larger arena
         // ---- long rows through the candidate-slot tiles
-        const uint64_t L = __ldcg(lt.count);
-        if (L > 0 && !long_rows_join<NT, VT>(a, st, ctl, lt, L, st->S + ll.f_off,
-                                             reinterpret_cast<int64_t *>(st->S + ll.part_off), ll.part_cap, cap,
-                                             bsum, wt))
-            return;
+        const uint64_t ctr = __ldcg(&st->nlong), L = ctr & ((1ull << lt.rbits) - 1ull), total = ctr >> lt.rbits;
+        if (L > 0) {
+            const unsigned warp = threadIdx.x >> 5;
+            // neighbouring runs of slots go to different SMs
+            long_rows_join(a, lt, L, total, (uint64_t)warp * G + blockIdx.x, (uint64_t)G * (NT / 32), out, cap, &st->count,
+                           smem + warp * long_warp_smem(t, a.s.d));
+            if (!grid_barrier(ctl, G)) return;
+        }
         if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) {      // survivors written (both models)
             const unsigned long long wbytes = 4ull * (uint64_t)(t + 1) * min((uint64_t)__ldcg(&st->count), cap);
             atomicAdd(a.stats, wbytes);
@@ -463,8 +381,7 @@ gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &s
         cfg[t].memo = nodedup ? nullptr : memo;
         cfg[t].memo_n = g->n;
         cfg[t].nodedup = nodedup ? 1 : 0;
-        cfg[t].rmax = LONG_RMAX;             // the tiles of k_query see long rows only
-        sm = std::max(sm, join_smem(cfg[t].rmax, steps[t].t, steps[t].d));
+        sm = std::max(sm, long_warp_smem(steps[t].t, steps[t].d) * (JOIN_NT / 32));
         sm = std::max(sm, rows_smem(JOIN_NT, steps[t].t));
     }
     if (sm > 200 * 1024) {
@@ -476,11 +393,11 @@ gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &s
 }
 
 gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bitmap, size_t sm, void *cfg_dev,
-                             DStep *dsteps, QueryCtl *ctl, unsigned long long *bsum, int *grid_out, bool listwise,
+                             DStep *dsteps, QueryCtl *ctl, int *grid_out, bool listwise,
                              cudaStream_t st) {
     // the variant that also counts whole-list bytes costs registers: only on request
-    const void *kern = listwise ? (const void *)k_query<JOIN_NT, JOIN_VT, true>
-                                : (const void *)k_query<JOIN_NT, JOIN_VT, false>;
+    const void *kern = listwise ? (const void *)k_query<JOIN_NT, true>
+                                : (const void *)k_query<JOIN_NT, false>;
     int dev = 0;
     cudaGetDevice(&dev);
     // occupancy depends only on the dynamic shared memory: looked up once per
@@ -492,9 +409,9 @@ gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bit
     {
         std::lock_guard<std::mutex> lk(mu);
         if (dev >= 0 && dev < 64 && !nsm[dev]) {
-            GSI_CUDA_TRY(cudaFuncSetAttribute(k_query<JOIN_NT, JOIN_VT, false>,
+            GSI_CUDA_TRY(cudaFuncSetAttribute(k_query<JOIN_NT, false>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
-            GSI_CUDA_TRY(cudaFuncSetAttribute(k_query<JOIN_NT, JOIN_VT, true>,
+            GSI_CUDA_TRY(cudaFuncSetAttribute(k_query<JOIN_NT, true>,
                                               cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024));
             GSI_CUDA_TRY(cudaDeviceGetAttribute(&nsm[dev], cudaDevAttrMultiProcessorCount, dev));
         }
@@ -516,8 +433,7 @@ gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bit
     *grid_out = grid;
     const JoinArgs *cfgp = static_cast<const JoinArgs *>(cfg_dev);
     int64_t nwords = g->nwords;
-    void *args[] = {(void *)&cfgp, (void *)&dsteps, (void *)&k, (void *)&ctl, (void *)&seed_bitmap, (void *)&nwords,
-                    (void *)&bsum};
+    void *args[] = {(void *)&cfgp, (void *)&dsteps, (void *)&k, (void *)&ctl, (void *)&seed_bitmap, (void *)&nwords};
     GSI_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(JOIN_NT), args, sm, st));
     return GSI_OK;
 }

@@ -14,10 +14,11 @@
 //     (bitmap of C(u), set subtraction against the row, membership in the
 //     other linking lists: Alg. 3's set operations) and keeps a bit mask of
 //     survivors;
-//   * otherwise the row, with its bound record (length, linking edge, start),
-//     is appended to a long-row table that the slot tiles process after a
-//     grid barrier (a hub row then spreads over many CTAs, Sec. VI-A's load
-//     balancing done by the tiles);
+//   * otherwise the row, with its bound record (length, linking edge, start)
+//     and its place among the step's candidate slots, is appended to a
+//     long-row table that the slot tiles process after a grid barrier (a hub
+//     row then spreads over many warps, Sec. VI-A's load balancing done by the
+//     tiles);
 //   * one block-wide scan and one atomic per CTA and batch place the batch's
 //     survivors in M', which the CTA writes as one coalesced run
 //     (Prealloc-Combine without a second join: each survivor is written
@@ -45,35 +46,40 @@
 namespace gsi {
 
 constexpr int SHORT_MAX = 16;     // rows with at most this many candidates are joined inline
-// Rows of one slot tile of long rows: every long row spans at least
-// SHORT_MAX + 1 + W slots, plus a partial row at each end of the tile.
-constexpr int LONG_RMAX = JOIN_NV / (SHORT_MAX + 1 + JOIN_ROW_WEIGHT) + 2;
 
 // Rows whose bound exceeds SHORT_MAX, copied (t columns) with their bound
-// records, for the slot tiles.  count is a device counter.
+// records, for the slot tiles.  Their candidates are slots of a flat index
+// space: row i's begin at F[i], the sum of the earlier rows' lengths.  A CTA
+// that sets rows aside reserves their places in the table and in the slot
+// space with one atomic add on `ctr`, rows in the low rbits bits and slots
+// above them, so that F ascends with the row index and is written with the
+// row: no scan over the table, no pass that cuts it into tiles, and no grid
+// barriers between them (they cost 14-20 us a step, more than the join of most
+// steps).  rbits holds the step's row count; a step whose slots do not fit the
+// other bits fails like one whose table is full.
 struct LongTable {
     int32_t *rows;
+    uint64_t *F;
     uint32_t *bnd;                // length | linking edge << BOUND_LEN_BITS
     uint32_t *blo;                // start of the shortest sub-list
     uint64_t cap;                 // rows the table holds
-    unsigned long long *count;
+    unsigned long long *ctr;
+    int rbits;
 };
 
-// Layout of the long-row table of step t in a scratch region of S_words
-// 8-byte words: rows, bound records, then F; the tile partition takes what is
-// left (at least an eighth of the region).
-struct LongLayout {
-    uint64_t cap, f_off, part_off, part_cap;    // offsets in words
-};
-__host__ __device__ inline LongLayout long_layout(uint64_t S_words, int t) {
-    LongLayout l;
-    const uint64_t avail = S_words > 64 ? S_words - S_words / 8 - 8 : 0;
-    l.cap = avail * 8 / (4ull * (uint64_t)t + 16ull);
-    const uint64_t rec_words = (l.cap * (4ull * (uint64_t)t + 8ull) + 7) / 8;
-    l.f_off = rec_words;
-    l.part_off = l.f_off + l.cap + 1;
-    l.part_cap = S_words > l.part_off ? S_words - l.part_off : 0;
-    return l;
+// The long-row table of step t, whose input has R rows, in a scratch region of
+// S_words 8-byte words: F, rows, bound records.
+__device__ __forceinline__ LongTable long_table(uint64_t *S, uint64_t S_words, int t, uint64_t R,
+                                                unsigned long long *ctr) {
+    LongTable lt;
+    lt.cap = S_words > 8 ? (S_words - 8) * 8 / (4ull * (uint64_t)t + 16ull) : 0;
+    lt.F = S;
+    lt.rows = reinterpret_cast<int32_t *>(S + lt.cap);
+    lt.bnd = reinterpret_cast<uint32_t *>(lt.rows + lt.cap * (uint64_t)t);
+    lt.blo = lt.bnd + lt.cap;
+    lt.ctr = ctr;
+    lt.rbits = 64 - __clzll((long long)(R | 1));
+    return lt;
 }
 
 constexpr int ROW_RPT = 2;        // rows per thread in one batch of the row pass
@@ -123,6 +129,17 @@ __device__ __forceinline__ void stage_rows(int32_t *dst, const int32_t *__restri
     } else {
         for (int e = threadIdx.x; e < n; e += NT) dst[e] = __ldcg(src + e);
     }
+}
+
+// Rows that one CTA takes at a time when R rows meet G CTAs: all of NB once
+// there are enough rows to fill every CTA, fewer below (a table of 9,000 rows
+// is spread over the whole GPU in pieces of 16, instead of over ten CTAs: a
+// step of so few rows is bound by the latency of one batch, 12-20 us when its
+// threads were all in a few CTAs), in multiples of 8 so that a batch starts on
+// 16 bytes whatever its columns.
+__device__ __forceinline__ int batch_rows(uint64_t R, unsigned G, int NB) {
+    const uint64_t per = (R + G - 1) / G;
+    return per >= (uint64_t)NB ? NB : max(8, ((int)per + 7) & ~7);
 }
 
 // Length of the whole linking list N(v, lab[j]) (for the whole-list byte count).
@@ -392,22 +409,23 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
     }
 }
 
-// The row pass over rows [first, R) in batches of NT * RPT rows, batch
-// starts `stride` apart (a grid-strided pass: first = blockIdx.x * NB,
-// stride = gridDim.x * NB; one CTA alone: first = 0, stride = NB).  `a` should
-// live in shared memory.  Survivors go to out (up to cap rows; `count` is
+// The row pass over rows [first, R) in batches of nbatch <= NT * RPT rows,
+// batch starts `stride` apart (a grid-strided pass: first = blockIdx.x *
+// nbatch, stride = gridDim.x * nbatch; one CTA alone: first = 0, stride =
+// nbatch).  `a` should live in shared memory.  Survivors go to out (up to cap rows; `count` is
 // exact), long rows to lt.  Bit 1 of *fail is set when the long-row table is
 // full or a bound does not fit its record.  When a.stats is set, adds this
 // thread's algorithmic bytes (rows read, lists located and read; survivors
 // are counted by the caller) to *abytes, the same under the whole-list model
 // to *lbytes (only when LW), and its candidate slots to *items.
 template <int NT, bool DR = true, int RPT = ROW_RPT, bool LW = true>
-__device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64_t first, uint64_t stride,
+__device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64_t first, uint64_t stride, int nbatch,
                          int32_t *__restrict__ out, uint64_t cap, unsigned long long *count, const LongTable &lt,
                          unsigned *fail, unsigned char *smem, unsigned long long *abytes,
                          unsigned long long *items, unsigned long long *lbytes) {
     constexpr int NW = NT / 32, NB = NT * RPT, CCAP = NB * ROW_SURV;
     __shared__ uint32_t wt[NW];
+    __shared__ unsigned long long wts[NW];              // slots of each warp's long rows
     __shared__ unsigned long long base_s, lbase_s;
     const int t = a.s.t, W1 = t + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -421,10 +439,10 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
     const int rpw = 32 / W1, rs = lane / W1, oc = lane - rs * W1;
     const int src_col = a.iperm[oc < W1 ? oc : 0];
     for (uint64_t r0 = first; r0 < R; r0 += stride) {
-        const int nb = (int)min((uint64_t)NB, R - r0);
+        const int nb = (int)min((uint64_t)nbatch, R - r0);
         const int32_t *src = M + r0 * (uint64_t)t;
         if (threadIdx.x == 0 && r0 + stride < R)      // the next batch's rows, while this one runs
-            prefetch_l2(M + (r0 + stride) * (uint64_t)t, min((uint64_t)NB, R - r0 - stride) * (uint64_t)t * 4);
+            prefetch_l2(M + (r0 + stride) * (uint64_t)t, min((uint64_t)nbatch, R - r0 - stride) * (uint64_t)t * 4);
         stage_rows<NT>(rowv, src, nb * t);
         __syncthreads();
         // this thread's rows q * NT + tid, q < RPT (a warp's lanes hold
@@ -432,6 +450,7 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
         uint32_t mask[RPT], best[RPT], lob[RPT];
         int jb[RPT];
         uint32_t n = 0, nl = 0;
+        unsigned long long sl = 0;                    // slots of this thread's long rows, then their exclusive prefix
         if (DR && a.s.d == 1 && !a.nodedup) {
             rows_join_single<NT, RPT, LW>(a, rowv, nb, lane, best, lob, mask, abytes, items, lbytes);
 #pragma unroll
@@ -449,11 +468,14 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
 #pragma unroll
         for (int q = 0; q < RPT; ++q) {
             n += __popc(mask[q]);
-            nl += best[q] > (uint32_t)SHORT_MAX;
+            const bool lng = best[q] > (uint32_t)SHORT_MAX;
+            nl += lng;
+            sl += lng ? best[q] : 0u;
         }
         // one barrier: warp scans, warp totals through shared memory (wt is
         // written again only after the next batch's staging barrier)
         uint32_t ex, tot;
+        unsigned long long stot = 0;
         {
             const uint32_t v = n | (nl << 16);
             uint32_t x = v;
@@ -462,9 +484,21 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
                 const uint32_t y = __shfl_up_sync(FULL_MASK, x, o);
                 if (lane >= o) x += y;
             }
-            if (lane == 31) wt[warp] = x;
+            const unsigned long long own = sl;
+            if (__any_sync(FULL_MASK, nl != 0)) {
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const unsigned long long y = __shfl_up_sync(FULL_MASK, sl, o);
+                    if (lane >= o) sl += y;
+                }
+            }
+            if (lane == 31) {
+                wt[warp] = x;
+                wts[warp] = sl;
+            }
             __syncthreads();
             uint32_t pre = 0;
+            unsigned long long spre = 0;
             tot = 0;
 #pragma unroll
             for (int w = 0; w < NW; ++w) {
@@ -473,15 +507,28 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
                 tot += y;
             }
             ex = pre + x - v;
+            if (tot >> 16) {                          // the batch has long rows
+                for (int w = 0; w < NW; ++w) {
+                    const unsigned long long y = wts[w];
+                    spre += w < warp ? y : 0ull;
+                    stot += y;
+                }
+                sl = spre + sl - own;
+            }
         }
         const uint32_t ntot = tot & 0xffffu, ltot = tot >> 16;
         if (threadIdx.x == 0) {                 // read after the next barrier
             base_s = ntot ? atomicAdd(count, (unsigned long long)ntot) : 0ull;
-            lbase_s = ltot ? atomicAdd(lt.count, (unsigned long long)ltot) : 0ull;
+            if (ltot) {
+                const unsigned long long old = atomicAdd(lt.ctr, (stot << lt.rbits) | (unsigned long long)ltot);
+                if ((old >> lt.rbits) + stot >= 1ull << (64 - lt.rbits)) atomicOr(fail, 1u);
+                lbase_s = old;
+            }
         }
         // long rows to the table
         auto copy_long = [&]() {
-            unsigned long long li = lbase_s + (ex >> 16);
+            unsigned long long li = (lbase_s & ((1ull << lt.rbits) - 1ull)) + (ex >> 16);
+            unsigned long long f = (lbase_s >> lt.rbits) + sl;
 #pragma unroll
             for (int q = 0; q < RPT; ++q) {
                 if (best[q] <= (uint32_t)SHORT_MAX) continue;
@@ -491,10 +538,12 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
                     for (int c = 0; c < t; ++c) dst[c] = row[c];
                     lt.bnd[li] = best[q] | ((uint32_t)jb[q] << BOUND_LEN_BITS);
                     lt.blo[li] = lob[q];
+                    lt.F[li] = f;
                 } else {
                     atomicOr(fail, 1u);
                 }
                 ++li;
+                f += best[q];
             }
         };
         if (!write || ntot == 0) {
@@ -572,6 +621,152 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
             }
             __syncthreads();
         }
+    }
+}
+
+// ------------------------------------------------------------- long rows
+// The slot tiles: warp wi of nw takes an equal, contiguous run of the table's
+// slots, in tiles of LW_SLOTS, and works alone: no barrier, no map of the tile
+// in shared memory.  The warp finds its first row with one 32-way search of F
+// and from then on walks the table.  In each tile its lanes
+//   * load the records of the rows that meet the tile (at most LW_ROWS, as
+//     every long row has more than SHORT_MAX slots) and stage their columns;
+//   * find their slots' rows from one 32-bit mask of row starts per group of
+//     32 slots;
+//   * load LW_SLOTS / 32 candidates and then as many bitmap words each, all in
+//     flight together;
+//   * test set subtraction and the other lists (label sub-lists, from the
+//     step's memo or searched), and compact the survivors by ballots.
+// One atomic per tile places the survivors, which the warp writes as one
+// coalesced run.  What bounds it is the latency of the two rounds of loads
+// (candidates, bitmap words) times the warps in flight.  CTA-wide tiles of
+// 1,024 slots with five barriers each did 156 slots per ns on the medium graph
+// (R-MAT 2^20, 16M edges, 64 labels); with these tiles and the table above,
+// eight counting queries there went from 5558 to 4220 us and four large ones
+// (2^22, 64M edges) from 22.2 to 18.1 ms.
+constexpr int LW_SLOTS = 256;
+constexpr int LW_G = LW_SLOTS / 32;
+constexpr int LW_ROWS = LW_SLOTS / (SHORT_MAX + 1) + 2;
+
+// Shared memory of one warp: survivors (value, local row), rows, other lists.
+__host__ __device__ constexpr size_t long_warp_smem(int t, int d) {
+    return ((size_t)LW_SLOTS * 5 + (size_t)LW_ROWS * ((size_t)t * 4 + (size_t)(d - 1) * 8) + 15) / 16 * 16;
+}
+
+__device__ inline void long_rows_join(const JoinArgs &a, const LongTable &lt, uint64_t L, uint64_t total, uint64_t wi,
+                                      uint64_t nw, int32_t *__restrict__ out, uint64_t cap, unsigned long long *count,
+                                      unsigned char *smem) {
+    const int lane = threadIdx.x & 31;
+    const int t = a.s.t, d = a.s.d, dm1 = d - 1, W1 = t + 1;
+    int32_t *sw = reinterpret_cast<int32_t *>(smem);
+    int32_t *rowv = sw + LW_SLOTS;                                   // LW_ROWS * t
+    uint32_t *lst = reinterpret_cast<uint32_t *>(rowv + LW_ROWS * t);   // LW_ROWS * 2 * dm1
+    unsigned char *sr = reinterpret_cast<unsigned char *>(lst + LW_ROWS * 2 * dm1);
+    // small tables: at least 64 slots a warp, so that the search pays
+    const uint64_t per = max((uint64_t)64, ((total + nw - 1) / nw + 31) / 32 * 32);
+    uint64_t s = wi * per;
+    const uint64_t w1 = min(total, s + per);
+    if (s >= w1) return;
+    // the row that holds slot s: the last with F <= s
+    uint64_t r = 0;
+    for (uint64_t hi = L; hi - r > 1;) {
+        const uint64_t step = (hi - r + 31) / 32, p = r + (uint64_t)(lane + 1) * step;
+        const int c = __popc(__ballot_sync(FULL_MASK, p < hi && __ldcg(lt.F + p) <= s));
+        r += (uint64_t)c * step;
+        hi = min(hi, r + step);
+    }
+    const unsigned le = lanemask_lt() | (1u << lane);
+    const int rpw = 32 / W1, rs = lane / W1, oc = lane - rs * W1;
+    const int src_col = a.iperm[oc];
+    unsigned long long found = 0;                     // counting only: this lane's survivors
+    while (s < w1) {
+        const uint64_t e = min(s + (uint64_t)LW_SLOTS, w1);
+        // lane j: the record of row r + j
+        uint64_t Fj = ~0ull;
+        uint32_t len = 0, lo = 0, jb = 0;
+        if (r + (uint64_t)lane < L) {
+            Fj = __ldcg(lt.F + r + lane);
+            const uint32_t b = __ldcg(lt.bnd + r + lane);
+            lo = __ldcg(lt.blo + r + lane);
+            len = b & BOUND_LEN_MASK;
+            jb = b >> BOUND_LEN_BITS;
+        }
+        const int nr = __popc(__ballot_sync(FULL_MASK, Fj < e));
+        {
+            const int32_t *src = lt.rows + r * (uint64_t)t;
+            for (int i = lane; i < nr * t; i += 32) rowv[i] = __ldcg(src + i);
+        }
+        __syncwarp();
+        if (dm1 > 0 && lane < nr) {
+            uint32_t *l = lst + lane * 2 * dm1;
+            for (int j = 0; j < d; ++j) {
+                if (j == (int)jb) continue;
+                l[1] = sublist(a, j, rowv[lane * t + a.s.col[j]], &l[0]);
+                l += 2;
+            }
+        }
+        // the first slot of the row in the tile, and the list position of the
+        // tile's slot 0 (modulo 2^32)
+        const int start = (lane < nr && Fj > s) ? (int)(Fj - s) : 0;
+        const uint32_t base = lo + (uint32_t)(s - Fj);
+        const uint64_t endF = Fj + (uint64_t)len;
+        __syncwarp();
+        int32_t w[LW_G];
+        int row[LW_G];
+        int before = 0;
+#pragma unroll
+        for (int g = 0; g < LW_G; ++g) {
+            const unsigned m = __reduce_or_sync(FULL_MASK, start > 0 && (start >> 5) == g ? 1u << (start & 31) : 0u);
+            row[g] = before + __popc(m & le);
+            before += __popc(m);
+            const uint32_t o = (uint32_t)(g * 32 + lane);
+            const uint32_t cix = __shfl_sync(FULL_MASK, base, row[g]) + o;
+            w[g] = s + o < e ? __ldg(a.ci + cix) : -1;
+        }
+        uint32_t bw[LW_G];
+#pragma unroll
+        for (int g = 0; g < LW_G; ++g) bw[g] = w[g] >= 0 ? __ldg(a.cand + (w[g] >> 5)) : 0u;
+        unsigned ns = 0;
+#pragma unroll
+        for (int g = 0; g < LW_G; ++g) {
+            bool ok = w[g] >= 0 && ((bw[g] >> (w[g] & 31)) & 1u);
+            const int32_t *rv = rowv + row[g] * t;
+            for (uint32_t im = a.s.inj; ok && im; im &= im - 1) ok = rv[__ffs(im) - 1] != w[g];
+            const uint32_t *l = lst + row[g] * 2 * dm1;
+            for (int j = 0; j < dm1 && ok; ++j) ok = sorted_contains(a.ci + l[2 * j], l[2 * j + 1], w[g]);
+            const unsigned b = __ballot_sync(FULL_MASK, ok);
+            if (a.count_only) {
+                found += ok;
+            } else {
+                if (ok) {
+                    const unsigned i = ns + __popc(b & le) - 1;
+                    sw[i] = w[g];
+                    sr[i] = (unsigned char)row[g];
+                }
+                ns += __popc(b);
+            }
+        }
+        if (ns) {
+            unsigned long long at = 0;
+            if (lane == 0) at = atomicAdd(count, (unsigned long long)ns);
+            at = __shfl_sync(FULL_MASK, at, 0);       // also orders the list before its readers
+            __syncwarp();
+            const uint64_t room = cap > at ? cap - at : 0;
+            const unsigned nrow = (unsigned)min((uint64_t)ns, room);
+            int32_t *dst = out + at * (uint64_t)W1;
+            if (rs < rpw)
+                for (unsigned i = (unsigned)rs; i < nrow; i += (unsigned)rpw)
+                    dst[(uint64_t)i * W1 + oc] = src_col == t ? sw[i] : rowv[(int)sr[i] * t + src_col];
+        }
+        // a last row that ends with the tile is done
+        r += (uint64_t)(nr - (__shfl_sync(FULL_MASK, endF, nr - 1) > e ? 1 : 0));
+        s = e;
+        __syncwarp();                                 // the staged rows are free
+    }
+    if (a.count_only) {
+#pragma unroll
+        for (int o = 16; o; o >>= 1) found += __shfl_down_sync(FULL_MASK, found, o);
+        if (lane == 0 && found) atomicAdd(count, found);
     }
 }
 

@@ -1,5 +1,5 @@
-// The candidate-slot tile of a join step, shared by the host-sized launch,
-// the one-launch-per-query kernel and the batched kernel.
+// What the forms of a join step share, and the candidate-slot tile of the
+// host-sized one.
 #pragma once
 
 #include "common.cuh"
@@ -204,28 +204,14 @@ __device__ __forceinline__ uint32_t sublist(const JoinArgs &a, int j, int32_t v,
     return len;
 }
 
-// One tile of NV candidate slots.  The table-dependent inputs (M, R, F,
-// total, part, out, out_cap, out_count) are arguments so that the same code
-// serves host-sized launches (one CTA per tile) and device-sized persistent
-// launches (CTAs take tiles from a counter).  M and F can be rewritten within
-// one persistent launch (ping-pong table regions, one scratch region for
-// every step), so they are read through L2 (ld.global.cg) and never through
-// the non-coherent read-only path.
-//
-// With bounds (PRE: the long rows set aside by the row pass), each row's
-// shortest label sub-list is already known: bnd[r] holds its length and
-// linking-edge index (BOUND_LEN_BITS), blo[r] its start.  Staging then reads
-// those instead of searching, the other linking lists' label(u) sub-lists
-// come from the step's memo (filled by the row pass) or a label-range search,
-// and since every such row spans more than
-// SHORT_MAX + W slots a tile holds few rows, so each slot finds its row by a
-// binary search of the staged offsets instead of a block-wide scan.
-template <int NT, int VT, bool TILE_STATS = true, bool PRE = false>
+// One tile of NV candidate slots of the host-sized step (k_join).  Each row
+// takes W slots before its candidates, which pay for staging it and bound the
+// rows that one tile touches.
+template <int NT, int VT>
 __device__ __forceinline__ void join_tile(const JoinArgs &a, const int32_t *M, int64_t R,
                                           const uint64_t *F, uint64_t total, int64_t r_lo,
                                           int64_t r_next, int32_t *__restrict__ out, uint64_t out_cap,
-                                          unsigned long long *out_count, uint64_t tile,
-                                          const uint32_t *bnd = nullptr, const uint32_t *blo = nullptr) {
+                                          unsigned long long *out_count, uint64_t tile) {
     constexpr int NV = NT * VT;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wt[NT / 32];
@@ -251,8 +237,7 @@ __device__ __forceinline__ void join_tile(const JoinArgs &a, const int32_t *M, i
     const int nr = (int)(r_hi - r_lo + 1);
 
     // ---- stage the tile's rows: values, candidate sub-list, other sub-lists
-    if (!PRE)
-        for (int x = threadIdx.x; x < NV; x += NT) rowmap[x] = 0;
+    for (int x = threadIdx.x; x < NV; x += NT) rowmap[x] = 0;
     for (int lr = threadIdx.x; lr <= nr; lr += NT) Fs[lr] = __ldcg(F + r_lo + lr);
     __syncthreads();
     unsigned long long bytes = 0;
@@ -260,24 +245,6 @@ __device__ __forceinline__ void join_tile(const JoinArgs &a, const int32_t *M, i
         const int32_t *row = M + (r_lo + lr) * (int64_t)t;
         int32_t *rv = rowv + lr * t;
         for (int c = 0; c < t; ++c) rv[c] = __ldcg(row + c);
-        if (PRE) {
-            // the bound scan's record: candidates from the shortest sub-list;
-            // every other linking list restricted to label(u)
-            const uint32_t bw = __ldcg(bnd + r_lo + lr);
-            const uint32_t best = bw & BOUND_LEN_MASK;
-            const int jb = (int)(bw >> BOUND_LEN_BITS);
-            base0[lr] = __ldcg(blo + r_lo + lr);
-            int q = 0;
-            for (int j = 0; j < d && best > 0; ++j) {
-                if (j == jb) continue;
-                uint32_t lo;
-                const uint32_t len = sublist(a, j, rv[a.s.col[j]], &lo);
-                lst[(lr * dm1 + q) * 2] = lo;
-                lst[(lr * dm1 + q) * 2 + 1] = len;
-                ++q;
-            }
-            continue;
-        }
         // the row's lists: the shortest label sub-list supplies candidates
         uint32_t lo[GSI_MAX_QUERY_VERTICES], len[GSI_MAX_QUERY_VERTICES];
         uint32_t best = 0xffffffffu;
@@ -302,10 +269,10 @@ __device__ __forceinline__ void join_tile(const JoinArgs &a, const int32_t *M, i
         }
         const uint64_t fr = Fs[lr];
         if (fr > s0 && fr < s1) rowmap[fr - s0] = (uint16_t)lr;       // first slot of the row in this tile
-        if (TILE_STATS && a.stats && fr >= s0) bytes += 4ull * t + 8ull * d + 4ull * (lsum - best);   // row owned by this tile
+        if (a.stats && fr >= s0) bytes += 4ull * t + 8ull * d + 4ull * (lsum - best);   // row owned by this tile
     }
     __syncthreads();
-    if (!PRE) {   // slot -> row: inclusive max-scan of the row-start marks
+    {   // slot -> row: inclusive max-scan of the row-start marks
         int v[VT];
         int m = 0;
 #pragma unroll
@@ -344,20 +311,7 @@ __device__ __forceinline__ void join_tile(const JoinArgs &a, const int32_t *M, i
         lrv[k] = 0;
         cix[k] = 0;
         if (s >= s1) continue;
-        int lr;
-        if (PRE) {
-            // long rows only (each holds more than SHORT_MAX + W slots): few
-            // rows per tile, found by a search of the staged offsets
-            int l = 0, h = nr - 1;
-            while (l < h) {
-                const int mid = (l + h + 1) >> 1;
-                if (Fs[mid] <= s) l = mid;
-                else h = mid - 1;
-            }
-            lr = l;
-        } else {
-            lr = rowmap[s - s0];
-        }
+        const int lr = rowmap[s - s0];
         const int64_t p = (int64_t)(s - Fs[lr]) - a.W;
         lrv[k] = lr;
         if (p < 0) continue;            // a row-staging slot
@@ -426,7 +380,7 @@ __device__ __forceinline__ void join_tile(const JoinArgs &a, const int32_t *M, i
                 dst[(uint64_t)r * W1 + oc] = c == t ? sv.y : rowv[sv.x * t + c];
             }
     }
-    if (TILE_STATS && a.stats) {
+    if (a.stats) {
         bytes += 8ull * items;                                    // list element + bitmap probe
         if (!a.count_only && threadIdx.x == 0) bytes += 4ull * (t + 1) * nsurv;
         unsigned long long bsum = block_sum<NT, unsigned long long>(bytes, wt);

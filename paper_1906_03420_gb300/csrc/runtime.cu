@@ -430,7 +430,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     unsigned char *ctl = nullptr;
     const uint64_t memo_bytes = nodedup ? 0 : (uint64_t)query_memo_tables(steps, k) * (uint64_t)g->n * 8;
     const size_t ctl_bytes = (join_args_size() * (size_t)k + 255) / 256 * 256 +
-                             (sizeof(DStep) * (size_t)k + 255) / 256 * 256 + 256 + 8 * (size_t)QUERY_MAX_CTAS;
+                             (sizeof(DStep) * (size_t)k + 255) / 256 * 256 + 256;
     gsi_status rc = dalloc(*this, (void **)&S, s_bytes);
     if (rc == GSI_OK) rc = dalloc(*this, (void **)&reg[0], t_bytes);
     if (rc == GSI_OK) rc = dalloc(*this, (void **)&reg[1], t_bytes);
@@ -451,7 +451,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         return GSI_OK;
     }
     peak = std::max(peak, s_bytes + 2 * t_bytes);
-    // control block: [step configs][step records][barrier/status][per-CTA sums]
+    // control block: [step configs][step records][barrier/status]
     unsigned char *p = ctl;
     void *cfg_dev = p;
     p += (join_args_size() * (size_t)k + 255) / 256 * 256;
@@ -459,7 +459,6 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     p += (sizeof(DStep) * (size_t)k + 255) / 256 * 256;
     QueryCtl *qc = reinterpret_cast<QueryCtl *>(p);
     p += 256;
-    unsigned long long *bsum = reinterpret_cast<unsigned long long *>(p);
     // configurations, step records and zeroed control words staged in pinned
     // memory in the control block's layout: one upload, no staging copies
     const size_t up_bytes = (size_t)(p - ctl);
@@ -479,7 +478,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     std::memset(hs, 0, sizeof(DStep) * (size_t)k);
     std::memset(h_stage + (reinterpret_cast<unsigned char *>(qc) - ctl), 0, 256);
     for (int t = 1; t < k; ++t) {
-        DStep &h = hs[t];
+        DStepIn &h = hs[t].in;
         h.M = reg[(t - 1) & 1];
         h.out = reg[t & 1];
         h.out_bytes = t_bytes;
@@ -502,8 +501,8 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     int grid = 0;
     if (rc == GSI_OK) {
         tm.begin(1);
-        rc = launch_query_coop(g, k, bitmaps + (uint64_t)order[0] * (uint64_t)g->nwords, smem, cfg_dev, dst, qc, bsum,
-                               &grid, listwise && stats, st);
+        rc = launch_query_coop(g, k, bitmaps + (uint64_t)order[0] * (uint64_t)g->nwords, smem, cfg_dev, dst, qc, &grid,
+                               listwise && stats, st);
         tm.end();
         kernels += 1;
         tiles += (uint64_t)(k - 1);

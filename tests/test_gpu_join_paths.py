@@ -39,10 +39,64 @@ def test_lists_around_the_directory_length(pkg, n_labels, extra):
     edges = [(0, 2 + i) for i in range(deg)] + [(1, 2 + deg + i) for i in range(deg)]
     lab = [n_labels, n_labels] + [(i * 7) % n_labels for i in range(deg)] + [0 if i % 2 else n_labels - 1 for i in range(deg)]
     g = H.graph(n, edges, vlab=lab, elab=[0] * len(edges))
-    assert np.unique(g.vlab).shape[0] == n_labels + 1 or extra < 0
     G = pkg.Graph(g.vlab, g.src, g.dst, g.elab)
     for r in {0, n_labels // 2, n_labels - 1}:
         q = H.query(2, [(0, 1)], [n_labels, r], [0])
         assert same_rows(pkg, G, g, q, order=[0, 1]) == int((g.vlab[2:] == r).sum())
         q = H.query(3, [(0, 1), (0, 2)], [n_labels, r, 0], [0, 0])
         same_rows(pkg, G, g, q, order=[0, 1, 2])
+
+
+@pytest.mark.parametrize("degrees", [[16], [17], [1, 15, 16, 17, 18, 31, 63, 64, 65], [255, 256, 257, 17, 300, 2, 400]])
+def test_long_rows_around_the_tile_edges(pkg, degrees):
+    """Rows with as many candidates as the short rows' limit, the tile's slots and a warp's share, one more and one less;
+    every (hub, leaf) row of the second step is a long one again."""
+    edges, n = [], len(degrees)
+    for h, d in enumerate(degrees):
+        edges += [(h, n + i) for i in range(d)]
+        n += d
+    g = H.graph(n, edges, vlab=[0] * len(degrees) + [1] * (n - len(degrees)), elab=[0] * len(edges))
+    G = pkg.Graph(g.vlab, g.src, g.dst, g.elab)
+    q = H.query(3, [(0, 1), (0, 2)], [0, 1, 1], [0, 0])
+    for order in ([0, 1, 2], [1, 0, 2]):
+        assert same_rows(pkg, G, g, q, order=order) == sum(d * (d - 1) for d in degrees)
+    assert G.query(q, semantics=pkg.GSI_HOMOMORPHISM, count_only=True).count == sum(d * d for d in degrees)
+    r = G.query(q, row_cap=33)
+    assert r.count == sum(d * (d - 1) for d in degrees) and r.rows(33).shape[0] == min(33, r.count)
+
+
+@pytest.mark.parametrize("n", [40, 130])
+def test_long_rows_with_several_lists(pkg, n):
+    """Dense graph: the closing steps have two and three linking edges and more than 16 candidates each."""
+    g = H.random_graph(np.random.default_rng(n), n, 0.55, 1, 1)
+    G = pkg.Graph(g.vlab, g.src, g.dst, g.elab)
+    same_rows(pkg, G, g, H.clique_query(3))
+    if n < 100:
+        same_rows(pkg, G, g, H.clique_query(4))
+        same_rows(pkg, G, g, H.query(4, [(0, 1), (1, 2), (2, 3), (3, 0)]))
+
+
+@pytest.mark.parametrize("k", [9, 31, 32])
+def test_long_rows_of_many_columns(pkg, k):
+    """A chain of k - 1 vertices that ends in a hub with 40 leaves: the widest rows a long step can have."""
+    edges = [(i, i + 1) for i in range(k - 2)] + [(k - 2, k - 1 + i) for i in range(40)]
+    g = H.graph(k - 1 + 40, edges, vlab=list(range(k - 1)) + [99] * 40, elab=[0] * len(edges))
+    G = pkg.Graph(g.vlab, g.src, g.dst, g.elab)
+    q = H.query(k, [(i, i + 1) for i in range(k - 1)], list(range(k - 1)) + [99], [0] * (k - 1))
+    assert same_rows(pkg, G, g, q, order=list(range(k))) == 40
+    assert same_rows(pkg, G, g, q) == 40
+
+
+@pytest.mark.parametrize("rows", [1, 7, 8, 9, 607, 608 * 8, 608 * 8 + 1, 608 * 512 + 3])
+def test_tables_that_fill_some_or_all_of_the_grid(pkg, rows):
+    """One edge per row, so that the second table has `rows` rows: a batch of 8 rows, several, and full batches."""
+    n = 3 * rows
+    edges = [(i, rows + i) for i in range(rows)] + [(rows + i, 2 * rows + i) for i in range(rows)]
+    lab = [0] * rows + [1] * rows + [2] * rows
+    G = pkg.Graph(lab, [a for a, _ in edges], [b for _, b in edges], [0] * len(edges))
+    q = H.query(3, [(0, 1), (1, 2)], [0, 1, 2], [0, 0])
+    r = G.query(q)
+    got = r.rows()
+    got = got[np.argsort(got[:, 0])]
+    want = np.arange(rows, dtype=np.int32)[:, None] + np.array([0, rows, 2 * rows], np.int32)
+    assert r.count == rows and np.array_equal(got, want)
