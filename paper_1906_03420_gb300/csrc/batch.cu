@@ -5,12 +5,14 @@
 // seeds its table with the set bits of its word range and runs the query's
 // join steps on those rows depth-first inside its own slice of the batch
 // arena (a scratch region and two table regions used in turn), with CTA-local
-// long-row tables and survivor counters.  When a step leaves more than split_rows rows
-// and steps remain, the CTA keeps the first split_rows rows and moves the
-// rest, in pieces of split_rows rows, to a spill area and a spill queue; any
-// CTA continues such a piece from the next step.  Idle CTAs take spill units
-// before new seed units, so a query whose tables grow is spread over the GPU
-// instead of running on one CTA.
+// long-row tables and survivor counters.  When a step leaves more than
+// split_rows rows and steps remain, the CTA keeps the first split_rows rows
+// and moves the rest, in pieces of split_rows rows, to a spill area and a
+// spill queue; any CTA continues such a piece from the next step.  Long rows
+// with more than SPLIT_SLOTS candidates in all are handed over in the same
+// way before their join.  Idle CTAs take spill units before new seed units, so
+// a query whose tables grow is spread over the GPU instead of running on one
+// CTA.
 //
 // A unit's final rows are appended to a result arena shared by all units (one
 // atomic reservation per unit) and recorded in a unit record.  A unit whose
@@ -34,6 +36,13 @@ namespace {
 constexpr uint64_t SPILL_SLOTS = 1ull << 18;                  // spill queue capacity (units)
 constexpr unsigned long long WAIT_SPIN_LIMIT = 1ull << 26;    // x ~100 ns sleeps: several seconds
 constexpr long long UNIT_DONE = -(1ll << 62);
+// Candidate slots of a unit's long rows in one step above which the rows past
+// that many slots go to other CTAs.  8,192 slots are four tiles for each warp,
+// some 20 us, and handing a piece over costs about as much.  Without it one
+// CTA took all hub rows of its 1,024 (10^5 slots and more, whose survivors it
+// then queued: rows of many times the size), and a batch of 768 queries kept a
+// tenth of the GPU busy for most of its time.
+constexpr uint64_t SPLIT_SLOTS = 1ull << 13;
 
 struct BatchQuery {
     const uint32_t *seed_bm;       // bitmap of C(u_first)
@@ -52,10 +61,12 @@ struct BatchItem {                 // a seed unit
 
 struct SpillUnit {                 // rows of a table to continue from step t
     int32_t q;
-    int32_t t;
+    int32_t t;                     // step | COUNTED: the rows are already in the step's statistics
     unsigned long long off;        // int32 offset of the rows in the spill area
     unsigned long long rows;
 };
+
+constexpr int32_t COUNTED = 1 << 8;
 
 struct BatchRec {                  // one per unit that kept rows
     int32_t q;
@@ -102,23 +113,27 @@ __device__ __forceinline__ unsigned long long vload(const unsigned long long *p)
 
 // Thread 0 only: the next unit (seed item >= 0, spill slot s as -(s + 1)),
 // or UNIT_DONE once no unit is pending (or a wait ran out).
-__device__ long long next_unit(const BatchArgs &b) {
+//
+// Spill slots are dealt by tickets: a CTA that sees slots waiting takes the
+// next number with one atomic add and owns that slot.  Where several race for
+// the last one, the others' numbers are ahead of the queue: each keeps its
+// ticket (*ticket) and takes seed units meanwhile.  (A compare-and-swap on the
+// queue's head let one CTA through per round trip to L2: 0.55 us a unit,
+// however many CTAs were idle, which was all of the time of a batch with
+// 50,000 units.)
+__device__ long long next_unit(const BatchArgs &b, long long *ticket) {
     BatchCtl *c = b.ctl;
     unsigned long long spins = 0;
     for (;;) {
-        const unsigned long long h = vload(&c->sq_head), tl = vload(&c->sq_tail);
-        if (h < tl) {
-            if (atomicCAS(&c->sq_head, h, h + 1) != h) continue;
-            // the producer reserved slot h and is publishing it
-            while (*reinterpret_cast<volatile unsigned *>(&b.sq_ready[h]) == 0u) {
-                if (++spins > b.spin_limit) {
-                    atomicOr(&c->error, 1u);
-                    return UNIT_DONE;
-                }
-                __nanosleep(32);
-            }
+        if (*ticket < 0 && vload(&c->sq_head) < vload(&c->sq_tail))
+            *ticket = (long long)atomicAdd(&c->sq_head, 1ull);
+        // published (a number past the queue's end never is)
+        if (*ticket >= 0 && (unsigned long long)*ticket < b.sq_cap &&
+            *reinterpret_cast<volatile unsigned *>(&b.sq_ready[*ticket]) != 0u) {
             __threadfence();
-            return -(long long)h - 1;
+            const long long h = *ticket;
+            *ticket = -1;
+            return -h - 1;
         }
         if (vload(&c->next_item) < (unsigned long long)b.nitems) {
             const unsigned long long i = atomicAdd(&c->next_item, 1ull);
@@ -130,8 +145,86 @@ __device__ long long next_unit(const BatchArgs &b) {
             atomicOr(&c->error, 1u);
             return UNIT_DONE;
         }
-        __nanosleep(64);
+        // idle CTAs look less and less often: hundreds of them polling the
+        // control words slow down the atomics of those at work
+        __nanosleep(spins < 8 ? 64u : 500u);
     }
+}
+
+// Copies n int32, eight 16-byte pieces in flight per thread when both ends are
+// 16-byte aligned (one int32 per thread and round trip was 1 KB per
+// microsecond and CTA: 2.7 ms for the 3.3 MB that a unit queues at once).
+template <int NT>
+__device__ __forceinline__ void copy_ints(int32_t *__restrict__ dst, const int32_t *__restrict__ src, uint64_t n) {
+    uint64_t i = threadIdx.x;
+    if (((reinterpret_cast<uintptr_t>(dst) | reinterpret_cast<uintptr_t>(src)) & 15) == 0) {
+        const uint64_t nv = n >> 2;
+        const int4 *s4 = reinterpret_cast<const int4 *>(src);
+        int4 *d4 = reinterpret_cast<int4 *>(dst);
+        for (; i + 7 * NT < nv; i += 8 * NT) {
+            int4 v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = __ldcg(s4 + i + j * NT);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) d4[i + j * NT] = v[j];
+        }
+        for (; i < nv; i += NT) d4[i] = __ldcg(s4 + i);
+        i = nv * 4 + threadIdx.x;
+    }
+    for (; i + 3 * NT < n; i += 4 * NT) {
+        int32_t v[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) v[j] = __ldcg(src + i + j * NT);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) dst[i + j * NT] = v[j];
+    }
+    for (; i < n; i += NT) dst[i] = __ldcg(src + i);
+}
+
+// Moves `rows` rows of w columns at src to the spill area and queues them as
+// units of `per` rows that continue query q with step t (see SpillUnit).  All
+// threads call it; false, with nothing done, when the area or the queue is
+// full.  sh: two words of shared memory.
+template <int NT>
+__device__ bool queue_rows(const BatchArgs &b, int32_t q, int32_t t, const int32_t *src, uint64_t rows, uint64_t w,
+                           uint64_t per, unsigned long long *sh) {
+    BatchCtl *c = b.ctl;
+    const uint64_t nch = (rows + per - 1) / per;
+    if (threadIdx.x == 0) {
+        const uint64_t need = (rows * w + 3) & ~3ull;         // pieces of the area start on 16 bytes
+        sh[0] = ~0ull;
+        const unsigned long long sp = atomicAdd(&c->spill_used, need);
+        if (sp + need <= b.spill_cap) {
+            unsigned long long tl = vload(&c->sq_tail);
+            while (tl + nch <= b.sq_cap) {
+                const unsigned long long old = atomicCAS(&c->sq_tail, tl, tl + nch);
+                if (old == tl) {
+                    sh[0] = sp;
+                    sh[1] = tl;
+                    atomicAdd(&c->pending, (unsigned long long)nch);
+                    break;
+                }
+                tl = old;
+            }
+        }
+    }
+    __syncthreads();
+    const unsigned long long sp = sh[0], s0 = sh[1];
+    if (sp == ~0ull) return false;
+    copy_ints<NT>(b.spill + sp, src, rows * w);
+    __threadfence();                                  // the rows, before any unit that holds them
+    __syncthreads();
+    for (uint64_t ch = threadIdx.x; ch < nch; ch += NT) {
+        SpillUnit u;
+        u.q = q;
+        u.t = t;
+        u.off = sp + ch * per * w;
+        u.rows = min(per, rows - ch * per);
+        b.sq[s0 + ch] = u;
+        __threadfence();
+        atomicExch(&b.sq_ready[s0 + ch], 1u);
+    }
+    return true;
 }
 
 // Drops, without a write-back, the L2 lines that lie wholly inside
@@ -155,7 +248,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wt[BNT / 32];
     __shared__ long long unit_s;
-    __shared__ unsigned long long cnt_s, lctr_s, off_s, slot_s;
+    __shared__ unsigned long long cnt_s, lctr_s, off_s, queue_s[2];
     __shared__ unsigned rfail_s;
     __shared__ int fail_s, skip_s;
     __shared__ __align__(16) JoinArgs a_s;
@@ -168,12 +261,13 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
     int32_t *const result = c->result;
     const unsigned long long result_cap = c->result_cap;
 
+    long long ticket = -1;                            // thread 0: its spill slot to come
     for (;;) {
-        if (threadIdx.x == 0) unit_s = next_unit(b);
+        if (threadIdx.x == 0) unit_s = next_unit(b, &ticket);
         __syncthreads();
         const long long unit = unit_s;
         if (unit == UNIT_DONE) return;
-        int q, t0, oreg;
+        int q, t0, oreg, counted = 0;                 // counted: the step whose statistics hold this unit's rows
         const int32_t *M;
         uint64_t R = 0;
         if (unit >= 0) {
@@ -185,7 +279,8 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
         } else {
             const SpillUnit su = b.sq[-unit - 1];
             q = su.q;
-            t0 = su.t;
+            t0 = su.t & (COUNTED - 1);
+            counted = su.t & COUNTED ? t0 : 0;
             oreg = 0;
             M = b.spill + su.off;
             R = su.rows;
@@ -240,7 +335,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             unsigned long long abytes = 0, items = 0, lbytes = 0;
             row_pass<BNT, true, RPT, false>(a, M, R, 0, (uint64_t)BNT * RPT, BNT * RPT, out, cap, &cnt_s, lt, &rfail_s, smem,
                                             &abytes, &items, &lbytes);
-            if (a.stats) {                       // one add per step of a unit
+            if (a.stats && t != counted) {       // one add per step of a unit
                 abytes = block_sum<BNT, unsigned long long>(abytes, wt);
                 items = block_sum<BNT, unsigned long long>(items, wt);
                 lbytes = block_sum<BNT, unsigned long long>(lbytes, wt);
@@ -252,7 +347,22 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             }
             __syncthreads();
             if (rfail_s) { failed = true; break; }     // long-row table full: the plain path
-            const uint64_t L = lctr_s & ((1ull << lt.rbits) - 1ull), total = lctr_s >> lt.rbits;
+            uint64_t L = lctr_s & ((1ull << lt.rbits) - 1ull), total = lctr_s >> lt.rbits;
+            if (b.split_rows && total > SPLIT_SLOTS && L > 1) {
+                // rows whose slots begin past SPLIT_SLOTS go to other CTAs, which
+                // join them from this step on
+                unsigned long long keep = 0;
+                for (uint64_t i = threadIdx.x; i < L; i += BNT) keep += __ldcg(lt.F + i) < SPLIT_SLOTS;
+                keep = block_sum<BNT, unsigned long long>(keep, wt);
+                if (keep < L) {
+                    const uint64_t first = __ldcg(lt.F + keep), extra = L - keep;
+                    const uint64_t per = max((uint64_t)1, extra * SPLIT_SLOTS / (total - first));
+                    if (queue_rows<BNT>(b, q, t | COUNTED, lt.rows + keep * (uint64_t)t, extra, (uint64_t)t, per, queue_s)) {
+                        L = keep;
+                        total = first;
+                    }
+                }
+            }
             if (L > 0) {
                 // the long rows' slot tiles, CTA-local
                 const unsigned warp = threadIdx.x >> 5;
@@ -273,47 +383,9 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             if (!last && b.split_rows && R > b.split_rows) {
                 const uint64_t keep = b.split_rows, extra = R - keep;
                 const uint64_t w = (uint64_t)(t + 1);
-                const uint64_t nch = (extra + keep - 1) / keep;
-                if (threadIdx.x == 0) {
-                    off_s = ~0ull;
-                    const unsigned long long sp = atomicAdd(&c->spill_used, extra * w);
-                    if (sp + extra * w <= b.spill_cap) {
-                        unsigned long long tl = vload(&c->sq_tail);
-                        while (tl + nch <= b.sq_cap) {
-                            const unsigned long long old = atomicCAS(&c->sq_tail, tl, tl + nch);
-                            if (old == tl) {
-                                off_s = sp;
-                                slot_s = tl;
-                                atomicAdd(&c->pending, (unsigned long long)nch);
-                                break;
-                            }
-                            tl = old;
-                        }
-                    }
-                }
-                __syncthreads();
-                const unsigned long long sp = off_s;
-                if (sp != ~0ull) {
-                    const int32_t *src = M + keep * w;
-                    int32_t *dst = b.spill + sp;
-                    const uint64_t n = extra * w;
-                    for (uint64_t i = threadIdx.x; i < n; i += BNT) dst[i] = src[i];
+                if (queue_rows<BNT>(b, q, t + 1, M + keep * w, extra, w, keep, queue_s)) {
                     __syncthreads();
-                    discard_l2<BNT>(src, n * 4);       // the queued rows now live in the spill area
-                    if (threadIdx.x == 0) {
-                        __threadfence();
-                        const unsigned long long s0 = slot_s;
-                        for (uint64_t ch = 0; ch < nch; ++ch) {
-                            SpillUnit u;
-                            u.q = q;
-                            u.t = t + 1;
-                            u.off = sp + ch * keep * w;
-                            u.rows = min(keep, extra - ch * keep);
-                            b.sq[s0 + ch] = u;
-                        }
-                        __threadfence();
-                        for (uint64_t ch = 0; ch < nch; ++ch) atomicExch(&b.sq_ready[s0 + ch], 1u);
-                    }
+                    discard_l2<BNT>(M + keep * w, extra * w * 4);      // the queued rows now live in the spill area
                     R = keep;
                 }
             }
@@ -327,7 +399,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             fail_s = failed;
             off_s = 0;
             if (!skip && !failed && rows > 0) {
-                const unsigned long long need = rows * (unsigned long long)k;
+                const unsigned long long need = (rows * (unsigned long long)k + 3) & ~3ull;    // on 16 bytes
                 const unsigned long long o = atomicAdd(&c->result_used, need);
                 if (o + need > result_cap) fail_s = 1;
                 else off_s = o;
@@ -346,9 +418,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
         }
         __syncthreads();
         if (!fail_s && rows > 0) {
-            int32_t *dst = result + off_s;
-            const uint64_t n = rows * (uint64_t)k;
-            for (uint64_t i = threadIdx.x; i < n; i += BNT) dst[i] = __ldcg(M + i);
+            copy_ints<BNT>(result + off_s, M, rows * (uint64_t)k);
         }
         __syncthreads();
         if (!fail_s && rows > 0) discard_l2<BNT>(M, rows * (uint64_t)k * 4);   // copied out
