@@ -130,4 +130,39 @@ __device__ inline bool sorted_contains(const int32_t *__restrict__ a, uint32_t l
     return lo < len && __ldg(a + lo) == x;
 }
 
+// The same for the candidates ci[lo + p], p a set bit of `mask`: the bits
+// whose candidate is in ci[b .. b + len).  Four searches run in lockstep, so
+// that their probes are in flight together: one at a time, a row with several
+// candidates and a long other list was a chain of dozens of dependent loads
+// that its whole step waited for.
+__device__ __forceinline__ uint32_t contains_mask(const int32_t *__restrict__ ci, uint32_t lo, uint32_t mask, uint32_t b,
+                                                  uint32_t len) {
+    uint32_t keep = 0;
+    while (mask) {
+        uint32_t bit[4], at[4];
+        int32_t x[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            bit[q] = mask & (0u - mask);
+            mask &= mask - 1;
+            x[q] = bit[q] ? __ldg(ci + lo + (uint32_t)(__ffs(bit[q]) - 1)) : 0;
+            at[q] = b;
+        }
+        // lower bounds, halving the same length for all four
+        for (uint32_t n = len; n > 0;) {
+            const uint32_t h = n >> 1;
+            int32_t y[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) y[q] = bit[q] ? __ldg(ci + at[q] + h) : 0;
+#pragma unroll
+            for (int q = 0; q < 4; ++q) at[q] += y[q] < x[q] ? n - h : 0u;
+            n = h;
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (bit[q] && at[q] < b + len && __ldg(ci + at[q]) == x[q]) keep |= bit[q];
+    }
+    return keep;
+}
+
 }  // namespace gsi

@@ -29,16 +29,17 @@
 // row of M, and hubs recur everywhere.  Two mechanisms keep rows from
 // repeating each other's work:
 //   * a per-step memo holds, for each data vertex v and each of the first
-//     MEMO_EDGES linking edges, where the label(u) sub-list of N(v, l) starts
-//     and how long it is; a row whose vertex is in the memo skips the list
-//     lookup and the label-range search (entries carry the step number, so a
-//     stale entry is a miss, never a wrong answer);
-//   * in single-edge steps the lanes of a warp whose rows share the first-edge
-//     vertex v (found with __match_any_sync) elect one lane, which locates the
-//     sub-list and probes the candidate bitmap C(u) for the whole group once;
-//     the other lanes receive the bound and the bitmap mask by shuffle and
-//     only add their own set subtraction, as Alg. 5 shares one N(v, l0)
-//     fetch among the rows of a block that have the same m_i[u0'].
+//     MEMO_EDGES linking edges, where the label(u) sub-list of N(v, l) starts,
+//     how long it is and, for a short one, which of its entries are in C(u); a
+//     row whose vertex is in the memo skips the list lookup, the label-range
+//     search and the bitmap probes (entries carry the step number, so a stale
+//     entry is a miss, never a wrong answer);
+//   * without a memo, the lanes of a warp whose single-edge rows share the
+//     first-edge vertex v (found with __match_any_sync) elect one lane, which
+//     locates the sub-list and probes the candidate bitmap C(u) for the whole
+//     group once; the other lanes receive the bound and the bitmap mask by
+//     shuffle and only add their own set subtraction, as Alg. 5 shares one
+//     N(v, l0) fetch among the rows of a block that have the same m_i[u0'].
 #pragma once
 
 #include "join_tile.cuh"
@@ -182,11 +183,9 @@ __device__ __forceinline__ uint32_t subtract_row(const JoinArgs &a, const int32_
 
 // One row of the pass: its bound (shortest label sub-list: length *best,
 // start *lob, linking edge *jb) and the mask of its survivors among the
-// first *best candidates when best <= SHORT_MAX.  Lanes whose rows share the
-// first-edge vertex of a single-edge step share the lookup and the bitmap
-// probes (every lane of the warp must call this together).
-template <bool DR, bool LW = true>
-__device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *row, bool valid, int lane,
+// first *best candidates when best <= SHORT_MAX.
+template <bool LW = true>
+__device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *row, bool valid,
                                              uint32_t *best_out, uint32_t *lob_out, int *jb_out,
                                              unsigned long long *abytes, unsigned long long *items,
                                              unsigned long long *lbytes) {
@@ -194,50 +193,36 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
     const bool stats = a.stats != nullptr;
     uint32_t mask = 0, best = 0, lob = 0;
     int jb = 0;
-    if (DR && d == 1) {
-        const int32_t v = valid ? row[a.s.col[0]] : -1 - lane;
-        const unsigned peers = __match_any_sync(FULL_MASK, v);
-        const int leader = __ffs(peers) - 1;
-        uint32_t bm = 0;
-        if (lane == leader && valid) {
-            best = sublist(a, 0, v, &lob);
-            if (best <= (uint32_t)SHORT_MAX) bm = bitmap_mask(a, lob, best);
-        }
-        best = __shfl_sync(FULL_MASK, best, leader);
-        lob = __shfl_sync(FULL_MASK, lob, leader);
-        bm = __shfl_sync(FULL_MASK, bm, leader);
-        if (valid && best <= (uint32_t)SHORT_MAX) mask = subtract_row(a, row, lob, bm);
-        if (valid && stats) {
-            *abytes += row_alg_bytes(t, 1, best, best);
-            if (LW) *lbytes += row_list_bytes(t, 1, whole_len(a, 0, v), best);
-            *items += best;
-        }
-    } else if (valid) {
+    if (valid) {
         uint32_t lo4[MEMO_EDGES], len4[MEMO_EDGES];
         uint64_t lsum = 0;
+        uint32_t known = NO_MASK;                     // the best list's mask, if the memo has it
         best = 0xffffffffu;
 #pragma unroll
         for (int j = 0; j < MEMO_EDGES; ++j) {
             lo4[j] = 0;
             len4[j] = 0;
             if (j < d) {
-                len4[j] = sublist(a, j, row[a.s.col[j]], &lo4[j]);
+                uint32_t m;
+                len4[j] = sublist(a, j, row[a.s.col[j]], &lo4[j], &m);
                 lsum += len4[j];
                 if (len4[j] < best) {
                     best = len4[j];
                     lob = lo4[j];
                     jb = j;
+                    known = m;
                 }
             }
         }
         for (int j = MEMO_EDGES; j < d; ++j) {
-            uint32_t l;
-            const uint32_t n = sublist(a, j, row[a.s.col[j]], &l);
+            uint32_t l, m;
+            const uint32_t n = sublist(a, j, row[a.s.col[j]], &l, &m);
             lsum += n;
             if (n < best) {
                 best = n;
                 lob = l;
                 jb = j;
+                known = m;
             }
         }
         if (stats) {
@@ -250,18 +235,18 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
             *items += best;
         }
         if (best > 0 && best <= (uint32_t)SHORT_MAX) {
-            mask = subtract_row(a, row, lob, bitmap_mask(a, lob, best));
+            if (known == NO_MASK) {
+                known = bitmap_mask(a, lob, best);
+                if (a.memo && jb < MEMO_EDGES)
+                    a.memo[(uint64_t)jb * (uint64_t)a.memo_n + (uint32_t)row[a.s.col[jb]]] =
+                        memo_entry(t, lob, best, known);
+            }
+            mask = subtract_row(a, row, lob, known);
             // every other linking list must hold the candidate (Alg. 3)
             if (a.isect == ISECT_BSEARCH) {
-                for (uint32_t m = mask; m; m &= m - 1) {
-                    const int p = __ffs(m) - 1;
-                    const int32_t w = __ldg(a.ci + lob + (uint32_t)p);
-                    bool ok = true;
 #pragma unroll
-                    for (int j = 0; j < MEMO_EDGES; ++j)
-                        if (ok && j < d && j != jb) ok = sorted_contains(a.ci + lo4[j], len4[j], w);
-                    if (!ok) mask &= ~(1u << p);
-                }
+                for (int j = 0; j < MEMO_EDGES; ++j)
+                    if (mask && j < d && j != jb) mask = contains_mask(a.ci, lob, mask, lo4[j], len4[j]);
             } else {
 #pragma unroll
                 for (int j = 0; j < MEMO_EDGES; ++j) {
@@ -313,11 +298,14 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
 }
 
 // The single-edge rows of one thread (RPT of them, rows q * NT + tid) in
-// lockstep, so that each round of loads is issued for all of them at once:
-// first-edge vertices and their warp groups, memo lookups (the leader of each
-// group), candidate values, bitmap probes, then the group's bound and bitmap
-// mask to every lane, and each lane's own set subtraction.  Sets best[q],
-// lob[q] and mask[q]; rows past nb get best 0.
+// lockstep, so that each round of loads is issued for all of them at once.
+// Sets best[q], lob[q] and mask[q]; rows past nb get best 0.
+//
+// With a memo (one query's launch), each row looks its vertex up: an entry
+// with a mask is all it needs, and large steps meet each vertex many times.
+// On a miss it finds the sub-list, probes the bitmap and leaves both there.
+// Without one (batches), the lanes of a warp whose rows share the vertex elect
+// a leader that does this for the group.
 constexpr int ROW_C = 8;          // candidate values of a single-edge group loaded in the first round
 
 template <int NT, int RPT, bool LW = true>
@@ -327,6 +315,7 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
                                                  unsigned long long *lbytes) {
     constexpr int C = ROW_C;
     const int t = a.s.t;
+    const bool memo = a.memo != nullptr;
     int32_t v[RPT];
     bool lead[RPT];
     int leader[RPT];
@@ -334,73 +323,72 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
     for (int q = 0; q < RPT; ++q) {
         const int lr = q * NT + (int)threadIdx.x;
         v[q] = lr < nb ? rowv[lr * t + a.s.col[0]] : -1 - lane;
-        const unsigned peers = __match_any_sync(FULL_MASK, v[q]);
-        leader[q] = __ffs(peers) - 1;
+        leader[q] = memo ? lane : __ffs(__match_any_sync(FULL_MASK, v[q])) - 1;
         lead[q] = lane == leader[q] && lr < nb;
     }
-    // memo lookups of the group leaders, with the list offsets beside them
-    // (used on a miss)
-    uint64_t e[RPT];
+    // memo lookups, with the list offsets beside them (used on a miss)
     uint32_t x0[RPT], x1[RPT];
+    uint64_t e[RPT];
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        e[q] = (lead[q] && a.memo) ? a.memo[(uint32_t)v[q]] : 0ull;
+        e[q] = (lead[q] && memo) ? a.memo[(uint32_t)v[q]] : 0ull;
         const uint64_t seg = (uint64_t)(uint32_t)(lead[q] ? v[q] : 0) * (uint64_t)a.s.L + (uint64_t)a.s.lab[0];
         x0[q] = lead[q] ? __ldg(a.off + seg) : 0u;
         x1[q] = lead[q] ? __ldg(a.off + seg + 1) : 0u;
     }
-    uint32_t len[RPT], lo[RPT];
+    bool probe[RPT], store[RPT];
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        len[q] = 0;
-        lo[q] = 0;
+        best[q] = 0;
+        lob[q] = 0;
+        mask[q] = 0;
+        probe[q] = store[q] = false;
         if (!lead[q]) continue;
-        if (a.memo && (uint32_t)(e[q] >> MEMO_TAG_SHIFT) == (uint32_t)a.s.t) {
-            lo[q] = (uint32_t)e[q];
-            len[q] = (uint32_t)(e[q] >> 32) & BOUND_LEN_MASK;
+        if (memo_hit(e[q], t)) {
+            lob[q] = (uint32_t)e[q];
+            best[q] = memo_len(e[q]);
+            mask[q] = memo_mask(e[q]);
+            probe[q] = mask[q] == NO_MASK && best[q] <= (uint32_t)SHORT_MAX;
+            if (mask[q] == NO_MASK) mask[q] = 0;
         } else {
             uint32_t h;
-            label_range(a.cl, x0[q], x1[q], (uint32_t)a.s.ulab, &lo[q], &h);
-            len[q] = h - lo[q];
-            if (a.memo && len[q] <= BOUND_LEN_MASK)
-                a.memo[(uint32_t)v[q]] = (uint64_t)lo[q] | ((uint64_t)len[q] << 32) |
-                                         ((uint64_t)(uint32_t)a.s.t << MEMO_TAG_SHIFT);
+            label_range(a.cl, x0[q], x1[q], (uint32_t)a.s.ulab, &lob[q], &h);
+            best[q] = h - lob[q];
+            probe[q] = best[q] <= (uint32_t)SHORT_MAX;
+            store[q] = memo && best[q] <= MEMO_LEN_MASK;
         }
     }
-    // the first C candidates of every short group, then their bitmap probes
+    // the first C candidates of every short list to probe, then their bitmap
+    // words
     int32_t w[RPT][C];
 #pragma unroll
     for (int q = 0; q < RPT; ++q)
 #pragma unroll
         for (int p = 0; p < C; ++p)
-            w[q][p] = (lead[q] && (uint32_t)p < len[q] && len[q] <= (uint32_t)SHORT_MAX)
-                          ? __ldg(a.ci + lo[q] + (uint32_t)p) : -1;
-    uint32_t bm[RPT];
+            w[q][p] = probe[q] && (uint32_t)p < best[q] ? __ldg(a.ci + lob[q] + (uint32_t)p) : -1;
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
-        bm[q] = 0;
 #pragma unroll
         for (int p = 0; p < C; ++p)
-            if (w[q][p] >= 0 && ((__ldg(a.cand + (w[q][p] >> 5)) >> (w[q][p] & 31)) & 1u)) bm[q] |= 1u << p;
+            if (w[q][p] >= 0 && ((__ldg(a.cand + (w[q][p] >> 5)) >> (w[q][p] & 31)) & 1u)) mask[q] |= 1u << p;
+        // candidates past the first C
+        if (probe[q] && best[q] > (uint32_t)C) mask[q] |= bitmap_mask(a, lob[q] + C, best[q] - C) << C;
+        if ((probe[q] && memo) || store[q])
+            a.memo[(uint32_t)v[q]] = memo_entry(t, lob[q], best[q], probe[q] ? mask[q] : NO_MASK);
     }
-#pragma unroll
-    for (int q = 0; q < RPT; ++q)                     // candidates past the first C (groups with C < len <= SHORT_MAX)
-        if (lead[q] && len[q] > (uint32_t)C && len[q] <= (uint32_t)SHORT_MAX)
-            bm[q] |= bitmap_mask(a, lo[q] + C, len[q] - C) << C;
 #pragma unroll
     for (int q = 0; q < RPT; ++q) {
         const int lr = q * NT + (int)threadIdx.x;
         const bool valid = lr < nb;
-        best[q] = __shfl_sync(FULL_MASK, len[q], leader[q]);
-        lob[q] = __shfl_sync(FULL_MASK, lo[q], leader[q]);
-        const uint32_t b = __shfl_sync(FULL_MASK, bm[q], leader[q]);
-        if (!valid) best[q] = 0;
-        mask[q] = (valid && best[q] <= (uint32_t)SHORT_MAX) ? subtract_row(a, rowv + lr * t, lob[q], b) : 0u;
+        if (!memo) {
+            best[q] = __shfl_sync(FULL_MASK, best[q], leader[q]);
+            lob[q] = __shfl_sync(FULL_MASK, lob[q], leader[q]);
+            mask[q] = __shfl_sync(FULL_MASK, mask[q], leader[q]);
+            if (!valid) best[q] = mask[q] = 0;
+        }
+        if (mask[q]) mask[q] = subtract_row(a, rowv + lr * t, lob[q], mask[q]);
         if (a.stats) {
-            if (LW) {                                 // whole first-edge list, from the group leader
-                const uint32_t whole = __shfl_sync(FULL_MASK, lead[q] ? whole_len(a, 0, v[q]) : 0u, leader[q]);
-                if (valid) *lbytes += row_list_bytes(t, 1, whole, best[q]);
-            }
+            if (LW && valid) *lbytes += row_list_bytes(t, 1, whole_len(a, 0, v[q]), best[q]);
             if (valid) {
                 *abytes += row_alg_bytes(t, 1, best[q], best[q]);
                 *items += best[q];
@@ -460,7 +448,7 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
             for (int q = 0; q < RPT; ++q) {
                 const int lr = q * NT + (int)threadIdx.x;
                 const bool valid = lr < nb;
-                mask[q] = row_join<false, LW>(a, rowv + (valid ? lr : 0) * t, valid, lane, &best[q], &lob[q], &jb[q],
+                mask[q] = row_join<LW>(a, rowv + (valid ? lr : 0) * t, valid, &best[q], &lob[q], &jb[q],
                                           abytes, items, lbytes);
                 if (!valid) best[q] = 0;
             }
@@ -701,7 +689,8 @@ __device__ inline void long_rows_join(const JoinArgs &a, const LongTable &lt, ui
             uint32_t *l = lst + lane * 2 * dm1;
             for (int j = 0; j < d; ++j) {
                 if (j == (int)jb) continue;
-                l[1] = sublist(a, j, rowv[lane * t + a.s.col[j]], &l[0]);
+                uint32_t m;
+                l[1] = sublist(a, j, rowv[lane * t + a.s.col[j]], &l[0], &m);
                 l += 2;
             }
         }

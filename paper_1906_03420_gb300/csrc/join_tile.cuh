@@ -174,14 +174,37 @@ __device__ inline int block_inclusive_max(int v, int *wt) {
 }
 
 constexpr int MEMO_EDGES = 4;     // linking edges of a step with a sub-list memo
+
+// A memo entry (8 bytes) of a data vertex and linking edge:
+//   bits 63..59  the step it was made in (another step's entry is a miss)
+//   bit  58      1: the sub-list has at most 16 entries and `mask` tells which
+//                of them are in C(u)
+//   bits 31..0   start of the sub-list
+//   bits 57..32  its length; with bit 58: bits 36..32 length, 52..37 mask
+// Concurrent writers store equal values or one with and one without the mask,
+// and a load that sees an older entry only recomputes it.
 constexpr uint32_t MEMO_TAG_SHIFT = 59;
+constexpr uint32_t MEMO_LEN_MASK = (1u << 26) - 1;
+constexpr uint32_t NO_MASK = 0xffffffffu;
+
+__device__ __forceinline__ bool memo_hit(uint64_t e, int t) { return (uint32_t)(e >> MEMO_TAG_SHIFT) == (uint32_t)t; }
+__device__ __forceinline__ uint32_t memo_len(uint64_t e) {
+    const uint32_t h = (uint32_t)(e >> 32);
+    return (h >> 26) & 1u ? h & 31u : h & MEMO_LEN_MASK;
+}
+__device__ __forceinline__ uint32_t memo_mask(uint64_t e) {
+    const uint32_t h = (uint32_t)(e >> 32);
+    return (h >> 26) & 1u ? (h >> 5) & 0xffffu : NO_MASK;
+}
+__device__ __forceinline__ uint64_t memo_entry(int t, uint32_t lo, uint32_t len, uint32_t mask) {
+    const uint32_t h = mask == NO_MASK ? len : (1u << 26) | (mask << 5) | len;
+    return (uint64_t)lo | ((uint64_t)h << 32) | ((uint64_t)(uint32_t)t << MEMO_TAG_SHIFT);
+}
 
 // Start (*lo) and length (returned) of the label(u) sub-list of N(v, lab[j]),
-// through the memo when the step has one.  A memo entry is
-// start | length << 32 | step << MEMO_TAG_SHIFT; concurrent writers store the
-// same value, and a load that sees an older entry (another step's, or a
-// stale cached line) only recomputes it.
-__device__ __forceinline__ uint32_t sublist(const JoinArgs &a, int j, int32_t v, uint32_t *lo) {
+// through the memo when the step has one, and the sub-list's mask if the memo
+// knows it (else NO_MASK).
+__device__ __forceinline__ uint32_t sublist(const JoinArgs &a, int j, int32_t v, uint32_t *lo, uint32_t *mask) {
     uint64_t *slot = nullptr;
     uint64_t e = 0;
     const uint64_t seg = (uint64_t)(uint32_t)v * (uint64_t)a.s.L + (uint64_t)a.s.lab[j];
@@ -191,16 +214,17 @@ __device__ __forceinline__ uint32_t sublist(const JoinArgs &a, int j, int32_t v,
     }
     // the list's offsets are loaded beside the memo entry (used on a miss)
     const uint32_t x0 = __ldg(a.off + seg), x1 = __ldg(a.off + seg + 1);
-    if (slot && (uint32_t)(e >> MEMO_TAG_SHIFT) == (uint32_t)a.s.t) {
+    if (slot && memo_hit(e, a.s.t)) {
         *lo = (uint32_t)e;
-        return (uint32_t)(e >> 32) & BOUND_LEN_MASK;
+        *mask = memo_mask(e);
+        return memo_len(e);
     }
     uint32_t l, h;
     label_range(a.cl, x0, x1, (uint32_t)a.s.ulab, &l, &h);
     *lo = l;
+    *mask = NO_MASK;
     const uint32_t len = h - l;
-    if (slot && len <= BOUND_LEN_MASK)
-        *slot = (uint64_t)l | ((uint64_t)len << 32) | ((uint64_t)(uint32_t)a.s.t << MEMO_TAG_SHIFT);
+    if (slot && len <= MEMO_LEN_MASK) *slot = memo_entry(a.s.t, l, len, NO_MASK);
     return len;
 }
 
