@@ -163,6 +163,9 @@ gsi_status selftest_barrier_timeout(int dev, unsigned long long spin_limit, doub
 // memo: query_memo_tables(steps, k) tables of n 8-byte entries, zeroed before
 // the launch (per-vertex label sub-list locations, see join_rows.cuh), or null.
 int query_memo_tables(const std::vector<JoinStep> &steps, int k);
+// Whether the last step is counted without enumeration (count_tail): the memo
+// is then followed by one more zeroed table of n 8-byte entries.
+bool query_counts_tail(const std::vector<JoinStep> &steps, int k, int count_only, bool nodedup);
 gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &steps, int k, const uint32_t *bitmaps,
                               const int32_t *order, int count_only, unsigned long long *stats, uint64_t *memo, bool nodedup,
                               void *cfg_host, size_t *smem);

@@ -221,9 +221,16 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         if (blockIdx.x == 0 && threadIdx.x == 0) st->out_cap = cap;
         // ---- short rows joined inline, long rows set aside (one pass over M)
         unsigned long long abytes = 0, items = 0, lbytes = 0;
-        const int nb = batch_rows(R, G, NT * ROW_RPT);
-        row_pass<NT, true, ROW_RPT, LW>(a, in_s.M, R, (uint64_t)blockIdx.x * nb, (uint64_t)G * nb, nb, out, cap,
-                                        &st->count, lt, &ctl->fail, smem, &abytes, &items, &lbytes);
+        // neighbouring runs of warp work go to different SMs
+        const unsigned warp = threadIdx.x >> 5;
+        const uint64_t wi = (uint64_t)warp * G + blockIdx.x, nw = (uint64_t)G * (NT / 32);
+        if (a.mult) {                                         // a counting query's last step
+            count_tail<LW>(a, in_s.M, R, wi, nw, lt, &ctl->fail, &st->count, &abytes, &items, &lbytes);
+        } else {
+            const int nb = batch_rows(R, G, NT * ROW_RPT);
+            row_pass<NT, true, ROW_RPT, LW>(a, in_s.M, R, (uint64_t)blockIdx.x * nb, (uint64_t)G * nb, nb, out, cap,
+                                            &st->count, lt, &ctl->fail, smem, &abytes, &items, &lbytes);
+        }
         if (a.stats) {                       // one add per CTA and step
             abytes = block_sum<NT, unsigned long long>(abytes, wt);
             items = block_sum<NT, unsigned long long>(items, wt);
@@ -239,10 +246,9 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         // ---- long rows through the candidate-slot tiles
         const uint64_t ctr = __ldcg(&st->nlong), L = ctr & ((1ull << lt.rbits) - 1ull), total = ctr >> lt.rbits;
         if (L > 0) {
-            const unsigned warp = threadIdx.x >> 5;
-            // neighbouring runs of slots go to different SMs
-            long_rows_join(a, lt, L, total, (uint64_t)warp * G + blockIdx.x, (uint64_t)G * (NT / 32), out, cap, &st->count,
-                           smem + warp * long_warp_smem(t, a.s.d));
+            unsigned char *const sm = smem + warp * long_warp_smem(t, a.s.d);
+            if (a.mult) long_rows_join<true>(a, lt, L, total, wi, nw, out, 0, &st->count, sm);
+            else long_rows_join<false>(a, lt, L, total, wi, nw, out, cap, &st->count, sm);
             if (!grid_barrier(ctl, G)) return;
         }
         if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) {      // survivors written (both models)
@@ -369,6 +375,10 @@ int query_memo_tables(const std::vector<JoinStep> &steps, int k) {
     return m;
 }
 
+bool query_counts_tail(const std::vector<JoinStep> &steps, int k, int count_only, bool nodedup) {
+    return count_only && !nodedup && k > 1 && steps[k - 1].d == 1;
+}
+
 gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &steps, int k, const uint32_t *bitmaps,
                               const int32_t *order, int count_only, unsigned long long *stats, uint64_t *memo, bool nodedup,
                               void *cfg_host, size_t *smem) {
@@ -381,6 +391,8 @@ gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &s
         cfg[t].memo = nodedup ? nullptr : memo;
         cfg[t].memo_n = g->n;
         cfg[t].nodedup = nodedup ? 1 : 0;
+        if (co && query_counts_tail(steps, k, count_only, nodedup))
+            cfg[t].mult = reinterpret_cast<unsigned long long *>(memo + (uint64_t)query_memo_tables(steps, k) * (uint64_t)g->n);
         sm = std::max(sm, long_warp_smem(steps[t].t, steps[t].d) * (JOIN_NT / 32));
         sm = std::max(sm, rows_smem(JOIN_NT, steps[t].t));
     }

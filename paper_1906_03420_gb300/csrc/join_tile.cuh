@@ -133,6 +133,7 @@ struct JoinArgs {
     // (null: none); table j holds n entries, tagged with the step
     uint64_t *memo;
     int64_t memo_n;
+    unsigned long long *mult;   // counting tail (count_tail): rows per long-listed vertex, zeroed; null: none
     int32_t isect;              // intersection strategy of short multi-edge rows (ISECT_*)
     int32_t nodedup;            // 1: no duplicate removal in the row pass (no warp groups, no memo)
 };

@@ -428,7 +428,9 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     uint64_t *S = nullptr, *memo = nullptr;
     int32_t *reg[2] = {nullptr, nullptr};
     unsigned char *ctl = nullptr;
-    const uint64_t memo_bytes = nodedup ? 0 : (uint64_t)query_memo_tables(steps, k) * (uint64_t)g->n * 8;
+    const uint64_t memo_tables =
+        (uint64_t)query_memo_tables(steps, k) + (query_counts_tail(steps, k, count_only, nodedup) ? 1 : 0);
+    const uint64_t memo_bytes = nodedup ? 0 : memo_tables * (uint64_t)g->n * 8;
     const size_t ctl_bytes = (join_args_size() * (size_t)k + 255) / 256 * 256 +
                              (sizeof(DStep) * (size_t)k + 255) / 256 * 256 + 256;
     gsi_status rc = dalloc(*this, (void **)&S, s_bytes);
