@@ -11,6 +11,7 @@
 // bitmap word (consecutive, as ids ascend) OR their bits together and the
 // last of them sets them with one atomicOr.
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 #include <vector>
 
@@ -22,9 +23,96 @@ namespace {
 
 constexpr int FNT = 256;
 
+// One warp's 32 vertices against the query vertices of their label.
+//
+// A query vertex has few (edge label, neighbour label) pairs, so most of its
+// 15 group words are zero and hold for every vertex: only the words that some
+// query vertex of the label uses are read (gmask), and only a query vertex's
+// own are compared (qsig[s][0], where the label itself is not needed).  On the
+// medium graph (2^20 vertices, 64 labels) a 10-vertex query reads 3-6 words
+// instead of 15.
+__device__ __forceinline__ void filter_warp(const int32_t *__restrict__ gperm, const uint32_t *__restrict__ gsig,
+                                            int64_t np, int64_t p, const uint32_t *qsig, const int32_t *qid, int32_t s0,
+                                            int32_t s1, uint32_t gmask, uint32_t *scnt, int32_t nwords,
+                                            uint32_t *__restrict__ bitmaps, unsigned long long *__restrict__ counts) {
+    const int lane = threadIdx.x & 31;
+    const int32_t v = __ldg(gperm + p);
+    uint32_t x[GSI_SIG_WORDS - 1];
+#pragma unroll
+    for (int j = 0; j < GSI_SIG_WORDS - 1; ++j) x[j] = (gmask >> j) & 1u ? __ldg(gsig + (int64_t)j * np + p) : 0u;
+    const int32_t word = v >= 0 ? (v >> 5) : -1;
+    unsigned run = 0;                                 // lanes sharing my bitmap word, once needed
+    for (int32_t s = s0; s < s1; ++s) {
+        const uint32_t *q = qsig + (int64_t)s * GSI_SIG_WORDS;
+        const uint32_t qm = q[0];
+        bool pass = v >= 0;
+#pragma unroll
+        for (int j = 0; j < GSI_SIG_WORDS - 1; ++j)
+            if ((qm >> j) & 1u) {
+                const uint32_t qw = q[j + 1];
+                pass = pass && ((x[j] & qw) == qw);
+            }
+        const unsigned b = __ballot_sync(FULL_MASK, pass);
+        if (!b) continue;
+        uint32_t *bm = bitmaps + (int64_t)qid[s] * nwords;
+        uint32_t bit = pass ? 1u << (v & 31) : 0u;
+        if (__popc(b) <= 4) {                         // few: one atomic each
+            if (bit) atomicOr(&bm[word], bit);
+        } else {                                      // lanes that share a word OR their bits; the last one sets them
+            if (!run) run = __match_any_sync(FULL_MASK, word);
+            const int first = __ffs(run) - 1;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const uint32_t y = __shfl_up_sync(FULL_MASK, bit, o);
+                if (lane - o >= first) bit |= y;
+            }
+            if (31 - __clz(run) == lane && bit) atomicOr(&bm[word], bit);
+        }
+        if (lane == 0) {
+            if (scnt) atomicAdd(&scnt[s], (uint32_t)__popc(b));
+            else atomicAdd(&counts[qid[s]], (unsigned long long)__popc(b));
+        }
+    }
+}
+
 // meta: qid[nqv] (bitmap / counter index of sorted query vertex s),
 // gstart[ngroups + 1] (query vertices of group g), wbeg[ngroups] (first warp
-// of the group's label), wcum[ngroups + 1] (prefix of the groups' warps).
+// of the group's label), wcum[ngroups + 1] (prefix of the groups' warps),
+// gmask[ngroups] (words that the group's query vertices use).
+__device__ __forceinline__ void filter_body(const int32_t *__restrict__ gperm, const uint32_t *__restrict__ gsig,
+                                            int64_t np, const uint32_t *qsig, const int32_t *meta, int32_t ngroups,
+                                            int32_t nqv, int32_t shared_counts, int32_t nwords,
+                                            uint32_t *__restrict__ bitmaps, unsigned long long *__restrict__ counts,
+                                            uint32_t *scnt) {
+    const int32_t *qid = meta;
+    const int32_t *gstart = qid + nqv;
+    const int32_t *wbeg = gstart + ngroups + 1;
+    const int32_t *wcum = wbeg + ngroups;
+    const int32_t *gmask = wcum + ngroups + 1;
+    if (shared_counts)
+        for (int32_t s = threadIdx.x; s < nqv; s += FNT) scnt[s] = 0;
+    __syncthreads();
+    const int64_t total = wcum[ngroups];
+    const int64_t stride = (int64_t)gridDim.x * (FNT / 32);
+    for (int64_t aw = (int64_t)blockIdx.x * (FNT / 32) + (threadIdx.x >> 5); aw < total; aw += stride) {
+        int lo = 0, hi = ngroups - 1;                  // the group whose warps hold aw
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (wcum[mid] <= aw) lo = mid;
+            else hi = mid - 1;
+        }
+        const int64_t p = ((int64_t)wbeg[lo] + (aw - wcum[lo])) * 32 + (threadIdx.x & 31);
+        filter_warp(gperm, gsig, np, p, qsig, qid, gstart[lo], gstart[lo + 1], (uint32_t)gmask[lo],
+                    shared_counts ? scnt : nullptr, nwords, bitmaps, counts);
+    }
+    if (shared_counts) {
+        __syncthreads();
+        for (int32_t s = threadIdx.x; s < nqv; s += FNT)
+            if (scnt[s]) atomicAdd(&counts[qid[s]], (unsigned long long)scnt[s]);
+    }
+}
+
+// A batch's query vertices, from device memory.
 __global__ void __launch_bounds__(FNT) k_filter_groups(const int32_t *__restrict__ gperm,
                                                        const uint32_t *__restrict__ gsig, int64_t np,
                                                        const uint32_t *__restrict__ qsig,
@@ -33,61 +121,19 @@ __global__ void __launch_bounds__(FNT) k_filter_groups(const int32_t *__restrict
                                                        uint32_t *__restrict__ bitmaps,
                                                        unsigned long long *__restrict__ counts) {
     extern __shared__ uint32_t scnt[];
-    const int32_t *qid = meta;
-    const int32_t *gstart = qid + nqv;
-    const int32_t *wbeg = gstart + ngroups + 1;
-    const int32_t *wcum = wbeg + ngroups;
-    if (shared_counts)
-        for (int32_t s = threadIdx.x; s < nqv; s += FNT) scnt[s] = 0;
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
-    const int64_t total = __ldg(wcum + ngroups);
-    const int64_t stride = (int64_t)gridDim.x * (FNT / 32);
-    for (int64_t aw = (int64_t)blockIdx.x * (FNT / 32) + (threadIdx.x >> 5); aw < total; aw += stride) {
-        int lo = 0, hi = ngroups - 1;                  // the group whose warps hold aw
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (__ldg(wcum + mid) <= aw) lo = mid;
-            else hi = mid - 1;
-        }
-        const int g = lo;
-        const int64_t p = ((int64_t)__ldg(wbeg + g) + (aw - __ldg(wcum + g))) * 32 + lane;
-        const int32_t v = __ldg(gperm + p);
-        uint32_t x[GSI_SIG_WORDS - 1];
-#pragma unroll
-        for (int j = 0; j < GSI_SIG_WORDS - 1; ++j) x[j] = __ldg(gsig + (int64_t)j * np + p);
-        const int32_t word = v >= 0 ? (v >> 5) : -1;
-        const unsigned run = __match_any_sync(FULL_MASK, word);   // lanes sharing my bitmap word
-        const int first = __ffs(run) - 1;
-        const bool last = 31 - __clz(run) == lane;
-        const int32_t s1 = __ldg(gstart + g + 1);
-        for (int32_t s = __ldg(gstart + g); s < s1; ++s) {
-            const uint32_t *q = qsig + (int64_t)s * GSI_SIG_WORDS;
-            bool pass = v >= 0;
-#pragma unroll
-            for (int j = 1; j < GSI_SIG_WORDS; ++j) {
-                const uint32_t qw = __ldg(q + j);
-                pass = pass && ((x[j - 1] & qw) == qw);
-            }
-            uint32_t bit = pass ? 1u << (v & 31) : 0u;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint32_t y = __shfl_up_sync(FULL_MASK, bit, o);
-                if (lane - o >= first) bit |= y;
-            }
-            if (last && bit) atomicOr(&bitmaps[(int64_t)__ldg(qid + s) * nwords + word], bit);
-            const unsigned b = __ballot_sync(FULL_MASK, pass);
-            if (b && lane == 0) {
-                if (shared_counts) atomicAdd(&scnt[s], (uint32_t)__popc(b));
-                else atomicAdd(&counts[__ldg(qid + s)], (unsigned long long)__popc(b));
-            }
-        }
-    }
-    if (shared_counts) {
-        __syncthreads();
-        for (int32_t s = threadIdx.x; s < nqv; s += FNT)
-            if (scnt[s]) atomicAdd(&counts[__ldg(qid + s)], (unsigned long long)scnt[s]);
-    }
+    filter_body(gperm, gsig, np, qsig, meta, ngroups, nqv, shared_counts, nwords, bitmaps, counts, scnt);
+}
+
+// One query's, from the launch's own parameters: no buffer to allocate and
+// nothing to upload before the kernel (two pageable copies and an allocation
+// were 10 us of a single query's host time).
+__global__ void __launch_bounds__(FNT) k_filter_query(const int32_t *__restrict__ gperm,
+                                                      const uint32_t *__restrict__ gsig, int64_t np,
+                                                      const __grid_constant__ FilterInline f, int32_t ngroups,
+                                                      int32_t nqv, int32_t nwords, uint32_t *__restrict__ bitmaps,
+                                                      unsigned long long *__restrict__ counts) {
+    __shared__ uint32_t scnt[GSI_MAX_QUERY_VERTICES];
+    filter_body(gperm, gsig, np, f.sig, f.meta, ngroups, nqv, 1, nwords, bitmaps, counts, scnt);
 }
 
 struct PopcProducer {
@@ -145,7 +191,7 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
     for (int32_t i = 0; i < nqv; ++i) perm[i] = i;
     std::stable_sort(perm.begin(), perm.end(), [&](int32_t a, int32_t b) { return sigs[a][0] < sigs[b][0]; });
     std::vector<uint32_t> flat;
-    std::vector<int32_t> qid, gstart, wbeg, wcum;
+    std::vector<int32_t> qid, gstart, wbeg, wcum, gmask;
     flat.reserve((size_t)nqv * GSI_SIG_WORDS);
     int64_t warps = 0;
     for (int32_t i = 0; i < nqv;) {
@@ -157,9 +203,15 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
             wbeg.push_back((int32_t)(g->goff[r] / 32));
             wcum.push_back((int32_t)warps);
             warps += (g->goff[r + 1] - g->goff[r]) / 32;
+            gmask.push_back(0);
             for (int32_t t = i; t < j; ++t) {
+                const uint32_t *sig = sigs[perm[t]];
+                uint32_t used = 0;                    // its non-zero words, in the label's place
+                for (int w = 1; w < GSI_SIG_WORDS; ++w) used |= sig[w] ? 1u << (w - 1) : 0u;
                 qid.push_back(perm[t]);
-                flat.insert(flat.end(), sigs[perm[t]], sigs[perm[t]] + GSI_SIG_WORDS);
+                flat.push_back(used);
+                flat.insert(flat.end(), sig + 1, sig + GSI_SIG_WORDS);
+                gmask.back() |= (int32_t)used;
             }
         }
         i = j;
@@ -184,11 +236,18 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
     gstart.push_back(fp->nq);
     wcum.push_back((int32_t)warps);
     std::vector<int32_t> meta;
-    meta.reserve(qid.size() + gstart.size() + wbeg.size() + wcum.size());
+    meta.reserve(qid.size() + gstart.size() + wbeg.size() + wcum.size() + gmask.size());
     meta.insert(meta.end(), qid.begin(), qid.end());
     meta.insert(meta.end(), gstart.begin(), gstart.end());
     meta.insert(meta.end(), wbeg.begin(), wbeg.end());
     meta.insert(meta.end(), wcum.begin(), wcum.end());
+    meta.insert(meta.end(), gmask.begin(), gmask.end());
+    if (nqv <= GSI_MAX_QUERY_VERTICES) {              // one query: in the launch's parameters
+        fp->in.reset(new FilterInline());
+        std::memcpy(fp->in->sig, flat.data(), flat.size() * 4);
+        std::memcpy(fp->in->meta, meta.data(), meta.size() * 4);
+        return GSI_OK;
+    }
     const size_t qbytes = flat.size() * 4;
     GSI_CUDA_TRY(cudaMallocAsync(&fp->d_q, qbytes + meta.size() * 4, st));
     fp->d_meta = reinterpret_cast<int32_t *>(reinterpret_cast<unsigned char *>(fp->d_q) + qbytes);
@@ -208,6 +267,12 @@ gsi_status filter_enqueue(const gsi_graph *g, const FilterPlan &fp, uint32_t *bi
     int64_t blocks = (fp.warps + (FNT / 32) - 1) / (FNT / 32);
     if (blocks > 152 * 8) blocks = 152 * 8;
     if (blocks < 1) blocks = 1;
+    if (fp.in) {
+        k_filter_query<<<(unsigned)blocks, FNT, 0, st>>>(g->gperm, g->gsig, g->np, *fp.in, fp.ngroups, fp.nq, g->nwords,
+                                                         bitmaps, counts);
+        GSI_CUDA_TRY(cudaGetLastError());
+        return GSI_OK;
+    }
     // per-CTA counters in shared memory when they fit (else global atomics)
     const size_t smem = (size_t)fp.nq * 4;
     const int shared_counts = smem <= 96 * 1024 ? 1 : 0;

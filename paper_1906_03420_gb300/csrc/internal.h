@@ -2,6 +2,7 @@
 #pragma once
 
 #include <cstdint>
+#include <memory>
 #include <string>
 #include <vector>
 
@@ -72,7 +73,14 @@ gsi_status launch_filter_batch(const gsi_graph *g, const std::vector<QuerySig> &
 // and uploads their signatures (host work, stream-ordered allocation);
 // filter_enqueue zeroes bitmaps [nqv][nwords] and counters [nqv] and runs the
 // kernel (stream work only: capturable into a CUDA graph).
+// Up to GSI_MAX_QUERY_VERTICES grouped signatures and their group table go to
+// the kernel by value (FilterInline), larger calls through device memory.
+struct FilterInline {
+    uint32_t sig[GSI_MAX_QUERY_VERTICES * GSI_SIG_WORDS];
+    int32_t meta[5 * GSI_MAX_QUERY_VERTICES + 2];
+};
 struct FilterPlan {
+    std::shared_ptr<FilterInline> in;
     uint32_t *d_q = nullptr;    // grouped signatures, then the group table
     int32_t *d_meta = nullptr;
     int32_t nqv = 0, nq = 0, ngroups = 0;
