@@ -19,6 +19,7 @@
 // label) pair of v is hashed to a group whose state goes 00 -> 01 -> 11 as the
 // first and second pair arrive.
 #include <algorithm>
+#include <climits>
 #include <vector>
 
 #include "internal.h"
@@ -65,46 +66,143 @@ __global__ void k_adjacent_equal(const uint64_t *__restrict__ keys, int64_t n, u
     if (__any_sync(FULL_MASK, dup) && (threadIdx.x & 31) == 0) atomicOr(flags, (unsigned)DUP_PAIR);
 }
 
-// Dense rank of each vertex label (binary search in the sorted distinct labels).
-__global__ void k_vertex_rank(const int32_t *__restrict__ vlab, int32_t n, const int32_t *__restrict__ uniq, int32_t LV,
-                              uint16_t *__restrict__ rank) {
+// Smallest and largest vertex label (range[0], range[1]: INT_MAX and INT_MIN before).
+__global__ void k_label_range(const int32_t *__restrict__ vlab, int32_t n, int *range) {
+    int lo = INT_MAX, hi = INT_MIN;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x) {
-        int32_t x = vlab[v], lo = 0, hi = LV - 1;
-        while (lo < hi) {
-            int32_t mid = (lo + hi) >> 1;
-            if (uniq[mid] < x) lo = mid + 1;
-            else hi = mid;
+        lo = min(lo, vlab[v]);
+        hi = max(hi, vlab[v]);
+    }
+    lo = __reduce_min_sync(FULL_MASK, lo);
+    hi = __reduce_max_sync(FULL_MASK, hi);
+    if ((threadIdx.x & 31) == 0) {
+        atomicMin(range, lo);
+        atomicMax(range + 1, hi);
+    }
+}
+
+__global__ void k_vertex_keys(const int32_t *__restrict__ vlab, int32_t n, int32_t lo, int nb, uint64_t *__restrict__ keys) {
+    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
+        keys[v] = ((uint64_t)((uint32_t)vlab[v] - (uint32_t)lo) << nb) | (uint64_t)v;
+}
+
+// The vertices in the order of (label, id): position i holds vertex sv[i] of
+// label rank sr[i], gpos is the inverse of sv, and label rank r begins at
+// position start[r] and stands for label uniq[r].  One scan over the sorted
+// keys: a position that differs from the one before it in its label starts a
+// rank.  Ranks past MAX_LABELS are not written (the graph is refused).
+constexpr int32_t MAX_LABELS = 65535;
+
+struct LabelHead {
+    const uint64_t *keys;
+    int nb;
+    __device__ uint32_t operator()(int64_t i) const { return i == 0 || (keys[i] >> nb) != (keys[i - 1] >> nb); }
+};
+struct LabelRanks {
+    LabelHead head;
+    int64_t n;
+    int32_t lo;
+    int32_t *sv;
+    uint16_t *sr;
+    uint32_t *gpos;
+    uint32_t *nlabels;
+    int32_t *uniq, *start;
+    __device__ void operator()(int64_t i, uint32_t before) const {
+        if (i == n) {
+            *nlabels = before;
+            return;
         }
-        rank[v] = (uint16_t)lo;
+        const uint64_t k = head.keys[i];
+        const uint32_t h = head(i), r = before + h - 1;
+        const int32_t v = (int32_t)(k & ((1ull << head.nb) - 1));
+        sv[i] = v;
+        sr[i] = (uint16_t)r;
+        gpos[v] = (uint32_t)i;
+        if (h && r < (uint32_t)MAX_LABELS) {
+            uniq[r] = (int32_t)((uint32_t)(k >> head.nb) + (uint32_t)lo);
+            start[r] = (int32_t)i;
+        }
     }
+};
+
+// gperm: position i of the order above goes to its group's padded place.
+__global__ void k_group_perm(const int32_t *__restrict__ sv, const uint16_t *__restrict__ sr,
+                             const int64_t *__restrict__ shift, int32_t n, int32_t *__restrict__ gperm) {
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        gperm[i + shift[sr[i]]] = sv[i];
 }
 
-// Directed entry keys: (((v*L + l) << lb | rank(neighbour)) << nb) | neighbour, two per edge.
+// Directed entry keys, two per edge: ((v << Lb | l) << nb) | gpos(neighbour).
+// The neighbour stands as its position in the order of (label, id), which a
+// list is sorted by: one field of nb bits instead of a label rank and an id.
 __global__ void k_csr_keys(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
-                           const int32_t *__restrict__ elab, const uint16_t *__restrict__ vrank, int64_t m, int32_t L,
-                           int lb, int nb, uint64_t *__restrict__ keys) {
+                           const int32_t *__restrict__ elab, const uint32_t *__restrict__ gpos, int64_t m, int Lb,
+                           int nb, uint64_t *__restrict__ keys) {
+    ulonglong2 *out = reinterpret_cast<ulonglong2 *>(keys);
     for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t a = (uint32_t)src[e], b = (uint32_t)dst[e], l = (uint32_t)elab[e];
-        keys[2 * e] = ((((a * (uint64_t)L + l) << lb) | vrank[b]) << nb) | b;
-        keys[2 * e + 1] = ((((b * (uint64_t)L + l) << lb) | vrank[a]) << nb) | a;
+        const uint32_t a = (uint32_t)src[e], b = (uint32_t)dst[e];
+        const uint64_t l = (uint32_t)elab[e];
+        out[e] = make_ulonglong2((((uint64_t)a << Lb | l) << nb) | gpos[b], (((uint64_t)b << Lb | l) << nb) | gpos[a]);
     }
 }
 
-// From sorted keys: ci[p] = neighbour, cl[p] = its label rank, and off[s] =
-// first position of segment s = v*L + l.
-__global__ void k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int lb, int nb, uint64_t nseg,
-                           uint32_t *__restrict__ off, int32_t *__restrict__ ci, uint16_t *__restrict__ cl) {
-    const uint64_t mask = (1ull << nb) - 1, lmask = (1ull << lb) - 1;
-    const int sh = lb + nb;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n2; p += (int64_t)gridDim.x * blockDim.x) {
-        uint64_t k = keys[p];
-        ci[p] = (int32_t)(k & mask);
-        cl[p] = (uint16_t)((k >> nb) & lmask);
-        uint64_t s = k >> sh;
-        uint64_t prev = p == 0 ? 0 : (keys[p - 1] >> sh) + 1;
-        for (uint64_t x = prev; x <= s; ++x) off[x] = (uint32_t)p;
+// From sorted keys: ci[p] = neighbour, cl[p] = its label rank, off[s] = first
+// position of segment s = v*L + l, and the group bits of the signatures
+// (zeroed before).
+//
+// A pair's state needs its first two occurrences only, and equal pairs of a
+// vertex stand together here: the first entry of a run counts one, the second
+// sets both bits, the others do nothing.  32M entries take 389 us; going over
+// the edge list for the signatures instead, every entry hashed its pair and did
+// its atomic on a random vertex (349 us, and 110 for the rest).
+__global__ void k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int Lb, int nb, int32_t L, uint64_t nseg,
+                           const int32_t *__restrict__ sv, const uint16_t *__restrict__ sr,
+                           const int32_t *__restrict__ uniq, int32_t n, uint32_t *__restrict__ off,
+                           int32_t *__restrict__ ci, uint16_t *__restrict__ cl, uint32_t *__restrict__ sig) {
+    const uint64_t mask = (1ull << nb) - 1, lmask = (1ull << Lb) - 1;
+    const int lane = threadIdx.x & 31;
+    for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); p0 < n2;
+         p0 += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t p = p0 + lane;
+        const bool valid = p < n2;
+        const uint64_t k = valid ? keys[p] : 0ull;
+        const uint32_t r = sr[k & mask];
+        // the two entries before the warp's, in lanes 0 and 1
+        const bool xv = lane < 2 && p >= 2;
+        const uint64_t x = xv ? keys[p - 2] : 0ull;
+        const uint32_t xr = xv ? sr[x & mask] : 0u;
+        const uint64_t seg = k >> nb, xseg = x >> nb;
+        uint64_t s1 = __shfl_up_sync(FULL_MASK, seg, 1), s2 = __shfl_up_sync(FULL_MASK, seg, 2);
+        uint32_t r1 = __shfl_up_sync(FULL_MASK, r, 1), r2 = __shfl_up_sync(FULL_MASK, r, 2);
+        const uint64_t y = __shfl_sync(FULL_MASK, xseg, 1);
+        const uint32_t yr = __shfl_sync(FULL_MASK, xr, 1);
+        if (lane < 2) {
+            s2 = xseg;
+            r2 = xr;
+        }
+        if (lane == 0) {
+            s1 = y;
+            r1 = yr;
+        }
+        // lane 0 of the second entry on: the entry before it is lane 1's x
+        const bool same1 = p >= 1 && s1 == seg && r1 == r, same2 = p >= 2 && s2 == seg && r2 == r;
+        if (!valid) continue;
+        const int32_t w = sv[k & mask];
+        ci[p] = w;
+        cl[p] = (uint16_t)r;
+        const uint64_t v = seg >> Lb, l = seg & lmask, s = v * (uint64_t)L + l;
+        uint64_t prev = 0;
+        if (p > 0) prev = (s1 >> Lb) * (uint64_t)L + (s1 & lmask) + 1;
+        for (uint64_t q = prev; q <= s; ++q) off[q] = (uint32_t)p;
         if (p == n2 - 1)
-            for (uint64_t x = s + 1; x <= nseg; ++x) off[x] = (uint32_t)n2;
+            for (uint64_t q = s + 1; q <= nseg; ++q) off[q] = (uint32_t)n2;
+        if (!(same1 && same2)) {
+            const uint32_t g = sig_group((int32_t)l, uniq[r]);
+            uint32_t *word = sig + (int64_t)sig_word(g) * n + (int64_t)v;
+            const uint32_t bit = 1u << sig_bit(g);
+            if (same1) atomicOr(word, 3u * bit);
+            else if (atomicOr(word, bit) & bit) atomicOr(word, 2u * bit);
+        }
     }
 }
 
@@ -140,27 +238,6 @@ __global__ void k_fill_u32(uint32_t *a, uint64_t n, uint32_t v) {
         a[i] = v;
 }
 
-__global__ void k_sig_labels(const int32_t *__restrict__ vlab, int32_t n, uint32_t *__restrict__ sig) {
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (int64_t)gridDim.x * blockDim.x)
-        sig[v] = (uint32_t)vlab[v];
-}
-
-// One (edge label, neighbour label) pair per directed entry.
-__global__ void k_sig_pairs(const int32_t *__restrict__ src, const int32_t *__restrict__ dst,
-                            const int32_t *__restrict__ elab, const int32_t *__restrict__ vlab, int64_t m, int32_t n,
-                            uint32_t *__restrict__ sig) {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 2 * m; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t e = i >> 1;
-        int32_t v = (i & 1) ? dst[e] : src[e];
-        int32_t w = (i & 1) ? src[e] : dst[e];
-        uint32_t g = sig_group(elab[e], vlab[w]);
-        uint32_t word = sig_word(g), bit = sig_bit(g);
-        uint32_t *p = sig + (int64_t)word * n + v;
-        uint32_t old = atomicOr(p, 1u << bit);
-        if (old & (1u << bit)) atomicOr(p, 2u << bit);
-    }
-}
-
 // Words 1..15 of every grouped position's vertex (zero for padding).
 __global__ void k_group_sig(const uint32_t *__restrict__ sig, int32_t n, const int32_t *__restrict__ gperm,
                             int64_t np, uint32_t *__restrict__ gsig) {
@@ -171,21 +248,43 @@ __global__ void k_group_sig(const uint32_t *__restrict__ sig, int32_t n, const i
     }
 }
 
-__global__ void k_label_hist(const int32_t *__restrict__ elab, int64_t m, int32_t L, unsigned long long *freq) {
-    extern __shared__ unsigned long long h[];
-    const bool local = L <= 4096;
-    if (local)
-        for (int i = threadIdx.x; i < L; i += blockDim.x) h[i] = 0;
+// Directed entries per edge label, from the lists' lengths: a thread's
+// segments all have one label (the grid's threads are a multiple of L), so it
+// adds up in a register (one shared-memory atomic per edge, on 8 addresses,
+// took 198 us of 16M edges; this takes 33).
+__global__ void __launch_bounds__(NT) k_label_count(const uint32_t *__restrict__ off, uint64_t nseg, int32_t L,
+                                                    uint64_t step, unsigned long long *freq) {
+    constexpr int32_t LOCAL = 1024;
+    __shared__ unsigned long long h[LOCAL];
+    for (int32_t i = threadIdx.x; i < min(L, LOCAL); i += NT) h[i] = 0;
     __syncthreads();
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < m; e += (int64_t)gridDim.x * blockDim.x) {
-        if (local) atomicAdd(&h[elab[e]], 1ull);
-        else atomicAdd(&freq[elab[e]], 1ull);
-    }
+    const uint64_t t = (uint64_t)blockIdx.x * NT + threadIdx.x;
+    unsigned long long c = 0;
+    if (t < step)
+        for (uint64_t s = t; s < nseg; s += step) c += off[s + 1] - off[s];
+    const uint64_t l = t % (uint64_t)L;
+    if (c) atomicAdd(L <= LOCAL ? &h[l] : &freq[l], c);
     __syncthreads();
-    if (local)
-        for (int i = threadIdx.x; i < L; i += blockDim.x)
+    if (L <= LOCAL)
+        for (int32_t i = threadIdx.x; i < L; i += NT)
             if (h[i]) atomicAdd(&freq[i], h[i]);
 }
+
+// Device buffers of one build, released on its stream when it ends.
+struct Temps {
+    cudaStream_t st;
+    std::vector<void *> all;
+    explicit Temps(cudaStream_t s) : st(s) {}
+    ~Temps() {
+        for (void *p : all) cudaFreeAsync(p, st);
+    }
+    template <typename T>
+    gsi_status alloc(T **p, uint64_t count) {
+        GSI_CUDA_TRY(cudaMallocAsync(p, sizeof(T) * (size_t)(count + 1), st));
+        all.push_back(*p);
+        return GSI_OK;
+    }
+};
 
 unsigned grid_for(int64_t n) {
     int64_t b = (n + NT - 1) / NT;
@@ -219,161 +318,144 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_CUDA_TRY(cudaEventCreate(&e1));
     GSI_CUDA_TRY(cudaEventRecord(e0, st));
 
+    Temps tmps(st);
     int32_t *d_vlab = nullptr, *d_src = nullptr, *d_dst = nullptr, *d_elab = nullptr;
-    unsigned *d_flags = nullptr;
-    int *d_maxlab = nullptr;
-    GSI_CUDA_TRY(cudaMallocAsync(&d_vlab, sizeof(int32_t) * (size_t)n, st));
-    GSI_CUDA_TRY(cudaMallocAsync(&d_src, sizeof(int32_t) * (size_t)(m + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&d_dst, sizeof(int32_t) * (size_t)(m + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&d_elab, sizeof(int32_t) * (size_t)(m + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&d_flags, 16, st));
-    d_maxlab = reinterpret_cast<int *>(d_flags + 1);
+    // error bits, largest edge label, vertex label range, distinct vertex labels
+    struct Words {
+        unsigned flags;
+        int maxlab, lo, hi;
+        uint32_t nlabels;
+    } hw = {0u, -1, INT_MAX, INT_MIN, 0u};
+    Words *d_w = nullptr;
+    GSI_TRY(tmps.alloc(&d_vlab, (uint64_t)n));
+    GSI_TRY(tmps.alloc(&d_src, (uint64_t)m));
+    GSI_TRY(tmps.alloc(&d_dst, (uint64_t)m));
+    GSI_TRY(tmps.alloc(&d_elab, (uint64_t)m));
+    GSI_TRY(tmps.alloc(&d_w, 1));
+    GSI_CUDA_TRY(cudaMemcpyAsync(d_w, &hw, sizeof hw, cudaMemcpyHostToDevice, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_vlab, vlab, sizeof(int32_t) * (size_t)n, cudaMemcpyDefault, st));
+    k_label_range<<<grid_for(n), NT, 0, st>>>(d_vlab, n, &d_w->lo);
     if (m > 0) {
         GSI_CUDA_TRY(cudaMemcpyAsync(d_src, src, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
         GSI_CUDA_TRY(cudaMemcpyAsync(d_dst, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
         GSI_CUDA_TRY(cudaMemcpyAsync(d_elab, elab, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
+        k_validate<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, &d_w->flags, &d_w->maxlab);
     }
-    GSI_CUDA_TRY(cudaMemsetAsync(d_flags, 0, 4, st));
-    GSI_CUDA_TRY(cudaMemsetAsync(d_maxlab, 0xff, 4, st));   // -1
-    auto cleanup_inputs = [&]() {
-        cudaFreeAsync(d_vlab, st); cudaFreeAsync(d_src, st); cudaFreeAsync(d_dst, st);
-        cudaFreeAsync(d_elab, st); cudaFreeAsync(d_flags, st);
-    };
-    if (m > 0) k_validate<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, d_flags, d_maxlab);
-    unsigned h_flags[2] = {0, 0};
-    GSI_CUDA_TRY(cudaMemcpyAsync(h_flags, d_flags, 8, cudaMemcpyDeviceToHost, st));
+    GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
     GSI_CUDA_TRY(cudaStreamSynchronize(st));
-    int maxlab = (int)h_flags[1];
-    if (h_flags[0]) {
-        cleanup_inputs();
-        set_error(std::string("gsi_graph_create: ") + ((h_flags[0] & BAD_ID) ? "vertex id out of range " : "") +
-                  ((h_flags[0] & SELF_LOOP) ? "self-loop " : "") + ((h_flags[0] & NEG_LABEL) ? "negative edge label" : ""));
+    if (hw.flags) {
+        set_error(std::string("gsi_graph_create: ") + ((hw.flags & BAD_ID) ? "vertex id out of range " : "") +
+                  ((hw.flags & SELF_LOOP) ? "self-loop " : "") + ((hw.flags & NEG_LABEL) ? "negative edge label" : ""));
         return GSI_EINVAL;
     }
-    const int32_t L = maxlab < 0 ? 1 : maxlab + 1;
-    // sorted distinct vertex labels (host): dense ranks for the sub-list order
-    std::vector<int32_t> uniq;
-    {
-        int32_t mn = vlab[0], mx = vlab[0];
-        for (int32_t v = 1; v < n; ++v) { mn = std::min(mn, vlab[v]); mx = std::max(mx, vlab[v]); }
-        if ((int64_t)mx - (int64_t)mn < (1 << 24)) {
-            std::vector<uint8_t> seen((size_t)((int64_t)mx - mn + 1), 0);
-            for (int32_t v = 0; v < n; ++v) seen[(size_t)((int64_t)vlab[v] - mn)] = 1;
-            for (size_t i = 0; i < seen.size(); ++i)
-                if (seen[i]) uniq.push_back((int32_t)((int64_t)mn + (int64_t)i));
-        } else {
-            uniq.assign(vlab, vlab + n);
-            std::sort(uniq.begin(), uniq.end());
-            uniq.erase(std::unique(uniq.begin(), uniq.end()), uniq.end());
-        }
+    const int32_t L = hw.maxlab < 0 ? 1 : hw.maxlab + 1;
+    const int nb = ceil_log2_bits((uint64_t)(n > 1 ? n - 1 : 1));
+
+    // the vertices in the order of (label, id), the duplicate check of the
+    // pairs behind them on the stream, one readback for both
+    const uint64_t nkeys = std::max((uint64_t)(2 * m), (uint64_t)n);
+    uint64_t *keys = nullptr, *tmp = nullptr, *sorted = nullptr;
+    GSI_TRY(tmps.alloc(&keys, nkeys));
+    GSI_TRY(tmps.alloc(&tmp, nkeys));
+    int32_t *sv = nullptr, *d_labels = nullptr;
+    uint16_t *sr = nullptr;
+    uint32_t *gpos = nullptr, *scr = nullptr;
+    const int32_t most = (int32_t)std::min<int64_t>(n, MAX_LABELS);
+    GSI_TRY(tmps.alloc(&sv, (uint64_t)n));
+    GSI_TRY(tmps.alloc(&sr, (uint64_t)n));
+    GSI_TRY(tmps.alloc(&gpos, (uint64_t)n));
+    GSI_TRY(tmps.alloc(&d_labels, 2 * (uint64_t)most));
+    GSI_TRY(tmps.alloc(&scr, (uint64_t)scan_blocks(n) + 1));
+    const uint32_t range = (uint32_t)hw.hi - (uint32_t)hw.lo;
+    k_vertex_keys<<<grid_for(n), NT, 0, st>>>(d_vlab, n, hw.lo, nb, keys);
+    GSI_TRY(radix_sort_u64(keys, tmp, n, nb, range ? nb + ceil_log2_bits(range) : nb, &sorted, st));
+    const LabelHead head{sorted, nb};
+    GSI_CUDA_TRY(device_scan<uint32_t>(
+        head, n, LabelRanks{head, n, hw.lo, sv, sr, gpos, &d_w->nlabels, d_labels, d_labels + most}, scr, st));
+    if (m > 1) {
+        k_pair_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, m, nb, keys);
+        GSI_TRY(radix_sort_u64(keys, tmp, m, 0, 2 * nb, &sorted, st));
+        k_adjacent_equal<<<grid_for(m), NT, 0, st>>>(sorted, m, &d_w->flags);
     }
-    if (uniq.size() > 65535) {
-        cleanup_inputs();
+    std::vector<int32_t> labels(2 * (size_t)most);     // the distinct labels, then where each begins
+    GSI_CUDA_TRY(cudaMemcpyAsync(labels.data(), d_labels, sizeof(int32_t) * labels.size(), cudaMemcpyDeviceToHost, st));
+    GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
+    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    if (hw.nlabels > (uint32_t)MAX_LABELS) {
         set_error("gsi_graph_create: more than 65535 distinct vertex labels");
         return GSI_EINVAL;
     }
-    const int32_t LV = (int32_t)uniq.size();
-    const int nb = ceil_log2_bits((uint64_t)(n > 1 ? n - 1 : 1));
+    const int32_t LV = (int32_t)hw.nlabels;
     const int lb = ceil_log2_bits((uint64_t)(LV > 1 ? LV - 1 : 1));
     const uint64_t nseg = (uint64_t)n * (uint64_t)L;
     const int sb = ceil_log2_bits(nseg - 1);
     if (sb + lb + nb > 64 || nseg + 1 >= ((uint64_t)1 << 34)) {
-        cleanup_inputs();
         set_error("gsi_graph_create: n * L * labels too large for the label-partitioned layout");
         return GSI_EINVAL;
     }
-
-    // vertices grouped by label rank (host counting sort, ascending ids per
-    // group, each group padded to a multiple of 32 positions)
-    std::vector<int32_t> gperm;
-    std::vector<int64_t> goff((size_t)LV + 1, 0);
-    {
-        std::vector<int32_t> rank((size_t)n);
-        for (int32_t v = 0; v < n; ++v)
-            rank[v] = (int32_t)(std::lower_bound(uniq.begin(), uniq.end(), vlab[v]) - uniq.begin());
-        std::vector<int64_t> cnt((size_t)LV, 0);
-        for (int32_t v = 0; v < n; ++v) ++cnt[rank[v]];
-        for (int32_t r = 0; r < LV; ++r) goff[r + 1] = goff[r] + (cnt[r] + 31) / 32 * 32;
-        gperm.assign((size_t)goff[LV], -1);
-        std::vector<int64_t> pos(goff.begin(), goff.end() - 1);
-        for (int32_t v = 0; v < n; ++v) gperm[pos[rank[v]]++] = v;
+    if (hw.flags & DUP_PAIR) {
+        set_error("gsi_graph_create: a vertex pair appears more than once");
+        return GSI_EINVAL;
     }
 
-    // duplicate vertex pairs
-    uint64_t *keys = nullptr, *tmp = nullptr;
-    GSI_CUDA_TRY(cudaMallocAsync(&keys, sizeof(uint64_t) * (size_t)(2 * m + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&tmp, sizeof(uint64_t) * (size_t)(2 * m + 1), st));
-    if (m > 1) {
-        k_pair_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, m, nb, keys);
-        GSI_TRY(radix_sort_u64(keys, tmp, m, 2 * nb, st));
-        k_adjacent_equal<<<grid_for(m), NT, 0, st>>>(keys, m, d_flags);
-        GSI_CUDA_TRY(cudaMemcpyAsync(h_flags, d_flags, 4, cudaMemcpyDeviceToHost, st));
-        GSI_CUDA_TRY(cudaStreamSynchronize(st));
-        if (h_flags[0] & DUP_PAIR) {
-            cudaFreeAsync(keys, st); cudaFreeAsync(tmp, st);
-            cleanup_inputs();
-            set_error("gsi_graph_create: a vertex pair appears more than once");
-            return GSI_EINVAL;
-        }
+    // label groups, each padded to whole warps
+    std::vector<int64_t> goff((size_t)LV + 1, 0), shift((size_t)LV, 0);
+    for (int32_t r = 0; r < LV; ++r) {
+        const int64_t begin = labels[(size_t)(most + r)], end = r + 1 < LV ? labels[(size_t)(most + r + 1)] : n;
+        goff[r + 1] = goff[r] + (end - begin + 31) / 32 * 32;
+        shift[r] = goff[r] - begin;
     }
 
-    // CSR
+    // CSR and signatures
     g->n = n; g->m = m; g->L = L; g->LV = LV; g->nwords = (n + 31) / 32;
-    g->vlabels = uniq;
+    g->vlabels.assign(labels.begin(), labels.begin() + LV);
     GSI_CUDA_TRY(cudaMallocAsync(&g->off, sizeof(uint32_t) * (size_t)(nseg + 1), st));
     GSI_CUDA_TRY(cudaMallocAsync(&g->ci, sizeof(int32_t) * (size_t)(2 * m + 1), st));
     GSI_CUDA_TRY(cudaMallocAsync(&g->cl, sizeof(uint16_t) * (size_t)(2 * m + 1), st));
     GSI_CUDA_TRY(cudaMallocAsync(&g->dir, sizeof(uint32_t) * (size_t)(m + 1), st));
     g->dir_min = 2u * ((uint32_t)LV + 1u);
     GSI_CUDA_TRY(cudaMallocAsync(&g->sig, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
+    GSI_CUDA_TRY(cudaMemsetAsync(g->sig, 0, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
+    GSI_CUDA_TRY(cudaMemcpyAsync(g->sig, d_vlab, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st));
     if (m > 0) {
-        int32_t *d_uniq = nullptr;
-        uint16_t *d_vrank = nullptr;
-        GSI_CUDA_TRY(cudaMallocAsync(&d_uniq, sizeof(int32_t) * (size_t)LV, st));
-        GSI_CUDA_TRY(cudaMallocAsync(&d_vrank, sizeof(uint16_t) * (size_t)n, st));
-        GSI_CUDA_TRY(cudaMemcpyAsync(d_uniq, uniq.data(), sizeof(int32_t) * (size_t)LV, cudaMemcpyHostToDevice, st));
-        k_vertex_rank<<<grid_for(n), NT, 0, st>>>(d_vlab, n, d_uniq, LV, d_vrank);
-        k_csr_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, d_vrank, m, L, lb, nb, keys);
-        GSI_TRY(radix_sort_u64(keys, tmp, 2 * m, sb + lb + nb, st));
-        k_csr_fill<<<grid_for(2 * m), NT, 0, st>>>(keys, 2 * m, lb, nb, nseg, g->off, g->ci, g->cl);
+        // nb + Lb + nb is at most sb + 1 + nb, and lb at least 1: it fits 64 bits
+        const int Lb = L > 1 ? ceil_log2_bits((uint64_t)L - 1) : 0;
+        k_csr_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, gpos, m, Lb, nb, keys);
+        GSI_TRY(radix_sort_u64(keys, tmp, 2 * m, 0, nb + Lb + nb, &sorted, st));
+        k_csr_fill<<<grid_for(2 * m), NT, 0, st>>>(sorted, 2 * m, Lb, nb, L, nseg, sv, sr, d_labels, n, g->off, g->ci,
+                                                   g->cl, g->sig);
         k_label_dir<<<grid_for((int64_t)nseg), NT, 0, st>>>(g->off, g->cl, nseg, LV, g->dir_min, g->dir);
-        cudaFreeAsync(d_uniq, st);
-        cudaFreeAsync(d_vrank, st);
     } else {
         k_fill_u32<<<grid_for((int64_t)nseg + 1), NT, 0, st>>>(g->off, nseg + 1, 0u);
     }
-    cudaFreeAsync(keys, st);
-    cudaFreeAsync(tmp, st);
-
-    // signatures
-    GSI_CUDA_TRY(cudaMemsetAsync(g->sig, 0, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
-    k_sig_labels<<<grid_for(n), NT, 0, st>>>(d_vlab, n, g->sig);
-    if (m > 0) k_sig_pairs<<<grid_for(2 * m), NT, 0, st>>>(d_src, d_dst, d_elab, d_vlab, m, n, g->sig);
 
     // signatures grouped by label
     g->np = goff[LV];
     g->goff = goff;
     GSI_CUDA_TRY(cudaMallocAsync(&g->gperm, sizeof(int32_t) * (size_t)g->np, st));
     GSI_CUDA_TRY(cudaMallocAsync(&g->gsig, sizeof(uint32_t) * (size_t)(GSI_SIG_WORDS - 1) * (size_t)g->np, st));
-    GSI_CUDA_TRY(cudaMemcpyAsync(g->gperm, gperm.data(), sizeof(int32_t) * (size_t)g->np, cudaMemcpyHostToDevice, st));
+    int64_t *d_shift = nullptr;
+    GSI_TRY(tmps.alloc(&d_shift, (uint64_t)LV));
+    GSI_CUDA_TRY(cudaMemcpyAsync(d_shift, shift.data(), sizeof(int64_t) * (size_t)LV, cudaMemcpyHostToDevice, st));
+    GSI_CUDA_TRY(cudaMemsetAsync(g->gperm, 0xff, sizeof(int32_t) * (size_t)g->np, st));     // -1: padding
+    k_group_perm<<<grid_for(n), NT, 0, st>>>(sv, sr, d_shift, n, g->gperm);
     k_group_sig<<<grid_for(g->np), NT, 0, st>>>(g->sig, n, g->gperm, g->np, g->gsig);
 
-    // freq(l)
+    // freq(l): each edge has two entries
     unsigned long long *d_freq = nullptr;
-    GSI_CUDA_TRY(cudaMallocAsync(&d_freq, sizeof(unsigned long long) * (size_t)L, st));
+    GSI_TRY(tmps.alloc(&d_freq, (uint64_t)L));
     GSI_CUDA_TRY(cudaMemsetAsync(d_freq, 0, sizeof(unsigned long long) * (size_t)L, st));
-    if (m > 0) {
-        size_t sm = L <= 4096 ? sizeof(unsigned long long) * (size_t)L : 0;
-        k_label_hist<<<grid_for(m), NT, sm, st>>>(d_elab, m, L, d_freq);
+    {
+        const uint64_t threads = std::max<uint64_t>((uint64_t)L, 152 * 1024);
+        const uint64_t step = threads / (uint64_t)L * (uint64_t)L;
+        k_label_count<<<(unsigned)((step + NT - 1) / NT), NT, 0, st>>>(g->off, nseg, L, step, d_freq);
     }
     g->freq.assign((size_t)L, 0);
     GSI_CUDA_TRY(cudaMemcpyAsync(g->freq.data(), d_freq, sizeof(uint64_t) * (size_t)L, cudaMemcpyDeviceToHost, st));
-    cudaFreeAsync(d_freq, st);
-    cleanup_inputs();
     GSI_CUDA_TRY(cudaGetLastError());
     GSI_CUDA_TRY(cudaEventRecord(e1, st));
     GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    for (uint64_t &f : g->freq) f /= 2;
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
     cudaEventDestroy(e0);

@@ -45,10 +45,10 @@ struct gsi_graph {
 namespace gsi {
 
 // ------------------------------------------------------------------ sort
-// Ascending LSD radix sort of n keys over their low `bits` bits.  keys and
-// tmp hold n keys each; the result ends in keys.  Scratch is allocated
-// stream-ordered.
-gsi_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int bits, cudaStream_t st);
+// Ascending, stable LSD radix sort of n keys over their bits [lo, hi).  keys
+// and tmp hold n keys each; *sorted is the one that the result ends in.
+// Scratch is allocated stream-ordered.
+gsi_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int lo, int hi, uint64_t **sorted, cudaStream_t st);
 
 // ----------------------------------------------------------------- graph
 gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32_t *src, const int32_t *dst,
