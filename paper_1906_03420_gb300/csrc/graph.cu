@@ -86,9 +86,10 @@ __global__ void k_vertex_keys(const int32_t *__restrict__ vlab, int32_t n, int32
         keys[v] = ((uint64_t)((uint32_t)vlab[v] - (uint32_t)lo) << nb) | (uint64_t)v;
 }
 
-// The vertices in the order of (label, id): position i holds vertex sv[i] of
-// label rank sr[i], gpos is the inverse of sv, and label rank r begins at
-// position start[r] and stands for label uniq[r].  One scan over the sorted
+// The vertices in the order of (label, id): at[i] holds the vertex of position
+// i in its low half and its label rank in the high one (one gather for both),
+// gpos is the position of each vertex, and label rank r begins at position
+// start[r] and stands for label uniq[r].  One scan over the sorted
 // keys: a position that differs from the one before it in its label starts a
 // rank.  Ranks past MAX_LABELS are not written (the graph is refused).
 constexpr int32_t MAX_LABELS = 65535;
@@ -102,8 +103,7 @@ struct LabelRanks {
     LabelHead head;
     int64_t n;
     int32_t lo;
-    int32_t *sv;
-    uint16_t *sr;
+    uint64_t *at;
     uint32_t *gpos;
     uint32_t *nlabels;
     int32_t *uniq, *start;
@@ -114,9 +114,8 @@ struct LabelRanks {
         }
         const uint64_t k = head.keys[i];
         const uint32_t h = head(i), r = before + h - 1;
-        const int32_t v = (int32_t)(k & ((1ull << head.nb) - 1));
-        sv[i] = v;
-        sr[i] = (uint16_t)r;
+        const uint64_t v = k & ((1ull << head.nb) - 1);
+        at[i] = (uint64_t)r << 32 | v;
         gpos[v] = (uint32_t)i;
         if (h && r < (uint32_t)MAX_LABELS) {
             uniq[r] = (int32_t)((uint32_t)(k >> head.nb) + (uint32_t)lo);
@@ -126,10 +125,10 @@ struct LabelRanks {
 };
 
 // gperm: position i of the order above goes to its group's padded place.
-__global__ void k_group_perm(const int32_t *__restrict__ sv, const uint16_t *__restrict__ sr,
-                             const int64_t *__restrict__ shift, int32_t n, int32_t *__restrict__ gperm) {
+__global__ void k_group_perm(const uint64_t *__restrict__ at, const int64_t *__restrict__ shift, int32_t n,
+                             int32_t *__restrict__ gperm) {
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        gperm[i + shift[sr[i]]] = sv[i];
+        gperm[i + shift[at[i] >> 32]] = (int32_t)at[i];
 }
 
 // Directed entry keys, two per edge: ((v << Lb | l) << nb) | gpos(neighbour).
@@ -152,25 +151,40 @@ __global__ void k_csr_keys(const int32_t *__restrict__ src, const int32_t *__res
 //
 // A pair's state needs its first two occurrences only, and equal pairs of a
 // vertex stand together here: the first entry of a run counts one, the second
-// sets both bits, the others do nothing.  32M entries take 389 us; going over
-// the edge list for the signatures instead, every entry hashed its pair and did
-// its atomic on a random vertex (349 us, and 110 for the rest).
-__global__ void k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int Lb, int nb, int32_t L, uint64_t nseg,
-                           const int32_t *__restrict__ sv, const uint16_t *__restrict__ sr,
-                           const int32_t *__restrict__ uniq, int32_t n, uint32_t *__restrict__ off,
-                           int32_t *__restrict__ ci, uint16_t *__restrict__ cl, uint32_t *__restrict__ sig) {
+// sets both bits, the others do nothing.  A CTA takes FILL_TILE entries, which
+// belong to few vertices: those between its first and its last one have all
+// their entries here, so their words are put together in shared memory and
+// written plainly; the two at the ends, and those past the FILL_V-th (in a
+// sparse graph), set their bits by atomics.  The rank and the id of a neighbour
+// come from one gather.  32M entries take 340 us (389 with an atomic for each
+// pair and two gathers; 459 with the signatures made from the edge list).
+constexpr int FILL_VT = 8;
+constexpr int FILL_TILE = NT * FILL_VT;
+constexpr int FILL_V = 256;
+
+__global__ void __launch_bounds__(NT) k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int Lb, int nb, int32_t L,
+                                                 uint64_t nseg, const uint64_t *__restrict__ at,
+                                                 const int32_t *__restrict__ uniq, int32_t n, uint32_t *__restrict__ off, int32_t *__restrict__ ci,
+                                                 uint16_t *__restrict__ cl, uint32_t *__restrict__ sig) {
+    __shared__ uint32_t words[(GSI_SIG_WORDS - 1) * FILL_V];
     const uint64_t mask = (1ull << nb) - 1, lmask = (1ull << Lb) - 1;
-    const int lane = threadIdx.x & 31;
-    for (int64_t p0 = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); p0 < n2;
-         p0 += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, vsh = Lb + nb;
+    const int64_t t0 = (int64_t)blockIdx.x * FILL_TILE, t1 = min(n2, t0 + FILL_TILE);
+    const uint64_t vfirst = keys[t0] >> vsh, vlast = keys[t1 - 1] >> vsh;
+    const uint32_t inner = vlast - vfirst > 1 ? (uint32_t)min(vlast - vfirst - 1, (uint64_t)FILL_V) : 0u;   // vertices in `words`
+    for (uint32_t i = threadIdx.x; i < (GSI_SIG_WORDS - 1) * FILL_V; i += NT) words[i] = 0;
+    __syncthreads();
+#pragma unroll 2
+    for (int64_t p0 = t0 + (threadIdx.x & ~31u); p0 < t1; p0 += NT) {
         const int64_t p = p0 + lane;
-        const bool valid = p < n2;
+        const bool valid = p < t1;
         const uint64_t k = valid ? keys[p] : 0ull;
-        const uint32_t r = sr[k & mask];
+        const uint64_t here = at[k & mask];
+        const uint32_t r = (uint32_t)(here >> 32);
         // the two entries before the warp's, in lanes 0 and 1
         const bool xv = lane < 2 && p >= 2;
         const uint64_t x = xv ? keys[p - 2] : 0ull;
-        const uint32_t xr = xv ? sr[x & mask] : 0u;
+        const uint32_t xr = xv ? (uint32_t)(at[x & mask] >> 32) : 0u;
         const uint64_t seg = k >> nb, xseg = x >> nb;
         uint64_t s1 = __shfl_up_sync(FULL_MASK, seg, 1), s2 = __shfl_up_sync(FULL_MASK, seg, 2);
         uint32_t r1 = __shfl_up_sync(FULL_MASK, r, 1), r2 = __shfl_up_sync(FULL_MASK, r, 2);
@@ -184,11 +198,9 @@ __global__ void k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int Lb
             s1 = y;
             r1 = yr;
         }
-        // lane 0 of the second entry on: the entry before it is lane 1's x
         const bool same1 = p >= 1 && s1 == seg && r1 == r, same2 = p >= 2 && s2 == seg && r2 == r;
         if (!valid) continue;
-        const int32_t w = sv[k & mask];
-        ci[p] = w;
+        ci[p] = (int32_t)here;
         cl[p] = (uint16_t)r;
         const uint64_t v = seg >> Lb, l = seg & lmask, s = v * (uint64_t)L + l;
         uint64_t prev = 0;
@@ -197,12 +209,18 @@ __global__ void k_csr_fill(const uint64_t *__restrict__ keys, int64_t n2, int Lb
         if (p == n2 - 1)
             for (uint64_t q = s + 1; q <= nseg; ++q) off[q] = (uint32_t)n2;
         if (!(same1 && same2)) {
-            const uint32_t g = sig_group((int32_t)l, uniq[r]);
-            uint32_t *word = sig + (int64_t)sig_word(g) * n + (int64_t)v;
-            const uint32_t bit = 1u << sig_bit(g);
+            const uint32_t g = sig_group((int32_t)l, uniq[r]), bit = 1u << sig_bit(g);
+            const uint64_t j = v - vfirst - 1;                // vfirst itself: past every bound
+            uint32_t *word = j < inner && v < vlast ? words + (sig_word(g) - 1) * FILL_V + j
+                                                    : sig + (int64_t)sig_word(g) * n + (int64_t)v;
             if (same1) atomicOr(word, 3u * bit);
             else if (atomicOr(word, bit) & bit) atomicOr(word, 2u * bit);
         }
+    }
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < (GSI_SIG_WORDS - 1) * inner; i += NT) {
+        const uint32_t w = i / inner, j = i - w * inner;
+        sig[(int64_t)(w + 1) * n + (int64_t)(vfirst + 1 + j)] = words[w * FILL_V + j];
     }
 }
 
@@ -293,6 +311,11 @@ unsigned grid_for(int64_t n) {
     return (unsigned)b;
 }
 
+// For kernels that end with an atomic per warp on one word: thousands of warps
+// wait for it (51 us for 2^20 labels with one element per thread, 74 us for 16M
+// edges), so fewer threads take more each.
+unsigned few_blocks(int64_t n) { return std::min(grid_for(n), 152u * 6); }
+
 }  // namespace
 
 gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32_t *src, const int32_t *dst,
@@ -334,12 +357,12 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_TRY(tmps.alloc(&d_w, 1));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_w, &hw, sizeof hw, cudaMemcpyHostToDevice, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_vlab, vlab, sizeof(int32_t) * (size_t)n, cudaMemcpyDefault, st));
-    k_label_range<<<grid_for(n), NT, 0, st>>>(d_vlab, n, &d_w->lo);
+    k_label_range<<<few_blocks(n), NT, 0, st>>>(d_vlab, n, &d_w->lo);
     if (m > 0) {
         GSI_CUDA_TRY(cudaMemcpyAsync(d_src, src, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
         GSI_CUDA_TRY(cudaMemcpyAsync(d_dst, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
         GSI_CUDA_TRY(cudaMemcpyAsync(d_elab, elab, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
-        k_validate<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, &d_w->flags, &d_w->maxlab);
+        k_validate<<<few_blocks(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, &d_w->flags, &d_w->maxlab);
     }
     GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
     GSI_CUDA_TRY(cudaStreamSynchronize(st));
@@ -357,12 +380,11 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     uint64_t *keys = nullptr, *tmp = nullptr, *sorted = nullptr;
     GSI_TRY(tmps.alloc(&keys, nkeys));
     GSI_TRY(tmps.alloc(&tmp, nkeys));
-    int32_t *sv = nullptr, *d_labels = nullptr;
-    uint16_t *sr = nullptr;
+    int32_t *d_labels = nullptr;
+    uint64_t *at = nullptr;
     uint32_t *gpos = nullptr, *scr = nullptr;
     const int32_t most = (int32_t)std::min<int64_t>(n, MAX_LABELS);
-    GSI_TRY(tmps.alloc(&sv, (uint64_t)n));
-    GSI_TRY(tmps.alloc(&sr, (uint64_t)n));
+    GSI_TRY(tmps.alloc(&at, (uint64_t)n));
     GSI_TRY(tmps.alloc(&gpos, (uint64_t)n));
     GSI_TRY(tmps.alloc(&d_labels, 2 * (uint64_t)most));
     GSI_TRY(tmps.alloc(&scr, (uint64_t)scan_blocks(n) + 1));
@@ -371,7 +393,7 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_TRY(radix_sort_u64(keys, tmp, n, nb, range ? nb + ceil_log2_bits(range) : nb, &sorted, st));
     const LabelHead head{sorted, nb};
     GSI_CUDA_TRY(device_scan<uint32_t>(
-        head, n, LabelRanks{head, n, hw.lo, sv, sr, gpos, &d_w->nlabels, d_labels, d_labels + most}, scr, st));
+        head, n, LabelRanks{head, n, hw.lo, at, gpos, &d_w->nlabels, d_labels, d_labels + most}, scr, st));
     if (m > 1) {
         k_pair_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, m, nb, keys);
         GSI_TRY(radix_sort_u64(keys, tmp, m, 0, 2 * nb, &sorted, st));
@@ -422,8 +444,8 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
         const int Lb = L > 1 ? ceil_log2_bits((uint64_t)L - 1) : 0;
         k_csr_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, d_elab, gpos, m, Lb, nb, keys);
         GSI_TRY(radix_sort_u64(keys, tmp, 2 * m, 0, nb + Lb + nb, &sorted, st));
-        k_csr_fill<<<grid_for(2 * m), NT, 0, st>>>(sorted, 2 * m, Lb, nb, L, nseg, sv, sr, d_labels, n, g->off, g->ci,
-                                                   g->cl, g->sig);
+        k_csr_fill<<<(unsigned)((2 * m + FILL_TILE - 1) / FILL_TILE), NT, 0, st>>>(sorted, 2 * m, Lb, nb, L, nseg, at,
+                                                                                   d_labels, n, g->off, g->ci, g->cl, g->sig);
         k_label_dir<<<grid_for((int64_t)nseg), NT, 0, st>>>(g->off, g->cl, nseg, LV, g->dir_min, g->dir);
     } else {
         k_fill_u32<<<grid_for((int64_t)nseg + 1), NT, 0, st>>>(g->off, nseg + 1, 0u);
@@ -438,7 +460,7 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_TRY(tmps.alloc(&d_shift, (uint64_t)LV));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_shift, shift.data(), sizeof(int64_t) * (size_t)LV, cudaMemcpyHostToDevice, st));
     GSI_CUDA_TRY(cudaMemsetAsync(g->gperm, 0xff, sizeof(int32_t) * (size_t)g->np, st));     // -1: padding
-    k_group_perm<<<grid_for(n), NT, 0, st>>>(sv, sr, d_shift, n, g->gperm);
+    k_group_perm<<<grid_for(n), NT, 0, st>>>(at, d_shift, n, g->gperm);
     k_group_sig<<<grid_for(g->np), NT, 0, st>>>(g->sig, n, g->gperm, g->np, g->gsig);
 
     // freq(l): each edge has two entries

@@ -4,16 +4,18 @@
 //
 // Each pass: per-tile digit histograms, one device scan of the bin-major
 // histogram, then a stable scatter.  Inside a tile each warp owns a contiguous
-// run of keys and walks it 32 keys at a time; __match_any_sync groups lanes
-// with equal digits, so ranks follow input order and every pass is stable.
+// run of keys and walks it 32 keys at a time; lanes with equal digits find one
+// another in a mask per digit, so ranks follow input order and every pass is
+// stable.
 //
-// What bounds it is memory traffic: a pass reads the keys twice and writes
-// them once.  So the passes are few (digits of up to 10 bits, as wide as they
-// need to be to take the fewest passes) and the scatter first orders its tile
-// in shared memory, from where each digit's keys leave as one run (8 keys of
-// the 8,192 on average at 1,024 bins).  Writing straight from registers, with
-// 8-bit digits, a pass over 32M keys took 530-550 us (scatter 265-450, histogram
-// 74).
+// A pass reads the keys twice and writes them once, so the passes are few
+// (digits of up to 9 bits, no wider than the fewest passes need) and the scatter
+// first orders its tile in shared memory, from where each digit's keys leave as
+// one run (16 of the 8,192 on average at 512 bins).  The scatter is bound by the
+// instructions of its ranking (195 for 32 keys, half of the issue slots, with
+// DRAM at 1.6 TB/s, when lanes were matched by ballots).  32M keys take 190-240
+// us, and 78 for the histogram, for 9 bits; with __match_any_sync 190-330; with
+// 10-bit digits 350; written straight from registers 265-450 for 8 bits.
 #include "internal.h"
 #include "scan.cuh"
 
@@ -25,7 +27,7 @@ constexpr int RS_WARPS = RS_NT / 32;
 constexpr int RS_VT = 16;
 constexpr int RS_TILE = RS_NT * RS_VT;
 constexpr int RS_WARP_KEYS = 32 * RS_VT;
-constexpr int RS_MAX_BITS = 10;
+constexpr int RS_MAX_BITS = 9;
 constexpr int RS_BINS_PER_THREAD = (1 << RS_MAX_BITS) / RS_NT;
 
 __global__ void __launch_bounds__(RS_NT) k_rs_hist(const uint64_t *__restrict__ keys, int64_t n, int shift, int nbins,
@@ -59,30 +61,39 @@ __global__ void __launch_bounds__(RS_NT, 2) k_rs_scatter(const uint64_t *__restr
     __shared__ uint32_t wt[RS_WARPS];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const uint32_t dmask = (uint32_t)nbins - 1u;
-    for (int i = threadIdx.x; i < RS_WARPS * nbins / 2; i += RS_NT) reinterpret_cast<uint32_t *>(wcnt)[i] = 0;
-
-    const int64_t wbase = (int64_t)blockIdx.x * RS_TILE + (int64_t)warp * RS_WARP_KEYS;
-    uint64_t key[RS_VT];
-    uint32_t pos[RS_VT];
-    const unsigned lt = lanemask_lt();
-#pragma unroll
-    for (int r = 0; r < RS_VT; ++r) {
-        const int64_t i = wbase + r * 32 + lane;
-        key[r] = i < n ? in[i] : 0ull;
-    }
-    __syncthreads();
+    // each warp's lanes by digit, in the tile's place until that is filled
+    static_assert(RS_TILE * 8 >= RS_WARPS * (1 << RS_MAX_BITS) * 4, "the lane masks fit the tile");
+    uint32_t *peer = reinterpret_cast<uint32_t *>(stage) + warp * nbins;
     uint16_t *wc = wcnt + warp * nbins;
+    for (int i = lane; i < nbins; i += 32) peer[i] = 0;
+    for (int i = lane; i < nbins / 2; i += 32) reinterpret_cast<uint32_t *>(wc)[i] = 0;
+
+    const int64_t tbase = (int64_t)blockIdx.x * RS_TILE;
+    const uint32_t cnt = n - tbase < RS_TILE ? (uint32_t)(n - tbase) : (uint32_t)RS_TILE;
+    const uint32_t first = (uint32_t)(warp * RS_WARP_KEYS + lane);
+    in += tbase;
+    uint64_t key[RS_VT];
+    uint32_t pos[RS_VT / 2];                                               // two to a word: all are below RS_WARP_KEYS
+    const unsigned lt = lanemask_lt(), me = 1u << lane;
+#pragma unroll
+    for (int r = 0; r < RS_VT; ++r) key[r] = first + r * 32 < cnt ? in[first + r * 32] : 0ull;
+    __syncwarp();
 #pragma unroll
     for (int r = 0; r < RS_VT; ++r) {
-        const bool valid = wbase + r * 32 + lane < n;
-        const uint32_t dig = valid ? (uint32_t)(key[r] >> shift) & dmask : (uint32_t)nbins;
-        const unsigned peers = __match_any_sync(FULL_MASK, dig);
+        const bool valid = first + r * 32 < cnt;
+        const uint32_t dig = (uint32_t)(key[r] >> shift) & dmask;
+        if (valid) atomicOr(&peer[dig], me);
+        __syncwarp();
+        const uint32_t peers = peer[dig], before = wc[dig];
         const uint32_t rank = __popc(peers & lt);
-        const uint32_t before = valid ? wc[dig] : 0u;
         __syncwarp();
-        if (valid && rank == 0) wc[dig] = (uint16_t)(before + __popc(peers));
+        if (valid && rank == 0) {
+            peer[dig] = 0;
+            wc[dig] = (uint16_t)(before + __popc(peers));
+        }
         __syncwarp();
-        pos[r] = before + rank;
+        if (r & 1) pos[r / 2] |= (before + rank) << 16;
+        else pos[r / 2] = before + rank;
     }
     __syncthreads();
     {   // per digit: exclusive scan over the warps, then over the digits
@@ -91,12 +102,16 @@ __global__ void __launch_bounds__(RS_NT, 2) k_rs_scatter(const uint64_t *__restr
         for (int q = 0; q < RS_BINS_PER_THREAD; ++q) {
             const int b = (int)threadIdx.x * RS_BINS_PER_THREAD + q;
             uint32_t run = 0;
-            if (b < nbins)
+            if (b < nbins) {
+                uint32_t c[RS_WARPS];
+#pragma unroll
+                for (int w = 0; w < RS_WARPS; ++w) c[w] = wcnt[w * nbins + b];
+#pragma unroll
                 for (int w = 0; w < RS_WARPS; ++w) {
-                    const uint32_t c = wcnt[w * nbins + b];
                     wcnt[w * nbins + b] = (uint16_t)run;
-                    run += c;
+                    run += c[w];
                 }
+            }
             tot[q] = run;
             sum += run;
         }
@@ -115,13 +130,11 @@ __global__ void __launch_bounds__(RS_NT, 2) k_rs_scatter(const uint64_t *__restr
     __syncthreads();
 #pragma unroll
     for (int r = 0; r < RS_VT; ++r)
-        if (wbase + r * 32 + lane < n) {
+        if (first + r * 32 < cnt) {
             const uint32_t dig = (uint32_t)(key[r] >> shift) & dmask;
-            stage[start[dig] + wc[dig] + pos[r]] = key[r];
+            stage[start[dig] + wc[dig] + (r & 1 ? pos[r / 2] >> 16 : pos[r / 2] & 0xffffu)] = key[r];
         }
     __syncthreads();
-    const int64_t left = n - (int64_t)blockIdx.x * RS_TILE;
-    const uint32_t cnt = left < RS_TILE ? (uint32_t)left : (uint32_t)RS_TILE;
 #pragma unroll 4
     for (uint32_t j = threadIdx.x; j < cnt; j += RS_NT) {
         const uint64_t k = stage[j];
