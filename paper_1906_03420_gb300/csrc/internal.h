@@ -146,14 +146,15 @@ struct DStep {
     unsigned long long count;          // survivors (exact even past out_cap); [0]: seed size
     unsigned long long nlong;          // rows set aside for the slot tiles and their slots (LongTable::ctr)
     uint64_t out_cap;
+    unsigned fail;                     // 1: this step's long-row table was full (a step of its own reads it, so
+    unsigned pad;                      // that no CTA sees a later step's failure and leaves the others waiting)
 };
 
 // Grid-barrier and status words of one cooperative query launch.
 struct QueryCtl {
-    unsigned bar_count, bar_gen;
+    unsigned bar;         // arrivals at the barriers so far; BAR_FAIL: a wait gave up
     unsigned fail;        // 1 scratch too small (or a sub-list too long for a bound record),
                           // 2 table overflow, 4 barrier wait gave up
-    unsigned pad;
     unsigned long long spin_limit;   // sleeps before a barrier wait gives up (0 = default)
 };
 constexpr int QUERY_MAX_CTAS = 2048;

@@ -121,48 +121,65 @@ __global__ void __launch_bounds__(NT) k_join(const __grid_constant__ JoinArgs a)
 // every CTA that later sees the bit, so the kernel always terminates.
 
 constexpr unsigned long long BARRIER_SPIN_LIMIT = 1ull << 24;   // x ~64 ns sleeps: about a second
+constexpr unsigned BAR_FAIL = 1u << 31;
 
-__device__ __forceinline__ bool grid_barrier(QueryCtl *ctl, unsigned nblocks) {
-    const unsigned long long limit = ctl->spin_limit ? ctl->spin_limit : BARRIER_SPIN_LIMIT;
-    __shared__ int ok_s;
+// What a barrier hands to its CTA: the step's counters as of the barrier, read
+// by the thread that waited.
+struct BarrierView {
+    unsigned long long count, nlong;
+    unsigned fail;
+    int ok;
+};
+
+// One word counts the arrivals of all barriers of the launch, so a CTA knows
+// the number to wait for (epoch: barriers passed), the last one to arrive has
+// nothing to reset or release, and a wait that gave up shows in the same word.
+// A step of few rows costs little but its chain of L2 round trips (some 0.6 us
+// each): a generation word, a fail word and counters that all 4,864 warps read
+// for themselves took 2.3 us at least for a barrier and 2-3 us for the start of
+// a step; now 1.6 and 0.3 us (a 4-vertex query on 1,000 vertices: 42 -> 33 us).
+__device__ __forceinline__ bool grid_barrier(QueryCtl *ctl, unsigned nblocks, unsigned &epoch, const DStep *st,
+                                             BarrierView *view) {
     __syncthreads();
+    ++epoch;
     if (threadIdx.x == 0) {
-        volatile unsigned *gen = &ctl->bar_gen;
-        volatile unsigned *fail = &ctl->fail;
-        const unsigned g = *gen;
+        const unsigned long long limit = ctl->spin_limit ? ctl->spin_limit : BARRIER_SPIN_LIMIT;
+        const unsigned target = epoch * nblocks;
         __threadfence();
-        const unsigned arrived = atomicAdd(&ctl->bar_count, 1u);
-        int ok = 1;
-        if (arrived == nblocks - 1) {
-            ctl->bar_count = 0;
-            __threadfence();
-            atomicAdd(&ctl->bar_gen, 1u);
-        } else {
-            unsigned long long spins = 0;
-            while (*gen == g) {
-                if (*fail & 4u) { ok = 0; break; }
-                if (++spins > limit) {
-                    atomicOr(&ctl->fail, 4u);
-                    ok = 0;
-                    break;
-                }
-                __nanosleep(64);
+        unsigned v = atomicAdd(&ctl->bar, 1u) + 1u;
+        for (unsigned long long spins = 0; v < target;) {     // BAR_FAIL ends it too
+            if (++spins > limit) {
+                atomicOr(&ctl->fail, 4u);
+                v = atomicOr(&ctl->bar, BAR_FAIL) | BAR_FAIL;
+                break;
             }
+            if (spins > 1) __nanosleep(64);
+            asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&ctl->bar) : "memory");
         }
         __threadfence();
-        ok_s = ok && !(*fail & 4u);
+        view->ok = v < BAR_FAIL;
+        if (st) {
+            view->count = __ldcg(&st->count);
+            view->nlong = __ldcg(&st->nlong);
+            view->fail = __ldcg(&st->fail);
+        }
     }
     __syncthreads();
-    return ok_s != 0;
+    return view->ok != 0;
 }
 
-// Copies a struct of 4-byte words with the whole CTA.
+// Copies a struct of 8-byte words to shared memory with the whole CTA, behind
+// what it does next: complete after copy_wait and a barrier.
 template <int NT, typename T>
 __device__ __forceinline__ void copy_words(T *dst, const T *src) {
-    static_assert(sizeof(T) % 4 == 0, "whole words");
-    for (int i = threadIdx.x; i < (int)(sizeof(T) / 4); i += NT)
-        reinterpret_cast<uint32_t *>(dst)[i] = reinterpret_cast<const uint32_t *>(src)[i];
+    static_assert(sizeof(T) % 8 == 0 && alignof(T) >= 8, "whole words");
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    for (unsigned i = threadIdx.x; i < (unsigned)(sizeof(T) / 8); i += NT)
+        asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(d + 8 * i),
+                     "l"(reinterpret_cast<const unsigned char *>(src) + 8 * i)
+                     : "memory");
 }
+__device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int NT, bool LW>
 __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cfgs, DStep *steps, int k, QueryCtl *ctl,
@@ -172,7 +189,9 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
     __shared__ unsigned long long at_s;
     __shared__ __align__(16) JoinArgs args_s[2];      // this step's configuration and the next one's
     __shared__ __align__(16) DStepIn ins_s[2];
+    __shared__ BarrierView view_s;
     const unsigned G = gridDim.x;
+    unsigned epoch = 0;
     copy_words<NT>(&args_s[1], cfgs + 1);
     copy_words<NT>(&ins_s[1], &steps[1].in);
 
@@ -195,16 +214,18 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
             for (pos += at_s; x; x &= x - 1) seed_out[pos++] = (int32_t)(i * 32 + (uint64_t)(__ffs(x) - 1));
             __syncthreads();
         }
-        if (!grid_barrier(ctl, G)) return;
+        copy_wait();
+        if (!grid_barrier(ctl, G, epoch, steps, &view_s)) return;
     }
 
+    uint64_t prev_cap = ~0ull;                                // rows that the step's input region holds
     for (int t = 1; t < k; ++t) {
         DStep *st = steps + t;
         const JoinArgs &a = args_s[t & 1];
         const DStepIn &in_s = ins_s[t & 1];
-        const uint64_t R = __ldcg(&steps[t - 1].count);
+        const uint64_t R = view_s.count;
         // the previous table must have fit its region
-        if (t > 1 && R > __ldcg(&steps[t - 1].out_cap)) {
+        if (R > prev_cap) {
             if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->fail, 2u);
             return;
         }
@@ -219,17 +240,18 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         if (in_s.row_cap && in_s.row_cap < cap) cap = in_s.row_cap;
         if (in_s.count_only) cap = 0;
         if (blockIdx.x == 0 && threadIdx.x == 0) st->out_cap = cap;
+        prev_cap = cap;
         // ---- short rows joined inline, long rows set aside (one pass over M)
         unsigned long long abytes = 0, items = 0, lbytes = 0;
         // neighbouring runs of warp work go to different SMs
         const unsigned warp = threadIdx.x >> 5;
         const uint64_t wi = (uint64_t)warp * G + blockIdx.x, nw = (uint64_t)G * (NT / 32);
         if (a.mult) {                                         // a counting query's last step
-            count_tail<LW>(a, in_s.M, R, wi, nw, lt, &ctl->fail, &st->count, &abytes, &items, &lbytes);
+            count_tail<LW>(a, in_s.M, R, wi, nw, lt, &st->fail, &st->count, &abytes, &items, &lbytes);
         } else {
             const int nb = batch_rows(R, G, NT * ROW_RPT);
             row_pass<NT, true, ROW_RPT, LW>(a, in_s.M, R, (uint64_t)blockIdx.x * nb, (uint64_t)G * nb, nb, out, cap,
-                                            &st->count, lt, &ctl->fail, smem, &abytes, &items, &lbytes);
+                                            &st->count, lt, &st->fail, smem, &abytes, &items, &lbytes);
         }
         if (a.stats) {                       // one add per CTA and step
             abytes = block_sum<NT, unsigned long long>(abytes, wt);
@@ -241,18 +263,22 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
                 if (lbytes) atomicAdd(a.stats + 2, lbytes);
             }
         }
-        if (!grid_barrier(ctl, G)) return;
-        if (__ldcg(&ctl->fail) & 1u) return;                  // long-row table full: a larger arena
+        copy_wait();
+        if (!grid_barrier(ctl, G, epoch, st, &view_s)) return;
+        if (view_s.fail) {                                    // long-row table full: a larger arena
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->fail, 1u);
+            return;
+        }
         // ---- long rows through the candidate-slot tiles
-        const uint64_t ctr = __ldcg(&st->nlong), L = ctr & ((1ull << lt.rbits) - 1ull), total = ctr >> lt.rbits;
+        const uint64_t ctr = view_s.nlong, L = ctr & ((1ull << lt.rbits) - 1ull), total = ctr >> lt.rbits;
         if (L > 0) {
             unsigned char *const sm = smem + warp * long_warp_smem(t, a.s.d);
             if (a.mult) long_rows_join<true>(a, lt, L, total, wi, nw, out, 0, &st->count, sm);
             else long_rows_join<false>(a, lt, L, total, wi, nw, out, cap, &st->count, sm);
-            if (!grid_barrier(ctl, G)) return;
+            if (!grid_barrier(ctl, G, epoch, st, &view_s)) return;
         }
         if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) {      // survivors written (both models)
-            const unsigned long long wbytes = 4ull * (uint64_t)(t + 1) * min((uint64_t)__ldcg(&st->count), cap);
+            const unsigned long long wbytes = 4ull * (uint64_t)(t + 1) * min((uint64_t)view_s.count, cap);
             atomicAdd(a.stats, wbytes);
             if (LW) atomicAdd(a.stats + 2, wbytes);
         }
@@ -261,7 +287,9 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
 
 __global__ void k_barrier_selftest(QueryCtl *ctl, unsigned expect) {
     // every CTA waits at a barrier that expects one CTA more than exist
-    grid_barrier(ctl, expect);
+    __shared__ BarrierView view_s;
+    unsigned epoch = 0;
+    grid_barrier(ctl, expect, epoch, nullptr, &view_s);
 }
 
 std::once_flag g_join_attr_once[64];
