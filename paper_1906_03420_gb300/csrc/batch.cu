@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
             if (L > 0) {
                 // the long rows' slot tiles, CTA-local
                 const unsigned warp = threadIdx.x >> 5;
-                long_rows_join<false>(a, lt, L, total, warp, BNT / 32, out, cap, &cnt_s, smem + warp * long_warp_smem(t, a.s.d));
+                long_rows_join(a, lt, L, total, warp, BNT / 32, out, cap, &cnt_s, smem + warp * long_warp_smem(t, a.s.d));
             }
             __syncthreads();
             discard_l2<BNT>(M, R * (uint64_t)t * 4);    // this step's input is dead

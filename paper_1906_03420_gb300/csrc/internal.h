@@ -145,6 +145,7 @@ struct DStep {
     // set on the device
     unsigned long long count;          // survivors (exact even past out_cap); [0]: seed size
     unsigned long long nlong;          // rows set aside for the slot tiles and their slots (LongTable::ctr)
+    unsigned long long row_ticket, slot_ticket;   // the work handed out on demand (row_pass, long_rows_join)
     uint64_t out_cap;
     unsigned fail;                     // 1: this step's long-row table was full (a step of its own reads it, so
     unsigned pad;                      // that no CTA sees a later step's failure and leaves the others waiting)

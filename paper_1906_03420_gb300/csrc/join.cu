@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         } else {
             const int nb = batch_rows(R, G, NT * ROW_RPT);
             row_pass<NT, true, ROW_RPT, LW>(a, in_s.M, R, (uint64_t)blockIdx.x * nb, (uint64_t)G * nb, nb, out, cap,
-                                            &st->count, lt, &st->fail, smem, &abytes, &items, &lbytes);
+                                            &st->count, lt, &st->fail, smem, &abytes, &items, &lbytes, &st->row_ticket);
         }
         if (a.stats) {                       // one add per CTA and step
             abytes = block_sum<NT, unsigned long long>(abytes, wt);
@@ -273,8 +273,8 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         const uint64_t ctr = view_s.nlong, L = ctr & ((1ull << lt.rbits) - 1ull), total = ctr >> lt.rbits;
         if (L > 0) {
             unsigned char *const sm = smem + warp * long_warp_smem(t, a.s.d);
-            if (a.mult) long_rows_join<true>(a, lt, L, total, wi, nw, out, 0, &st->count, sm);
-            else long_rows_join<false>(a, lt, L, total, wi, nw, out, cap, &st->count, sm);
+            if (a.mult) long_rows_mode<LONG_TAIL>(a, lt, L, total, wi, nw, out, 0, &st->count, sm, &st->slot_ticket);
+            else long_rows_join(a, lt, L, total, wi, nw, out, cap, &st->count, sm, &st->slot_ticket);
             if (!grid_barrier(ctl, G, epoch, st, &view_s)) return;
         }
         if (a.stats && blockIdx.x == 0 && threadIdx.x == 0) {      // survivors written (both models)

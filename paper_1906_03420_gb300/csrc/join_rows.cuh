@@ -132,15 +132,15 @@ __device__ __forceinline__ void stage_rows(int32_t *dst, const int32_t *__restri
     }
 }
 
-// Rows that one CTA takes at a time when R rows meet G CTAs: all of NB once
-// there are enough rows to fill every CTA, fewer below (a table of 9,000 rows
-// is spread over the whole GPU in pieces of 16, instead of over ten CTAs: a
+// Rows that one CTA takes at a time when R rows meet G CTAs: at most NB, and
+// as few as make every CTA take the same number of batches (a table of 9,000
+// rows is spread over the whole GPU in pieces of 16, instead of over ten CTAs: a
 // step of so few rows is bound by the latency of one batch, 12-20 us when its
 // threads were all in a few CTAs), in multiples of 8 so that a batch starts on
 // 16 bytes whatever its columns.
 __device__ __forceinline__ int batch_rows(uint64_t R, unsigned G, int NB) {
-    const uint64_t per = (R + G - 1) / G;
-    return per >= (uint64_t)NB ? NB : max(8, ((int)per + 7) & ~7);
+    const uint64_t per = (R + G - 1) / G, rounds = (per + NB - 1) / NB;
+    return min(NB, max(8, ((int)((per + rounds - 1) / rounds) + 7) & ~7));
 }
 
 // Length of the whole linking list N(v, lab[j]) (for the whole-list byte count).
@@ -400,7 +400,10 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
 // The row pass over rows [first, R) in batches of nbatch <= NT * RPT rows,
 // batch starts `stride` apart (a grid-strided pass: first = blockIdx.x *
 // nbatch, stride = gridDim.x * nbatch; one CTA alone: first = 0, stride =
-// nbatch).  `a` should live in shared memory.  Survivors go to out (up to cap rows; `count` is
+// nbatch).  With a ticket counter (zero before the step) only three quarters of
+// the batches go out that way, at least two to a CTA, and the rest on demand:
+// rows differ in their lists, and of a step of millions of rows a quarter of
+// the time went by while the last CTAs worked alone.  `a` should live in shared memory.  Survivors go to out (up to cap rows; `count` is
 // exact), long rows to lt.  Bit 1 of *fail is set when the long-row table is
 // full or a bound does not fit its record.  When a.stats is set, adds this
 // thread's algorithmic bytes (rows read, lists located and read; survivors
@@ -410,11 +413,12 @@ template <int NT, bool DR = true, int RPT = ROW_RPT, bool LW = true>
 __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64_t first, uint64_t stride, int nbatch,
                          int32_t *__restrict__ out, uint64_t cap, unsigned long long *count, const LongTable &lt,
                          unsigned *fail, unsigned char *smem, unsigned long long *abytes,
-                         unsigned long long *items, unsigned long long *lbytes) {
+                         unsigned long long *items, unsigned long long *lbytes,
+                         unsigned long long *ticket = nullptr) {
     constexpr int NW = NT / 32, NB = NT * RPT, CCAP = NB * ROW_SURV;
     __shared__ uint32_t wt[NW];
     __shared__ unsigned long long wts[NW];              // slots of each warp's long rows
-    __shared__ unsigned long long base_s, lbase_s;
+    __shared__ unsigned long long base_s, lbase_s, after_s;
     const int t = a.s.t, W1 = t + 1;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     int32_t *rowv = reinterpret_cast<int32_t *>(smem);                  // NB * t
@@ -426,11 +430,13 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
     // the rs-th of the warp's rpw rows per round
     const int rpw = 32 / W1, rs = lane / W1, oc = lane - rs * W1;
     const int src_col = a.iperm[oc < W1 ? oc : 0];
-    for (uint64_t r0 = first; r0 < R; r0 += stride) {
+    const uint64_t fixed = ticket ? max(2 * stride, R / stride * 3 / 4 * stride) : R;     // rows dealt by stride
+    uint64_t next = first + stride;
+    for (uint64_t r0 = first; r0 < R; r0 = next, next = after_s) {
         const int nb = (int)min((uint64_t)nbatch, R - r0);
         const int32_t *src = M + r0 * (uint64_t)t;
-        if (threadIdx.x == 0 && r0 + stride < R)      // the next batch's rows, while this one runs
-            prefetch_l2(M + (r0 + stride) * (uint64_t)t, min((uint64_t)nbatch, R - r0 - stride) * (uint64_t)t * 4);
+        if (threadIdx.x == 0 && next < R)             // the next batch's rows, while this one runs
+            prefetch_l2(M + next * (uint64_t)t, min((uint64_t)nbatch, R - next) * (uint64_t)t * 4);
         stage_rows<NT>(rowv, src, nb * t);
         __syncthreads();
         // this thread's rows q * NT + tid, q < RPT (a warp's lanes hold
@@ -506,6 +512,9 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
         }
         const uint32_t ntot = tot & 0xffffu, ltot = tot >> 16;
         if (threadIdx.x == 0) {                 // read after the next barrier
+            after_s = next + stride;
+            if (after_s >= fixed && ticket && next < R)
+                after_s = fixed + atomicAdd(ticket, 1ull) * (uint64_t)nbatch;
             base_s = ntot ? atomicAdd(count, (unsigned long long)ntot) : 0ull;
             if (ltot) {
                 const unsigned long long old = atomicAdd(lt.ctr, (stot << lt.rbits) | (unsigned long long)ltot);
@@ -616,15 +625,25 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
 // The slot tiles: warp wi of nw takes an equal, contiguous run of the table's
 // slots, in tiles of LW_SLOTS, and works alone: no barrier, no map of the tile
 // in shared memory.  The warp finds its first row with one 32-way search of F
-// and from then on walks the table.  In each tile its lanes
+// and from then on walks the table.  With a ticket counter (zero before the
+// step) and runs long enough to pay for more searches (3 us each), a quarter of
+// the slots, three quarters of long runs, is left for pieces a thirty-second as
+// long that warps take on demand: slots differ in what they find, and the warps
+// had been waiting for the last ones for a quarter of the time.  In each tile its lanes
 //   * load the records of the rows that meet the tile (at most LW_ROWS, as
 //     every long row has more than SHORT_MAX slots) and stage their columns;
 //   * find their slots' rows from one 32-bit mask of row starts per group of
 //     32 slots;
 //   * load LW_SLOTS / 32 candidates and then as many bitmap words each, all in
 //     flight together;
-//   * test set subtraction and the other lists (label sub-lists, from the
-//     step's memo or searched), and compact the survivors by ballots.
+//   * test set subtraction and compact what is left by ballots;
+//   * search it in the other lists (label sub-lists, from the step's memo or
+//     searched), LW_Q candidates a lane in lockstep, and compact again: most
+//     candidates are not in C(u), and searched in their slots' lanes, one after
+//     the other, the rest kept few lanes and one load of each in flight (849M
+//     slots of rows with three lists took 15.3 ms, 14.0 with a part dealt on
+//     demand and 11.4 with both; steps of one list have a variant without it,
+//     as its registers cost them 10%).
 // One atomic per tile places the survivors, which the warp writes as one
 // coalesced run.  What bounds it is the latency of the two rounds of loads
 // (candidates, bitmap words) times the warps in flight.  CTA-wide tiles of
@@ -635,42 +654,61 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
 constexpr int LW_SLOTS = 256;
 constexpr int LW_G = LW_SLOTS / 32;
 constexpr int LW_ROWS = LW_SLOTS / (SHORT_MAX + 1) + 2;
+constexpr int LW_Q = 4;                               // candidates a lane searches for in lockstep
+constexpr uint64_t LW_DEAL = 1024;                    // slots a warp from which a part is dealt on demand
 
 // Shared memory of one warp: survivors (value, local row), rows, other lists.
 __host__ __device__ constexpr size_t long_warp_smem(int t, int d) {
     return ((size_t)LW_SLOTS * 5 + (size_t)LW_ROWS * ((size_t)t * 4 + (size_t)(d - 1) * 8) + 15) / 16 * 16;
 }
 
-// TAIL (see count_tail): the table's rows are vertices, each standing for
+// LONG_TAIL (see count_tail): the table's rows are vertices, each standing for
 // a.mult[v] rows; no set subtraction and no other lists.
-template <bool TAIL>
-__device__ inline void long_rows_join(const JoinArgs &a, const LongTable &lt, uint64_t L, uint64_t total, uint64_t wi,
+enum { LONG_SINGLE, LONG_MULTI, LONG_TAIL };
+
+template <int MODE>
+__device__ inline void long_rows_mode(const JoinArgs &a, const LongTable &lt, uint64_t L, uint64_t total, uint64_t wi,
                                       uint64_t nw, int32_t *__restrict__ out, uint64_t cap, unsigned long long *count,
-                                      unsigned char *smem) {
+                                      unsigned char *smem, unsigned long long *ticket = nullptr) {
     const int lane = threadIdx.x & 31;
-    const int t = TAIL ? 1 : a.s.t, d = TAIL ? 1 : a.s.d, dm1 = d - 1, W1 = t + 1;
+    constexpr bool TAIL = MODE == LONG_TAIL, MULTI = MODE == LONG_MULTI;
+    const int t = TAIL ? 1 : a.s.t, d = MULTI ? a.s.d : 1, dm1 = d - 1, W1 = t + 1;
     int32_t *sw = reinterpret_cast<int32_t *>(smem);
     int32_t *rowv = sw + LW_SLOTS;                                   // LW_ROWS * t
     uint32_t *lst = reinterpret_cast<uint32_t *>(rowv + LW_ROWS * t);   // LW_ROWS * 2 * dm1
     unsigned char *sr = reinterpret_cast<unsigned char *>(lst + LW_ROWS * 2 * dm1);
     // small tables: at least 64 slots a warp, so that the search pays
     const uint64_t per = max((uint64_t)64, ((total + nw - 1) / nw + 31) / 32 * 32);
-    uint64_t s = wi * per;
-    const uint64_t w1 = min(total, s + per);
-    if (s >= w1) return;
-    // the row that holds slot s: the last with F <= s
-    uint64_t r = 0;
-    for (uint64_t hi = L; hi - r > 1;) {
-        const uint64_t step = (hi - r + 31) / 32, p = r + (uint64_t)(lane + 1) * step;
-        const int c = __popc(__ballot_sync(FULL_MASK, p < hi && __ldcg(lt.F + p) <= s));
-        r += (uint64_t)c * step;
-        hi = min(hi, r + step);
-    }
+    const bool deal = ticket && per >= LW_DEAL;
+    const bool most = per >= 8 * LW_DEAL;
+    const uint64_t run = deal ? max((uint64_t)1, (most ? per : 3 * per) / (4 * LW_SLOTS)) * LW_SLOTS : per;
+    const uint64_t piece = max((uint64_t)1, per / (32 * LW_SLOTS)) * LW_SLOTS;
+    uint64_t s = wi * run, w1 = min(total, s + run), r = 0;
+    bool found_row = false;
     const unsigned le = lanemask_lt() | (1u << lane);
     const int rpw = 32 / W1, rs = lane / W1, oc = lane - rs * W1;
     const int src_col = a.iperm[oc];
     unsigned long long found = 0;                     // counting only: this lane's survivors
-    while (s < w1) {
+    for (;;) {
+        if (s >= w1) {
+            if (!deal) break;
+            unsigned long long k = 0;
+            if (lane == 0) k = atomicAdd(ticket, 1ull);
+            s = nw * run + __shfl_sync(FULL_MASK, k, 0) * piece;
+            if (s >= total) break;
+            w1 = min(total, s + piece);
+            found_row = false;
+        }
+        if (!found_row) {                             // the row that holds slot s: the last with F <= s
+            found_row = true;
+            r = 0;
+            for (uint64_t hi = L; hi - r > 1;) {
+                const uint64_t step = (hi - r + 31) / 32, p = r + (uint64_t)(lane + 1) * step;
+                const int c = __popc(__ballot_sync(FULL_MASK, p < hi && __ldcg(lt.F + p) <= s));
+                r += (uint64_t)c * step;
+                hi = min(hi, r + step);
+            }
+        }
         const uint64_t e = min(s + (uint64_t)LW_SLOTS, w1);
         // lane j: the record of row r + j
         uint64_t Fj = ~0ull;
@@ -688,7 +726,7 @@ __device__ inline void long_rows_join(const JoinArgs &a, const LongTable &lt, ui
             for (int i = lane; i < nr * t; i += 32) rowv[i] = __ldcg(src + i);
         }
         __syncwarp();
-        if (dm1 > 0 && lane < nr) {
+        if (MULTI && lane < nr) {
             uint32_t *l = lst + lane * 2 * dm1;
             for (int j = 0; j < d; ++j) {
                 if (j == (int)jb) continue;
@@ -730,18 +768,78 @@ __device__ inline void long_rows_join(const JoinArgs &a, const LongTable &lt, ui
             }
             const int32_t *rv = rowv + row[g] * t;
             for (uint32_t im = a.s.inj; ok && im; im &= im - 1) ok = rv[__ffs(im) - 1] != w[g];
-            const uint32_t *l = lst + row[g] * 2 * dm1;
-            for (int j = 0; j < dm1 && ok; ++j) ok = sorted_contains(a.ci + l[2 * j], l[2 * j + 1], w[g]);
-            const unsigned b = __ballot_sync(FULL_MASK, ok);
-            if (a.count_only) {
+            if (!MULTI && a.count_only) {
                 found += ok;
-            } else {
-                if (ok) {
-                    const unsigned i = ns + __popc(b & le) - 1;
-                    sw[i] = w[g];
-                    sr[i] = (unsigned char)row[g];
+                continue;
+            }
+            const unsigned b = __ballot_sync(FULL_MASK, ok);
+            if (ok) {
+                const unsigned i = ns + __popc(b & le) - 1;
+                sw[i] = w[g];
+                sr[i] = (unsigned char)row[g];
+            }
+            ns += __popc(b);
+        }
+        if (MULTI && ns > 0) {
+            __syncwarp();
+            const unsigned n = ns;
+            ns = 0;
+            for (unsigned i0 = 0; i0 < n; i0 += 32 * LW_Q) {
+                int32_t x[LW_Q];
+                uint32_t rr[LW_Q];
+                bool ok[LW_Q];
+#pragma unroll
+                for (int q = 0; q < LW_Q; ++q) {
+                    const unsigned i = i0 + (unsigned)(q * 32 + lane);
+                    ok[q] = i < n;
+                    x[q] = ok[q] ? sw[i] : 0;
+                    rr[q] = ok[q] ? sr[i] : 0u;
                 }
-                ns += __popc(b);
+                for (int j = 0; j < dm1; ++j) {
+                    uint32_t at[LW_Q], m[LW_Q], end[LW_Q], left = 0;
+#pragma unroll
+                    for (int q = 0; q < LW_Q; ++q) {
+                        const uint32_t *l = lst + (rr[q] * (uint32_t)dm1 + (uint32_t)j) * 2;
+                        at[q] = l[0];
+                        m[q] = ok[q] ? l[1] : 0u;
+                        end[q] = at[q] + m[q];
+                        left |= m[q];
+                    }
+                    while (left) {                    // lower bounds, in lockstep
+                        left = 0;
+                        int32_t y[LW_Q];
+#pragma unroll
+                        for (int q = 0; q < LW_Q; ++q) y[q] = m[q] ? __ldg(a.ci + at[q] + (m[q] >> 1)) : 0;
+#pragma unroll
+                        for (int q = 0; q < LW_Q; ++q) {
+                            const uint32_t h = m[q] >> 1;
+                            at[q] += m[q] && y[q] < x[q] ? m[q] - h : 0u;
+                            m[q] = h;
+                            left |= h;
+                        }
+                    }
+                    int32_t y[LW_Q];
+#pragma unroll
+                    for (int q = 0; q < LW_Q; ++q) y[q] = ok[q] && at[q] < end[q] ? __ldg(a.ci + at[q]) : -1;
+#pragma unroll
+                    for (int q = 0; q < LW_Q; ++q) ok[q] = ok[q] && y[q] == x[q];
+                }
+                if (a.count_only) {
+#pragma unroll
+                    for (int q = 0; q < LW_Q; ++q) found += ok[q];
+                    continue;
+                }
+                __syncwarp();                         // read: those that stay move to the front
+#pragma unroll
+                for (int q = 0; q < LW_Q; ++q) {
+                    const unsigned b = __ballot_sync(FULL_MASK, ok[q]);
+                    if (ok[q]) {
+                        const unsigned i = ns + __popc(b & le) - 1;
+                        sw[i] = x[q];
+                        sr[i] = (unsigned char)rr[q];
+                    }
+                    ns += __popc(b);
+                }
             }
         }
         if (ns) {
@@ -766,6 +864,14 @@ __device__ inline void long_rows_join(const JoinArgs &a, const LongTable &lt, ui
         for (int o = 16; o; o >>= 1) found += __shfl_down_sync(FULL_MASK, found, o);
         if (lane == 0 && found) atomicAdd(count, found);
     }
+}
+
+__device__ __forceinline__ void long_rows_join(const JoinArgs &a, const LongTable &lt, uint64_t L, uint64_t total,
+                                               uint64_t wi, uint64_t nw, int32_t *__restrict__ out, uint64_t cap,
+                                               unsigned long long *count, unsigned char *smem,
+                                               unsigned long long *ticket = nullptr) {
+    if (a.s.d == 1) long_rows_mode<LONG_SINGLE>(a, lt, L, total, wi, nw, out, cap, count, smem, ticket);
+    else long_rows_mode<LONG_MULTI>(a, lt, L, total, wi, nw, out, cap, count, smem, ticket);
 }
 
 // --------------------------------------------------------- counting tail
