@@ -170,6 +170,7 @@ gsi_status selftest_barrier_timeout(int dev, unsigned long long spin_limit, doub
 // memory the launch needs; the caller uploads them to cfg_dev together with
 // the k step records (host-initialised static fields) and the zeroed control
 // words.  launch_query_coop then launches; steps[0].count receives |seed|.
+// The launch runs the steps [t0, k), t0 = 1 for a query.
 // memo: query_memo_tables(steps, k) tables of n 8-byte entries, zeroed before
 // the launch (per-vertex label sub-list locations, see join_rows.cuh), or null.
 int query_memo_tables(const std::vector<JoinStep> &steps, int k);
@@ -179,10 +180,13 @@ bool query_counts_tail(const std::vector<JoinStep> &steps, int k, int count_only
 gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &steps, int k, const uint32_t *bitmaps,
                               const int32_t *order, int count_only, unsigned long long *stats, uint64_t *memo, bool nodedup,
                               void *cfg_host, size_t *smem);
+// One step over a table of the caller's on the same kernel; waits for it.
+gsi_status step_coop(const gsi_graph *g, const int32_t *M, uint64_t R, const JoinStep &s, const uint32_t *cand,
+                     int32_t *out, uint64_t out_cap, uint64_t *count, bool *ran, cudaStream_t st);
 // nodedup (configs): rows of single-edge steps are joined one by one (no
 // warp groups, no memo).  listwise (launch): the kernel variant that also
 // counts whole-list bytes (stats[2]).
-gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bitmap, size_t smem, void *cfg_dev,
+gsi_status launch_query_coop(const gsi_graph *g, int t0, int k, const uint32_t *seed_bitmap, size_t smem, void *cfg_dev,
                              DStep *dsteps, QueryCtl *ctl, int *grid_out, bool listwise,
                              cudaStream_t stream);
 

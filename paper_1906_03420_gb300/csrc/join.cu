@@ -43,6 +43,7 @@
 //     atomic per CTA, then written once as rows of M' (Prealloc-Combine: the
 //     join runs once; the output buffer is sized by F's total).
 #include <algorithm>
+#include <cstddef>
 #include <cstring>
 #include <map>
 #include <mutex>
@@ -182,8 +183,8 @@ __device__ __forceinline__ void copy_words(T *dst, const T *src) {
 __device__ __forceinline__ void copy_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 template <int NT, bool LW>
-__global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cfgs, DStep *steps, int k, QueryCtl *ctl,
-                                              const uint32_t *__restrict__ seed_bitmap, int64_t nwords) {
+__global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cfgs, DStep *steps, int t0, int k,
+                                              QueryCtl *ctl, const uint32_t *__restrict__ seed_bitmap, int64_t nwords) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wt[NT / 32];
     __shared__ unsigned long long at_s;
@@ -192,14 +193,19 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
     __shared__ BarrierView view_s;
     const unsigned G = gridDim.x;
     unsigned epoch = 0;
-    copy_words<NT>(&args_s[1], cfgs + 1);
-    copy_words<NT>(&ins_s[1], &steps[1].in);
+    copy_words<NT>(&args_s[t0 & 1], cfgs + 1);
+    copy_words<NT>(&ins_s[t0 & 1], &steps[1].in);
 
     // ---- seed: C(u_first) as the one-column table in the first region (Alg.
     // 2).  Each CTA lists the set bits of an equal share of the words, at a
     // place that one atomic reserves (the order of rows is free): one read of
-    // the bitmap and one grid barrier.
-    {
+    // the bitmap and one grid barrier.  Without a seed bitmap (step_coop) the
+    // first step's table is there, and steps[0] has its row count.
+    if (!seed_bitmap) {
+        copy_wait();
+        if (threadIdx.x == 0) view_s.count = steps[0].count;
+        __syncthreads();
+    } else {
         int32_t *seed_out = const_cast<int32_t *>(steps[1].in.M);
         const uint64_t chunk = (((uint64_t)nwords + G - 1) / G + 31) & ~31ull;
         const uint64_t lo = (uint64_t)blockIdx.x * chunk, hi = min((uint64_t)nwords, lo + chunk);
@@ -219,8 +225,8 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
     }
 
     uint64_t prev_cap = ~0ull;                                // rows that the step's input region holds
-    for (int t = 1; t < k; ++t) {
-        DStep *st = steps + t;
+    for (int t = t0; t < k; ++t) {                            // cfgs[1] and steps[1] are step t0's
+        DStep *st = steps + (t - t0 + 1);
         const JoinArgs &a = args_s[t & 1];
         const DStepIn &in_s = ins_s[t & 1];
         const uint64_t R = view_s.count;
@@ -231,8 +237,8 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         }
         if (R == 0) return;                                   // no embeddings: the counts stay zero
         if (t + 1 < k) {                                      // read behind this step's barriers
-            copy_words<NT>(&args_s[(t + 1) & 1], cfgs + t + 1);
-            copy_words<NT>(&ins_s[(t + 1) & 1], &steps[t + 1].in);
+            copy_words<NT>(&args_s[(t + 1) & 1], cfgs + (t - t0 + 2));
+            copy_words<NT>(&ins_s[(t + 1) & 1], &st[1].in);
         }
         const LongTable lt = long_table(in_s.S, in_s.S_words, t, R, &st->nlong);
         int32_t *const out = in_s.out;
@@ -432,7 +438,7 @@ gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &s
     return GSI_OK;
 }
 
-gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bitmap, size_t sm, void *cfg_dev,
+gsi_status launch_query_coop(const gsi_graph *g, int t0, int k, const uint32_t *seed_bitmap, size_t sm, void *cfg_dev,
                              DStep *dsteps, QueryCtl *ctl, int *grid_out, bool listwise,
                              cudaStream_t st) {
     // the variant that also counts whole-list bytes costs registers: only on request
@@ -473,9 +479,73 @@ gsi_status launch_query_coop(const gsi_graph *g, int k, const uint32_t *seed_bit
     *grid_out = grid;
     const JoinArgs *cfgp = static_cast<const JoinArgs *>(cfg_dev);
     int64_t nwords = g->nwords;
-    void *args[] = {(void *)&cfgp, (void *)&dsteps, (void *)&k, (void *)&ctl, (void *)&seed_bitmap, (void *)&nwords};
+    void *args[] = {(void *)&cfgp, (void *)&dsteps, (void *)&t0, (void *)&k, (void *)&ctl, (void *)&seed_bitmap, (void *)&nwords};
     GSI_CUDA_TRY(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(JOIN_NT), args, sm, st));
     return GSI_OK;
+}
+
+// One step over the caller's table as a launch of k_query without the seed.
+// Device memory in one block: configurations (the second is the step's), step
+// records and control words, the memo, the long-row table with room for every
+// row.  *ran is false, with nothing written but rows of `out`, when the block
+// could not be reserved or the long rows' candidates do not fit their counter.
+gsi_status step_coop(const gsi_graph *g, const int32_t *M, uint64_t R, const JoinStep &s, const uint32_t *cand,
+                     int32_t *out, uint64_t out_cap, uint64_t *count, bool *ran, cudaStream_t st) {
+    *ran = false;
+    struct Head {
+        JoinArgs cfg[2];
+        DStep steps[2];
+        QueryCtl ctl;
+    } h;
+    std::memset(static_cast<void *>(&h), 0, sizeof h);
+    const size_t sm = std::max(long_warp_smem(s.t, s.d) * (JOIN_NT / 32), rows_smem(JOIN_NT, s.t));
+    if (sm > 200 * 1024 || R >> 40) return GSI_OK;
+    // a memo once each vertex is met by a row on average: its clearing is 8
+    // bytes a vertex and list
+    const uint64_t tables = R >= (uint64_t)g->n ? (uint64_t)std::min(s.d, MEMO_EDGES) : 0;
+    const uint64_t head = (sizeof h + 255) / 256 * 256, memo = tables * (uint64_t)g->n * 8;
+    const uint64_t scratch = (R * (4 * (uint64_t)s.t + 16) + 64 + 15) / 16 * 16;
+    unsigned char *d = nullptr;
+    if (cudaMallocAsync(&d, head + memo + scratch, st) != cudaSuccess) {
+        (void)cudaGetLastError();
+        return GSI_OK;
+    }
+    h.cfg[1] = make_join_args(g, s, cand, out_cap == 0, nullptr);
+    if (tables) h.cfg[1].memo = reinterpret_cast<uint64_t *>(d + head);
+    h.cfg[1].memo_n = g->n;
+    DStepIn &in = h.steps[1].in;
+    in.M = M;
+    in.out = out;
+    in.out_bytes = out_cap * 4 * (uint64_t)(s.t + 1);
+    in.S = reinterpret_cast<uint64_t *>(d + head + memo);
+    in.S_words = scratch / 8;
+    in.t = s.t;
+    in.count_only = out_cap == 0;
+    h.steps[0].count = R;
+    Head *hd = reinterpret_cast<Head *>(d);
+    int grid = 0;
+    gsi_status rc = GSI_OK;
+    if ((memo && cudaMemsetAsync(d + head, 0, memo, st) != cudaSuccess) ||
+        cudaMemcpyAsync(d, &h, sizeof h, cudaMemcpyHostToDevice, st) != cudaSuccess) {
+        set_error("join step: scratch setup failed");
+        rc = GSI_ECUDA;
+    }
+    if (rc == GSI_OK)
+        rc = launch_query_coop(g, s.t, s.t + 1, nullptr, sm, hd->cfg, hd->steps, &hd->ctl, &grid, false, st);
+    if (rc == GSI_OK && (cudaMemcpyAsync(&h.steps[1], &hd->steps[1], sizeof h - offsetof(Head, steps[1]),
+                                         cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+                         cudaStreamSynchronize(st) != cudaSuccess)) {
+        set_error("join step: kernel or readback failed");
+        rc = GSI_ECUDA;
+    }
+    cudaFreeAsync(d, st);
+    if (rc == GSI_OK && (h.ctl.fail & 4u)) {
+        set_error("join step: a grid barrier wait ran past its limit");
+        rc = GSI_ETIMEOUT;
+    }
+    *ran = rc == GSI_OK && h.ctl.fail == 0;
+    if (*ran) *count = h.steps[1].count;
+    return rc;
 }
 
 gsi_status selftest_barrier_timeout(int dev, unsigned long long spin_limit, double *ms) {

@@ -503,7 +503,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     int grid = 0;
     if (rc == GSI_OK) {
         tm.begin(1);
-        rc = launch_query_coop(g, k, bitmaps + (uint64_t)order[0] * (uint64_t)g->nwords, smem, cfg_dev, dst, qc, &grid,
+        rc = launch_query_coop(g, 1, k, bitmaps + (uint64_t)order[0] * (uint64_t)g->nwords, smem, cfg_dev, dst, qc, &grid,
                                listwise && stats, st);
         tm.end();
         kernels += 1;

@@ -100,3 +100,35 @@ def test_tables_that_fill_some_or_all_of_the_grid(pkg, rows):
     got = got[np.argsort(got[:, 0])]
     want = np.arange(rows, dtype=np.int32)[:, None] + np.array([0, rows, 2 * rows], np.int32)
     assert r.count == rows and np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("t,d,rows,shift", [(1, 1, 63, 0), (1, 1, 5000, 1), (2, 2, 64, 3), (3, 3, 4097, 0), (6, 5, 9001, 1),
+                                            (31, 7, 700, 2), (4, 2, 40_000, 0)])
+def test_step_in_one_launch_against_the_scan_path(pkg, t, d, rows, shift):
+    """A step over the caller's table, with fewer and with more rows than vertices (with and without a memo), more lists than
+    the memo has, buffers off a 16-byte boundary, and out_cap short, exact and zero: the allocation-free call still
+    takes the scan and the slot tiles."""
+    import torch
+    rng = np.random.default_rng(1000 * t + d)
+    g = H.random_graph(rng, 220, 0.45, 2, 2)
+    G = pkg.Graph(g.vlab, g.src, g.dst, g.elab)
+    flat = torch.zeros(shift + rows * t, dtype=torch.int32, device="cuda")
+    flat[shift:] = torch.from_numpy(rng.integers(0, 220, rows * t).astype(np.int32)).cuda()
+    ptr = flat.data_ptr() + 4 * shift
+    cand = torch.from_numpy(rng.integers(-2**31, 2**31, 7).astype(np.int32)).cuda()
+    cols, labs = sorted(rng.choice(t, d, replace=False).tolist()), rng.integers(0, 2, d).tolist()
+    full = G.join_step_noalloc(ptr, rows, t, cand.data_ptr(), 1, cols, labs, 0, 0)
+    assert G.join_step(ptr, rows, t, cand.data_ptr(), 1, cols, labs, 0, 0) == full
+
+    def out_of(call, cap):
+        out = torch.full((shift + cap * (t + 1) + 1,), -7, dtype=torch.int32, device="cuda")
+        assert call(ptr, rows, t, cand.data_ptr(), 1, cols, labs, out.data_ptr() + 4 * shift, cap) == full
+        torch.cuda.synchronize()
+        assert int(out[-1]) == -7                     # nothing past the last row
+        return out[shift:-1].cpu().numpy().reshape(cap, t + 1)
+
+    want = oracle.sort_rows(out_of(G.join_step_noalloc, full))
+    assert np.array_equal(oracle.sort_rows(out_of(G.join_step, full)), want)
+    short = out_of(G.join_step, full // 2)
+    have = {r.tobytes() for r in np.ascontiguousarray(want)}
+    assert all(r.tobytes() in have for r in np.ascontiguousarray(short))
