@@ -28,7 +28,8 @@ gsi_result::~gsi_result() {
     if (cur != device) cudaSetDevice(device);
     cudaStream_t rs = own_stream ? stream : release_stream(device);
     for (auto &c : chunks) {
-        if (c.owned) cudaFreeAsync(c.rows, rs);
+        if (c.owned && c.block) gsi::block_put(device, c.rows, c.block, rs, false);
+        else if (c.owned) cudaFreeAsync(c.rows, rs);
         if (c.held) gsi::release_region(device, c.held);
     }
     arena.reset();
@@ -104,6 +105,7 @@ gsi_status gsi_graph_create(const int32_t *vlab, int32_t n, const int32_t *src, 
         if (g->gsig) cudaFree(g->gsig);
         return rc;
     }
+    block_users(dev, 1);
     *out = g.release();
     return GSI_OK;
     GSI_API_END
@@ -122,6 +124,7 @@ void gsi_graph_destroy(gsi_graph *g) {
     cudaFree(g->sig);
     cudaFree(g->gperm);
     cudaFree(g->gsig);
+    block_users(g->device, -1);
     if (cur >= 0) cudaSetDevice(cur);
     delete g;
 }
@@ -300,21 +303,26 @@ gsi_status gsi_filter(gsi_graph *g, const int32_t *qvlab, int32_t k, const int32
     QuerySig qs;
     query_signatures(qvlab, k, qsrc, qdst, qelab, qm, &qs);
     uint32_t *d_bm = nullptr;
-    unsigned long long *d_cnt = nullptr;
     const uint64_t words = (uint64_t)k * (uint64_t)g->nwords;
-    GSI_CUDA_TRY(cudaMallocAsync(&d_bm, words * 4 + 16, st));
-    GSI_CUDA_TRY(cudaMallocAsync(&d_cnt, 8 * (size_t)k, st));
+    const size_t bm_bytes = filter_bitmap_bytes(g, k), cnt_bytes = 8 * (size_t)k;
+    GSI_CUDA_TRY(device_alloc(&d_bm, bm_bytes + cnt_bytes, st));
+    unsigned long long *d_cnt = reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(d_bm) + bm_bytes);
     gsi_status rc = launch_filter(g, qs, d_bm, d_cnt, st);
+    // counts on the host go through pinned memory, ahead of the bitmaps: a
+    // copy to pageable memory waits for the device by itself (9 us)
+    cudaPointerAttributes pa;
+    unsigned char *pinned = cudaPointerGetAttributes(&pa, counts) == cudaSuccess && pa.type == cudaMemoryTypeUnregistered
+                                ? thread_pinned() : nullptr;
     if (rc == GSI_OK) {
-        if (cudaMemcpyAsync(bitmaps, d_bm, words * 4, cudaMemcpyDefault, st) != cudaSuccess ||
-            cudaMemcpyAsync(counts, d_cnt, 8 * (size_t)k, cudaMemcpyDefault, st) != cudaSuccess) {
+        if (cudaMemcpyAsync(pinned ? (void *)pinned : (void *)counts, d_cnt, cnt_bytes, cudaMemcpyDefault, st) != cudaSuccess ||
+            cudaMemcpyAsync(bitmaps, d_bm, words * 4, cudaMemcpyDefault, st) != cudaSuccess) {
             set_error("gsi_filter: copy-out failed");
             rc = GSI_ECUDA;
         }
     }
     cudaFreeAsync(d_bm, st);
-    cudaFreeAsync(d_cnt, st);
     GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    if (rc == GSI_OK && pinned) std::memcpy(counts, pinned, cnt_bytes);
     return rc;
     GSI_API_END
 }
@@ -339,9 +347,9 @@ gsi_status gsi_join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, 
     uint64_t h[2] = {0, 0};
     int64_t *part = nullptr;
     unsigned long long *d_cnt = nullptr;
-    GSI_CUDA_TRY(cudaMallocAsync(&F, 8 * (R + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&scr, 8 * (uint64_t)join_scan_scratch(R), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&d_cnt, 8, st));
+    GSI_CUDA_TRY(device_alloc(&F, 8 * (R + 1), st));
+    GSI_CUDA_TRY(device_alloc(&scr, 8 * (uint64_t)join_scan_scratch(R), st));
+    GSI_CUDA_TRY(device_alloc(&d_cnt, 8, st));
     gsi_status rc = launch_join_scan(g, M, R, s, F, scr, st);
     uint64_t total = 0;
     if (rc == GSI_OK) {
@@ -354,7 +362,7 @@ gsi_status gsi_join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, 
     }
     if (rc == GSI_OK) {
         const uint64_t ntiles = join_tiles(total);
-        if (cudaMallocAsync(&part, 8 * (ntiles + 1), st) != cudaSuccess ||
+        if (device_alloc(&part, 8 * (ntiles + 1), st) != cudaSuccess ||
             cudaMemsetAsync(d_cnt, 0, 8, st) != cudaSuccess) {
             set_error("gsi_join_step: scratch allocation failed");
             rc = GSI_ENOMEM;

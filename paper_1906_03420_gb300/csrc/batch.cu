@@ -476,7 +476,7 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     L.nt = o.block_threads ? o.block_threads : 256;
     L.rpt = o.rows_per_thread ? o.rows_per_thread : 2;
     if (stats) {
-        GSI_CUDA_TRY(cudaMallocAsync(&L.dstats, 24, st));
+        GSI_CUDA_TRY(device_alloc(&L.dstats, 24, st));
     }
     size_t sm = long_warp_smem(1, 1) * (size_t)(L.nt / 32);
     for (int i = 0; i < nq; ++i) {
@@ -526,6 +526,11 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     std::vector<BatchQuery> bqs((size_t)nq);
     std::vector<JoinArgs> cfg;
     std::vector<BatchItem> items;
+    {
+        size_t total = 0;
+        for (const BatchPlan &p : plans) total += p.active ? (size_t)p.k : 0;
+        cfg.reserve(total);
+    }
     const uint64_t max_words = std::max<uint64_t>(1, (L.t_bytes - 1024) / 128);   // seeds fit a table region
     for (int i = 0; i < nq; ++i) {
         BatchPlan &p = plans[i];
@@ -574,7 +579,7 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     L.o_ctl = L.o_ready + up(sizeof(unsigned) * L.sq_cap);
     L.ctl_bytes = L.o_ctl + up(sizeof(BatchCtl));
     L.has_template = keep_template;
-    if (cudaMallocAsync(&L.ctl, L.ctl_bytes, st) != cudaSuccess) {
+    if (device_alloc(&L.ctl, L.ctl_bytes, st) != cudaSuccess) {
         (void)cudaGetLastError();
         L.ctl = nullptr;
         set_error("batch: could not reserve the control block");
@@ -583,7 +588,7 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     if (ws) {
         L.arena = ws->arena;
     } else {
-        if (cudaMallocAsync(&L.arena, L.work_bytes, st) != cudaSuccess) {
+        if (device_alloc(&L.arena, L.work_bytes, st) != cudaSuccess) {
             (void)cudaGetLastError();
             L.arena = nullptr;
             set_error("batch: could not reserve the batch arena");
@@ -730,7 +735,7 @@ gsi_status batch_collect(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &p
         gsi_status rc = GSI_OK;
         if (tot > 0) {
             unsigned long long *d_dst = reinterpret_cast<unsigned long long *>(L.ctl + L.o_dst);
-            if (cudaMallocAsync(&buf, tot * 4, st) != cudaSuccess ||
+            if (device_alloc(&buf, tot * 4, st) != cudaSuccess ||
                 cudaMemcpyAsync(d_dst, dst.data(), sizeof(unsigned long long) * dst.size(), cudaMemcpyHostToDevice,
                                 st) != cudaSuccess) {
                 (void)cudaGetLastError();
@@ -793,7 +798,7 @@ gsi_status batch_run_device(gsi_graph *g, std::vector<BatchPlan> &plans, const g
     if (rc == GSI_OK && !L.all_plain) {
         if (ws) {
             result = ws->result;
-        } else if (cudaMallocAsync(&result, L.result_bytes, st) != cudaSuccess) {
+        } else if (device_alloc(&result, L.result_bytes, st) != cudaSuccess) {
             (void)cudaGetLastError();
             result = nullptr;
             set_error("batch: could not reserve the result arena");

@@ -160,21 +160,19 @@ struct SeedWriter {
 void query_signatures(const int32_t *qvlab, int32_t k, const int32_t *qsrc, const int32_t *qdst,
                       const int32_t *qelab, int32_t qm, QuerySig *out, bool hom) {
     out->k = k;
-    uint32_t counts[GSI_MAX_QUERY_VERTICES][GSI_SIG_GROUPS];
-    for (int u = 0; u < k; ++u)
-        for (int gidx = 0; gidx < GSI_SIG_GROUPS; ++gidx) counts[u][gidx] = 0;
-    for (int e = 0; e < qm; ++e) {
-        int a = qsrc[e], b = qdst[e];
-        counts[a][sig_group(qelab[e], qvlab[b])]++;
-        counts[b][sig_group(qelab[e], qvlab[a])]++;
-    }
     for (int u = 0; u < k; ++u) {
         for (int w = 0; w < GSI_SIG_WORDS; ++w) out->sig[u][w] = 0;
         out->sig[u][0] = (uint32_t)qvlab[u];
-        for (uint32_t gidx = 0; gidx < GSI_SIG_GROUPS; ++gidx) {
-            if (counts[u][gidx] >= 1) out->sig[u][sig_word(gidx)] |= 1u << sig_bit(gidx);
-            if (counts[u][gidx] >= 2 && !hom) out->sig[u][sig_word(gidx)] |= 2u << sig_bit(gidx);
-        }
+    }
+    // a group's first pair sets its first bit, a second one the other
+    auto add = [&](int u, int32_t elab, int32_t nlab) {
+        const uint32_t g = sig_group(elab, nlab), bit = 1u << sig_bit(g);
+        uint32_t &w = out->sig[u][sig_word(g)];
+        w |= (w & bit) && !hom ? 2u * bit : bit;
+    };
+    for (int e = 0; e < qm; ++e) {
+        add(qsrc[e], qelab[e], qvlab[qdst[e]]);
+        add(qdst[e], qelab[e], qvlab[qsrc[e]]);
     }
 }
 
@@ -249,7 +247,7 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
         return GSI_OK;
     }
     const size_t qbytes = flat.size() * 4;
-    GSI_CUDA_TRY(cudaMallocAsync(&fp->d_q, qbytes + meta.size() * 4, st));
+    GSI_CUDA_TRY(device_alloc(&fp->d_q, qbytes + meta.size() * 4, st));
     fp->d_meta = reinterpret_cast<int32_t *>(reinterpret_cast<unsigned char *>(fp->d_q) + qbytes);
     GSI_CUDA_TRY(cudaMemcpyAsync(fp->d_q, flat.data(), qbytes, cudaMemcpyHostToDevice, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(fp->d_meta, meta.data(), meta.size() * 4, cudaMemcpyHostToDevice, st));
@@ -261,8 +259,13 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
 gsi_status filter_enqueue(const gsi_graph *g, const FilterPlan &fp, uint32_t *bitmaps, unsigned long long *counts,
                           cudaStream_t st) {
     if (fp.nqv == 0) return GSI_OK;
-    GSI_CUDA_TRY(cudaMemsetAsync(bitmaps, 0, (size_t)fp.nqv * (size_t)g->nwords * 4, st));
-    GSI_CUDA_TRY(cudaMemsetAsync(counts, 0, (size_t)fp.nqv * 8, st));
+    const size_t bm_bytes = filter_bitmap_bytes(g, fp.nqv);
+    if (reinterpret_cast<unsigned char *>(bitmaps) + bm_bytes == reinterpret_cast<unsigned char *>(counts)) {
+        GSI_CUDA_TRY(cudaMemsetAsync(bitmaps, 0, bm_bytes + (size_t)fp.nqv * 8, st));       // one block of the caller's
+    } else {
+        GSI_CUDA_TRY(cudaMemsetAsync(bitmaps, 0, (size_t)fp.nqv * (size_t)g->nwords * 4, st));
+        GSI_CUDA_TRY(cudaMemsetAsync(counts, 0, (size_t)fp.nqv * 8, st));
+    }
     if (fp.ngroups == 0) return GSI_OK;
     int64_t blocks = (fp.warps + (FNT / 32) - 1) / (FNT / 32);
     if (blocks > 152 * 8) blocks = 152 * 8;

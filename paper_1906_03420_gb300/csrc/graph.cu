@@ -298,7 +298,7 @@ struct Temps {
     }
     template <typename T>
     gsi_status alloc(T **p, uint64_t count) {
-        GSI_CUDA_TRY(cudaMallocAsync(p, sizeof(T) * (size_t)(count + 1), st));
+        GSI_CUDA_TRY(device_alloc(p, sizeof(T) * (size_t)(count + 1), st));
         all.push_back(*p);
         return GSI_OK;
     }
@@ -431,12 +431,12 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     // CSR and signatures
     g->n = n; g->m = m; g->L = L; g->LV = LV; g->nwords = (n + 31) / 32;
     g->vlabels.assign(labels.begin(), labels.begin() + LV);
-    GSI_CUDA_TRY(cudaMallocAsync(&g->off, sizeof(uint32_t) * (size_t)(nseg + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&g->ci, sizeof(int32_t) * (size_t)(2 * m + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&g->cl, sizeof(uint16_t) * (size_t)(2 * m + 1), st));
-    GSI_CUDA_TRY(cudaMallocAsync(&g->dir, sizeof(uint32_t) * (size_t)(m + 1), st));
+    GSI_CUDA_TRY(device_alloc(&g->off, sizeof(uint32_t) * (size_t)(nseg + 1), st));
+    GSI_CUDA_TRY(device_alloc(&g->ci, sizeof(int32_t) * (size_t)(2 * m + 1), st));
+    GSI_CUDA_TRY(device_alloc(&g->cl, sizeof(uint16_t) * (size_t)(2 * m + 1), st));
+    GSI_CUDA_TRY(device_alloc(&g->dir, sizeof(uint32_t) * (size_t)(m + 1), st));
     g->dir_min = 2u * ((uint32_t)LV + 1u);
-    GSI_CUDA_TRY(cudaMallocAsync(&g->sig, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
+    GSI_CUDA_TRY(device_alloc(&g->sig, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
     GSI_CUDA_TRY(cudaMemsetAsync(g->sig, 0, sizeof(uint32_t) * (size_t)GSI_SIG_WORDS * (size_t)n, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(g->sig, d_vlab, sizeof(uint32_t) * (size_t)n, cudaMemcpyDeviceToDevice, st));
     if (m > 0) {
@@ -454,8 +454,8 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     // signatures grouped by label
     g->np = goff[LV];
     g->goff = goff;
-    GSI_CUDA_TRY(cudaMallocAsync(&g->gperm, sizeof(int32_t) * (size_t)g->np, st));
-    GSI_CUDA_TRY(cudaMallocAsync(&g->gsig, sizeof(uint32_t) * (size_t)(GSI_SIG_WORDS - 1) * (size_t)g->np, st));
+    GSI_CUDA_TRY(device_alloc(&g->gperm, sizeof(int32_t) * (size_t)g->np, st));
+    GSI_CUDA_TRY(device_alloc(&g->gsig, sizeof(uint32_t) * (size_t)(GSI_SIG_WORDS - 1) * (size_t)g->np, st));
     int64_t *d_shift = nullptr;
     GSI_TRY(tmps.alloc(&d_shift, (uint64_t)LV));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_shift, shift.data(), sizeof(int64_t) * (size_t)LV, cudaMemcpyHostToDevice, st));

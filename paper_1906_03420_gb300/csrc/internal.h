@@ -44,6 +44,27 @@ struct gsi_graph {
 
 namespace gsi {
 
+// ---------------------------------------------------------------- memory
+// cudaMallocAsync; where that fails, the blocks kept by the device's cache are
+// given back first.
+cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st);
+template <typename T>
+cudaError_t device_alloc(T **p, size_t bytes, cudaStream_t st) { return device_alloc(reinterpret_cast<void **>(p), bytes, st); }
+
+// Blocks of the single queries' arenas, kept for the next query: a few sizes
+// only, gigabytes each.  The stream-ordered pool serves them well as long as no
+// smaller request is cut out of a free one; then the next query waits
+// milliseconds for new memory (four queries with rows took 14 to 25 ms instead
+// of 2).  Any thread and stream may take a block that another gave back: `idle`
+// says that the stream had completed, otherwise an event orders the two.  At
+// most an eighth of the device's memory is kept, nothing under BLOCK_MIN, and
+// nothing at all without a graph on the device.
+constexpr uint64_t BLOCK_MIN = 64ull << 20;
+cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p);
+void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle);
+// A graph was made on the device (+1) or destroyed (-1, with the device idle).
+void block_users(int dev, int change);
+
 // ------------------------------------------------------------------ sort
 // Ascending, stable LSD radix sort of n keys over their bits [lo, hi).  keys
 // and tmp hold n keys each; *sorted is the one that the result ends in.
@@ -91,6 +112,11 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
 gsi_status filter_enqueue(const gsi_graph *g, const FilterPlan &fp, uint32_t *bitmaps, unsigned long long *counts,
                           cudaStream_t st);
 void filter_plan_free(FilterPlan &fp, cudaStream_t st);
+// Bytes of nqv bitmaps, up to the 8-byte boundary where counters that stand in
+// the same block begin (they are then zeroed together).
+inline size_t filter_bitmap_bytes(const gsi_graph *g, int32_t nqv) {
+    return ((size_t)nqv * (size_t)g->nwords * 4 + 7) / 8 * 8;
+}
 // Algorithmic bytes of one filter call over query vertices with these labels.
 uint64_t filter_alg_bytes(const gsi_graph *g, const std::vector<int32_t> &labels);
 // Compact the bitmap of C(u) into the int32 list out (ascending); scratch: uint32[scan_blocks+1].
@@ -110,6 +136,7 @@ struct JoinStep {
     uint32_t inj = 0xffffffffu;          // columns whose query vertex has u's label (set subtraction)
 };
 
+constexpr int MEMO_EDGES = 4;           // linking edges of a step with a sub-list memo
 constexpr int JOIN_NT = 256;
 constexpr int JOIN_VT = 4;
 constexpr int JOIN_NV = JOIN_NT * JOIN_VT;

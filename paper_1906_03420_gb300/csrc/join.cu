@@ -506,7 +506,7 @@ gsi_status step_coop(const gsi_graph *g, const int32_t *M, uint64_t R, const Joi
     const uint64_t head = (sizeof h + 255) / 256 * 256, memo = tables * (uint64_t)g->n * 8;
     const uint64_t scratch = (R * (4 * (uint64_t)s.t + 16) + 64 + 15) / 16 * 16;
     unsigned char *d = nullptr;
-    if (cudaMallocAsync(&d, head + memo + scratch, st) != cudaSuccess) {
+    if (device_alloc(&d, head + memo + scratch, st) != cudaSuccess) {
         (void)cudaGetLastError();
         return GSI_OK;
     }

@@ -174,8 +174,6 @@ __device__ inline int block_inclusive_max(int v, int *wt) {
     return r;
 }
 
-constexpr int MEMO_EDGES = 4;     // linking edges of a step with a sub-list memo
-
 // A memo entry (8 bytes) of a data vertex and linking edge:
 //   bits 63..59  the step it was made in (another step's entry is a miss)
 //   bit  58      1: the sub-list has at most 16 entries and `mask` tells which

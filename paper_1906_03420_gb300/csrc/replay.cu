@@ -129,7 +129,7 @@ extern "C" gsi_status gsi_batch_replay(gsi_batch *b, gsi_result **outs, int32_t 
         int32_t *result = nullptr;
         std::shared_ptr<ResultArena> arena;
         if (!b->L.all_plain && b->L.result_bytes) {
-            if (cudaMallocAsync(&result, b->L.result_bytes, st) != cudaSuccess) {
+            if (device_alloc(&result, b->L.result_bytes, st) != cudaSuccess) {
                 (void)cudaGetLastError();
                 set_error("gsi_batch_replay: could not reserve the result arena");
                 return GSI_ENOMEM;

@@ -239,6 +239,9 @@ void Timer::resolve(gsi_stats *s) {
 // default budget (a large share of HBM) from the stream-ordered pool costs
 // milliseconds per query; arenas up to tens of GB cost well under one.
 constexpr uint64_t DEVICE_ARENA_START = 16ull << 30;
+// Largest memo that is cleared before the plan is known, behind the host's
+// work: 32 MB take 8 us, about as long as that.
+constexpr uint64_t EARLY_MEMO = 32ull << 20;
 
 static std::atomic<uint64_t> g_total_mem[64];
 static std::atomic<uint64_t> g_held[64];
@@ -271,13 +274,126 @@ void release_region(int dev, uint64_t bytes) {
     if (dev >= 0 && dev < 64) g_held[dev].fetch_sub(bytes);
 }
 
+namespace {
+struct KeptBlock {
+    void *p;
+    uint64_t bytes;
+    cudaEvent_t done;                // null: idle
+};
+struct BlockCache {
+    std::mutex mu;
+    std::vector<KeptBlock> kept;     // oldest first
+    uint64_t bytes = 0;
+    int users = 0;
+};
+BlockCache &block_cache(int dev) {   // never destroyed: results may outlive static objects
+    static BlockCache *const c = new BlockCache[64];
+    return c[dev];
+}
+// Gives the first `n` kept blocks back to the pool, behind their last use.
+void block_release(BlockCache &c, size_t n, cudaStream_t st) {
+    for (size_t i = 0; i < n; ++i) {
+        KeptBlock &b = c.kept[i];
+        if (b.done) {
+            cudaStreamWaitEvent(st, b.done, 0);
+            cudaEventDestroy(b.done);
+        }
+        cudaFreeAsync(b.p, st);
+        c.bytes -= b.bytes;
+    }
+    c.kept.erase(c.kept.begin(), c.kept.begin() + (std::ptrdiff_t)n);
+}
+}  // namespace
+
+cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st) {
+    cudaError_t e = cudaMallocAsync(p, bytes, st);
+    int dev = 0;
+    if (e != cudaErrorMemoryAllocation || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return e;
+    BlockCache &c = block_cache(dev);
+    {
+        std::lock_guard<std::mutex> lk(c.mu);
+        if (c.kept.empty()) return e;
+        block_release(c, c.kept.size(), st);
+    }
+    (void)cudaGetLastError();
+    return cudaMallocAsync(p, bytes, st);
+}
+
+cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p) {
+    if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
+        BlockCache &c = block_cache(dev);
+        std::lock_guard<std::mutex> lk(c.mu);
+        for (size_t i = c.kept.size(); i-- > 0;) {
+            const KeptBlock b = c.kept[i];
+            if (b.bytes != bytes) continue;
+            if (b.done) {
+                const cudaError_t e = cudaStreamWaitEvent(st, b.done, 0);
+                if (e != cudaSuccess) return e;
+                cudaEventDestroy(b.done);
+            }
+            c.kept.erase(c.kept.begin() + (std::ptrdiff_t)i);
+            c.bytes -= bytes;
+            *p = b.p;
+            return cudaSuccess;
+        }
+    }
+    return device_alloc(p, bytes, st);
+}
+
+void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle) {
+    if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
+        const uint64_t most = device_total_mem(dev) / 8;
+        BlockCache &c = block_cache(dev);
+        std::lock_guard<std::mutex> lk(c.mu);
+        if (c.users > 0 && bytes <= most) {
+            cudaEvent_t done = nullptr;
+            if (!idle && (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess ||
+                          cudaEventRecord(done, st) != cudaSuccess)) {
+                (void)cudaGetLastError();
+                if (done) cudaEventDestroy(done);
+                done = nullptr;
+                cudaDeviceSynchronize();              // the stream is gone: wait for what it had
+            }
+            c.kept.push_back({p, bytes, done});
+            c.bytes += bytes;
+            size_t n = 0;
+            for (uint64_t left = c.bytes; left > most; ++n) left -= c.kept[n].bytes;
+            if (n) block_release(c, n, st);
+            return;
+        }
+    }
+    cudaFreeAsync(p, st);
+}
+
+void block_users(int dev, int change) {
+    if (dev < 0 || dev >= 64) return;
+    BlockCache &c = block_cache(dev);
+    std::lock_guard<std::mutex> lk(c.mu);
+    c.users += change;
+    if (c.users == 0) block_release(c, c.kept.size(), nullptr);
+}
+
 static gsi_status dalloc(Exec &x, void **p, uint64_t bytes) {
-    cudaError_t e = cudaMallocAsync(p, bytes ? bytes : 16, x.st);
+    cudaError_t e = device_alloc(p, bytes ? bytes : 16, x.st);
     if (e != cudaSuccess) {
         set_error(std::string("device allocation of ") + std::to_string(bytes) + " bytes: " + cudaGetErrorString(e));
         return GSI_ENOMEM;
     }
     return GSI_OK;
+}
+
+unsigned char *thread_pinned() {
+    static thread_local unsigned char *p = nullptr;
+    if (!p && cudaMallocHost(&p, PINNED_READ + PINNED_STAGE) != cudaSuccess) p = nullptr;
+    return p;
+}
+
+// The calling thread's event on a device, for waits within one entry point.
+static cudaEvent_t thread_event(int dev) {
+    static thread_local cudaEvent_t ev[64];
+    if (dev < 0 || dev >= 64) return nullptr;
+    if (!ev[dev] && cudaEventCreateWithFlags(&ev[dev], cudaEventDisableTiming) != cudaSuccess) ev[dev] = nullptr;
+    return ev[dev];
 }
 
 static gsi_status read_u64(Exec &x, const void *dptr, uint64_t *val) {
@@ -427,23 +543,26 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     }
     uint64_t *S = nullptr, *memo = nullptr;
     int32_t *reg[2] = {nullptr, nullptr};
-    unsigned char *ctl = nullptr;
-    const uint64_t memo_tables =
-        (uint64_t)query_memo_tables(steps, k) + (query_counts_tail(steps, k, count_only, nodedup) ? 1 : 0);
-    const uint64_t memo_bytes = nodedup ? 0 : memo_tables * (uint64_t)g->n * 8;
-    const size_t ctl_bytes = (join_args_size() * (size_t)k + 255) / 256 * 256 +
-                             (sizeof(DStep) * (size_t)k + 255) / 256 * 256 + 256;
-    gsi_status rc = dalloc(*this, (void **)&S, s_bytes);
-    if (rc == GSI_OK) rc = dalloc(*this, (void **)&reg[0], t_bytes);
-    if (rc == GSI_OK) rc = dalloc(*this, (void **)&reg[1], t_bytes);
-    if (rc == GSI_OK) rc = dalloc(*this, (void **)&ctl, ctl_bytes);
-    if (rc == GSI_OK && memo_bytes) rc = dalloc(*this, (void **)&memo, memo_bytes);
+    const uint64_t tables =
+        nodedup ? 0 : (uint64_t)query_memo_tables(steps, k) + (query_counts_tail(steps, k, count_only, nodedup) ? 1 : 0);
+    const uint64_t memo_bytes = tables * (uint64_t)g->n * 8;
+    if (this->memo && memo_tables >= tables) {
+        memo = this->memo;
+        this->memo = nullptr;
+    }
+    const bool cleared = memo != nullptr;
+    // the control block stands behind the scratch region; all three blocks
+    // have one size, so that a kept one serves as any of them
+    const uint64_t block = std::max(s_bytes + PINNED_STAGE, t_bytes);
+    gsi_status rc = GSI_OK;
+    for (void **p : {(void **)&S, (void **)&reg[0], (void **)&reg[1]})
+        if (rc == GSI_OK && block_get(g->device, block, st, p) != cudaSuccess) rc = GSI_ENOMEM;
+    if (rc == GSI_OK && memo_bytes && !memo) rc = dalloc(*this, (void **)&memo, memo_bytes);
+    unsigned char *const ctl = reinterpret_cast<unsigned char *>(S) + s_bytes;
     auto release = [&]() {
         if (memo) cudaFreeAsync(memo, st);
-        if (S) cudaFreeAsync(S, st);
-        if (reg[0]) cudaFreeAsync(reg[0], st);
-        if (reg[1]) cudaFreeAsync(reg[1], st);
-        if (ctl) cudaFreeAsync(ctl, st);
+        for (void *p : {(void *)S, (void *)reg[0], (void *)reg[1]})
+            if (p) block_put(g->device, p, block, st, !pending);
     };
     if (rc != GSI_OK) {
         release();
@@ -492,7 +611,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         h.t = t;
     }
     rc = GSI_OK;
-    if (memo_bytes && cudaMemsetAsync(memo, 0, memo_bytes, st) != cudaSuccess) {
+    if (memo_bytes && !cleared && cudaMemsetAsync(memo, 0, memo_bytes, st) != cudaSuccess) {
         set_error("device-driven join: clearing the sub-list memo failed");
         rc = GSI_ECUDA;
     }
@@ -509,20 +628,26 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         kernels += 1;
         tiles += (uint64_t)(k - 1);
     }
-    // read back: status, and the final count / capacity
+    // read back: the last step's record (final count, capacity) and, behind
+    // it, the status
     uint64_t fin[3] = {0, 0, 0};
     if (rc == GSI_OK) {
-        if (cudaMemcpyAsync(h_pinned, &qc->fail, 4, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemcpyAsync(h_pinned + 1, &dst[k - 1].count, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaMemcpyAsync(h_pinned + 2, &dst[k - 1].out_cap, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+        unsigned char *const back = reinterpret_cast<unsigned char *>(h_pinned + 8);
+        const size_t qc_at = (size_t)(reinterpret_cast<unsigned char *>(qc) - reinterpret_cast<unsigned char *>(dst + k - 1));
+        if (cudaMemcpyAsync(back, dst + k - 1, qc_at + sizeof(QueryCtl), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             (stats && cudaMemcpyAsync(h_pinned + 3, d_scalars + 1, 24, cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
             cudaStreamSynchronize(st) != cudaSuccess) {
             set_error("device-driven join: kernel or readback failed");
             rc = GSI_ECUDA;
         }
-        fin[0] = h_pinned[0] & 0xffffffffu;
-        fin[1] = h_pinned[1];
-        fin[2] = h_pinned[2];
+        pending = false;
+        DStep last;
+        QueryCtl status;
+        std::memcpy(&last, back, sizeof last);
+        std::memcpy(&status, back + qc_at, sizeof status);
+        fin[0] = status.fail;
+        fin[1] = last.count;
+        fin[2] = last.out_cap;
         if (rc == GSI_OK && stats && fin[0] == 0) {   // the join's counters, read with the status
             join_bytes = h_pinned[3];
             join_items = h_pinned[4];
@@ -560,12 +685,14 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         if (!tight_rows && (big || hold_region(g->device, t_bytes))) {
             gsi_result::Chunk ch{final_reg, rows};
             ch.held = big ? 0 : t_bytes;
+            ch.block = block;
             res->chunks.push_back(ch);
             res->materialised += rows;
             reg[(k - 1) & 1] = nullptr;
         } else {
             int32_t *tight = nullptr;
             rc = dalloc(*this, (void **)&tight, bytes);
+            pending = true;
             if (rc == GSI_OK && cudaMemcpyAsync(tight, final_reg, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
                 set_error("device-driven join: result copy failed");
                 rc = GSI_ECUDA;
@@ -651,32 +778,31 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
     QuerySig qs;
     const bool hom = o.semantics == GSI_HOMOMORPHISM;
     query_signatures(q.vl.data(), q.k, q.src.data(), q.dst.data(), q.lab.data(), q.qm, &qs, hom);
-    const uint64_t bm_words = (uint64_t)q.k * (uint64_t)g->nwords;
-    // per-thread pinned staging: small readbacks first, then the upload area
-    // of the device-driven control block (cudaFreeHost would synchronise the
-    // whole device, so the buffer lives as long as the thread).  Every use is
-    // complete before run_query returns (the stream is synchronised).
-    static thread_local unsigned char *t_pinned = nullptr;
-    constexpr size_t PINNED_READ = 4096, PINNED_STAGE = 60 * 1024;
-    if (!t_pinned) GSI_CUDA_TRY(cudaMallocHost(&t_pinned, PINNED_READ + PINNED_STAGE));
-    x.h_pinned = reinterpret_cast<uint64_t *>(t_pinned);
-    x.h_stage = t_pinned + PINNED_READ;
+    const size_t bm_bytes = filter_bitmap_bytes(g, q.k);
+    unsigned char *const pinned = thread_pinned();
+    if (!pinned) {
+        set_error("query: no pinned memory");
+        return GSI_ENOMEM;
+    }
+    x.h_pinned = reinterpret_cast<uint64_t *>(pinned);
+    x.h_stage = pinned + PINNED_READ;
     x.h_stage_bytes = PINNED_STAGE;
-    unsigned long long *d_counts = nullptr;
-    gsi_status rc = dalloc(x, (void **)&x.bitmaps, bm_words * 4);
-    if (rc == GSI_OK) rc = dalloc(x, (void **)&d_counts, 8 * GSI_MAX_QUERY_VERTICES + 32);
+    // one block: bitmaps, their counts, the counters
+    gsi_status rc = dalloc(x, (void **)&x.bitmaps, bm_bytes + 8 * (size_t)q.k + 32);
+    unsigned long long *const d_counts =
+        reinterpret_cast<unsigned long long *>(reinterpret_cast<unsigned char *>(x.bitmaps) + bm_bytes);
     if (rc == GSI_OK) {
-        x.d_scalars = d_counts + GSI_MAX_QUERY_VERTICES;
-        if (cudaMemsetAsync(x.d_scalars, 0, 32, x.st) != cudaSuccess) {
+        x.d_scalars = d_counts + q.k;
+        if (x.stats && cudaMemsetAsync(x.d_scalars, 0, 32, x.st) != cudaSuccess) {
             set_error("query: clearing the counters failed");
             rc = GSI_ECUDA;
         }
     }
     if (rc != GSI_OK) {                     // nothing was launched: release what was reserved
         if (x.bitmaps) cudaFreeAsync(x.bitmaps, x.st);
-        if (d_counts) cudaFreeAsync(d_counts, x.st);
         return rc;
     }
+    x.pending = true;
 
     x.tm.begin(0);
     rc = launch_filter(g, qs, x.bitmaps, d_counts, x.st);
@@ -684,8 +810,32 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
     x.kernels += 1;
     uint64_t cand_h[GSI_MAX_QUERY_VERTICES] = {0};
     if (rc == GSI_OK) {
-        if (cudaMemcpyAsync(x.h_pinned, d_counts, 8 * (size_t)q.k, cudaMemcpyDeviceToHost, x.st) != cudaSuccess ||
-            cudaStreamSynchronize(x.st) != cudaSuccess) {
+        bool ok = cudaMemcpyAsync(x.h_pinned, d_counts, 8 * (size_t)q.k, cudaMemcpyDeviceToHost, x.st) == cudaSuccess;
+        // a small memo is cleared while the host takes the counts and plans (it
+        // waits for an event before the clearing): no step has more linking edges than a vertex has edges, nor more than
+        // the query has beyond a tree's
+        const cudaEvent_t counted = thread_event(g->device);
+        if (ok && counted) ok = cudaEventRecord(counted, x.st) == cudaSuccess;
+        if (ok && counted && !o.host_driven && !x.nodedup && q.k > 1) {
+            int deg = 0;
+            for (int u = 0; u < q.k; ++u) {
+                int c = 0;
+                for (int w = 0; w < q.k; ++w) c += q.elab[u][w] >= 0;
+                deg = std::max(deg, c);
+            }
+            const uint64_t t = (uint64_t)std::min({deg, q.qm - q.k + 2, MEMO_EDGES}) + (x.count_only ? 1 : 0);
+            const uint64_t bytes = t * (uint64_t)g->n * 8;
+            if (bytes <= EARLY_MEMO) {
+                if (dalloc(x, (void **)&x.memo, bytes) == GSI_OK) {
+                    x.memo_tables = t;
+                    ok = cudaMemsetAsync(x.memo, 0, bytes, x.st) == cudaSuccess;
+                } else {
+                    x.memo = nullptr;
+                    (void)cudaGetLastError();
+                }
+            }
+        }
+        if (!ok || (counted ? cudaEventSynchronize(counted) : cudaStreamSynchronize(x.st)) != cudaSuccess) {
             set_error("filter: readback failed");
             rc = GSI_ECUDA;
         } else {
@@ -748,6 +898,7 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
         const uint64_t R0 = cand_h[order[0]];
         int32_t *M0 = nullptr;
         if (rc == GSI_OK && overflow) {
+            x.pending = true;
             // seed: M = C(u_first) as a one-column table (Alg. 2)
             uint32_t *sscr = nullptr;
             rc = dalloc(x, (void **)&M0, R0 * 4);
@@ -785,8 +936,9 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
         }
     }
     cudaFreeAsync(x.bitmaps, x.st);
-    cudaFreeAsync(d_counts, x.st);
-    cudaError_t se = cudaStreamSynchronize(x.st);
+    if (x.memo) cudaFreeAsync(x.memo, x.st);
+    // the device path has waited for its stream
+    const cudaError_t se = x.pending ? cudaStreamSynchronize(x.st) : cudaSuccess;
     if (rc == GSI_OK && se != cudaSuccess) {
         set_error(std::string("query: ") + cudaGetErrorString(se));
         rc = GSI_ECUDA;

@@ -28,6 +28,7 @@ struct gsi_result {
         bool owned = true;   // false: the rows live in a shared arena
         uint64_t held = 0;   // > 0: a whole table region kept without a tight copy,
                              // counted against the device's held-region allowance
+        uint64_t block = 0;  // > 0: the rows lie in an arena block of that size (block_put)
     };
     int32_t k = 0;
     int device = 0;
@@ -119,6 +120,11 @@ struct Exec {
     // arena_bytes: scratch + two table regions; *overflow: a table did not
     // fit (or the arena could not be reserved: *no_memory as well)
     gsi_status run_device(uint64_t arena_bytes, bool *overflow, bool *no_memory);
+    // The memo of the first run_device call, reserved and cleared ahead of it
+    // (tables its size; 0: not yet).
+    uint64_t *memo = nullptr;
+    uint64_t memo_tables = 0;
+    bool pending = false;            // work was enqueued after the last wait for the stream
     gsi_status add_chunk(int32_t *rows, uint64_t nrows, uint64_t alloc_rows);
     const uint32_t *cand(const JoinStep &s, int t) const;
 };
@@ -202,6 +208,12 @@ gsi_status batch_execute(gsi_graph *g, std::vector<BatchPlan> &plans, const gsi_
 gsi_status batch_run_device(gsi_graph *g, std::vector<BatchPlan> &plans, const gsi_batch_opts &o, uint64_t budget,
                             cudaStream_t st, gsi_stats *stats, BatchWorkspace *ws = nullptr);
 gsi_status prepare_device(int dev);
+// PINNED_READ + PINNED_STAGE bytes of pinned memory of the calling thread:
+// small readbacks first, then an upload area.  Every use is complete before the
+// entry point that makes it returns (cudaFreeHost would synchronise the whole
+// device, so the buffer lives as long as the thread).  Null without memory.
+constexpr size_t PINNED_READ = 4096, PINNED_STAGE = 60 * 1024;
+unsigned char *thread_pinned();
 gsi_status validate_query(const int32_t *qvlab, int32_t k, const int32_t *qsrc, const int32_t *qdst,
                           const int32_t *qelab, int32_t qm, QueryGraph *q);
 void plan_order(const QueryGraph &q, const uint64_t *cand, const uint64_t *freq, int32_t nlabels, int32_t *order,

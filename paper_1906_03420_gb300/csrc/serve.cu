@@ -56,8 +56,8 @@ gsi_status batch_plan_all(gsi_graph *g, std::vector<BatchPlan> &plans, gsi_stats
     }
     in.nk = nk;
     if (nk == 0) return GSI_OK;
-    GSI_CUDA_TRY(cudaMallocAsync(&in.bitmaps, bm_words * 4 + 16, st));
-    GSI_CUDA_TRY(cudaMallocAsync(&in.counts, nk * 8, st));
+    GSI_CUDA_TRY(device_alloc(&in.bitmaps, bm_words * 4 + 16, st));
+    GSI_CUDA_TRY(device_alloc(&in.counts, nk * 8, st));
     std::vector<QuerySig> sigs;
     sigs.reserve((size_t)nq);
     for (int32_t i = 0; i < nq; ++i) {
@@ -497,8 +497,8 @@ static void serve_batch(gsi_server *s, cudaStream_t st, uint64_t reserve, size_t
     BatchWorkspace ws;
     ws.result_bytes = (reserve / 5) / 256 * 256;
     ws.arena_bytes = (reserve - ws.result_bytes) / 256 * 256;
-    if (cudaMallocAsync((void **)&ws.arena, ws.arena_bytes, st) != cudaSuccess ||
-        cudaMallocAsync((void **)&ws.result, ws.result_bytes, st) != cudaSuccess) {
+    if (device_alloc((void **)&ws.arena, ws.arena_bytes, st) != cudaSuccess ||
+        device_alloc((void **)&ws.result, ws.result_bytes, st) != cudaSuccess) {
         (void)cudaGetLastError();
         if (ws.arena) cudaFreeAsync(ws.arena, st);
         ws = BatchWorkspace();             // the batch reserves its own memory
@@ -655,9 +655,9 @@ static gsi_status pair_counts(gsi_server *s) {
     unsigned long long *tab = nullptr;
     int64_t *goff = nullptr;
     cudaStream_t st = s->streams[0];
-    GSI_CUDA_TRY(cudaMallocAsync(&tab, cells * 8, st));
+    GSI_CUDA_TRY(device_alloc(&tab, cells * 8, st));
     gsi_status rc = GSI_OK;
-    if (cudaMallocAsync(&goff, sizeof(int64_t) * g->goff.size(), st) != cudaSuccess ||
+    if (device_alloc(&goff, sizeof(int64_t) * g->goff.size(), st) != cudaSuccess ||
         cudaMemsetAsync(tab, 0, cells * 8, st) != cudaSuccess ||
         cudaMemcpyAsync(goff, g->goff.data(), sizeof(int64_t) * g->goff.size(), cudaMemcpyHostToDevice, st) !=
             cudaSuccess) {

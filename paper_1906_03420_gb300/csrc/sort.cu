@@ -157,8 +157,8 @@ gsi_status radix_sort_u64(uint64_t *keys, uint64_t *tmp, int64_t n, int lo, int 
     GSI_CUDA_TRY(cudaFuncSetAttribute(k_rs_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                       (int)rs_smem(1 << RS_MAX_BITS)));
     uint32_t *hist = nullptr, *scr = nullptr;
-    GSI_CUDA_TRY(cudaMallocAsync(&hist, sizeof(uint32_t) * (size_t)(nh + 1), st));
-    if (cudaMallocAsync(&scr, sizeof(uint32_t) * (size_t)(scan_blocks(nh) + 1), st) != cudaSuccess) {
+    GSI_CUDA_TRY(device_alloc(&hist, sizeof(uint32_t) * (size_t)(nh + 1), st));
+    if (device_alloc(&scr, sizeof(uint32_t) * (size_t)(scan_blocks(nh) + 1), st) != cudaSuccess) {
         cudaFreeAsync(hist, st);
         set_error("radix sort: no memory for the scan");
         return GSI_ENOMEM;
