@@ -12,8 +12,9 @@ using namespace gsi;
 
 // Result memory is released stream-ordered on a library stream: cudaFree
 // would wait for every kernel on the device, stalling concurrent queries.
-// The producing stream has always completed before a result is handed out.
-static cudaStream_t release_stream(int dev) {
+// The producing stream has always completed before a result is handed out. A
+// graph build copies its edge arrays there.
+cudaStream_t gsi::library_stream(int dev) {
     static std::mutex mu;
     static cudaStream_t streams[64];
     std::lock_guard<std::mutex> lk(mu);
@@ -26,7 +27,7 @@ gsi_result::~gsi_result() {
     int cur = -1;
     cudaGetDevice(&cur);
     if (cur != device) cudaSetDevice(device);
-    cudaStream_t rs = own_stream ? stream : release_stream(device);
+    cudaStream_t rs = own_stream ? stream : gsi::library_stream(device);
     for (auto &c : chunks) {
         if (c.owned && c.block) gsi::block_put(device, c.rows, c.block, rs, false);
         else if (c.owned) cudaFreeAsync(c.rows, rs);
@@ -41,7 +42,7 @@ gsi::ResultArena::~ResultArena() {
     int cur = -1;
     cudaGetDevice(&cur);
     if (cur != device) cudaSetDevice(device);
-    cudaFreeAsync(ptr, own_stream ? stream : release_stream(device));
+    cudaFreeAsync(ptr, own_stream ? stream : gsi::library_stream(device));
     if (cur >= 0 && cur != device) cudaSetDevice(cur);
 }
 

@@ -29,6 +29,7 @@ namespace gsi {
 namespace {
 
 constexpr int NT = 256;
+constexpr int64_t COPY_APART = 1 << 20;               // below, an array arrives in 25 us
 
 enum : unsigned { BAD_ID = 1u, SELF_LOOP = 2u, NEG_LABEL = 4u, DUP_PAIR = 8u };
 
@@ -294,7 +295,26 @@ struct Temps {
     std::vector<void *> all;
     explicit Temps(cudaStream_t s) : st(s) {}
     ~Temps() {
+        if (other) cudaStreamSynchronize(other);      // an error may leave copies behind
+        if (ev) cudaEventDestroy(ev);
         for (void *p : all) cudaFreeAsync(p, st);
+    }
+    // A second stream, behind what this one has so far; join() orders the first
+    // behind it.
+    cudaStream_t other = nullptr;
+    cudaEvent_t ev = nullptr;
+    gsi_status beside(cudaStream_t s) {
+        GSI_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+        GSI_CUDA_TRY(cudaEventRecord(ev, st));
+        GSI_CUDA_TRY(cudaStreamWaitEvent(s, ev, 0));
+        other = s;
+        return GSI_OK;
+    }
+    gsi_status join() {
+        if (!other) return GSI_OK;
+        GSI_CUDA_TRY(cudaEventRecord(ev, other));
+        GSI_CUDA_TRY(cudaStreamWaitEvent(st, ev, 0));
+        return GSI_OK;
     }
     template <typename T>
     gsi_status alloc(T **p, uint64_t count) {
@@ -358,24 +378,17 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_CUDA_TRY(cudaMemcpyAsync(d_w, &hw, sizeof hw, cudaMemcpyHostToDevice, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_vlab, vlab, sizeof(int32_t) * (size_t)n, cudaMemcpyDefault, st));
     k_label_range<<<few_blocks(n), NT, 0, st>>>(d_vlab, n, &d_w->lo);
-    if (m > 0) {
-        GSI_CUDA_TRY(cudaMemcpyAsync(d_src, src, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
-        GSI_CUDA_TRY(cudaMemcpyAsync(d_dst, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
-        GSI_CUDA_TRY(cudaMemcpyAsync(d_elab, elab, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, st));
-        k_validate<<<few_blocks(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, &d_w->flags, &d_w->maxlab);
-    }
+    // a large edge list is copied on the library's own stream: the vertices
+    // are sorted meanwhile, and the pairs while the edge labels arrive (16M
+    // edges: 365 us an array; 4.58 -> 4.26 ms)
+    const cudaStream_t cs = m >= COPY_APART ? library_stream(g->device) : st;
+    if (cs != st) GSI_TRY(tmps.beside(cs));
     GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
     GSI_CUDA_TRY(cudaStreamSynchronize(st));
-    if (hw.flags) {
-        set_error(std::string("gsi_graph_create: ") + ((hw.flags & BAD_ID) ? "vertex id out of range " : "") +
-                  ((hw.flags & SELF_LOOP) ? "self-loop " : "") + ((hw.flags & NEG_LABEL) ? "negative edge label" : ""));
-        return GSI_EINVAL;
-    }
-    const int32_t L = hw.maxlab < 0 ? 1 : hw.maxlab + 1;
     const int nb = ceil_log2_bits((uint64_t)(n > 1 ? n - 1 : 1));
 
-    // the vertices in the order of (label, id), the duplicate check of the
-    // pairs behind them on the stream, one readback for both
+    // the vertices in the order of (label, id), the checks of the edges behind
+    // them on the stream, one readback for all
     const uint64_t nkeys = std::max((uint64_t)(2 * m), (uint64_t)n);
     uint64_t *keys = nullptr, *tmp = nullptr, *sorted = nullptr;
     GSI_TRY(tmps.alloc(&keys, nkeys));
@@ -394,15 +407,31 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     const LabelHead head{sorted, nb};
     GSI_CUDA_TRY(device_scan<uint32_t>(
         head, n, LabelRanks{head, n, hw.lo, at, gpos, &d_w->nlabels, d_labels, d_labels + most}, scr, st));
-    if (m > 1) {
+    if (m > 0) {
+        GSI_CUDA_TRY(cudaMemcpyAsync(d_src, src, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, cs));
+        GSI_CUDA_TRY(cudaMemcpyAsync(d_dst, dst, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, cs));
+        GSI_TRY(tmps.join());
+    }
+    if (m > 1) {                                      // of ids that may yet turn out to be bad
         k_pair_keys<<<grid_for(m), NT, 0, st>>>(d_src, d_dst, m, nb, keys);
         GSI_TRY(radix_sort_u64(keys, tmp, m, 0, 2 * nb, &sorted, st));
         k_adjacent_equal<<<grid_for(m), NT, 0, st>>>(sorted, m, &d_w->flags);
+    }
+    if (m > 0) {
+        GSI_CUDA_TRY(cudaMemcpyAsync(d_elab, elab, sizeof(int32_t) * (size_t)m, cudaMemcpyDefault, cs));
+        GSI_TRY(tmps.join());
+        k_validate<<<few_blocks(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, &d_w->flags, &d_w->maxlab);
     }
     std::vector<int32_t> labels(2 * (size_t)most);     // the distinct labels, then where each begins
     GSI_CUDA_TRY(cudaMemcpyAsync(labels.data(), d_labels, sizeof(int32_t) * labels.size(), cudaMemcpyDeviceToHost, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
     GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    if (hw.flags & ~(unsigned)DUP_PAIR) {
+        set_error(std::string("gsi_graph_create: ") + ((hw.flags & BAD_ID) ? "vertex id out of range " : "") +
+                  ((hw.flags & SELF_LOOP) ? "self-loop " : "") + ((hw.flags & NEG_LABEL) ? "negative edge label" : ""));
+        return GSI_EINVAL;
+    }
+    const int32_t L = hw.maxlab < 0 ? 1 : hw.maxlab + 1;
     if (hw.nlabels > (uint32_t)MAX_LABELS) {
         set_error("gsi_graph_create: more than 65535 distinct vertex labels");
         return GSI_EINVAL;

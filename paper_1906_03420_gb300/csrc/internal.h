@@ -44,6 +44,9 @@ struct gsi_graph {
 
 namespace gsi {
 
+// The library's own stream on a device (null: none).
+cudaStream_t library_stream(int dev);
+
 // ---------------------------------------------------------------- memory
 // cudaMallocAsync; where that fails, the blocks kept by the device's cache are
 // given back first.
