@@ -42,7 +42,9 @@ gsi::ResultArena::~ResultArena() {
     int cur = -1;
     cudaGetDevice(&cur);
     if (cur != device) cudaSetDevice(device);
-    cudaFreeAsync(ptr, own_stream ? stream : gsi::library_stream(device));
+    cudaStream_t rs = own_stream ? stream : gsi::library_stream(device);
+    if (block) gsi::block_put(device, ptr, block, rs, false);
+    else cudaFreeAsync(ptr, rs);
     if (cur >= 0 && cur != device) cudaSetDevice(cur);
 }
 

@@ -467,6 +467,7 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     L = BatchLaunch();
     const int nq = (int)plans.size();
     L.nq = (size_t)nq;
+    L.device = g->device;
     if ((o.block_threads != 0 && o.block_threads != 128 && o.block_threads != 256) ||
         (o.rows_per_thread != 0 && o.rows_per_thread != 1 && o.rows_per_thread != 2) || o.isect < 0 ||
         o.isect > ISECT_BITMAP) {
@@ -588,7 +589,7 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     if (ws) {
         L.arena = ws->arena;
     } else {
-        if (device_alloc(&L.arena, L.work_bytes, st) != cudaSuccess) {
+        if (block_get(g->device, L.work_bytes, st, reinterpret_cast<void **>(&L.arena)) != cudaSuccess) {
             (void)cudaGetLastError();
             L.arena = nullptr;
             set_error("batch: could not reserve the batch arena");
@@ -782,7 +783,7 @@ gsi_status batch_collect(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &p
 
 void batch_release(BatchLaunch &L, cudaStream_t st) {
     if (L.ctl) cudaFreeAsync(L.ctl, st);
-    if (L.own_arena && L.arena) cudaFreeAsync(L.arena, st);
+    if (L.own_arena && L.arena) block_put(L.device, L.arena, L.work_bytes, st, false);
     if (L.dstats) cudaFreeAsync(L.dstats, st);
     L = BatchLaunch();
 }
@@ -798,7 +799,7 @@ gsi_status batch_run_device(gsi_graph *g, std::vector<BatchPlan> &plans, const g
     if (rc == GSI_OK && !L.all_plain) {
         if (ws) {
             result = ws->result;
-        } else if (device_alloc(&result, L.result_bytes, st) != cudaSuccess) {
+        } else if (block_get(g->device, L.result_bytes, st, reinterpret_cast<void **>(&result)) != cudaSuccess) {
             (void)cudaGetLastError();
             result = nullptr;
             set_error("batch: could not reserve the result arena");
@@ -809,6 +810,7 @@ gsi_status batch_run_device(gsi_graph *g, std::vector<BatchPlan> &plans, const g
             arena->device = g->device;
             arena->stream = st;
             arena->own_stream = true;
+            arena->block = L.result_bytes;
         }
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;

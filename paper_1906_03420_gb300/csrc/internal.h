@@ -54,13 +54,13 @@ cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st);
 template <typename T>
 cudaError_t device_alloc(T **p, size_t bytes, cudaStream_t st) { return device_alloc(reinterpret_cast<void **>(p), bytes, st); }
 
-// Blocks of the single queries' arenas, kept for the next query: a few sizes
-// only, gigabytes each.  The stream-ordered pool serves them well as long as no
+// Blocks of the arenas of queries and batches, kept for the next call: a few
+// sizes only, gigabytes each.  The stream-ordered pool serves them well as long as no
 // smaller request is cut out of a free one; then the next query waits
 // milliseconds for new memory (four queries with rows took 14 to 25 ms instead
 // of 2).  Any thread and stream may take a block that another gave back: `idle`
 // says that the stream had completed, otherwise an event orders the two.  At
-// most an eighth of the device's memory is kept, nothing under BLOCK_MIN, and
+// most a quarter of the device's memory is kept, nothing under BLOCK_MIN, and
 // nothing at all without a graph on the device.
 constexpr uint64_t BLOCK_MIN = 64ull << 20;
 cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p);

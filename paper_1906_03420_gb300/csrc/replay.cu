@@ -129,7 +129,7 @@ extern "C" gsi_status gsi_batch_replay(gsi_batch *b, gsi_result **outs, int32_t 
         int32_t *result = nullptr;
         std::shared_ptr<ResultArena> arena;
         if (!b->L.all_plain && b->L.result_bytes) {
-            if (device_alloc(&result, b->L.result_bytes, st) != cudaSuccess) {
+            if (block_get(g->device, b->L.result_bytes, st, reinterpret_cast<void **>(&result)) != cudaSuccess) {
                 (void)cudaGetLastError();
                 set_error("gsi_batch_replay: could not reserve the result arena");
                 return GSI_ENOMEM;
@@ -139,6 +139,7 @@ extern "C" gsi_status gsi_batch_replay(gsi_batch *b, gsi_result **outs, int32_t 
             arena->device = g->device;
             arena->stream = st;
             arena->own_stream = !b->own_stream;           // a private stream dies with the batch
+            arena->block = b->L.result_bytes;
         }
         GSI_TRY(batch_enqueue_ctl(b->L, result, b->L.result_bytes, st));
         GSI_CUDA_TRY(cudaGraphLaunch(b->exec, st));

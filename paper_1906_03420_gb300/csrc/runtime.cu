@@ -342,7 +342,7 @@ cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p) {
 
 void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle) {
     if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
-        const uint64_t most = device_total_mem(dev) / 8;
+        const uint64_t most = device_total_mem(dev) / 4;
         BlockCache &c = block_cache(dev);
         std::lock_guard<std::mutex> lk(c.mu);
         if (c.users > 0 && bytes <= most) {

@@ -17,6 +17,7 @@ struct ResultArena {
     int device = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
+    uint64_t block = 0;              // > 0: a block of that size for block_put
     ~ResultArena();
 };
 }  // namespace gsi
@@ -164,7 +165,7 @@ struct BatchWorkspace {
 // work only when the launch keeps a template, hence capturable);
 // batch_collect reads the outcome back into the plans.
 struct BatchLaunch {
-    int grid = 0, nsm = 152;
+    int grid = 0, nsm = 152, device = 0;
     int nt = 256, rpt = 2;                   // block shape of the batch kernel
     size_t sm = 0;
     uint64_t result_bytes = 0, work_bytes = 0, spill_bytes = 0, slices_bytes = 0;
