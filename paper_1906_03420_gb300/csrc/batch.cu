@@ -125,7 +125,9 @@ __device__ long long next_unit(const BatchArgs &b, long long *ticket) {
     BatchCtl *c = b.ctl;
     unsigned long long spins = 0;
     for (;;) {
-        if (*ticket < 0 && vload(&c->sq_head) < vload(&c->sq_tail))
+        // read together: one round trip to L2, not one for each queue
+        const unsigned long long head = vload(&c->sq_head), tail = vload(&c->sq_tail), item = vload(&c->next_item);
+        if (*ticket < 0 && head < tail)
             *ticket = (long long)atomicAdd(&c->sq_head, 1ull);
         // published (a number past the queue's end never is)
         if (*ticket >= 0 && (unsigned long long)*ticket < b.sq_cap &&
@@ -135,7 +137,7 @@ __device__ long long next_unit(const BatchArgs &b, long long *ticket) {
             *ticket = -1;
             return -h - 1;
         }
-        if (vload(&c->next_item) < (unsigned long long)b.nitems) {
+        if (item < (unsigned long long)b.nitems) {
             const unsigned long long i = atomicAdd(&c->next_item, 1ull);
             if (i < (unsigned long long)b.nitems) return (long long)i;
         }
