@@ -516,7 +516,8 @@ gsi_status step_coop(const gsi_graph *g, const int32_t *M, uint64_t R, const Joi
     DStepIn &in = h.steps[1].in;
     in.M = M;
     in.out = out;
-    in.out_bytes = out_cap * 4 * (uint64_t)(s.t + 1);
+    in.out_bytes = ~0ull;                             // the limit is in rows: as bytes a large one ("all of
+    in.row_cap = out_cap;                             // them") would wrap to a small one
     in.S = reinterpret_cast<uint64_t *>(d + head + memo);
     in.S_words = scratch / 8;
     in.t = s.t;
