@@ -1,0 +1,69 @@
+// Device memory: stream-ordered allocations, and the arena blocks of queries
+// and batches that are kept for the next call.  Host code only.
+#pragma once
+
+#include <cstddef>
+#include <cstdint>
+
+#include <cuda_runtime.h>
+
+namespace gsi {
+
+// Total memory of a device (looked up once per device).
+uint64_t device_total_mem(int dev);
+
+// cudaMallocAsync; where that fails, the blocks kept by the device's cache are
+// given back first.
+cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st);
+template <typename T>
+cudaError_t device_alloc(T **p, size_t bytes, cudaStream_t st) { return device_alloc(reinterpret_cast<void **>(p), bytes, st); }
+
+// Blocks of the arenas of queries and batches, kept for the next call: a few
+// sizes only, gigabytes each.  The stream-ordered pool serves them well as long as no
+// smaller request is cut out of a free one; then the next query waits
+// milliseconds for new memory (four queries with rows took 14 to 25 ms instead
+// of 2).  Any thread and stream may take a block that another gave back: `idle`
+// says that the stream had completed, otherwise an event orders the two.  At
+// most a quarter of the device's memory is kept, nothing under BLOCK_MIN, and
+// nothing at all without a graph on the device.
+constexpr uint64_t BLOCK_MIN = 64ull << 20;
+cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p);
+void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle);
+// A graph was made on the device (+1) or destroyed (-1, with the device idle).
+void block_users(int dev, int change);
+
+// The blocks of one attempt on a stream, given back when it ends.  A block that
+// another thread gave back may still be in use by the work that `st` was made
+// to wait for, so the set counts as in use from its first get(); it goes back
+// as idle only if a wait for the stream has succeeded since and nothing was
+// enqueued after it.
+class BlockSet {
+public:
+    BlockSet(int dev, cudaStream_t st) : dev_(dev), st_(st) {}
+    BlockSet(const BlockSet &) = delete;
+    BlockSet &operator=(const BlockSet &) = delete;
+    ~BlockSet();
+    cudaError_t get(uint64_t bytes, void **p);
+    void enqueued() { busy_ = true; }
+    // The outcome of a wait for the stream.
+    bool waited(cudaError_t e) {
+        if (e == cudaSuccess) busy_ = false;
+        return e == cudaSuccess;
+    }
+    bool busy() const { return busy_; }
+    // Leaves the block at p to the caller, who gives it back by block_put.
+    void take(void *p);
+
+private:
+    static constexpr int MOST = 4;
+    struct Held {
+        void *p;
+        uint64_t bytes;
+    };
+    int dev_, n_ = 0;
+    cudaStream_t st_;
+    bool busy_ = false;
+    Held held_[MOST];
+};
+
+}  // namespace gsi

@@ -9,6 +9,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/gsi.h"
+#include "blocks.h"
 
 struct gsi_graph {
     int device = 0;
@@ -46,27 +47,6 @@ namespace gsi {
 
 // The library's own stream on a device (null: none).
 cudaStream_t library_stream(int dev);
-
-// ---------------------------------------------------------------- memory
-// cudaMallocAsync; where that fails, the blocks kept by the device's cache are
-// given back first.
-cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st);
-template <typename T>
-cudaError_t device_alloc(T **p, size_t bytes, cudaStream_t st) { return device_alloc(reinterpret_cast<void **>(p), bytes, st); }
-
-// Blocks of the arenas of queries and batches, kept for the next call: a few
-// sizes only, gigabytes each.  The stream-ordered pool serves them well as long as no
-// smaller request is cut out of a free one; then the next query waits
-// milliseconds for new memory (four queries with rows took 14 to 25 ms instead
-// of 2).  Any thread and stream may take a block that another gave back: `idle`
-// says that the stream had completed, otherwise an event orders the two.  At
-// most a quarter of the device's memory is kept, nothing under BLOCK_MIN, and
-// nothing at all without a graph on the device.
-constexpr uint64_t BLOCK_MIN = 64ull << 20;
-cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p);
-void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle);
-// A graph was made on the device (+1) or destroyed (-1, with the device idle).
-void block_users(int dev, int change);
 
 // ------------------------------------------------------------------ sort
 // Ascending, stable LSD radix sort of n keys over their bits [lo, hi).  keys

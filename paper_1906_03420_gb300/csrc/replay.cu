@@ -141,10 +141,20 @@ extern "C" gsi_status gsi_batch_replay(gsi_batch *b, gsi_result **outs, int32_t 
             arena->own_stream = !b->own_stream;           // a private stream dies with the batch
             arena->block = b->L.result_bytes;
         }
+        // a private stream's arena goes back on the library's: if this ends early,
+        // not before the stream's work has
+        struct Early {
+            cudaStream_t st;
+            bool on = true;
+            ~Early() {
+                if (on) cudaStreamSynchronize(st);
+            }
+        } early{st};
         GSI_TRY(batch_enqueue_ctl(b->L, result, b->L.result_bytes, st));
         GSI_CUDA_TRY(cudaGraphLaunch(b->exec, st));
         gsi_status rc = batch_collect(b->L, g, b->plans, result, arena, st, stats, nullptr);
         if (rc != GSI_OK) return rc;
+        early.on = false;
         if (stats) {
             float fms = 0, jms = 0;
             cudaEventElapsedTime(&fms, b->ev[0], b->ev[1]);

@@ -274,105 +274,6 @@ void release_region(int dev, uint64_t bytes) {
     if (dev >= 0 && dev < 64) g_held[dev].fetch_sub(bytes);
 }
 
-namespace {
-struct KeptBlock {
-    void *p;
-    uint64_t bytes;
-    cudaEvent_t done;                // null: idle
-};
-struct BlockCache {
-    std::mutex mu;
-    std::vector<KeptBlock> kept;     // oldest first
-    uint64_t bytes = 0;
-    int users = 0;
-};
-BlockCache &block_cache(int dev) {   // never destroyed: results may outlive static objects
-    static BlockCache *const c = new BlockCache[64];
-    return c[dev];
-}
-// Gives the first `n` kept blocks back to the pool, behind their last use.
-void block_release(BlockCache &c, size_t n, cudaStream_t st) {
-    for (size_t i = 0; i < n; ++i) {
-        KeptBlock &b = c.kept[i];
-        if (b.done) {
-            cudaStreamWaitEvent(st, b.done, 0);
-            cudaEventDestroy(b.done);
-        }
-        cudaFreeAsync(b.p, st);
-        c.bytes -= b.bytes;
-    }
-    c.kept.erase(c.kept.begin(), c.kept.begin() + (std::ptrdiff_t)n);
-}
-}  // namespace
-
-cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st) {
-    cudaError_t e = cudaMallocAsync(p, bytes, st);
-    int dev = 0;
-    if (e != cudaErrorMemoryAllocation || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return e;
-    BlockCache &c = block_cache(dev);
-    {
-        std::lock_guard<std::mutex> lk(c.mu);
-        if (c.kept.empty()) return e;
-        block_release(c, c.kept.size(), st);
-    }
-    (void)cudaGetLastError();
-    return cudaMallocAsync(p, bytes, st);
-}
-
-cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p) {
-    if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
-        BlockCache &c = block_cache(dev);
-        std::lock_guard<std::mutex> lk(c.mu);
-        for (size_t i = c.kept.size(); i-- > 0;) {
-            const KeptBlock b = c.kept[i];
-            if (b.bytes != bytes) continue;
-            if (b.done) {
-                const cudaError_t e = cudaStreamWaitEvent(st, b.done, 0);
-                if (e != cudaSuccess) return e;
-                cudaEventDestroy(b.done);
-            }
-            c.kept.erase(c.kept.begin() + (std::ptrdiff_t)i);
-            c.bytes -= bytes;
-            *p = b.p;
-            return cudaSuccess;
-        }
-    }
-    return device_alloc(p, bytes, st);
-}
-
-void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle) {
-    if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
-        const uint64_t most = device_total_mem(dev) / 4;
-        BlockCache &c = block_cache(dev);
-        std::lock_guard<std::mutex> lk(c.mu);
-        if (c.users > 0 && bytes <= most) {
-            cudaEvent_t done = nullptr;
-            if (!idle && (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess ||
-                          cudaEventRecord(done, st) != cudaSuccess)) {
-                (void)cudaGetLastError();
-                if (done) cudaEventDestroy(done);
-                done = nullptr;
-                cudaDeviceSynchronize();              // the stream is gone: wait for what it had
-            }
-            c.kept.push_back({p, bytes, done});
-            c.bytes += bytes;
-            size_t n = 0;
-            for (uint64_t left = c.bytes; left > most; ++n) left -= c.kept[n].bytes;
-            if (n) block_release(c, n, st);
-            return;
-        }
-    }
-    cudaFreeAsync(p, st);
-}
-
-void block_users(int dev, int change) {
-    if (dev < 0 || dev >= 64) return;
-    BlockCache &c = block_cache(dev);
-    std::lock_guard<std::mutex> lk(c.mu);
-    c.users += change;
-    if (c.users == 0) block_release(c, c.kept.size(), nullptr);
-}
-
 static gsi_status dalloc(Exec &x, void **p, uint64_t bytes) {
     cudaError_t e = device_alloc(p, bytes ? bytes : 16, x.st);
     if (e != cudaSuccess) {
@@ -555,14 +456,16 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     // have one size, so that a kept one serves as any of them
     const uint64_t block = std::max(s_bytes + PINNED_STAGE, t_bytes);
     gsi_status rc = GSI_OK;
+    // from here on the stream may hold work, be it a wait for a block's last
+    // user: the blocks go back behind it unless a wait for it succeeds
+    pending = true;
+    BlockSet blocks(g->device, st);
     for (void **p : {(void **)&S, (void **)&reg[0], (void **)&reg[1]})
-        if (rc == GSI_OK && block_get(g->device, block, st, p) != cudaSuccess) rc = GSI_ENOMEM;
+        if (rc == GSI_OK && blocks.get(block, p) != cudaSuccess) rc = GSI_ENOMEM;
     if (rc == GSI_OK && memo_bytes && !memo) rc = dalloc(*this, (void **)&memo, memo_bytes);
     unsigned char *const ctl = reinterpret_cast<unsigned char *>(S) + s_bytes;
     auto release = [&]() {
         if (memo) cudaFreeAsync(memo, st);
-        for (void *p : {(void *)S, (void *)reg[0], (void *)reg[1]})
-            if (p) block_put(g->device, p, block, st, !pending);
     };
     if (rc != GSI_OK) {
         release();
@@ -636,11 +539,11 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         const size_t qc_at = (size_t)(reinterpret_cast<unsigned char *>(qc) - reinterpret_cast<unsigned char *>(dst + k - 1));
         if (cudaMemcpyAsync(back, dst + k - 1, qc_at + sizeof(QueryCtl), cudaMemcpyDeviceToHost, st) != cudaSuccess ||
             (stats && cudaMemcpyAsync(h_pinned + 3, d_scalars + 1, 24, cudaMemcpyDeviceToHost, st) != cudaSuccess) ||
-            cudaStreamSynchronize(st) != cudaSuccess) {
+            !blocks.waited(cudaStreamSynchronize(st))) {
             set_error("device-driven join: kernel or readback failed");
             rc = GSI_ECUDA;
         }
-        pending = false;
+        pending = blocks.busy();
         DStep last;
         QueryCtl status;
         std::memcpy(&last, back, sizeof last);
@@ -688,10 +591,11 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
             ch.block = block;
             res->chunks.push_back(ch);
             res->materialised += rows;
-            reg[(k - 1) & 1] = nullptr;
+            blocks.take(final_reg);
         } else {
             int32_t *tight = nullptr;
             rc = dalloc(*this, (void **)&tight, bytes);
+            blocks.enqueued();
             pending = true;
             if (rc == GSI_OK && cudaMemcpyAsync(tight, final_reg, bytes, cudaMemcpyDeviceToDevice, st) != cudaSuccess) {
                 set_error("device-driven join: result copy failed");

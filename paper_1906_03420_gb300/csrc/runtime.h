@@ -60,8 +60,6 @@ struct gsi_result {
 
 namespace gsi {
 
-// Total memory of a device (looked up once per device).
-uint64_t device_total_mem(int dev);
 // Held table regions: a result may keep the whole region its rows were
 // written in (no tight copy) while the regions held on the device stay within
 // a quarter of its memory.  hold_region reserves `bytes` of that allowance
