@@ -104,6 +104,8 @@ typedef struct {
  */
 gsi_status gsi_graph_create(const int32_t *vlab, int32_t n, const int32_t *src, const int32_t *dst,
                             const int32_t *elab, int64_t m, const gsi_graph_opts *opts, gsi_graph **out);
+/* Waits for the device and frees the graph.  With the device's last graph go
+   the arena blocks kept there (gsi_memory_trim). */
 void gsi_graph_destroy(gsi_graph *g);
 gsi_status gsi_graph_get_info(const gsi_graph *g, gsi_graph_info *info);
 /*
@@ -239,8 +241,26 @@ gsi_status gsi_result_copy(const gsi_result *r, int32_t *dst, uint64_t max_rows,
 gsi_status gsi_result_copy_async(const gsi_result *r, int32_t *dst, uint64_t max_rows, uint64_t *rows,
                                  void *stream);
 /* Releases the result's device memory stream-ordered on the stream it was
-   produced on: destroy results before destroying that stream. */
+   produced on: destroy results before destroying that stream.  A table region
+   or batch arena that the rows lie in may be kept for a later call
+   (gsi_memory_trim). */
 void gsi_result_destroy(gsi_result *r);
+
+/*
+ * Device memory kept between calls.  The arena blocks of queries and batches
+ * (scratch and table regions, 64 MB and more each) are not freed with the call
+ * or the result that used them but kept for the next one: at most 64 blocks and
+ * a quarter of the device's memory, while a graph lives on the device.  They
+ * come on top of what mem_budget and a server's budget allow for the calls that
+ * run.  Everything else goes back to the device's default memory pool, whose
+ * release threshold the library raises, so that it keeps it.
+ * gsi_memory_trim gives the kept blocks of a device back to that pool and waits
+ * until they have arrived, so that other stream-ordered allocations can use
+ * them and cudaMemPoolTrimTo can return them to the device; *bytes (may be
+ * NULL) receives their size.  Blocks in use are not touched.  The library does
+ * the same by itself when one of its allocations fails.
+ */
+gsi_status gsi_memory_trim(int32_t device, uint64_t *bytes);
 
 /* ------------------------------------------------------- step-level calls */
 /*

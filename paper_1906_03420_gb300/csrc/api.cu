@@ -29,7 +29,7 @@ gsi_result::~gsi_result() {
     if (cur != device) cudaSetDevice(device);
     cudaStream_t rs = own_stream ? stream : gsi::library_stream(device);
     for (auto &c : chunks) {
-        if (c.owned && c.block) gsi::block_put(device, c.rows, c.block, rs, false);
+        if (c.owned && c.block) gsi::block_put(device, {c.rows, c.block}, rs, false);
         else if (c.owned) cudaFreeAsync(c.rows, rs);
         if (c.held) gsi::release_region(device, c.held);
     }
@@ -43,7 +43,7 @@ gsi::ResultArena::~ResultArena() {
     cudaGetDevice(&cur);
     if (cur != device) cudaSetDevice(device);
     cudaStream_t rs = own_stream ? stream : gsi::library_stream(device);
-    if (block) gsi::block_put(device, ptr, block, rs, false);
+    if (block) gsi::block_put(device, {ptr, block}, rs, false);
     else cudaFreeAsync(ptr, rs);
     if (cur >= 0 && cur != device) cudaSetDevice(cur);
 }
@@ -404,6 +404,18 @@ gsi_status gsi_plan_order(int32_t k, const int32_t *qsrc, const int32_t *qdst, c
     QueryGraph q;
     GSI_TRY(validate_query(vl, k, qsrc, qdst, qelab, qm, &q));
     plan_order(q, cand, freq, n_labels, order_out, first_edge);
+    return GSI_OK;
+    GSI_API_END
+}
+
+gsi_status gsi_memory_trim(int32_t device, uint64_t *bytes) {
+    GSI_API_BEGIN
+    if (bytes) *bytes = 0;
+    GSI_TRY(prepare_device(device));
+    const cudaStream_t st = library_stream(device);
+    const uint64_t n = block_trim(device, st);
+    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    if (bytes) *bytes = n;
     return GSI_OK;
     GSI_API_END
 }

@@ -591,13 +591,13 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
     if (ws) {
         L.arena = ws->arena;
     } else {
-        if (block_get(g->device, L.work_bytes, st, reinterpret_cast<void **>(&L.arena)) != cudaSuccess) {
+        if (block_get(g->device, L.work_bytes, st, &L.own_arena) != cudaSuccess) {
             (void)cudaGetLastError();
-            L.arena = nullptr;
+            L.own_arena = Block();
             set_error("batch: could not reserve the batch arena");
             return GSI_ENOMEM;
         }
-        L.own_arena = true;
+        L.arena = static_cast<unsigned char *>(L.own_arena.p);
     }
     GSI_CUDA_TRY(cudaMemcpyAsync(L.ctl, cfg.data(), sizeof(JoinArgs) * cfg.size(), cudaMemcpyHostToDevice, st));
     if (items.size())
@@ -785,7 +785,7 @@ gsi_status batch_collect(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &p
 
 void batch_release(BatchLaunch &L, cudaStream_t st) {
     if (L.ctl) cudaFreeAsync(L.ctl, st);
-    if (L.own_arena && L.arena) block_put(L.device, L.arena, L.work_bytes, st, false);
+    if (L.own_arena.p) block_put(L.device, L.own_arena, st, false);
     if (L.dstats) cudaFreeAsync(L.dstats, st);
     L = BatchLaunch();
 }
@@ -797,22 +797,23 @@ gsi_status batch_run_device(gsi_graph *g, std::vector<BatchPlan> &plans, const g
     BatchLaunch L;
     gsi_status rc = batch_setup(L, g, plans, o, budget, st, ws, stats != nullptr, false);
     int32_t *result = nullptr;
+    Block blk;
     std::shared_ptr<ResultArena> arena;
     if (rc == GSI_OK && !L.all_plain) {
         if (ws) {
             result = ws->result;
-        } else if (block_get(g->device, L.result_bytes, st, reinterpret_cast<void **>(&result)) != cudaSuccess) {
+        } else if (block_get(g->device, L.result_bytes, st, &blk) != cudaSuccess) {
             (void)cudaGetLastError();
-            result = nullptr;
             set_error("batch: could not reserve the result arena");
             rc = GSI_ENOMEM;
         } else {
+            result = static_cast<int32_t *>(blk.p);
             arena = std::make_shared<ResultArena>();     // the last result to go releases it
             arena->ptr = result;
             arena->device = g->device;
             arena->stream = st;
             arena->own_stream = true;
-            arena->block = L.result_bytes;
+            arena->block = blk.bytes;
         }
     }
     cudaEvent_t e0 = nullptr, e1 = nullptr;

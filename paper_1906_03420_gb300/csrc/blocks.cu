@@ -2,82 +2,99 @@
 #include "blocks.h"
 
 #include <mutex>
-#include <vector>
 
 namespace gsi {
-
 namespace {
+
 struct KeptBlock {
     void *p;
     uint64_t bytes;
     cudaEvent_t done;                // null: idle
+    uint64_t turn;                   // requests before it was given back
 };
 struct BlockCache {
     std::mutex mu;
-    std::vector<KeptBlock> kept;     // oldest first
-    uint64_t bytes = 0;
-    int users = 0;
+    KeptBlock kept[KEPT_MOST];       // oldest first; no allocation, as results are destroyed without exceptions
+    int n = 0, users = 0;
+    uint64_t bytes = 0, turn = 0;
 };
+
 BlockCache &block_cache(int dev) {   // never destroyed: results may outlive static objects
     static BlockCache *const c = new BlockCache[64];
     return c[dev];
 }
-// Gives the first `n` kept blocks back to the pool, behind their last use.
-void block_release(BlockCache &c, size_t n, cudaStream_t st) {
-    for (size_t i = 0; i < n; ++i) {
-        KeptBlock &b = c.kept[i];
-        if (b.done) {
-            cudaStreamWaitEvent(st, b.done, 0);
-            cudaEventDestroy(b.done);
-        }
-        cudaFreeAsync(b.p, st);
-        c.bytes -= b.bytes;
-    }
-    c.kept.erase(c.kept.begin(), c.kept.begin() + (std::ptrdiff_t)n);
+
+void block_remove(BlockCache &c, int i) {
+    c.bytes -= c.kept[i].bytes;
+    for (--c.n; i < c.n; ++i) c.kept[i] = c.kept[i + 1];
 }
+
+// Gives kept block i back to the pool, behind its last use.
+void block_release(BlockCache &c, int i, cudaStream_t st) {
+    const KeptBlock b = c.kept[i];
+    if (b.done) {
+        cudaStreamWaitEvent(st, b.done, 0);
+        cudaEventDestroy(b.done);
+    }
+    cudaFreeAsync(b.p, st);
+    block_remove(c, i);
+}
+
 }  // namespace
 
 cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st) {
     cudaError_t e = cudaMallocAsync(p, bytes, st);
     int dev = 0;
     if (e != cudaErrorMemoryAllocation || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return e;
-    BlockCache &c = block_cache(dev);
-    {
-        std::lock_guard<std::mutex> lk(c.mu);
-        if (c.kept.empty()) return e;
-        block_release(c, c.kept.size(), st);
-    }
+    if (!block_trim(dev, st)) return e;
     (void)cudaGetLastError();
     return cudaMallocAsync(p, bytes, st);
 }
 
-cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p) {
+cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, Block *b) {
     if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
         BlockCache &c = block_cache(dev);
         std::lock_guard<std::mutex> lk(c.mu);
-        for (size_t i = c.kept.size(); i-- > 0;) {
-            const KeptBlock b = c.kept[i];
-            if (b.bytes != bytes) continue;
-            if (b.done) {
-                const cudaError_t e = cudaStreamWaitEvent(st, b.done, 0);
+        ++c.turn;
+        int at = -1;
+        for (int i = 0; i < c.n; ++i) {
+            const KeptBlock &k = c.kept[i];
+            if (k.bytes < bytes || k.bytes - bytes > bytes / 2) continue;
+            const KeptBlock *best = at < 0 ? nullptr : &c.kept[at];
+            if (!best || (best->done && !k.done) || (!best->done == !k.done && k.bytes < best->bytes)) at = i;
+        }
+        if (at >= 0) {
+            const KeptBlock k = c.kept[at];
+            if (k.done) {
+                const cudaError_t e = cudaStreamWaitEvent(st, k.done, 0);
                 if (e != cudaSuccess) return e;
-                cudaEventDestroy(b.done);
+                cudaEventDestroy(k.done);
             }
-            c.kept.erase(c.kept.begin() + (std::ptrdiff_t)i);
-            c.bytes -= bytes;
-            *p = b.p;
+            block_remove(c, at);
+            *b = {k.p, k.bytes};
             return cudaSuccess;
         }
+        // a new block: one a little too small, which it will serve in place of,
+        // goes back to the pool, and so do those passed over for long
+        int less = -1, old = 0;
+        for (int i = 0; i < c.n; ++i)
+            if (c.kept[i].bytes < bytes && bytes - c.kept[i].bytes <= c.kept[i].bytes / 2 &&
+                (less < 0 || c.kept[i].bytes > c.kept[less].bytes))
+                less = i;
+        if (less >= 0) block_release(c, less, st);
+        while (old < c.n && c.turn - c.kept[old].turn > KEPT_TURNS) ++old;
+        while (old-- > 0) block_release(c, 0, st);
     }
-    return device_alloc(p, bytes, st);
+    b->bytes = bytes;
+    return device_alloc(&b->p, bytes, st);
 }
 
-void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle) {
-    if (bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
+void block_put(int dev, Block b, cudaStream_t st, bool idle) {
+    if (b.bytes >= BLOCK_MIN && dev >= 0 && dev < 64) {
         const uint64_t most = device_total_mem(dev) / 4;
         BlockCache &c = block_cache(dev);
         std::lock_guard<std::mutex> lk(c.mu);
-        if (c.users > 0 && bytes <= most) {
+        if (c.users > 0 && b.bytes <= most) {
             cudaEvent_t done = nullptr;
             if (!idle && (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess ||
                           cudaEventRecord(done, st) != cudaSuccess)) {
@@ -86,15 +103,22 @@ void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle) {
                 done = nullptr;
                 cudaDeviceSynchronize();              // the stream is gone: wait for what it had
             }
-            c.kept.push_back({p, bytes, done});
-            c.bytes += bytes;
-            size_t n = 0;
-            for (uint64_t left = c.bytes; left > most; ++n) left -= c.kept[n].bytes;
-            if (n) block_release(c, n, st);
+            while (c.n == KEPT_MOST || c.bytes + b.bytes > most) block_release(c, 0, st);
+            c.kept[c.n++] = {b.p, b.bytes, done, c.turn};
+            c.bytes += b.bytes;
             return;
         }
     }
-    cudaFreeAsync(p, st);
+    cudaFreeAsync(b.p, st);
+}
+
+uint64_t block_trim(int dev, cudaStream_t st) {
+    if (dev < 0 || dev >= 64) return 0;
+    BlockCache &c = block_cache(dev);
+    std::lock_guard<std::mutex> lk(c.mu);
+    const uint64_t bytes = c.bytes;
+    while (c.n) block_release(c, 0, st);
+    return bytes;
 }
 
 void block_users(int dev, int change) {
@@ -102,22 +126,22 @@ void block_users(int dev, int change) {
     BlockCache &c = block_cache(dev);
     std::lock_guard<std::mutex> lk(c.mu);
     c.users += change;
-    if (c.users == 0) block_release(c, c.kept.size(), nullptr);
+    while (c.users == 0 && c.n) block_release(c, 0, nullptr);
 }
 
 BlockSet::~BlockSet() {
-    for (int i = 0; i < n_; ++i) block_put(dev_, held_[i].p, held_[i].bytes, st_, !busy_);
+    for (int i = 0; i < n_; ++i) block_put(dev_, held_[i], st_, !busy_);
 }
 
-cudaError_t BlockSet::get(uint64_t bytes, void **p) {
+cudaError_t BlockSet::get(uint64_t bytes, Block *b) {
     if (n_ == MOST) return cudaErrorInvalidValue;
     busy_ = true;
-    const cudaError_t e = block_get(dev_, bytes, st_, p);
-    if (e == cudaSuccess) held_[n_++] = {*p, bytes};
+    const cudaError_t e = block_get(dev_, bytes, st_, b);
+    if (e == cudaSuccess) held_[n_++] = *b;
     return e;
 }
 
-void BlockSet::take(void *p) {
+void BlockSet::take(const void *p) {
     for (int i = 0; i < n_; ++i)
         if (held_[i].p == p) {
             held_[i] = held_[--n_];

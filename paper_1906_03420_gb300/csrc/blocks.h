@@ -18,17 +18,32 @@ cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st);
 template <typename T>
 cudaError_t device_alloc(T **p, size_t bytes, cudaStream_t st) { return device_alloc(reinterpret_cast<void **>(p), bytes, st); }
 
-// Blocks of the arenas of queries and batches, kept for the next call: a few
-// sizes only, gigabytes each.  The stream-ordered pool serves them well as long as no
-// smaller request is cut out of a free one; then the next query waits
-// milliseconds for new memory (four queries with rows took 14 to 25 ms instead
-// of 2).  Any thread and stream may take a block that another gave back: `idle`
-// says that the stream had completed, otherwise an event orders the two.  At
-// most a quarter of the device's memory is kept, nothing under BLOCK_MIN, and
-// nothing at all without a graph on the device.
+// Blocks of the arenas of queries and batches, gigabytes each, kept for the
+// next call.  The stream-ordered pool serves them well as long as no smaller
+// request is cut out of a free one; then the next query waits milliseconds for
+// new memory (four queries with rows took 14 to 25 ms instead of 2).
+//
+// Any thread and stream may take a block that another gave back: `idle` says
+// that the stream had completed, otherwise an event orders the two.  A call
+// takes the smallest kept block that holds what it asks for and is at most half
+// as large again, an idle one first: calls whose budgets differ a little share
+// blocks, and none ties up twice what it asked for.  A request that finds none
+// gives back to the pool one that is a little too small, as the new block will
+// serve in its place, and those that KEPT_TURNS requests have passed over: there
+// they can be cut for other sizes.  At most KEPT_MOST blocks and a quarter of
+// the device's memory are kept, none under BLOCK_MIN, and none at all without a
+// graph on the device.
 constexpr uint64_t BLOCK_MIN = 64ull << 20;
-cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, void **p);
-void block_put(int dev, void *p, uint64_t bytes, cudaStream_t st, bool idle);
+constexpr int KEPT_MOST = 64;
+constexpr uint64_t KEPT_TURNS = 256;
+struct Block {
+    void *p = nullptr;
+    uint64_t bytes = 0;              // of the whole block, which may be larger than asked for
+};
+cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, Block *b);
+void block_put(int dev, Block b, cudaStream_t st, bool idle);
+// Gives every kept block back to the pool, behind the work on `st`; their bytes.
+uint64_t block_trim(int dev, cudaStream_t st);
 // A graph was made on the device (+1) or destroyed (-1, with the device idle).
 void block_users(int dev, int change);
 
@@ -43,7 +58,7 @@ public:
     BlockSet(const BlockSet &) = delete;
     BlockSet &operator=(const BlockSet &) = delete;
     ~BlockSet();
-    cudaError_t get(uint64_t bytes, void **p);
+    cudaError_t get(uint64_t bytes, Block *b);
     void enqueued() { busy_ = true; }
     // The outcome of a wait for the stream.
     bool waited(cudaError_t e) {
@@ -52,18 +67,14 @@ public:
     }
     bool busy() const { return busy_; }
     // Leaves the block at p to the caller, who gives it back by block_put.
-    void take(void *p);
+    void take(const void *p);
 
 private:
     static constexpr int MOST = 4;
-    struct Held {
-        void *p;
-        uint64_t bytes;
-    };
     int dev_, n_ = 0;
     cudaStream_t st_;
     bool busy_ = false;
-    Held held_[MOST];
+    Block held_[MOST];
 };
 
 }  // namespace gsi

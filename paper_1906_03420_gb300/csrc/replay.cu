@@ -129,17 +129,19 @@ extern "C" gsi_status gsi_batch_replay(gsi_batch *b, gsi_result **outs, int32_t 
         int32_t *result = nullptr;
         std::shared_ptr<ResultArena> arena;
         if (!b->L.all_plain && b->L.result_bytes) {
-            if (block_get(g->device, b->L.result_bytes, st, reinterpret_cast<void **>(&result)) != cudaSuccess) {
+            Block blk;
+            if (block_get(g->device, b->L.result_bytes, st, &blk) != cudaSuccess) {
                 (void)cudaGetLastError();
                 set_error("gsi_batch_replay: could not reserve the result arena");
                 return GSI_ENOMEM;
             }
+            result = static_cast<int32_t *>(blk.p);
             arena = std::make_shared<ResultArena>();     // the last result to go releases it
             arena->ptr = result;
             arena->device = g->device;
             arena->stream = st;
             arena->own_stream = !b->own_stream;           // a private stream dies with the batch
-            arena->block = b->L.result_bytes;
+            arena->block = blk.bytes;
         }
         // a private stream's arena goes back on the library's: if this ends early,
         // not before the stream's work has

@@ -453,15 +453,21 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     }
     const bool cleared = memo != nullptr;
     // the control block stands behind the scratch region; all three blocks
-    // have one size, so that a kept one serves as any of them
+    // are asked for in one size, so that a kept one serves as any of them
     const uint64_t block = std::max(s_bytes + PINNED_STAGE, t_bytes);
     gsi_status rc = GSI_OK;
     // from here on the stream may hold work, be it a wait for a block's last
     // user: the blocks go back behind it unless a wait for it succeeds
     pending = true;
     BlockSet blocks(g->device, st);
-    for (void **p : {(void **)&S, (void **)&reg[0], (void **)&reg[1]})
-        if (rc == GSI_OK && blocks.get(block, p) != cudaSuccess) rc = GSI_ENOMEM;
+    Block got[3];
+    for (Block &b : got)
+        if (rc == GSI_OK && blocks.get(block, &b) != cudaSuccess) rc = GSI_ENOMEM;
+    if (rc == GSI_OK) {
+        S = static_cast<uint64_t *>(got[0].p);
+        reg[0] = static_cast<int32_t *>(got[1].p);
+        reg[1] = static_cast<int32_t *>(got[2].p);
+    }
     if (rc == GSI_OK && memo_bytes && !memo) rc = dalloc(*this, (void **)&memo, memo_bytes);
     unsigned char *const ctl = reinterpret_cast<unsigned char *>(S) + s_bytes;
     auto release = [&]() {
@@ -578,6 +584,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     }
     const uint64_t rows = std::min(count, fin[2]);
     int32_t *final_reg = reg[(k - 1) & 1];
+    const uint64_t final_bytes = got[1 + ((k - 1) & 1)].bytes;
     res->count += count;
     if (rows > 0) {
         const uint64_t bytes = rows * (uint64_t)k * 4;
@@ -585,10 +592,10 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         // while the device's allowance for held regions lasts; otherwise (and
         // always when asked for tight rows) the rows move to a tight buffer
         const bool big = bytes * 4 >= t_bytes;
-        if (!tight_rows && (big || hold_region(g->device, t_bytes))) {
+        if (!tight_rows && (big || hold_region(g->device, final_bytes))) {
             gsi_result::Chunk ch{final_reg, rows};
-            ch.held = big ? 0 : t_bytes;
-            ch.block = block;
+            ch.held = big ? 0 : final_bytes;
+            ch.block = final_bytes;
             res->chunks.push_back(ch);
             res->materialised += rows;
             blocks.take(final_reg);

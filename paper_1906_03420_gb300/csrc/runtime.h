@@ -172,7 +172,7 @@ struct BatchLaunch {
     size_t o_q = 0, o_tpl = 0, o_items = 0, o_recs = 0, o_dst = 0, o_sq = 0, o_ready = 0, o_ctl = 0, ctl_bytes = 0;
     unsigned char *ctl = nullptr;            // control block
     unsigned char *arena = nullptr;          // work area: per-CTA slices, then the spill area
-    bool own_arena = false;
+    Block own_arena;                         // its block, unless a workspace brought it
     unsigned long long *dstats = nullptr;    // algorithmic bytes and candidates (optional)
     bool all_plain = false;                  // the budget holds no slice: every query on the plain path
     bool has_template = false;               // the initial query records also live on the device

@@ -30,7 +30,7 @@ EXPORTED = [
     "gsi_query_run", "gsi_result_count", "gsi_result_columns", "gsi_result_copy", "gsi_result_copy_async", "gsi_result_destroy", "gsi_server_estimate",
     "gsi_filter", "gsi_query_signatures", "gsi_join_step", "gsi_join_step_noalloc", "gsi_plan_order",
     "gsi_batch_run", "gsi_batch_autotune", "gsi_batch_autotune_full", "gsi_batch_prepare", "gsi_batch_replay", "gsi_batch_destroy", "gsi_server_create", "gsi_server_submit", "gsi_server_poll", "gsi_server_cancel",
-    "gsi_server_destroy", "gsi_last_error", "gsi_version", "gsi_selftest_wait_timeout",
+    "gsi_server_destroy", "gsi_last_error", "gsi_version", "gsi_memory_trim", "gsi_selftest_wait_timeout",
     "gsi_edge_graph_create", "gsi_edge_graph_destroy", "gsi_edge_graph_line", "gsi_edge_graph_device",
     "gsi_edge_query_line", "gsi_edge_query_run",
 ]
@@ -205,6 +205,8 @@ def load(build_if_missing: bool = False):
     L.gsi_edge_query_run.restype = st
     L.gsi_last_error.argtypes = []
     L.gsi_last_error.restype = ctypes.c_char_p
+    L.gsi_memory_trim.argtypes = [ctypes.c_int32, ctypes.POINTER(ctypes.c_uint64)]
+    L.gsi_memory_trim.restype = st
     L.gsi_selftest_wait_timeout.argtypes = [ctypes.c_int32, ctypes.c_uint64, ctypes.POINTER(ctypes.c_double)]
     L.gsi_selftest_wait_timeout.restype = st
     L.gsi_version.argtypes = []
@@ -678,6 +680,13 @@ class Server:
 
     def __del__(self):
         self.close()
+
+
+def memory_trim(device: int = 0) -> int:
+    """Give the device memory kept between calls back to the device's default pool; returns its bytes."""
+    n = ctypes.c_uint64()
+    _check(load().gsi_memory_trim(device, ctypes.byref(n)), "gsi_memory_trim")
+    return int(n.value)
 
 
 def selftest_wait_timeout(device: int = 0, spin_limit: int = 4096) -> tuple[int, float]:

@@ -97,89 +97,181 @@ using namespace gsi;
 static cudaStream_t S(long i) { return reinterpret_cast<cudaStream_t>(i); }
 constexpr uint64_t MB = 1ull << 20, GB = 1ull << 30;
 
+static Block get(cudaStream_t s, uint64_t bytes) {
+    Block b;
+    CHECK(block_get(0, bytes, s, &b) == cudaSuccess && b.bytes >= bytes && live[b.p] == b.bytes);
+    return b;
+}
 // A block that stream 1 gave back with work on it.
 static void *from_stream_1(uint64_t bytes) {
-    void *p = nullptr;
-    CHECK(block_get(0, bytes, S(1), &p) == cudaSuccess);
-    use(S(1), p);
-    block_put(0, p, bytes, S(1), false);
-    return p;
+    const Block b = get(S(1), bytes);
+    use(S(1), b.p);
+    block_put(0, b, S(1), false);
+    return b.p;
 }
 
 int main(int, char **argv) {
     const std::string what = argv[1];
-    void *p = nullptr, *q = nullptr;
+    Block a, b, c;
     block_users(0, 1);
     if (what == "abandoned set") {                // its stream waits for stream 1, but nobody has waited for it
-        void *b = from_stream_1(GB);
+        void *p = from_stream_1(GB);
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &p) == cudaSuccess && p == b);
+            CHECK(set.get(GB, &a) == cudaSuccess && a.p == p);
             deny = 1;
-            CHECK(set.get(GB, &q) != cudaSuccess);
+            CHECK(set.get(GB, &b) != cudaSuccess);
         }
         deny = 0;
-        CHECK(block_get(0, GB, S(3), &q) == cudaSuccess);
-        use(S(3), q);
+        use(S(3), get(S(3), GB).p);
     } else if (what == "failed wait") {
         from_stream_1(GB);
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &p) == cudaSuccess);
-            use(S(2), p);
+            CHECK(set.get(GB, &a) == cudaSuccess);
+            use(S(2), a.p);
             CHECK(!set.waited(cudaErrorUnknown) && set.busy());
         }
-        CHECK(block_get(0, GB, S(3), &q) == cudaSuccess && q == p);
-        use(S(3), q);
+        b = get(S(3), GB);
+        CHECK(b.p == a.p);
+        use(S(3), b.p);
     } else if (what == "work after the wait") {
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &p) == cudaSuccess);
-            use(S(2), p);
+            CHECK(set.get(GB, &a) == cudaSuccess);
+            use(S(2), a.p);
             wait_host(S(2));
             CHECK(set.waited(cudaSuccess) && !set.busy());
             set.enqueued();
-            use(S(2), p);
+            use(S(2), a.p);
         }
-        CHECK(block_get(0, GB, S(3), &q) == cudaSuccess && q == p);
-        use(S(3), q);
+        b = get(S(3), GB);
+        CHECK(b.p == a.p);
+        use(S(3), b.p);
     } else if (what == "second attempt") {        // a retry takes blocks of an attempt that was waited for
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &p) == cudaSuccess);
-            use(S(2), p);
+            CHECK(set.get(GB, &a) == cudaSuccess);
+            use(S(2), a.p);
             wait_host(S(2));
             set.waited(cudaSuccess);
         }
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &q) == cudaSuccess && q == p);
-            use(S(2), q);                         // and ends without a wait
+            CHECK(set.get(GB, &b) == cudaSuccess && b.p == a.p);
+            use(S(2), b.p);                       // and ends without a wait
         }
-        CHECK(block_get(0, GB, S(3), &q) == cudaSuccess && q == p);
-        use(S(3), q);
+        b = get(S(3), GB);
+        CHECK(b.p == a.p);
+        use(S(3), b.p);
     } else if (what == "waited for") {            // no event between the two
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &p) == cudaSuccess);
-            use(S(2), p);
+            CHECK(set.get(GB, &a) == cudaSuccess);
+            use(S(2), a.p);
             wait_host(S(2));
             set.waited(cudaSuccess);
         }
         const size_t before = waits;
-        CHECK(block_get(0, GB, S(3), &q) == cudaSuccess && q == p);
-        use(S(3), q);
-        CHECK(waits == before);
+        b = get(S(3), GB);
+        CHECK(b.p == a.p && waits == before);
+        use(S(3), b.p);
     } else if (what == "taken block") {           // a result keeps it: the set does not give it back
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &p) == cudaSuccess && set.get(GB, &q) == cudaSuccess);
-            set.take(p);
+            CHECK(set.get(GB, &a) == cudaSuccess && set.get(GB, &b) == cudaSuccess);
+            set.take(a.p);
         }
-        void *r = nullptr, *t = nullptr;
-        CHECK(block_get(0, GB, S(2), &r) == cudaSuccess && block_get(0, GB, S(2), &t) == cudaSuccess);
-        CHECK(r != p && t != p && live.count(p));
-        block_put(0, p, GB, S(2), false);
+        CHECK(get(S(2), GB).p == b.p && get(S(2), GB).p != a.p && live.count(a.p));
+        block_put(0, a, S(2), false);
+    } else if (what == "near size") {             // taken, with its own size; not one half as large again or more
+        a = get(S(1), 3 * GB);
+        block_put(0, a, S(1), true);
+        b = get(S(1), 2 * GB);
+        CHECK(b.p == a.p && b.bytes == 3 * GB);
+        block_put(0, b, S(1), true);
+        CHECK(get(S(1), 2 * GB - 1).p != a.p);
+        CHECK(live.count(a.p) && get(S(1), 3 * GB + 1).p != a.p && !live.count(a.p));     // the larger one replaces it
+    } else if (what == "smallest that fits") {
+        Block x[3];
+        for (int i = 0; i < 3; ++i) x[i] = get(S(1), (24 + 4 * ((i + 1) % 3)) * GB / 8);     // 3.5, 4, 3
+        for (Block &k : x) block_put(0, k, S(1), true);
+        CHECK(get(S(1), 3 * GB).p == x[2].p && get(S(1), 3 * GB).p == x[0].p && get(S(1), 3 * GB).p == x[1].p);
+    } else if (what == "idle first") {            // a larger idle block goes before one with work on it
+        a = get(S(1), GB);
+        b = get(S(1), GB + 64 * MB);
+        block_put(0, b, S(1), true);
+        use(S(1), a.p);
+        block_put(0, a, S(1), false);
+        const size_t before = waits;
+        CHECK(get(S(2), GB).p == b.p && waits == before);
+        c = get(S(2), GB);
+        CHECK(c.p == a.p && waits == before + 1);
+        use(S(2), c.p);
+    } else if (what == "changing budgets") {      // no two calls of one size: what is kept stays a few blocks
+        size_t most = 0;
+        for (uint64_t i = 0; i < 400; ++i) {
+            const uint64_t bytes = 64 * MB + (i * 7919 % 400) * 2 * MB;
+            BlockSet set(0, S(1));
+            for (Block *k : {&a, &b, &c}) CHECK(set.get(bytes, k) == cudaSuccess && k->bytes <= bytes + bytes / 2);
+            set.waited(cudaSuccess);
+            most = std::max(most, live.size());
+        }
+        // no two of a call's three blocks are kept in sizes nearer than half as large again, and from 64 to 862 MB there
+        // are at most seven such sizes
+        CHECK(most <= 3 * 7);
+        CHECK(mallocs <= 3 * 400 / 10);
+    } else if (what == "passed over") {           // sizes that nobody asks for any more go back to the pool
+        for (uint64_t i = 0; i < 10; ++i) a = get(S(1), (2 + 2 * i) * GB / 2 + GB), block_put(0, a, S(1), true);
+        for (uint64_t i = 0; i <= 2 * KEPT_TURNS; ++i) {
+            b = get(S(1), 100 * MB);
+            block_put(0, b, S(1), true);
+        }
+        c = get(S(1), 300 * MB);                  // the miss on which they go
+        CHECK(live.size() == 2);
+    } else if (what == "a quarter of the memory") {
+        total = 16 * GB;
+        Block x[6];
+        for (Block &k : x) k = get(S(1), GB);
+        use(S(1), x[0].p);
+        for (Block &k : x) block_put(0, k, S(1), false);
+        CHECK(live.size() == 4 && !live.count(x[0].p) && !live.count(x[1].p));     // the oldest two went
+        a = get(S(1), 5 * GB);
+        block_put(0, a, S(1), true);              // larger than the share: not kept
+        CHECK(live.size() == 4);
+    } else if (what == "number of blocks") {
+        total = 1024 * GB;
+        std::vector<Block> x(KEPT_MOST + 3);
+        for (Block &k : x) k = get(S(1), 64 * MB);
+        for (Block &k : x) block_put(0, k, S(1), true);
+        CHECK(live.size() == (size_t)KEPT_MOST && !live.count(x[2].p) && live.count(x[3].p));
+    } else if (what == "small ones") {            // left to the pool
+        a = get(S(1), 64 * MB - 1);
+        block_put(0, a, S(1), true);
+        CHECK(live.empty());
+    } else if (what == "out of memory") {         // any failed allocation gives the kept blocks back and tries again
+        total = 8 * GB;
+        from_stream_1(GB);
+        from_stream_1(GB + GB / 8);
+        void *p = nullptr;
+        CHECK(device_alloc(&p, 7 * GB, S(2)) == cudaSuccess && live.size() == 1);
+        CHECK(device_alloc(&p, 2 * GB, S(2)) == cudaErrorMemoryAllocation);
+    } else if (what == "trim") {
+        from_stream_1(GB);
+        a = get(S(2), 5 * GB);
+        block_put(0, a, S(2), true);
+        CHECK(block_trim(0, S(3)) == 6 * GB && live.empty() && events.empty() && block_trim(0, S(3)) == 0);
+    } else if (what == "last graph") {            // nothing is kept without one; a result that outlives it frees its block
+        block_users(0, 1);
+        a = get(S(1), GB);
+        from_stream_1(GB);
+        wait_host(S(1));                          // a graph goes with the device idle
+        block_users(0, -1);
+        CHECK(live.size() == 2);
+        block_users(0, -1);
+        CHECK(live.size() == 1);
+        block_put(0, a, S(1), false);
+        CHECK(live.empty() && events.empty());
     } else {
         std::printf("no such case\n");
         return 1;
