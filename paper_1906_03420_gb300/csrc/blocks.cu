@@ -17,11 +17,27 @@ struct BlockCache {
     KeptBlock kept[KEPT_MOST];       // oldest first; no allocation, as results are destroyed without exceptions
     int n = 0, users = 0;
     uint64_t bytes = 0, turn = 0;
+    // events that no block has: creating or destroying one waits for any thread
+    // that is in a copy to pageable memory, until that copy's stream gets there
+    cudaEvent_t spare[KEPT_MOST];
+    int nspare = 0;
 };
 
 BlockCache &block_cache(int dev) {   // never destroyed: results may outlive static objects
     static BlockCache *const c = new BlockCache[64];
     return c[dev];
+}
+
+// An event recorded on st; null, with the device waited for, if there is none.
+cudaEvent_t take_event(BlockCache &c, cudaStream_t st) {
+    cudaEvent_t e = nullptr;
+    if (c.nspare) e = c.spare[--c.nspare];
+    else if (cudaEventCreateWithFlags(&e, cudaEventDisableTiming) != cudaSuccess) e = nullptr;
+    if (e && cudaEventRecord(e, st) == cudaSuccess) return e;
+    (void)cudaGetLastError();
+    if (e) c.spare[c.nspare++] = e;
+    cudaDeviceSynchronize();                          // the stream is gone: wait for what it had
+    return nullptr;
 }
 
 void block_remove(BlockCache &c, int i) {
@@ -34,7 +50,7 @@ void block_release(BlockCache &c, int i, cudaStream_t st) {
     const KeptBlock b = c.kept[i];
     if (b.done) {
         cudaStreamWaitEvent(st, b.done, 0);
-        cudaEventDestroy(b.done);
+        c.spare[c.nspare++] = b.done;
     }
     cudaFreeAsync(b.p, st);
     block_remove(c, i);
@@ -68,7 +84,7 @@ cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, Block *b) {
             if (k.done) {
                 const cudaError_t e = cudaStreamWaitEvent(st, k.done, 0);
                 if (e != cudaSuccess) return e;
-                cudaEventDestroy(k.done);
+                c.spare[c.nspare++] = k.done;
             }
             block_remove(c, at);
             *b = {k.p, k.bytes};
@@ -95,15 +111,8 @@ void block_put(int dev, Block b, cudaStream_t st, bool idle) {
         BlockCache &c = block_cache(dev);
         std::lock_guard<std::mutex> lk(c.mu);
         if (c.users > 0 && b.bytes <= most) {
-            cudaEvent_t done = nullptr;
-            if (!idle && (cudaEventCreateWithFlags(&done, cudaEventDisableTiming) != cudaSuccess ||
-                          cudaEventRecord(done, st) != cudaSuccess)) {
-                (void)cudaGetLastError();
-                if (done) cudaEventDestroy(done);
-                done = nullptr;
-                cudaDeviceSynchronize();              // the stream is gone: wait for what it had
-            }
             while (c.n == KEPT_MOST || c.bytes + b.bytes > most) block_release(c, 0, st);
+            const cudaEvent_t done = idle ? nullptr : take_event(c, st);
             c.kept[c.n++] = {b.p, b.bytes, done, c.turn};
             c.bytes += b.bytes;
             return;
@@ -126,7 +135,9 @@ void block_users(int dev, int change) {
     BlockCache &c = block_cache(dev);
     std::lock_guard<std::mutex> lk(c.mu);
     c.users += change;
-    while (c.users == 0 && c.n) block_release(c, 0, nullptr);
+    if (c.users) return;
+    while (c.n) block_release(c, 0, nullptr);
+    while (c.nspare) cudaEventDestroy(c.spare[--c.nspare]);
 }
 
 BlockSet::~BlockSet() {

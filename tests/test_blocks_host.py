@@ -24,7 +24,7 @@ def program(tmp_path_factory):
 @pytest.mark.parametrize("case", ["abandoned set", "failed wait", "work after the wait", "second attempt", "waited for",
                                   "taken block", "near size", "smallest that fits", "idle first", "changing budgets",
                                   "passed over", "a quarter of the memory", "number of blocks", "small ones", "out of memory",
-                                  "trim", "last graph"])
+                                  "trim", "events", "last graph"])
 def test_blocks(program, case):
     r = subprocess.run([program, case], capture_output=True, text=True, timeout=60)
     assert r.returncode == 0, r.stdout + r.stderr
