@@ -12,8 +12,8 @@ using namespace gsi;
 
 // Result memory is released stream-ordered on a library stream: cudaFree
 // would wait for every kernel on the device, stalling concurrent queries.
-// The producing stream has always completed before a result is handed out. A
-// graph build copies its edge arrays there.
+// The producing stream has always completed before a result is handed out.
+// Nothing is put there that waits for a caller's stream.
 cudaStream_t gsi::library_stream(int dev) {
     static std::mutex mu;
     static cudaStream_t streams[64];

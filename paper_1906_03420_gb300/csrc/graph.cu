@@ -295,19 +295,23 @@ struct Temps {
     std::vector<void *> all;
     explicit Temps(cudaStream_t s) : st(s) {}
     ~Temps() {
-        if (other) cudaStreamSynchronize(other);      // an error may leave copies behind
+        if (other) {
+            cudaStreamSynchronize(other);             // an error may leave copies behind
+            cudaStreamDestroy(other);
+        }
         if (ev) cudaEventDestroy(ev);
         for (void *p : all) cudaFreeAsync(p, st);
     }
     // A second stream, behind what this one has so far; join() orders the first
-    // behind it.
+    // behind it.  It is the build's own: on a shared one, whatever else goes
+    // there (results that are released) would wait for the caller's stream too.
     cudaStream_t other = nullptr;
     cudaEvent_t ev = nullptr;
-    gsi_status beside(cudaStream_t s) {
+    gsi_status beside() {
+        GSI_CUDA_TRY(cudaStreamCreateWithFlags(&other, cudaStreamNonBlocking));
         GSI_CUDA_TRY(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
         GSI_CUDA_TRY(cudaEventRecord(ev, st));
-        GSI_CUDA_TRY(cudaStreamWaitEvent(s, ev, 0));
-        other = s;
+        GSI_CUDA_TRY(cudaStreamWaitEvent(other, ev, 0));
         return GSI_OK;
     }
     gsi_status join() {
@@ -323,6 +327,16 @@ struct Temps {
         return GSI_OK;
     }
 };
+
+// Reads device memory once the stream's work is done.  The wait comes first: a
+// copy to pageable memory waits for it inside the driver, where other threads'
+// calls that create or destroy an event then wait too.
+gsi_status read_back(void *dst, const void *src, size_t bytes, cudaStream_t st) {
+    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    GSI_CUDA_TRY(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDeviceToHost, st));
+    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    return GSI_OK;
+}
 
 unsigned grid_for(int64_t n) {
     int64_t b = (n + NT - 1) / NT;
@@ -378,13 +392,12 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
     GSI_CUDA_TRY(cudaMemcpyAsync(d_w, &hw, sizeof hw, cudaMemcpyHostToDevice, st));
     GSI_CUDA_TRY(cudaMemcpyAsync(d_vlab, vlab, sizeof(int32_t) * (size_t)n, cudaMemcpyDefault, st));
     k_label_range<<<few_blocks(n), NT, 0, st>>>(d_vlab, n, &d_w->lo);
-    // a large edge list is copied on the library's own stream: the vertices
-    // are sorted meanwhile, and the pairs while the edge labels arrive (16M
-    // edges: 365 us an array; 4.58 -> 4.26 ms)
-    const cudaStream_t cs = m >= COPY_APART ? library_stream(g->device) : st;
-    if (cs != st) GSI_TRY(tmps.beside(cs));
-    GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
-    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    // a large edge list is copied on a stream of its own: the vertices are
+    // sorted meanwhile, and the pairs while the edge labels arrive (16M edges:
+    // 365 us an array; 4.58 -> 4.26 ms)
+    if (m >= COPY_APART) GSI_TRY(tmps.beside());
+    const cudaStream_t cs = tmps.other ? tmps.other : st;
+    GSI_TRY(read_back(&hw, d_w, sizeof hw, st));
     const int nb = ceil_log2_bits((uint64_t)(n > 1 ? n - 1 : 1));
 
     // the vertices in the order of (label, id), the checks of the edges behind
@@ -423,9 +436,8 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
         k_validate<<<few_blocks(m), NT, 0, st>>>(d_src, d_dst, d_elab, m, n, &d_w->flags, &d_w->maxlab);
     }
     std::vector<int32_t> labels(2 * (size_t)most);     // the distinct labels, then where each begins
-    GSI_CUDA_TRY(cudaMemcpyAsync(labels.data(), d_labels, sizeof(int32_t) * labels.size(), cudaMemcpyDeviceToHost, st));
-    GSI_CUDA_TRY(cudaMemcpyAsync(&hw, d_w, sizeof hw, cudaMemcpyDeviceToHost, st));
-    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    GSI_TRY(read_back(&hw, d_w, sizeof hw, st));
+    GSI_TRY(read_back(labels.data(), d_labels, sizeof(int32_t) * labels.size(), st));
     if (hw.flags & ~(unsigned)DUP_PAIR) {
         set_error(std::string("gsi_graph_create: ") + ((hw.flags & BAD_ID) ? "vertex id out of range " : "") +
                   ((hw.flags & SELF_LOOP) ? "self-loop " : "") + ((hw.flags & NEG_LABEL) ? "negative edge label" : ""));
@@ -502,10 +514,9 @@ gsi_status build_graph(gsi_graph *g, const int32_t *vlab, int32_t n, const int32
         k_label_count<<<(unsigned)((step + NT - 1) / NT), NT, 0, st>>>(g->off, nseg, L, step, d_freq);
     }
     g->freq.assign((size_t)L, 0);
-    GSI_CUDA_TRY(cudaMemcpyAsync(g->freq.data(), d_freq, sizeof(uint64_t) * (size_t)L, cudaMemcpyDeviceToHost, st));
     GSI_CUDA_TRY(cudaGetLastError());
     GSI_CUDA_TRY(cudaEventRecord(e1, st));
-    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    GSI_TRY(read_back(g->freq.data(), d_freq, sizeof(uint64_t) * (size_t)L, st));
     for (uint64_t &f : g->freq) f /= 2;
     float ms = 0;
     cudaEventElapsedTime(&ms, e0, e1);
