@@ -284,9 +284,13 @@ gsi_status gsi_query_signatures(const int32_t *qvlab, int32_t k, const int32_t *
  * bounded by its shortest linking list restricted to ulabel (the Alg. 4
  * bound, chosen per row).  Writes rows (m || w) to out (int32[out_cap][t+1])
  * and the number of rows found to *count (host).  Rows beyond out_cap are
- * counted, not written.  Scratch memory is allocated stream-ordered on
- * `stream`.  Errors: GSI_EINVAL for t < 1, t >= 32, d < 1, d > t, a column
- * outside [0,t) or a label < 0.
+ * counted, not written.  The step runs as one cooperative launch; if its
+ * scratch cannot be reserved or one of its grid barriers gives up, it runs again
+ * over a scan of the rows' bounds, without barriers.  Scratch is allocated
+ * stream-ordered on `stream`: 4t + 16 bytes a row, and 8 n min(d, 4) bytes when R
+ * >= n (second form: 12 bytes a row, and 8 for every 1024 candidate slots).
+ * Errors: GSI_EINVAL for t < 1, t >= 32, d < 1, d > t, a column outside [0,t) or
+ * a label < 0; GSI_ENOMEM / GSI_ECUDA for device failures.
  */
 gsi_status gsi_join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, const uint32_t *cand,
                          int32_t ulabel, const int32_t *col, const int32_t *lab, int32_t d, int32_t *out,
@@ -594,6 +598,12 @@ gsi_status gsi_edge_query_run(gsi_edge_graph *g, const int32_t *qvlab, int32_t k
  * outcome), GSI_OK if it did not, GSI_ECUDA on launch failure.
  */
 gsi_status gsi_selftest_wait_timeout(int32_t device, uint64_t spin_limit, double *elapsed_ms);
+
+/* gsi_join_step as it runs when a grid barrier of its cooperative launch has
+   given up (the kernel finds the barrier in that state and waits nowhere). */
+gsi_status gsi_selftest_join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, const uint32_t *cand,
+                                  int32_t ulabel, const int32_t *col, const int32_t *lab, int32_t d, int32_t *out,
+                                  uint64_t out_cap, uint64_t *count, void *stream);
 
 /* Message of the calling thread's last failure ("" if none). */
 const char *gsi_last_error(void);

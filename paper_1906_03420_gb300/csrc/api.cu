@@ -80,6 +80,67 @@ gsi_status join_step_args(const char *who, gsi_graph *g, const int32_t *M, uint6
 }
 }  // namespace gsi
 
+// gsi_join_step; give_up: the cooperative launch as if a barrier wait had run
+// past its limit.
+static gsi_status join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, const uint32_t *cand, int32_t ulabel,
+                            const int32_t *col, const int32_t *lab, int32_t d, int32_t *out, uint64_t out_cap, uint64_t *count,
+                            cudaStream_t st, bool give_up) {
+    JoinStep s;
+    bool empty = false;
+    GSI_TRY(join_step_args("gsi_join_step", g, M, R, t, cand, ulabel, col, lab, d, out, out_cap, count, &s, &empty));
+    if (empty) return GSI_OK;
+    GSI_TRY(prepare_device(g->device));
+    // one launch of the query kernel; where that cannot take the step, the
+    // slot tiles over a scan of the rows' bounds (3M rows of 4 columns, two
+    // lists: 233 us of kernels and two waits of the host between them, now 124)
+    bool ran = false;
+    GSI_TRY(step_coop(g, M, R, s, cand, out, out_cap, count, give_up, &ran, st));
+    if (ran) return GSI_OK;
+    uint64_t *F = nullptr, *scr = nullptr;
+    uint64_t h[2] = {0, 0};
+    int64_t *part = nullptr;
+    unsigned long long *d_cnt = nullptr;
+    GSI_CUDA_TRY(device_alloc(&F, 8 * (R + 1), st));
+    GSI_CUDA_TRY(device_alloc(&scr, 8 * (uint64_t)join_scan_scratch(R), st));
+    GSI_CUDA_TRY(device_alloc(&d_cnt, 8, st));
+    gsi_status rc = launch_join_scan(g, M, R, s, F, scr, st);
+    uint64_t total = 0;
+    if (rc == GSI_OK) {
+        if (cudaMemcpyAsync(h, F + R, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess) {
+            set_error("gsi_join_step: readback failed");
+            rc = GSI_ECUDA;
+        }
+        total = h[0];
+    }
+    if (rc == GSI_OK) {
+        const uint64_t ntiles = join_tiles(total);
+        if (device_alloc(&part, 8 * (ntiles + 1), st) != cudaSuccess ||
+            cudaMemsetAsync(d_cnt, 0, 8, st) != cudaSuccess) {
+            set_error("gsi_join_step: scratch allocation failed");
+            rc = GSI_ENOMEM;
+        }
+    }
+    if (rc == GSI_OK) rc = launch_partition(F, R, total, part, st);
+    if (rc == GSI_OK)
+        rc = launch_join(g, M, R, s, F, total, part, cand, out, out_cap, d_cnt, out_cap == 0 ? 1 : 0, nullptr, st);
+    if (rc == GSI_OK) {
+        if (cudaMemcpyAsync(h, d_cnt, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
+            cudaStreamSynchronize(st) != cudaSuccess) {
+            set_error("gsi_join_step: kernel or readback failed");
+            rc = GSI_ECUDA;
+        } else {
+            *count = h[0];
+        }
+    }
+    cudaFreeAsync(F, st);
+    cudaFreeAsync(scr, st);
+    if (part) cudaFreeAsync(part, st);
+    cudaFreeAsync(d_cnt, st);
+    cudaStreamSynchronize(st);
+    return rc;
+}
+
 extern "C" {
 
 const char *gsi_version(void) { return "gsi-gb300 0.1 (sm_103a)"; }
@@ -334,61 +395,15 @@ gsi_status gsi_join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, 
                          int32_t ulabel, const int32_t *col, const int32_t *lab, int32_t d, int32_t *out,
                          uint64_t out_cap, uint64_t *count, void *stream) {
     GSI_API_BEGIN
-    JoinStep s;
-    bool empty = false;
-    GSI_TRY(join_step_args("gsi_join_step", g, M, R, t, cand, ulabel, col, lab, d, out, out_cap, count, &s, &empty));
-    if (empty) return GSI_OK;
-    GSI_TRY(prepare_device(g->device));
-    cudaStream_t st = (cudaStream_t)stream;
-    // one launch of the query kernel; where that cannot take the step, the
-    // slot tiles over a scan of the rows' bounds (3M rows of 4 columns, two
-    // lists: 233 us of kernels and two waits of the host between them, now 124)
-    bool ran = false;
-    GSI_TRY(step_coop(g, M, R, s, cand, out, out_cap, count, &ran, st));
-    if (ran) return GSI_OK;
-    uint64_t *F = nullptr, *scr = nullptr;
-    uint64_t h[2] = {0, 0};
-    int64_t *part = nullptr;
-    unsigned long long *d_cnt = nullptr;
-    GSI_CUDA_TRY(device_alloc(&F, 8 * (R + 1), st));
-    GSI_CUDA_TRY(device_alloc(&scr, 8 * (uint64_t)join_scan_scratch(R), st));
-    GSI_CUDA_TRY(device_alloc(&d_cnt, 8, st));
-    gsi_status rc = launch_join_scan(g, M, R, s, F, scr, st);
-    uint64_t total = 0;
-    if (rc == GSI_OK) {
-        if (cudaMemcpyAsync(h, F + R, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess) {
-            set_error("gsi_join_step: readback failed");
-            rc = GSI_ECUDA;
-        }
-        total = h[0];
-    }
-    if (rc == GSI_OK) {
-        const uint64_t ntiles = join_tiles(total);
-        if (device_alloc(&part, 8 * (ntiles + 1), st) != cudaSuccess ||
-            cudaMemsetAsync(d_cnt, 0, 8, st) != cudaSuccess) {
-            set_error("gsi_join_step: scratch allocation failed");
-            rc = GSI_ENOMEM;
-        }
-    }
-    if (rc == GSI_OK) rc = launch_partition(F, R, total, part, st);
-    if (rc == GSI_OK)
-        rc = launch_join(g, M, R, s, F, total, part, cand, out, out_cap, d_cnt, out_cap == 0 ? 1 : 0, nullptr, st);
-    if (rc == GSI_OK) {
-        if (cudaMemcpyAsync(h, d_cnt, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-            cudaStreamSynchronize(st) != cudaSuccess) {
-            set_error("gsi_join_step: kernel or readback failed");
-            rc = GSI_ECUDA;
-        } else {
-            *count = h[0];
-        }
-    }
-    cudaFreeAsync(F, st);
-    cudaFreeAsync(scr, st);
-    if (part) cudaFreeAsync(part, st);
-    cudaFreeAsync(d_cnt, st);
-    cudaStreamSynchronize(st);
-    return rc;
+    return join_step(g, M, R, t, cand, ulabel, col, lab, d, out, out_cap, count, (cudaStream_t)stream, false);
+    GSI_API_END
+}
+
+gsi_status gsi_selftest_join_step(gsi_graph *g, const int32_t *M, uint64_t R, int32_t t, const uint32_t *cand,
+                                  int32_t ulabel, const int32_t *col, const int32_t *lab, int32_t d, int32_t *out,
+                                  uint64_t out_cap, uint64_t *count, void *stream) {
+    GSI_API_BEGIN
+    return join_step(g, M, R, t, cand, ulabel, col, lab, d, out, out_cap, count, (cudaStream_t)stream, true);
     GSI_API_END
 }
 

@@ -190,9 +190,10 @@ bool query_counts_tail(const std::vector<JoinStep> &steps, int k, int count_only
 gsi_status query_coop_configs(const gsi_graph *g, const std::vector<JoinStep> &steps, int k, const uint32_t *bitmaps,
                               const int32_t *order, int count_only, unsigned long long *stats, uint64_t *memo, bool nodedup,
                               void *cfg_host, size_t *smem);
-// One step over a table of the caller's on the same kernel; waits for it.
+// One step over a table of the caller's on the same kernel; waits for it.  *ran:
+// it was done (see join.cu).
 gsi_status step_coop(const gsi_graph *g, const int32_t *M, uint64_t R, const JoinStep &s, const uint32_t *cand,
-                     int32_t *out, uint64_t out_cap, uint64_t *count, bool *ran, cudaStream_t st);
+                     int32_t *out, uint64_t out_cap, uint64_t *count, bool give_up, bool *ran, cudaStream_t st);
 // nodedup (configs): rows of single-edge steps are joined one by one (no
 // warp groups, no memo).  listwise (launch): the kernel variant that also
 // counts whole-list bytes (stats[2]).

@@ -30,7 +30,7 @@ EXPORTED = [
     "gsi_query_run", "gsi_result_count", "gsi_result_columns", "gsi_result_copy", "gsi_result_copy_async", "gsi_result_destroy", "gsi_server_estimate",
     "gsi_filter", "gsi_query_signatures", "gsi_join_step", "gsi_join_step_noalloc", "gsi_plan_order",
     "gsi_batch_run", "gsi_batch_autotune", "gsi_batch_autotune_full", "gsi_batch_prepare", "gsi_batch_replay", "gsi_batch_destroy", "gsi_server_create", "gsi_server_submit", "gsi_server_poll", "gsi_server_cancel",
-    "gsi_server_destroy", "gsi_last_error", "gsi_version", "gsi_memory_trim", "gsi_selftest_wait_timeout",
+    "gsi_server_destroy", "gsi_last_error", "gsi_version", "gsi_memory_trim", "gsi_selftest_wait_timeout", "gsi_selftest_join_step",
     "gsi_edge_graph_create", "gsi_edge_graph_destroy", "gsi_edge_graph_line", "gsi_edge_graph_device",
     "gsi_edge_query_line", "gsi_edge_query_run",
 ]
@@ -153,6 +153,8 @@ def load(build_if_missing: bool = False):
                                 ctypes.c_int32, VP, ctypes.c_uint64, U64P, VP]
     L.gsi_join_step.restype = st
     L.gsi_join_step_noalloc.argtypes = L.gsi_join_step.argtypes
+    L.gsi_selftest_join_step.argtypes = L.gsi_join_step.argtypes
+    L.gsi_selftest_join_step.restype = st
     L.gsi_join_step_noalloc.restype = st
     L.gsi_plan_order.argtypes = [ctypes.c_int32, I32P, I32P, I32P, ctypes.c_int32, U64P, U64P, ctypes.c_int32,
                                  I32P, I32P]
@@ -418,6 +420,17 @@ class Graph:
         cnt = ctypes.c_uint64()
         _check(load().gsi_join_step(self._h, M_ptr, R, t, cand_ptr, ulabel, _p32(c), _p32(l), c.shape[0], out_ptr,
                                     out_cap, ctypes.byref(cnt), _stream_handle(stream)), "gsi_join_step")
+        return int(cnt.value)
+
+    def selftest_join_step(self, M_ptr: int, R: int, t: int, cand_ptr: int, ulabel: int, cols, labs, out_ptr: int,
+                           out_cap: int, stream=None) -> int:
+        """join_step as it runs when a grid barrier of its cooperative launch has given up."""
+        c = _i32(cols)
+        l = _i32(labs)
+        cnt = ctypes.c_uint64()
+        _check(load().gsi_selftest_join_step(self._h, M_ptr, R, t, cand_ptr, ulabel, _p32(c), _p32(l), c.shape[0],
+                                             out_ptr, out_cap, ctypes.byref(cnt), _stream_handle(stream)),
+               "gsi_selftest_join_step")
         return int(cnt.value)
 
     def join_step_noalloc(self, M_ptr: int, R: int, t: int, cand_ptr: int, ulabel: int, cols, labs, out_ptr: int,

@@ -63,3 +63,19 @@ def test_a_row_limit_past_every_buffer_writes_all_rows(step, t, cap):
     got, out = run(G.join_step, args, n, cap)
     assert got == want == n
     assert np.array_equal(oracle.sort_rows(out), oracle.sort_rows(rows))
+
+
+@pytest.mark.parametrize("rows,t,links", [(1, 1, 1), (2000, 1, 1), (2000, 3, 2), (2000, 7, 7), (400_003, 2, 2)])
+@pytest.mark.parametrize("counted", [False, True])
+def test_a_barrier_that_gave_up_leaves_the_step_to_the_scan(step, rows, t, links, counted):
+    """The cooperative launch finds its barrier given up; the call still returns every row, or their number."""
+    G, make = step
+    args = make(rows, t, links)
+    n, _ = run(G.join_step_noalloc, args, 1, 0)
+    cap = 0 if counted else n
+    want, rows_want = run(G.join_step_noalloc, args, max(n, 1), cap)
+    got, out = run(G.selftest_join_step, args, max(n, 1), cap)
+    assert got == want == n
+    assert np.array_equal(oracle.sort_rows(out), oracle.sort_rows(rows_want))
+    got, out = run(G.join_step, args, max(n, 1), cap)
+    assert got == n and np.array_equal(oracle.sort_rows(out), oracle.sort_rows(rows_want))
