@@ -157,15 +157,15 @@ struct DStep {
     unsigned long long nlong;          // rows set aside for the slot tiles and their slots (LongTable::ctr)
     unsigned long long row_ticket, slot_ticket;   // the work handed out on demand (row_pass, long_rows_join)
     uint64_t out_cap;
-    unsigned fail;                     // 1: this step's long-row table was full (a step of its own reads it, so
+    unsigned fail;                     // LONG_*: this step's long rows did not fit (a step of its own reads it, so
     unsigned pad;                      // that no CTA sees a later step's failure and leaves the others waiting)
 };
 
 // Grid-barrier and status words of one cooperative query launch.
 struct QueryCtl {
     unsigned bar;         // arrivals at the barriers so far; BAR_FAIL: a wait gave up
-    unsigned fail;        // 1 scratch too small (or a sub-list too long for a bound record),
-                          // 2 table overflow, 4 barrier wait gave up
+    unsigned fail;        // 1 scratch too small, 2 table overflow, 4 barrier wait gave up, 8 too many
+                          // candidate slots in a step or too long a sub-list, whatever the arena
     unsigned long long spin_limit;   // sleeps before a barrier wait gives up (0 = default)
 };
 constexpr int QUERY_MAX_CTAS = 2048;

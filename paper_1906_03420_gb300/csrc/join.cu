@@ -271,8 +271,8 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
         }
         copy_wait();
         if (!grid_barrier(ctl, G, epoch, st, &view_s)) return;
-        if (view_s.fail) {                                    // long-row table full: a larger arena
-            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->fail, 1u);
+        if (view_s.fail) {                                    // the long rows do not fit
+            if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&ctl->fail, view_s.fail & LONG_NEVER ? 8u : 1u);
             return;
         }
         // ---- long rows through the candidate-slot tiles

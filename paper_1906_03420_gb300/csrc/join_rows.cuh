@@ -56,8 +56,12 @@ constexpr int SHORT_MAX = 16;     // rows with at most this many candidates are 
 // above them, so that F ascends with the row index and is written with the
 // row: no scan over the table, no pass that cuts it into tiles, and no grid
 // barriers between them (they cost 14-20 us a step, more than the join of most
-// steps).  rbits holds the step's row count; a step whose slots do not fit the
-// other bits fails like one whose table is full.
+// steps).  rbits holds the step's row count, or the table's room where that is
+// less: the reservation that leaves the room sees that it does, so a count that
+// runs into the slots' bits is always of a step that has failed.  A table that is
+// full fails the step with LONG_FULL, and more room helps; slots that do not fit
+// the other bits (2^37 of them for the 10^8 rows of a first arena) or a sub-list
+// that does not fit a bound record fail it with LONG_NEVER, and it does not.
 struct LongTable {
     int32_t *rows;
     uint64_t *F;
@@ -67,6 +71,22 @@ struct LongTable {
     unsigned long long *ctr;
     int rbits;
 };
+
+constexpr unsigned LONG_FULL = 1u, LONG_NEVER = 2u;
+
+__host__ __device__ inline int long_row_bits(uint64_t R, uint64_t cap) {
+    int b = 1;
+    for (uint64_t x = R < cap ? R : cap; x >> b;) ++b;
+    return b;
+}
+// How a reservation of `rows` rows and `slots` slots (below 2^63) on a counter
+// that stood at `old` fails: 0 if it does not.
+__host__ __device__ __forceinline__ unsigned long_fails(unsigned long long old, uint64_t rows, uint64_t slots, int rbits,
+                                                        uint64_t cap) {
+    const uint64_t at = old & ((1ull << rbits) - 1ull);
+    return (at + rows > cap ? LONG_FULL : 0u) |
+           ((old >> rbits) + slots >= 1ull << (64 - rbits) ? LONG_NEVER : 0u);
+}
 
 // The long-row table of step t, whose input has R rows, in a scratch region of
 // S_words 8-byte words: F, rows, bound records.
@@ -79,7 +99,7 @@ __device__ __forceinline__ LongTable long_table(uint64_t *S, uint64_t S_words, i
     lt.bnd = reinterpret_cast<uint32_t *>(lt.rows + lt.cap * (uint64_t)t);
     lt.blo = lt.bnd + lt.cap;
     lt.ctr = ctr;
-    lt.rbits = 64 - __clzll((long long)(R | 1));
+    lt.rbits = 64 - __clzll((long long)(min(R, lt.cap) | 1));      // long_row_bits, without its loop
     return lt;
 }
 
@@ -404,8 +424,7 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
 // the batches go out that way, at least two to a CTA, and the rest on demand:
 // rows differ in their lists, and of a step of millions of rows a quarter of
 // the time went by while the last CTAs worked alone.  `a` should live in shared memory.  Survivors go to out (up to cap rows; `count` is
-// exact), long rows to lt.  Bit 1 of *fail is set when the long-row table is
-// full or a bound does not fit its record.  When a.stats is set, adds this
+// exact), long rows to lt.  *fail gets LONG_* bits when they do not fit.  When a.stats is set, adds this
 // thread's algorithmic bytes (rows read, lists located and read; survivors
 // are counted by the caller) to *abytes, the same under the whole-list model
 // to *lbytes (only when LW), and its candidate slots to *items.
@@ -518,7 +537,8 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
             base_s = ntot ? atomicAdd(count, (unsigned long long)ntot) : 0ull;
             if (ltot) {
                 const unsigned long long old = atomicAdd(lt.ctr, (stot << lt.rbits) | (unsigned long long)ltot);
-                if ((old >> lt.rbits) + stot >= 1ull << (64 - lt.rbits)) atomicOr(fail, 1u);
+                const unsigned f = long_fails(old, ltot, stot, lt.rbits, lt.cap);
+                if (f) atomicOr(fail, f);
                 lbase_s = old;
             }
         }
@@ -530,14 +550,14 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
             for (int q = 0; q < RPT; ++q) {
                 if (best[q] <= (uint32_t)SHORT_MAX) continue;
                 const int32_t *row = rowv + (q * NT + (int)threadIdx.x) * t;
-                if (li < lt.cap && best[q] <= BOUND_LEN_MASK) {
+                if (best[q] > BOUND_LEN_MASK) {
+                    atomicOr(fail, LONG_NEVER);
+                } else if (li < lt.cap) {
                     int32_t *dst = lt.rows + li * (uint64_t)t;
                     for (int c = 0; c < t; ++c) dst[c] = row[c];
                     lt.bnd[li] = best[q] | ((uint32_t)jb[q] << BOUND_LEN_BITS);
                     lt.blo[li] = lob[q];
                     lt.F[li] = f;
-                } else {
-                    atomicOr(fail, 1u);
                 }
                 ++li;
                 f += best[q];
@@ -982,13 +1002,15 @@ __device__ __noinline__ void count_tail(const JoinArgs &a, const int32_t *M, uin
                     atomicAdd(a.mult + (uint32_t)v[q], (unsigned long long)__popc(peers)) == 0ull) {
                     const unsigned long long old = atomicAdd(lt.ctr, ((unsigned long long)len[q] << lt.rbits) | 1ull);
                     const unsigned long long li = old & ((1ull << lt.rbits) - 1ull), f = old >> lt.rbits;
-                    if (li < lt.cap && len[q] <= BOUND_LEN_MASK && f + len[q] < 1ull << (64 - lt.rbits)) {
+                    const unsigned bad = long_fails(old, 1, len[q], lt.rbits, lt.cap) |
+                                         (len[q] > BOUND_LEN_MASK ? LONG_NEVER : 0u);
+                    if (!bad) {
                         lt.rows[li] = v[q];
                         lt.bnd[li] = len[q];
                         lt.blo[li] = lo[q];
                         lt.F[li] = f;
                     } else {
-                        atomicOr(fail, 1u);
+                        atomicOr(fail, bad);
                     }
                 }
             }

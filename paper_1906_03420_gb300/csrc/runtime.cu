@@ -427,9 +427,9 @@ gsi_status Exec::run(int t, const int32_t *M, uint64_t R) {
 // region and two table regions used in turn), every step's sizes computed on
 // the device, no host wait until the end.  The final table's region is handed
 // to the result when it is well used, or its rows are copied to a tight buffer.
-gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memory) {
+gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *larger_helps) {
     *overflow = false;
-    *no_memory = false;
+    *larger_helps = true;
     const uint64_t B = arena_bytes;
     const uint64_t align = 256;
     // a third each: scratch (16 bytes per input row: offsets and bound
@@ -439,7 +439,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     const uint64_t t_bytes = ((B - s_bytes) / 2) / align * align;
     if (s_bytes < (1 << 16) || t_bytes < (uint64_t)g->n * 4 + 1024) {
         *overflow = true;
-        *no_memory = true;
+        *larger_helps = false;
         return GSI_OK;
     }
     uint64_t *S = nullptr, *memo = nullptr;
@@ -477,7 +477,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
         release();
         (void)cudaGetLastError();
         *overflow = true;              // could not reserve the arena: use the splitting path
-        *no_memory = true;
+        *larger_helps = false;
         return GSI_OK;
     }
     peak = std::max(peak, s_bytes + 2 * t_bytes);
@@ -572,6 +572,7 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *no_memor
     if (rc != GSI_OK || fin[0] != 0) {
         release();
         if (rc == GSI_OK) *overflow = true;
+        if (fin[0] & 8u) *larger_helps = false;
         return rc;
     }
     const uint64_t count = fin[1];
@@ -799,9 +800,9 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
             // arenas of 16 GiB, then x4 per overflow, up to the budget
             uint64_t arena = std::min<uint64_t>(x.budget, DEVICE_ARENA_START);
             for (;;) {
-                bool no_memory = false;
-                rc = x.run_device(arena, &overflow, &no_memory);
-                if (rc != GSI_OK || !overflow || no_memory || arena >= x.budget) break;
+                bool larger_helps = false;
+                rc = x.run_device(arena, &overflow, &larger_helps);
+                if (rc != GSI_OK || !overflow || !larger_helps || arena >= x.budget) break;
                 arena = std::min<uint64_t>(x.budget, arena * 4);
             }
         }

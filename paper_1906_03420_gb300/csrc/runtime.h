@@ -117,8 +117,9 @@ struct Exec {
     // All steps enqueued with device-resident sizes; *overflow is set when a
     // table or the scratch did not fit its region (nothing is added to res).
     // arena_bytes: scratch + two table regions; *overflow: a table did not
-    // fit (or the arena could not be reserved: *no_memory as well)
-    gsi_status run_device(uint64_t arena_bytes, bool *overflow, bool *no_memory);
+    // fit; *larger_helps is false when it would not fit a larger arena either
+    // (that cannot be reserved, or the step is past what its counters hold)
+    gsi_status run_device(uint64_t arena_bytes, bool *overflow, bool *larger_helps);
     // The memo of the first run_device call, reserved and cleared ahead of it
     // (tables its size; 0: not yet).
     uint64_t *memo = nullptr;
