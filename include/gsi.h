@@ -121,13 +121,22 @@ typedef struct {
     /* device time (CUDA events on the query's stream) and work, accumulated */
     double filter_ms, join_ms, other_ms;
     uint64_t filter_launches, join_launches, other_launches;
-    uint64_t filter_bytes;   /* algorithmic bytes of the filter */
+    uint64_t filter_bytes;   /* algorithmic bytes of the filter: of each label
+                                asked for, the vertex ids and the signature
+                                words that its query vertices use, and the
+                                bitmaps */
     uint64_t join_bytes;     /* algorithmic bytes of the join steps: per row
                                 the row, 16 bytes per linking list (its offset
                                 pair and label sub-range), the label
                                 sub-lists (the shortest once per candidate
                                 slot, with the bitmap word), and 4(t+1) per
-                                survivor written */
+                                survivor written.  Where the step's memo knows
+                                which entries of a list are candidates, 4 bytes
+                                for each of those stand in place of the slots
+                                (and, in a single-list row, 8 for the memo
+                                entry in place of 16); the last step of a
+                                counting query reads a long list once for all
+                                rows that share it, and it is counted once */
     uint64_t join_items;     /* candidate slots: sum over rows of the length
                                 of the row's shortest linking list restricted
                                 to the new vertex's label (a bound at most

@@ -184,6 +184,7 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
     *fp = FilterPlan();
     const int32_t nqv = (int32_t)sigs.size();
     fp->nqv = nqv;
+    fp->bytes = (uint64_t)nqv * (uint64_t)g->nwords * 4ull;
     if (nqv == 0) return GSI_OK;
     std::vector<int32_t> perm((size_t)nqv);
     for (int32_t i = 0; i < nqv; ++i) perm[i] = i;
@@ -211,6 +212,7 @@ gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &
                 flat.insert(flat.end(), sig + 1, sig + GSI_SIG_WORDS);
                 gmask.back() |= (int32_t)used;
             }
+            fp->bytes += (uint64_t)(g->goff[r + 1] - g->goff[r]) * 4ull * (uint64_t)(1 + __builtin_popcount((unsigned)gmask.back()));
         }
         i = j;
     }
@@ -291,19 +293,21 @@ void filter_plan_free(FilterPlan &fp, cudaStream_t st) {
 }
 
 static gsi_status launch_filter_groups(const gsi_graph *g, const std::vector<const uint32_t *> &sigs,
-                                       uint32_t *bitmaps, unsigned long long *counts, cudaStream_t st) {
+                                       uint32_t *bitmaps, unsigned long long *counts, cudaStream_t st,
+                                       uint64_t *bytes = nullptr) {
     FilterPlan fp;
     gsi_status rc = filter_plan(g, sigs, &fp, st);
+    if (bytes) *bytes = fp.bytes;
     if (rc == GSI_OK) rc = filter_enqueue(g, fp, bitmaps, counts, st);
     filter_plan_free(fp, st);
     return rc;
 }
 
 gsi_status launch_filter(const gsi_graph *g, const QuerySig &q, uint32_t *bitmaps, unsigned long long *counts,
-                         cudaStream_t st) {
+                         cudaStream_t st, uint64_t *bytes) {
     std::vector<const uint32_t *> sigs;
     for (int u = 0; u < q.k; ++u) sigs.push_back(q.sig[u]);
-    return launch_filter_groups(g, sigs, bitmaps, counts, st);
+    return launch_filter_groups(g, sigs, bitmaps, counts, st, bytes);
 }
 
 gsi_status launch_filter_batch(const gsi_graph *g, const std::vector<QuerySig> &qs, uint32_t *bitmaps,
@@ -312,20 +316,6 @@ gsi_status launch_filter_batch(const gsi_graph *g, const std::vector<QuerySig> &
     for (const QuerySig &q : qs)
         for (int u = 0; u < q.k; ++u) sigs.push_back(q.sig[u]);
     return launch_filter_groups(g, sigs, bitmaps, counts, st);
-}
-
-// Bytes the filter must move for these query vertices: the grouped words of
-// every label they carry (ids and 15 signature words) and their bitmaps.
-uint64_t filter_alg_bytes(const gsi_graph *g, const std::vector<int32_t> &labels) {
-    std::vector<int32_t> l(labels);
-    std::sort(l.begin(), l.end());
-    l.erase(std::unique(l.begin(), l.end()), l.end());
-    uint64_t b = 0;
-    for (int32_t x : l) {
-        const int32_t r = g->label_rank(x);
-        if (r >= 0) b += (uint64_t)(g->goff[r + 1] - g->goff[r]) * 4ull * GSI_SIG_WORDS;
-    }
-    return b + (uint64_t)labels.size() * (uint64_t)g->nwords * 4ull;
 }
 
 int64_t seed_scratch_words(const gsi_graph *g) { return scan_blocks(g->nwords) + 1; }

@@ -67,8 +67,9 @@ struct QuerySig {
 void query_signatures(const int32_t *qvlab, int32_t k, const int32_t *qsrc, const int32_t *qdst,
                       const int32_t *qelab, int32_t qm, QuerySig *out, bool hom = false);
 // bitmaps: device uint32[k][nwords]; counts: device unsigned long long[k] (both zeroed here).
+// *bytes (optional): FilterPlan::bytes.
 gsi_status launch_filter(const gsi_graph *g, const QuerySig &q, uint32_t *bitmaps, unsigned long long *counts,
-                         cudaStream_t st);
+                         cudaStream_t st, uint64_t *bytes = nullptr);
 // Every query vertex of a batch in one pass: bitmaps [sum k][nwords] and
 // counts [sum k] in query order (zeroed here).
 gsi_status launch_filter_batch(const gsi_graph *g, const std::vector<QuerySig> &qs, uint32_t *bitmaps,
@@ -89,6 +90,8 @@ struct FilterPlan {
     int32_t *d_meta = nullptr;
     int32_t nqv = 0, nq = 0, ngroups = 0;
     int64_t warps = 0;
+    uint64_t bytes = 0;         // what the call cannot do without: of each label it asks for, the ids and the
+                                // signature words that its query vertices use, and the bitmaps
 };
 gsi_status filter_plan(const gsi_graph *g, const std::vector<const uint32_t *> &sigs, FilterPlan *fp,
                        cudaStream_t st);
@@ -100,8 +103,6 @@ void filter_plan_free(FilterPlan &fp, cudaStream_t st);
 inline size_t filter_bitmap_bytes(const gsi_graph *g, int32_t nqv) {
     return ((size_t)nqv * (size_t)g->nwords * 4 + 7) / 8 * 8;
 }
-// Algorithmic bytes of one filter call over query vertices with these labels.
-uint64_t filter_alg_bytes(const gsi_graph *g, const std::vector<int32_t> &labels);
 // Compact the bitmap of C(u) into the int32 list out (ascending); scratch: uint32[scan_blocks+1].
 gsi_status launch_seed(const gsi_graph *g, const uint32_t *bitmap, int32_t *out, uint32_t *scratch,
                        cudaStream_t st);

@@ -252,6 +252,7 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
                 *lbytes += row_list_bytes(t, d, wsum, best);
             }
             *abytes += row_alg_bytes(t, d, lsum, best);
+            if (known != NO_MASK) *abytes -= 8ull * best - 4ull * (unsigned)__popc(known);
             *items += best;
         }
         if (best > 0 && best <= (uint32_t)SHORT_MAX) {
@@ -410,7 +411,8 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
         if (a.stats) {
             if (LW && valid) *lbytes += row_list_bytes(t, 1, whole_len(a, 0, v[q]), best[q]);
             if (valid) {
-                *abytes += row_alg_bytes(t, 1, best[q], best[q]);
+                const bool masked = memo && !probe[q] && best[q] <= (uint32_t)SHORT_MAX;
+                *abytes += masked ? row_memo_bytes(t, mask[q]) : row_alg_bytes(t, 1, best[q], best[q]);
                 *items += best[q];
             }
         }
@@ -945,6 +947,7 @@ __device__ __noinline__ void count_tail(const JoinArgs &a, const int32_t *M, uin
                 len[q] = h - lo[q];
                 mask[q] = len[q] <= (uint32_t)SHORT_MAX ? bitmap_mask(a, lo[q], len[q]) : NO_MASK;
                 if (len[q] <= MEMO_LEN_MASK) a.memo[(uint32_t)v[q]] = memo_entry(t, lo[q], len[q], mask[q]);
+                if (a.stats) *abytes += 16ull + (mask[q] != NO_MASK ? 8ull * len[q] : 0ull);
             }
         }
         // the rows' own values among the candidates: long lists are searched
@@ -990,8 +993,8 @@ __device__ __noinline__ void count_tail(const JoinArgs &a, const int32_t *M, uin
         for (int q = 0; q < TAIL_Q; ++q) {
             const bool lng = len[q] > (uint32_t)SHORT_MAX;
             if (!lng) found += __popc(mask[q]);
-            if (a.stats && v[q] >= 0) {
-                *abytes += row_alg_bytes(t, 1, len[q], len[q]);
+            if (a.stats && v[q] >= 0) {               // long lists are counted where they are read, once for all their rows
+                *abytes += row_memo_bytes(t, 0);
                 *items += len[q];
                 if (LW) *lbytes += row_list_bytes(t, 1, whole_len(a, 0, v[q]), len[q]);
             }
@@ -1009,6 +1012,7 @@ __device__ __noinline__ void count_tail(const JoinArgs &a, const int32_t *M, uin
                         lt.bnd[li] = len[q];
                         lt.blo[li] = lo[q];
                         lt.F[li] = f;
+                        if (a.stats) *abytes += 8ull * len[q];
                     } else {
                         atomicOr(fail, bad);
                     }

@@ -104,6 +104,12 @@ __device__ __forceinline__ unsigned long long row_alg_bytes(int t, int d, uint64
     return 4ull * t + 16ull * d + 4ull * (lsum - best) + 8ull * best;
 }
 
+// One row whose list the step's memo has with its mask: read the row, the memo
+// entry and the entries of the list that the mask keeps.
+__device__ __forceinline__ unsigned long long row_memo_bytes(int t, uint32_t mask) {
+    return 4ull * t + 8ull + 4ull * (unsigned)__popc(mask);
+}
+
 // The same row under the whole-list model: read the row, locate each linking
 // list with one 8-byte offset pair, read every linking list N(v, l) whole
 // (wsum elements, the merge-intersection bound), and probe the bitmap once

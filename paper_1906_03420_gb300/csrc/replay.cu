@@ -167,7 +167,7 @@ extern "C" gsi_status gsi_batch_replay(gsi_batch *b, gsi_result **outs, int32_t 
             stats->filter_launches += b->in.fp.ngroups ? 1 : 0;
             stats->join_launches += b->L.nitems ? 1 : 0;
             stats->kernels += (b->in.fp.ngroups ? 1 : 0) + (b->L.nitems ? 1 : 0);
-            stats->filter_bytes += filter_alg_bytes(g, b->in.labels);
+            stats->filter_bytes += b->in.fp.bytes;
         }
         gsi_batch_opts bo = b->opts;
         bo.stats = stats;

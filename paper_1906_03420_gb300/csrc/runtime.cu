@@ -717,7 +717,8 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
     x.pending = true;
 
     x.tm.begin(0);
-    rc = launch_filter(g, qs, x.bitmaps, d_counts, x.st);
+    uint64_t filter_bytes = 0;
+    rc = launch_filter(g, qs, x.bitmaps, d_counts, x.st, &filter_bytes);
     x.tm.end();
     x.kernels += 1;
     uint64_t cand_h[GSI_MAX_QUERY_VERTICES] = {0};
@@ -863,7 +864,7 @@ gsi_status run_query(gsi_graph *g, const QueryGraph &q, const gsi_query_opts &o,
         for (int p = 0; p < q.k; ++p) s->order[p] = (rc == GSI_OK && !empty) ? order[p] : -1;
         s->tiles += x.tiles;
         s->peak_bytes = std::max<uint64_t>(s->peak_bytes, x.peak);
-        s->filter_bytes += filter_alg_bytes(g, std::vector<int32_t>(q.vlab, q.vlab + q.k));
+        s->filter_bytes += filter_bytes;
         s->join_bytes += x.join_bytes;
         s->join_items += x.join_items;
         s->join_bytes_listwise += x.join_bytes_listwise;

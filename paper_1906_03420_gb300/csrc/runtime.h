@@ -193,7 +193,6 @@ struct BatchInputs {
     unsigned long long *counts = nullptr;
     FilterPlan fp;
     uint64_t nk = 0;
-    std::vector<int32_t> labels;             // query vertex labels (filter bytes)
 };
 gsi_status batch_plan_all(gsi_graph *g, std::vector<BatchPlan> &plans, gsi_stats *stats, cudaStream_t st,
                           BatchInputs &in);

@@ -66,7 +66,6 @@ gsi_status batch_plan_all(gsi_graph *g, std::vector<BatchPlan> &plans, gsi_stats
         sigs.emplace_back();
         query_signatures(p.q.vl.data(), p.k, p.q.src.data(), p.q.dst.data(), p.q.lab.data(), p.q.qm, &sigs.back());
         p.bitmaps = in.bitmaps + bm_off[i];
-        in.labels.insert(in.labels.end(), p.q.vlab, p.q.vlab + p.k);
     }
     std::vector<const uint32_t *> sp;
     for (const QuerySig &q : sigs)
@@ -92,7 +91,7 @@ gsi_status batch_plan_all(gsi_graph *g, std::vector<BatchPlan> &plans, gsi_stats
         stats->filter_ms += ms;
         stats->filter_launches += 1;
         stats->kernels += 1;
-        stats->filter_bytes += filter_alg_bytes(g, in.labels);
+        stats->filter_bytes += in.fp.bytes;
         cudaEventDestroy(f0);
         cudaEventDestroy(f1);
     }
