@@ -7,6 +7,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "runtime.h"
+#include "thread_kit.h"
 
 using namespace gsi;
 

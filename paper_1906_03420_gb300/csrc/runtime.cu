@@ -11,6 +11,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "runtime.h"
+#include "thread_kit.h"
 
 int32_t gsi_graph::label_rank(int32_t label) const {
     auto it = std::lower_bound(vlabels.begin(), vlabels.end(), label);
@@ -281,20 +282,6 @@ static gsi_status dalloc(Exec &x, void **p, uint64_t bytes) {
         return GSI_ENOMEM;
     }
     return GSI_OK;
-}
-
-unsigned char *thread_pinned() {
-    static thread_local unsigned char *p = nullptr;
-    if (!p && cudaMallocHost(&p, PINNED_READ + PINNED_STAGE) != cudaSuccess) p = nullptr;
-    return p;
-}
-
-// The calling thread's event on a device, for waits within one entry point.
-static cudaEvent_t thread_event(int dev) {
-    static thread_local cudaEvent_t ev[64];
-    if (dev < 0 || dev >= 64) return nullptr;
-    if (!ev[dev] && cudaEventCreateWithFlags(&ev[dev], cudaEventDisableTiming) != cudaSuccess) ev[dev] = nullptr;
-    return ev[dev];
 }
 
 static gsi_status read_u64(Exec &x, const void *dptr, uint64_t *val) {

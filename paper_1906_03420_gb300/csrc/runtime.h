@@ -207,12 +207,6 @@ gsi_status batch_execute(gsi_graph *g, std::vector<BatchPlan> &plans, const gsi_
 gsi_status batch_run_device(gsi_graph *g, std::vector<BatchPlan> &plans, const gsi_batch_opts &o, uint64_t budget,
                             cudaStream_t st, gsi_stats *stats, BatchWorkspace *ws = nullptr);
 gsi_status prepare_device(int dev);
-// PINNED_READ + PINNED_STAGE bytes of pinned memory of the calling thread:
-// small readbacks first, then an upload area.  Every use is complete before the
-// entry point that makes it returns (cudaFreeHost would synchronise the whole
-// device, so the buffer lives as long as the thread).  Null without memory.
-constexpr size_t PINNED_READ = 4096, PINNED_STAGE = 60 * 1024;
-unsigned char *thread_pinned();
 gsi_status validate_query(const int32_t *qvlab, int32_t k, const int32_t *qsrc, const int32_t *qdst,
                           const int32_t *qelab, int32_t qm, QueryGraph *q);
 void plan_order(const QueryGraph &q, const uint64_t *cand, const uint64_t *freq, int32_t nlabels, int32_t *order,
