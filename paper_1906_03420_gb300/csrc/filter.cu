@@ -31,6 +31,14 @@ constexpr int FNT = 256;
 // own are compared (qsig[s][0], where the label itself is not needed).  On the
 // medium graph (2^20 vertices, 64 labels) a 10-vertex query reads 3-6 words
 // instead of 15.
+//
+// That choice of words pays where a query vertex's own come from the launch's
+// parameters.  In a batch (WIDE) they come from memory, hundreds to a label, and
+// a branch for each word made their loads wait for one another: there each
+// signature is four 16-byte loads and 15 and-nots without branches.  233 queries
+// of 7-8 vertices on 410,886 vertices: 219 us with 15 4-byte loads, 277 with the
+// branches, 136 so.
+template <bool WIDE>
 __device__ __forceinline__ void filter_warp(const int32_t *__restrict__ gperm, const uint32_t *__restrict__ gsig,
                                             int64_t np, int64_t p, const uint32_t *qsig, const int32_t *qid, int32_t s0,
                                             int32_t s1, uint32_t gmask, uint32_t *scnt, int32_t nwords,
@@ -44,14 +52,25 @@ __device__ __forceinline__ void filter_warp(const int32_t *__restrict__ gperm, c
     unsigned run = 0;                                 // lanes sharing my bitmap word, once needed
     for (int32_t s = s0; s < s1; ++s) {
         const uint32_t *q = qsig + (int64_t)s * GSI_SIG_WORDS;
-        const uint32_t qm = q[0];
         bool pass = v >= 0;
+        if (WIDE) {                                   // a word that is not read (gmask) is zero in q too
+            uint32_t miss = 0;
 #pragma unroll
-        for (int j = 0; j < GSI_SIG_WORDS - 1; ++j)
-            if ((qm >> j) & 1u) {
-                const uint32_t qw = q[j + 1];
-                pass = pass && ((x[j] & qw) == qw);
+            for (int h = 0; h < GSI_SIG_WORDS / 4; ++h) {
+                const uint4 y = __ldg(reinterpret_cast<const uint4 *>(q) + h);
+                if (h) miss |= y.x & ~x[4 * h - 1];   // word 0 is the mask of the words in use
+                miss |= (y.y & ~x[4 * h]) | (y.z & ~x[4 * h + 1]) | (y.w & ~x[4 * h + 2]);
             }
+            pass = pass && miss == 0;
+        } else {
+            const uint32_t qm = q[0];
+#pragma unroll
+            for (int j = 0; j < GSI_SIG_WORDS - 1; ++j)
+                if ((qm >> j) & 1u) {
+                    const uint32_t qw = q[j + 1];
+                    pass = pass && ((x[j] & qw) == qw);
+                }
+        }
         const unsigned b = __ballot_sync(FULL_MASK, pass);
         if (!b) continue;
         uint32_t *bm = bitmaps + (int64_t)qid[s] * nwords;
@@ -79,6 +98,7 @@ __device__ __forceinline__ void filter_warp(const int32_t *__restrict__ gperm, c
 // gstart[ngroups + 1] (query vertices of group g), wbeg[ngroups] (first warp
 // of the group's label), wcum[ngroups + 1] (prefix of the groups' warps),
 // gmask[ngroups] (words that the group's query vertices use).
+template <bool WIDE>
 __device__ __forceinline__ void filter_body(const int32_t *__restrict__ gperm, const uint32_t *__restrict__ gsig,
                                             int64_t np, const uint32_t *qsig, const int32_t *meta, int32_t ngroups,
                                             int32_t nqv, int32_t shared_counts, int32_t nwords,
@@ -102,7 +122,7 @@ __device__ __forceinline__ void filter_body(const int32_t *__restrict__ gperm, c
             else hi = mid - 1;
         }
         const int64_t p = ((int64_t)wbeg[lo] + (aw - wcum[lo])) * 32 + (threadIdx.x & 31);
-        filter_warp(gperm, gsig, np, p, qsig, qid, gstart[lo], gstart[lo + 1], (uint32_t)gmask[lo],
+        filter_warp<WIDE>(gperm, gsig, np, p, qsig, qid, gstart[lo], gstart[lo + 1], (uint32_t)gmask[lo],
                     shared_counts ? scnt : nullptr, nwords, bitmaps, counts);
     }
     if (shared_counts) {
@@ -121,7 +141,7 @@ __global__ void __launch_bounds__(FNT) k_filter_groups(const int32_t *__restrict
                                                        uint32_t *__restrict__ bitmaps,
                                                        unsigned long long *__restrict__ counts) {
     extern __shared__ uint32_t scnt[];
-    filter_body(gperm, gsig, np, qsig, meta, ngroups, nqv, shared_counts, nwords, bitmaps, counts, scnt);
+    filter_body<true>(gperm, gsig, np, qsig, meta, ngroups, nqv, shared_counts, nwords, bitmaps, counts, scnt);
 }
 
 // One query's, from the launch's own parameters: no buffer to allocate and
@@ -133,7 +153,7 @@ __global__ void __launch_bounds__(FNT) k_filter_query(const int32_t *__restrict_
                                                       int32_t nqv, int32_t nwords, uint32_t *__restrict__ bitmaps,
                                                       unsigned long long *__restrict__ counts) {
     __shared__ uint32_t scnt[GSI_MAX_QUERY_VERTICES];
-    filter_body(gperm, gsig, np, f.sig, f.meta, ngroups, nqv, 1, nwords, bitmaps, counts, scnt);
+    filter_body<false>(gperm, gsig, np, f.sig, f.meta, ngroups, nqv, 1, nwords, bitmaps, counts, scnt);
 }
 
 struct PopcProducer {
