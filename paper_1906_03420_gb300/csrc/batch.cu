@@ -163,12 +163,12 @@ __device__ __forceinline__ void copy_ints(int32_t *__restrict__ dst, const int32
         const uint64_t nv = n >> 2;
         const int4 *s4 = reinterpret_cast<const int4 *>(src);
         int4 *d4 = reinterpret_cast<int4 *>(dst);
-        for (; i + 7 * NT < nv; i += 8 * NT) {
-            int4 v[8];
+        for (; i + 3 * NT < nv; i += 4 * NT) {
+            int4 v[4];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = __ldcg(s4 + i + j * NT);
+            for (int j = 0; j < 4; ++j) v[j] = __ldcg(s4 + i + j * NT);
 #pragma unroll
-            for (int j = 0; j < 8; ++j) d4[i + j * NT] = v[j];
+            for (int j = 0; j < 4; ++j) d4[i + j * NT] = v[j];
         }
         for (; i < nv; i += NT) d4[i] = __ldcg(s4 + i);
         i = nv * 4 + threadIdx.x;
@@ -242,6 +242,86 @@ __device__ __forceinline__ void discard_l2(const void *p, uint64_t bytes) {
         asm volatile("discard.global.L2 [%0], 128;" ::"l"(x) : "memory");
 }
 
+// This CTA's slice of the arena, and its two table regions behind the scratch.
+__device__ __forceinline__ unsigned char *slice(const BatchArgs &b) { return b.arena + (uint64_t)blockIdx.x * b.slice_bytes; }
+__device__ __forceinline__ int32_t *table(const BatchArgs &b, int i) {
+    return reinterpret_cast<int32_t *>(slice(b) + b.s_bytes + (i ? b.t_bytes : 0));
+}
+
+// The unit that a CTA works on, in shared memory: what stays the same through
+// its steps and what one step leaves to the next.  Thread 0 writes it between
+// barriers.  Held in registers beside the row pass and the slot tiles, which
+// need all 64, it was spilled: 334 bytes of stores and 478 of loads a thread, now
+// 24 and 48.  768 counting queries on 2^20 vertices: 9.5 -> 8.55 ms; 233 small
+// ones on 410,886: join 172 -> 149 us.
+struct Work {
+    long long unit;                // seed item, -(spill slot + 1) or UNIT_DONE
+    long long ticket;              // this CTA's spill slot to come, or -1
+    struct {
+        const int32_t *M;
+        uint64_t R;
+    } in[2];                       // input table and its rows of the even and the odd steps
+    const uint32_t *seed_bm;
+    uint64_t cap;                  // rows that the step's output table holds
+    unsigned long long cnt;        // survivors of the step
+    unsigned long long lctr;       // its long rows and their slots (LongTable::ctr)
+    unsigned long long off, queue[2];
+    uint64_t rows;                 // rows that go to the result arena
+    int64_t word_lo, word_hi;
+    int32_t q, k, t, cfg0, count_only;
+    int32_t counted;               // the step whose statistics hold this unit's rows already
+    unsigned rfail;
+    int32_t skip;                  // the query already failed: its rerun redoes this work
+    int32_t failed;
+};
+
+// Thread 0: takes the next unit.
+__device__ void take_unit(const BatchArgs &b, Work &u) {
+    const long long unit = next_unit(b, &u.ticket);
+    u.unit = unit;
+    if (unit == UNIT_DONE) return;
+    u.counted = 0;
+    u.failed = 0;
+    if (unit >= 0) {
+        const BatchItem it = b.items[unit];
+        u.q = it.q;
+        u.t = 1;
+        u.word_lo = it.word_lo;
+        u.word_hi = it.word_hi;
+        u.in[1] = {table(b, 0), 0};
+    } else {
+        const SpillUnit su = b.sq[-unit - 1];
+        u.q = su.q;
+        u.t = su.t & (COUNTED - 1);
+        u.counted = su.t & COUNTED ? u.t : 0;
+        u.in[u.t & 1] = {b.spill + su.off, su.rows};
+    }
+    const BatchQuery *bq = b.queries + u.q;
+    u.k = bq->k;
+    u.cfg0 = bq->cfg0;
+    u.count_only = bq->count_only;
+    u.seed_bm = bq->seed_bm;
+    u.skip = *reinterpret_cast<const volatile unsigned *>(&bq->status) != 0u;
+    u.cap = u.count_only ? 0 : b.t_bytes / 4;         // of a one-vertex query
+}
+
+// Rows whose slots begin past SPLIT_SLOTS go to other CTAs, which join them
+// from this step on; *L and *total are what is left.
+template <int NT>
+__device__ __noinline__ void share_long(const BatchArgs &b, Work &u, const LongTable &lt, int t, uint64_t *L, uint64_t *total,
+                                        unsigned long long *wt) {
+    unsigned long long keep = 0;
+    for (uint64_t i = threadIdx.x; i < *L; i += NT) keep += __ldcg(lt.F + i) < SPLIT_SLOTS;
+    keep = block_sum<NT, unsigned long long>(keep, wt);
+    if (keep == *L) return;
+    const uint64_t first = __ldcg(lt.F + keep), extra = *L - keep;
+    const uint64_t per = max((uint64_t)1, extra * SPLIT_SLOTS / (*total - first));
+    if (queue_rows<NT>(b, u.q, t | COUNTED, lt.rows + keep * (uint64_t)t, extra, (uint64_t)t, per, u.queue)) {
+        *L = keep;
+        *total = first;
+    }
+}
+
 // One instance per block shape: NT threads per CTA, RPT rows per thread in
 // the row pass (the batched autotuner picks one).
 template <int NT, int RPT>
@@ -249,95 +329,60 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
     constexpr int BNT = NT;
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ unsigned long long wt[BNT / 32];
-    __shared__ long long unit_s;
-    __shared__ unsigned long long cnt_s, lctr_s, off_s, queue_s[2];
-    __shared__ unsigned rfail_s;
-    __shared__ int fail_s, skip_s;
+    __shared__ Work u;
+    __shared__ LongTable lt;
     __shared__ __align__(16) JoinArgs a_s;
-    unsigned char *slice = b.arena + (uint64_t)blockIdx.x * b.slice_bytes;
-    uint64_t *S = reinterpret_cast<uint64_t *>(slice);
-    int32_t *reg[2] = {reinterpret_cast<int32_t *>(slice + b.s_bytes),
-                       reinterpret_cast<int32_t *>(slice + b.s_bytes + b.t_bytes)};
-    const uint64_t S_words = b.s_bytes / 8;
-    BatchCtl *c = b.ctl;
-    int32_t *const result = c->result;
-    const unsigned long long result_cap = c->result_cap;
+    const JoinArgs &a = a_s;
 
-    long long ticket = -1;                            // thread 0: its spill slot to come
+    if (threadIdx.x == 0) u.ticket = -1;
     for (;;) {
-        if (threadIdx.x == 0) unit_s = next_unit(b, &ticket);
+        if (threadIdx.x == 0) take_unit(b, u);
         __syncthreads();
-        const long long unit = unit_s;
-        if (unit == UNIT_DONE) return;
-        int q, t0, oreg, counted = 0;                 // counted: the step whose statistics hold this unit's rows
-        const int32_t *M;
-        uint64_t R = 0;
-        if (unit >= 0) {
-            const BatchItem it = b.items[unit];
-            q = it.q;
-            t0 = 1;
-            oreg = 1;
-            M = reg[0];
-        } else {
-            const SpillUnit su = b.sq[-unit - 1];
-            q = su.q;
-            t0 = su.t & (COUNTED - 1);
-            counted = su.t & COUNTED ? t0 : 0;
-            oreg = 0;
-            M = b.spill + su.off;
-            R = su.rows;
-        }
-        BatchQuery *bq = b.queries + q;
-        const int k = bq->k;
-        if (threadIdx.x == 0) skip_s = *reinterpret_cast<volatile unsigned *>(&bq->status) != 0u;
-        __syncthreads();
-        const bool skip = skip_s != 0;            // the query already failed: its rerun redoes this work
-        if (unit >= 0 && !skip) {
+        if (u.unit == UNIT_DONE) return;
+        if (u.unit >= 0 && !u.skip) {
             // ---- seed: set bits of the item's words, ascending
-            const BatchItem it = b.items[unit];
+            int32_t *const seeds = table(b, 0);
             unsigned long long run = 0;
-            for (int64_t base = it.word_lo; base < it.word_hi; base += BNT) {
+            for (int64_t base = u.word_lo; base < u.word_hi; base += BNT) {
                 const int64_t i = base + threadIdx.x;
-                const uint32_t w = i < it.word_hi ? bq->seed_bm[i] : 0u;
+                uint32_t x = i < u.word_hi ? u.seed_bm[i] : 0u;
                 unsigned long long tot;
-                unsigned long long pos = block_exclusive_scan<BNT, unsigned long long>(__popc(w), wt, &tot) + run;
-                uint32_t x = w;
+                unsigned long long pos = block_exclusive_scan<BNT, unsigned long long>(__popc(x), wt, &tot) + run;
                 while (x) {
-                    reg[0][pos++] = (int32_t)(i * 32 + (int64_t)(__ffs(x) - 1));
+                    seeds[pos++] = (int32_t)(i * 32 + (int64_t)(__ffs(x) - 1));
                     x &= x - 1;
                 }
                 run += tot;
             }
-            R = run;
-            __syncthreads();                      // step 1 reads seeds written by other threads
+            if (threadIdx.x == 0) u.in[1].R = run;
         }
-        bool failed = false;
-        uint64_t cap = 0;
-        for (int t = t0; t < k && R > 0 && !skip; ++t) {
-            __syncthreads();                      // the previous step's readers of a_s are done
+        int t = u.t;
+        for (; t < u.k && !u.skip; ++t) {
+            __syncthreads();                      // the step's input is there, the previous step's readers are done
+            const auto &in = u.in[t & 1];
+            if (in.R == 0) break;
+            int32_t *const out = table(b, t & 1);
             {   // this step's configuration in shared memory
-                const uint32_t *src = reinterpret_cast<const uint32_t *>(b.cfgs + bq->cfg0 + t);
+                const uint32_t *src = reinterpret_cast<const uint32_t *>(b.cfgs + u.cfg0 + t);
                 uint32_t *dst = reinterpret_cast<uint32_t *>(&a_s);
                 for (int i = threadIdx.x; i < (int)(sizeof(JoinArgs) / 4); i += BNT) dst[i] = src[i];
             }
-            const JoinArgs &a = a_s;
-            int32_t *out = reg[oreg];
-            const bool last = t == k - 1;
-            cap = b.t_bytes / (4ull * (uint64_t)(t + 1));
-            if (last && bq->count_only) cap = 0;
-            // long rows (bound above SHORT_MAX) in the scratch region
-            const LongTable lt = long_table(S, S_words, t, R, &lctr_s);
-            if (threadIdx.x == 0) {
-                cnt_s = 0;
-                lctr_s = 0;
-                rfail_s = 0;
+            if (threadIdx.x == BNT - 1) {         // in a warp that has little to copy
+                u.cnt = 0;
+                u.lctr = 0;
+                u.rfail = 0;
+                const JoinArgs *const cfg = b.cfgs + u.cfg0 + t;
+                u.cap = cfg->out_cap;
+                // long rows (bound above SHORT_MAX) in the scratch region; its
+                // room from the host, as a 64-bit division takes as long as the copy
+                lt = long_table(reinterpret_cast<uint64_t *>(slice(b)), cfg->total, t, in.R, &u.lctr);
             }
             __syncthreads();
             // short rows joined inline, long rows set aside
             unsigned long long abytes = 0, items = 0, lbytes = 0;
-            row_pass<BNT, true, RPT, false>(a, M, R, 0, (uint64_t)BNT * RPT, BNT * RPT, out, cap, &cnt_s, lt, &rfail_s, smem,
-                                            &abytes, &items, &lbytes);
-            if (a.stats && t != counted) {       // one add per step of a unit
+            row_pass<BNT, true, RPT, false, false>(a, in.M, in.R, 0, (uint64_t)BNT * RPT, BNT * RPT, out, u.cap, &u.cnt, lt,
+                                                   &u.rfail, smem, &abytes, &items, &lbytes);
+            if (a.stats && t != u.counted) {     // one add per step of a unit
                 abytes = block_sum<BNT, unsigned long long>(abytes, wt);
                 items = block_sum<BNT, unsigned long long>(items, wt);
                 lbytes = block_sum<BNT, unsigned long long>(lbytes, wt);
@@ -348,83 +393,82 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_batch(const __grid_constant__
                 }
             }
             __syncthreads();
-            if (rfail_s) { failed = true; break; }     // long-row table full: the plain path
-            uint64_t L = lctr_s & ((1ull << lt.rbits) - 1ull), total = lctr_s >> lt.rbits;
-            if (b.split_rows && total > SPLIT_SLOTS && L > 1) {
-                // rows whose slots begin past SPLIT_SLOTS go to other CTAs, which
-                // join them from this step on
-                unsigned long long keep = 0;
-                for (uint64_t i = threadIdx.x; i < L; i += BNT) keep += __ldcg(lt.F + i) < SPLIT_SLOTS;
-                keep = block_sum<BNT, unsigned long long>(keep, wt);
-                if (keep < L) {
-                    const uint64_t first = __ldcg(lt.F + keep), extra = L - keep;
-                    const uint64_t per = max((uint64_t)1, extra * SPLIT_SLOTS / (total - first));
-                    if (queue_rows<BNT>(b, q, t | COUNTED, lt.rows + keep * (uint64_t)t, extra, (uint64_t)t, per, queue_s)) {
-                        L = keep;
-                        total = first;
-                    }
-                }
+            if (u.rfail) {                        // long-row table full: the plain path
+                if (threadIdx.x == 0) u.failed = 1;
+                break;
             }
-            if (L > 0) {
+            if (u.lctr) {
+                uint64_t L = u.lctr & ((1ull << lt.rbits) - 1ull), total = u.lctr >> lt.rbits;
+                if (b.split_rows && total > SPLIT_SLOTS && L > 1) share_long<BNT>(b, u, lt, t, &L, &total, wt);
                 // the long rows' slot tiles, CTA-local
                 const unsigned warp = threadIdx.x >> 5;
-                long_rows_join(a, lt, L, total, warp, BNT / 32, out, cap, &cnt_s, smem + warp * long_warp_smem(t, a.s.d));
+                long_rows_join<false>(a, lt, L, total, warp, BNT / 32, out, u.cap, &u.cnt, smem + warp * long_warp_smem(t, a.s.d));
+                __syncthreads();
             }
-            __syncthreads();
-            discard_l2<BNT>(M, R * (uint64_t)t * 4);    // this step's input is dead
-            const uint64_t cnt = cnt_s;
+            discard_l2<BNT>(in.M, in.R * (uint64_t)t * 4);    // this step's input is dead
+            uint64_t R = u.cnt;
             if (a.stats && threadIdx.x == 0) {   // survivors written (both models)
-                atomicAdd(a.stats, 4ull * (uint64_t)(t + 1) * min(cnt, cap));
-                atomicAdd(a.stats + 2, 4ull * (uint64_t)(t + 1) * min(cnt, cap));
+                atomicAdd(a.stats, 4ull * (uint64_t)(t + 1) * min(R, u.cap));
+                atomicAdd(a.stats + 2, 4ull * (uint64_t)(t + 1) * min(R, u.cap));
             }
-            if (!last && cnt > cap) { failed = true; break; }
-            M = out;
-            oreg ^= 1;
-            R = cnt;
+            const bool last = t == u.k - 1;
+            if (!last && R > u.cap) {
+                if (threadIdx.x == 0) u.failed = 1;
+                break;
+            }
             // ---- split: keep split_rows rows, queue the rest for other CTAs
             if (!last && b.split_rows && R > b.split_rows) {
-                const uint64_t keep = b.split_rows, extra = R - keep;
-                const uint64_t w = (uint64_t)(t + 1);
-                if (queue_rows<BNT>(b, q, t + 1, M + keep * w, extra, w, keep, queue_s)) {
+                const uint64_t keep = b.split_rows, w = (uint64_t)(t + 1);
+                if (queue_rows<BNT>(b, u.q, t + 1, out + keep * w, R - keep, w, keep, u.queue)) {
                     __syncthreads();
-                    discard_l2<BNT>(M + keep * w, extra * w * 4);      // the queued rows now live in the spill area
+                    discard_l2<BNT>(out + keep * w, (R - keep) * w * 4);      // the queued rows now live in the spill area
                     R = keep;
                 }
             }
+            if (threadIdx.x == 0) u.in[(t + 1) & 1] = {out, R};
         }
-        if (!skip && k == 1) cap = bq->count_only ? 0 : b.t_bytes / 4;
-        // the final table must also have fit (rows past the region are lost)
-        if (!skip && !failed && !bq->count_only && R > cap) failed = true;
+        __syncthreads();                          // readers of the last step's state are done
         // ---- final rows to the result arena
-        const uint64_t rows = (skip || failed) ? 0 : min(R, cap);
+        const auto &fin = u.in[t & 1];
         if (threadIdx.x == 0) {
-            fail_s = failed;
-            off_s = 0;
-            if (!skip && !failed && rows > 0) {
-                const unsigned long long need = (rows * (unsigned long long)k + 3) & ~3ull;    // on 16 bytes
+            // the final table must also have fit (rows past the region are lost)
+            if (!u.skip && !u.count_only && fin.R > u.cap) u.failed = 1;
+            BatchCtl *const c = b.ctl;
+            BatchQuery *const bq = b.queries + u.q;
+            uint64_t rows = (u.skip || u.failed) ? 0 : min(fin.R, u.cap);
+            u.off = 0;
+            if (rows > 0) {
+                const unsigned long long need = (rows * (unsigned long long)u.k + 3) & ~3ull;    // on 16 bytes
                 const unsigned long long o = atomicAdd(&c->result_used, need);
-                if (o + need > result_cap) fail_s = 1;
-                else off_s = o;
+                if (o + need > c->result_cap) u.failed = 1;
+                else u.off = o;
             }
-            if (fail_s) atomicOr(&bq->status, 1u);
-            else if (!skip) atomicAdd(&bq->count, (unsigned long long)R);
-            if (!fail_s && rows > 0) {
+            if (u.failed) {
+                rows = 0;
+                atomicOr(&bq->status, 1u);
+            } else if (!u.skip) {
+                atomicAdd(&bq->count, (unsigned long long)fin.R);
+            }
+            if (rows > 0) {
                 const unsigned long long r = atomicAdd(&c->nrecs, 1ull);
                 BatchRec rec;
-                rec.q = q;
+                rec.q = u.q;
                 rec.pad = 0;
-                rec.off = off_s;
+                rec.off = u.off;
                 rec.rows = rows;
                 b.recs[r] = rec;
             }
+            u.rows = rows;
         }
         __syncthreads();
-        if (!fail_s && rows > 0) {
-            copy_ints<BNT>(result + off_s, M, rows * (uint64_t)k);
+        if (u.rows > 0) {
+            copy_ints<BNT>(b.ctl->result + u.off, fin.M, u.rows * (uint64_t)u.k);
+            __syncthreads();
+            discard_l2<BNT>(fin.M, u.rows * (uint64_t)u.k * 4);   // copied out
         }
         __syncthreads();
-        if (!fail_s && rows > 0) discard_l2<BNT>(M, rows * (uint64_t)k * 4);   // copied out
         if (threadIdx.x == 0) {
+            BatchCtl *const c = b.ctl;
             atomicAdd(&c->units, 1ull);
             __threadfence();
             atomicAdd(&c->pending, ~0ull);        // this unit is finished (its children were added first)
@@ -548,7 +592,10 @@ gsi_status batch_setup(BatchLaunch &L, gsi_graph *g, std::vector<BatchPlan> &pla
             const int co = (t == p.k - 1) && o.count_only;
             cfg[(size_t)bqs[i].cfg0 + t] =
                 make_join_args(g, p.steps[t], p.bitmaps + (uint64_t)p.order[t] * (uint64_t)g->nwords, co, L.dstats);
-            cfg[(size_t)bqs[i].cfg0 + t].isect = o.isect;
+            JoinArgs &c = cfg[(size_t)bqs[i].cfg0 + t];
+            c.isect = o.isect;
+            c.out_cap = co ? 0 : L.t_bytes / (4ull * (uint64_t)(t + 1));
+            c.total = long_room(L.s_bytes / 8, t);
         }
         // word ranges of the seed bitmap holding about seeds_per_item seeds each
         const uint64_t nw = (uint64_t)g->nwords;

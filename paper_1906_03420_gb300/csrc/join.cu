@@ -240,7 +240,7 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
             copy_words<NT>(&args_s[(t + 1) & 1], cfgs + (t - t0 + 2));
             copy_words<NT>(&ins_s[(t + 1) & 1], &st[1].in);
         }
-        const LongTable lt = long_table(in_s.S, in_s.S_words, t, R, &st->nlong);
+        const LongTable lt = long_table(in_s.S, long_room(in_s.S_words, t), t, R, &st->nlong);
         int32_t *const out = in_s.out;
         uint64_t cap = in_s.out_bytes / (4ull * (uint64_t)(t + 1));
         if (in_s.row_cap && in_s.row_cap < cap) cap = in_s.row_cap;

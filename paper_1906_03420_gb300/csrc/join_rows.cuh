@@ -88,12 +88,17 @@ __host__ __device__ __forceinline__ unsigned long_fails(unsigned long long old, 
            ((old >> rbits) + slots >= 1ull << (64 - rbits) ? LONG_NEVER : 0u);
 }
 
-// The long-row table of step t, whose input has R rows, in a scratch region of
-// S_words 8-byte words: F, rows, bound records.
-__device__ __forceinline__ LongTable long_table(uint64_t *S, uint64_t S_words, int t, uint64_t R,
-                                                unsigned long long *ctr) {
+// Rows that the long-row table of step t holds in a scratch region of S_words
+// 8-byte words.
+__host__ __device__ inline uint64_t long_room(uint64_t S_words, int t) {
+    return S_words > 8 ? (S_words - 8) * 8 / (4ull * (uint64_t)t + 16ull) : 0;
+}
+
+// The long-row table of step t, whose input has R rows, with room for `room`
+// rows in the scratch region S: F, rows, bound records.
+__device__ __forceinline__ LongTable long_table(uint64_t *S, uint64_t room, int t, uint64_t R, unsigned long long *ctr) {
     LongTable lt;
-    lt.cap = S_words > 8 ? (S_words - 8) * 8 / (4ull * (uint64_t)t + 16ull) : 0;
+    lt.cap = room;
     lt.F = S;
     lt.rows = reinterpret_cast<int32_t *>(S + lt.cap);
     lt.bnd = reinterpret_cast<uint32_t *>(lt.rows + lt.cap * (uint64_t)t);
@@ -204,7 +209,7 @@ __device__ __forceinline__ uint32_t subtract_row(const JoinArgs &a, const int32_
 // One row of the pass: its bound (shortest label sub-list: length *best,
 // start *lob, linking edge *jb) and the mask of its survivors among the
 // first *best candidates when best <= SHORT_MAX.
-template <bool LW = true>
+template <bool LW = true, bool MEMO = true>
 __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *row, bool valid,
                                              uint32_t *best_out, uint32_t *lob_out, int *jb_out,
                                              unsigned long long *abytes, unsigned long long *items,
@@ -224,7 +229,7 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
             len4[j] = 0;
             if (j < d) {
                 uint32_t m;
-                len4[j] = sublist(a, j, row[a.s.col[j]], &lo4[j], &m);
+                len4[j] = sublist<MEMO>(a, j, row[a.s.col[j]], &lo4[j], &m);
                 lsum += len4[j];
                 if (len4[j] < best) {
                     best = len4[j];
@@ -236,7 +241,7 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
         }
         for (int j = MEMO_EDGES; j < d; ++j) {
             uint32_t l, m;
-            const uint32_t n = sublist(a, j, row[a.s.col[j]], &l, &m);
+            const uint32_t n = sublist<MEMO>(a, j, row[a.s.col[j]], &l, &m);
             lsum += n;
             if (n < best) {
                 best = n;
@@ -258,16 +263,28 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
         if (best > 0 && best <= (uint32_t)SHORT_MAX) {
             if (known == NO_MASK) {
                 known = bitmap_mask(a, lob, best);
-                if (a.memo && jb < MEMO_EDGES)
+                if (MEMO && a.memo && jb < MEMO_EDGES)
                     a.memo[(uint64_t)jb * (uint64_t)a.memo_n + (uint32_t)row[a.s.col[jb]]] =
                         memo_entry(t, lob, best, known);
             }
             mask = subtract_row(a, row, lob, known);
             // every other linking list must hold the candidate (Alg. 3)
             if (a.isect == ISECT_BSEARCH) {
+                if (MEMO) {
 #pragma unroll
-                for (int j = 0; j < MEMO_EDGES; ++j)
-                    if (mask && j < d && j != jb) mask = contains_mask(a.ci, lob, mask, lo4[j], len4[j]);
+                    for (int j = 0; j < MEMO_EDGES; ++j)
+                        if (mask && j < d && j != jb) mask = contains_mask(a.ci, lob, mask, lo4[j], len4[j]);
+                } else {                              // rows of small units: one candidate, seldom two
+                    for (uint32_t m = mask; m; m &= m - 1) {
+                        const int p = __ffs(m) - 1;
+                        const int32_t w = __ldg(a.ci + lob + (uint32_t)p);
+                        bool ok = true;
+#pragma unroll
+                        for (int j = 0; j < MEMO_EDGES; ++j)
+                            if (ok && j < d && j != jb) ok = sorted_contains(a.ci + lo4[j], len4[j], w);
+                        if (!ok) mask &= ~(1u << p);
+                    }
+                }
             } else {
 #pragma unroll
                 for (int j = 0; j < MEMO_EDGES; ++j) {
@@ -329,14 +346,14 @@ __device__ __forceinline__ uint32_t row_join(const JoinArgs &a, const int32_t *r
 // a leader that does this for the group.
 constexpr int ROW_C = 8;          // candidate values of a single-edge group loaded in the first round
 
-template <int NT, int RPT, bool LW = true>
+template <int NT, int RPT, bool LW = true, bool MEMO = true>
 __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_t *rowv, int nb, int lane,
                                                  uint32_t *best, uint32_t *lob, uint32_t *mask,
                                                  unsigned long long *abytes, unsigned long long *items,
                                                  unsigned long long *lbytes) {
     constexpr int C = ROW_C;
     const int t = a.s.t;
-    const bool memo = a.memo != nullptr;
+    const bool memo = MEMO && a.memo != nullptr;
     int32_t v[RPT];
     bool lead[RPT];
     int leader[RPT];
@@ -365,7 +382,7 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
         mask[q] = 0;
         probe[q] = store[q] = false;
         if (!lead[q]) continue;
-        if (memo_hit(e[q], t)) {
+        if (MEMO && memo_hit(e[q], t)) {
             lob[q] = (uint32_t)e[q];
             best[q] = memo_len(e[q]);
             mask[q] = memo_mask(e[q]);
@@ -425,12 +442,14 @@ __device__ __forceinline__ void rows_join_single(const JoinArgs &a, const int32_
 // nbatch).  With a ticket counter (zero before the step) only three quarters of
 // the batches go out that way, at least two to a CTA, and the rest on demand:
 // rows differ in their lists, and of a step of millions of rows a quarter of
-// the time went by while the last CTAs worked alone.  `a` should live in shared memory.  Survivors go to out (up to cap rows; `count` is
-// exact), long rows to lt.  *fail gets LONG_* bits when they do not fit.  When a.stats is set, adds this
-// thread's algorithmic bytes (rows read, lists located and read; survivors
-// are counted by the caller) to *abytes, the same under the whole-list model
-// to *lbytes (only when LW), and its candidate slots to *items.
-template <int NT, bool DR = true, int RPT = ROW_RPT, bool LW = true>
+// the time went by while the last CTAs worked alone.  `a` should live in shared
+// memory.  Survivors go to out (up to cap rows; `count` is exact), long rows to
+// lt; *fail gets LONG_* bits when they do not fit.  MEMO false: the steps have no
+// memo (batches).  When a.stats is set, adds this thread's algorithmic bytes
+// (rows read, lists located and read; survivors are counted by the caller) to
+// *abytes, the same under the whole-list model to *lbytes (only when LW), and its
+// candidate slots to *items.
+template <int NT, bool DR = true, int RPT = ROW_RPT, bool LW = true, bool MEMO = true>
 __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64_t first, uint64_t stride, int nbatch,
                          int32_t *__restrict__ out, uint64_t cap, unsigned long long *count, const LongTable &lt,
                          unsigned *fail, unsigned char *smem, unsigned long long *abytes,
@@ -467,7 +486,7 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
         uint32_t n = 0, nl = 0;
         unsigned long long sl = 0;                    // slots of this thread's long rows, then their exclusive prefix
         if (DR && a.s.d == 1 && !a.nodedup) {
-            rows_join_single<NT, RPT, LW>(a, rowv, nb, lane, best, lob, mask, abytes, items, lbytes);
+            rows_join_single<NT, RPT, LW, MEMO>(a, rowv, nb, lane, best, lob, mask, abytes, items, lbytes);
 #pragma unroll
             for (int q = 0; q < RPT; ++q) jb[q] = 0;
         } else {
@@ -475,7 +494,7 @@ __device__ void row_pass(const JoinArgs &a, const int32_t *M, uint64_t R, uint64
             for (int q = 0; q < RPT; ++q) {
                 const int lr = q * NT + (int)threadIdx.x;
                 const bool valid = lr < nb;
-                mask[q] = row_join<LW>(a, rowv + (valid ? lr : 0) * t, valid, &best[q], &lob[q], &jb[q],
+                mask[q] = row_join<LW, MEMO>(a, rowv + (valid ? lr : 0) * t, valid, &best[q], &lob[q], &jb[q],
                                           abytes, items, lbytes);
                 if (!valid) best[q] = 0;
             }
@@ -688,7 +707,7 @@ __host__ __device__ constexpr size_t long_warp_smem(int t, int d) {
 // a.mult[v] rows; no set subtraction and no other lists.
 enum { LONG_SINGLE, LONG_MULTI, LONG_TAIL };
 
-template <int MODE>
+template <int MODE, bool MEMO = true>
 __device__ inline void long_rows_mode(const JoinArgs &a, const LongTable &lt, uint64_t L, uint64_t total, uint64_t wi,
                                       uint64_t nw, int32_t *__restrict__ out, uint64_t cap, unsigned long long *count,
                                       unsigned char *smem, unsigned long long *ticket = nullptr) {
@@ -753,7 +772,7 @@ __device__ inline void long_rows_mode(const JoinArgs &a, const LongTable &lt, ui
             for (int j = 0; j < d; ++j) {
                 if (j == (int)jb) continue;
                 uint32_t m;
-                l[1] = sublist(a, j, rowv[lane * t + a.s.col[j]], &l[0], &m);
+                l[1] = sublist<MEMO>(a, j, rowv[lane * t + a.s.col[j]], &l[0], &m);
                 l += 2;
             }
         }
@@ -888,12 +907,13 @@ __device__ inline void long_rows_mode(const JoinArgs &a, const LongTable &lt, ui
     }
 }
 
+template <bool MEMO = true>
 __device__ __forceinline__ void long_rows_join(const JoinArgs &a, const LongTable &lt, uint64_t L, uint64_t total,
                                                uint64_t wi, uint64_t nw, int32_t *__restrict__ out, uint64_t cap,
                                                unsigned long long *count, unsigned char *smem,
                                                unsigned long long *ticket = nullptr) {
-    if (a.s.d == 1) long_rows_mode<LONG_SINGLE>(a, lt, L, total, wi, nw, out, cap, count, smem, ticket);
-    else long_rows_mode<LONG_MULTI>(a, lt, L, total, wi, nw, out, cap, count, smem, ticket);
+    if (a.s.d == 1) long_rows_mode<LONG_SINGLE, MEMO>(a, lt, L, total, wi, nw, out, cap, count, smem, ticket);
+    else long_rows_mode<LONG_MULTI, MEMO>(a, lt, L, total, wi, nw, out, cap, count, smem, ticket);
 }
 
 // --------------------------------------------------------- counting tail

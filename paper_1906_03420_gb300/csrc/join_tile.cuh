@@ -122,14 +122,14 @@ struct JoinArgs {
     const int32_t *M;
     int64_t R;
     const uint64_t *F;
-    uint64_t total;
+    uint64_t total;             // slots of the host-sized step; of a batch's step: the room of its long-row table
     const int64_t *part;
     const uint32_t *off;
     const int32_t *ci;
     LabelIndex cl;
     const uint32_t *cand;
     int32_t *out;
-    uint64_t out_cap;
+    uint64_t out_cap;           // rows of the output table (host-sized steps and batches)
     unsigned long long *out_count;
     unsigned long long *stats;
     int32_t W, rmax, count_only;
@@ -208,12 +208,14 @@ __device__ __forceinline__ uint64_t memo_entry(int t, uint32_t lo, uint32_t len,
 
 // Start (*lo) and length (returned) of the label(u) sub-list of N(v, lab[j]),
 // through the memo when the step has one, and the sub-list's mask if the memo
-// knows it (else NO_MASK).
+// knows it (else NO_MASK).  MEMO false: the step has none, which spares a batch
+// the code for it.
+template <bool MEMO = true>
 __device__ __forceinline__ uint32_t sublist(const JoinArgs &a, int j, int32_t v, uint32_t *lo, uint32_t *mask) {
     uint64_t *slot = nullptr;
     uint64_t e = 0;
     const uint64_t seg = (uint64_t)(uint32_t)v * (uint64_t)a.s.L + (uint64_t)a.s.lab[j];
-    if (a.memo && j < MEMO_EDGES) {
+    if (MEMO && a.memo && j < MEMO_EDGES) {
         slot = a.memo + (uint64_t)j * (uint64_t)a.memo_n + (uint32_t)v;
         e = *slot;
     }
