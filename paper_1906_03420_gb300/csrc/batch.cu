@@ -34,7 +34,7 @@ namespace gsi {
 namespace {
 
 constexpr uint64_t SPILL_SLOTS = 1ull << 18;                  // spill queue capacity (units)
-constexpr unsigned long long WAIT_SPIN_LIMIT = 1ull << 26;    // x ~100 ns sleeps: several seconds
+constexpr unsigned long long WAIT_SPIN_LIMIT = 1ull << 26;    // x a 500 ns sleep and two round trips: half a minute at least
 constexpr long long UNIT_DONE = -(1ll << 62);
 // Candidate slots of a unit's long rows in one step above which the rows past
 // that many slots go to other CTAs.  8,192 slots are four tiles for each warp,
@@ -114,21 +114,27 @@ __device__ __forceinline__ unsigned long long vload(const unsigned long long *p)
 // Thread 0 only: the next unit (seed item >= 0, spill slot s as -(s + 1)),
 // or UNIT_DONE once no unit is pending (or a wait ran out).
 //
-// Spill slots are dealt by tickets: a CTA that sees slots waiting takes the
-// next number with one atomic add and owns that slot.  Where several race for
-// the last one, the others' numbers are ahead of the queue: each keeps its
-// ticket (*ticket) and takes seed units meanwhile.  (A compare-and-swap on the
-// queue's head let one CTA through per round trip to L2: 0.55 us a unit,
-// however many CTAs were idle, which was all of the time of a batch with
-// 50,000 units.)
+// Spill slots go before seed units.  While there are seed units, a CTA takes a
+// slot that it sees waiting by compare-and-swap, and a seed unit where another
+// was faster.  Once there are none, slots are dealt by tickets: a CTA takes the
+// next number with one atomic add and owns that slot; where several race for the
+// last one, the others' numbers are ahead of the queue, and each keeps its ticket
+// (*ticket) until the slot is there.  So a CTA at work never holds a slot.
+// (Compare-and-swap alone lets one CTA through per round trip to L2: 0.55 us a
+// unit, however many CTAs were idle, which was all of the time of a batch with
+// 50,000 units.  With tickets alone a slot could wait for its owner to finish a
+// seed unit: 768 counting queries on 2^20 vertices took 8.55 ms, now 8.22.)
 __device__ long long next_unit(const BatchArgs &b, long long *ticket) {
     BatchCtl *c = b.ctl;
     unsigned long long spins = 0;
     for (;;) {
         // read together: one round trip to L2, not one for each queue
         const unsigned long long head = vload(&c->sq_head), tail = vload(&c->sq_tail), item = vload(&c->next_item);
-        if (*ticket < 0 && head < tail)
-            *ticket = (long long)atomicAdd(&c->sq_head, 1ull);
+        const bool seeds = item < (unsigned long long)b.nitems;
+        if (*ticket < 0 && head < tail) {
+            if (!seeds) *ticket = (long long)atomicAdd(&c->sq_head, 1ull);
+            else if (atomicCAS(&c->sq_head, head, head + 1) == head) *ticket = (long long)head;
+        }
         // published (a number past the queue's end never is)
         if (*ticket >= 0 && (unsigned long long)*ticket < b.sq_cap &&
             *reinterpret_cast<volatile unsigned *>(&b.sq_ready[*ticket]) != 0u) {
@@ -137,7 +143,7 @@ __device__ long long next_unit(const BatchArgs &b, long long *ticket) {
             *ticket = -1;
             return -h - 1;
         }
-        if (item < (unsigned long long)b.nitems) {
+        if (seeds && *ticket < 0) {
             const unsigned long long i = atomicAdd(&c->next_item, 1ull);
             if (i < (unsigned long long)b.nitems) return (long long)i;
         }
