@@ -140,16 +140,21 @@ gsi_status launch_join(const gsi_graph *g, const int32_t *M, uint64_t R, const J
                        unsigned long long *out_count, int count_only, unsigned long long *stats, cudaStream_t st);
 inline uint64_t join_tiles(uint64_t total) { return (total + JOIN_NV - 1) / JOIN_NV; }
 
+// Rows that the long-row table of a step of t columns holds in a scratch region
+// of S_words 8-byte words (LongTable).
+inline uint64_t long_room(uint64_t S_words, int t) {
+    return S_words > 8 ? (S_words - 8) * 8 / (4ull * (uint64_t)t + 16ull) : 0;
+}
+
 // One join step of a cooperative query launch (see join.cu): the host sets
 // the regions, the device the sizes.
 struct DStepIn {                       // set by the host
     const int32_t *M;                  // input table (t columns)
     int32_t *out;                      // output table region
-    uint64_t out_bytes;                // bytes of the output region
-    uint64_t row_cap;                  // output rows allowed (0 = no limit)
+    uint64_t out_rows;                 // rows that may be written there (0: counted only)
     uint64_t *S;                       // scratch region: the long-row table
-    uint64_t S_words;
-    int32_t t, count_only;
+    uint64_t S_rows;                   // rows that it holds (long_room)
+    int32_t t, pad;
 };
 struct DStep {
     DStepIn in;

@@ -1,7 +1,8 @@
 // Join iterations (Sec. V, Algs. 3-4), in two forms.
 //
-// Host-sized (gsi_join_step, and the splitting path of the memory-bounded
-// driver): one iteration as three launches,
+// Host-sized (the splitting path of the memory-bounded driver, the
+// allocation-free join step, and gsi_join_step where its cooperative launch
+// cannot take the step): one iteration as three launches,
 //   1. scan   F[i] = sum_{r<i} (cap_r + W), where cap_r bounds row r's output
 //             (Alg. 4's preallocation bound), plus W "row slots" per row that
 //             pay for staging the row (load balancing, below);
@@ -9,9 +10,10 @@
 //   3. join   the fused kernel: one CTA per tile of NV slots.
 //
 // Device-driven (k_query): the seed and every iteration of one query in one
-// cooperative launch: per step the row pass (join_rows.cuh), which joins short
-// rows and sets long ones aside with their slot offsets, and the long rows'
-// slot tiles, with a bounded grid barrier after each.
+// cooperative launch, or one iteration over a caller's table (gsi_join_step):
+// per step the row pass (join_rows.cuh), which joins short rows and sets long
+// ones aside with their slot offsets, and the long rows' slot tiles, with a
+// bounded grid barrier after each.
 //
 // Output bound.  Every neighbour list N(v,l) is stored sorted by (label rank
 // of the neighbour, neighbour id), so the neighbours of v via l that carry
@@ -117,11 +119,11 @@ __global__ void __launch_bounds__(NT) k_join(const __grid_constant__ JoinArgs a)
 // The whole join of one query in a single cooperative launch: the seed, then
 // for every step the row pass and, when it set rows aside, the long rows'
 // tiles, with a grid barrier after each.  All CTAs are co-resident (cooperative
-// launch), so the barrier is a counter and a generation word; every wait is
-// bounded, and a CTA that gives up sets an error bit and returns, as does
-// every CTA that later sees the bit, so the kernel always terminates.
+// launch), so the barrier is one counter of arrivals; every wait is bounded,
+// and a CTA that gives up sets a bit in that word and returns, as does every
+// CTA that later sees the bit, so the kernel always terminates.
 
-constexpr unsigned long long BARRIER_SPIN_LIMIT = 1ull << 24;   // x ~64 ns sleeps: about a second
+constexpr unsigned long long BARRIER_SPIN_LIMIT = 1ull << 24;   // x a 64 ns sleep and a read of L2: a second at least
 constexpr unsigned BAR_FAIL = 1u << 31;
 
 // What a barrier hands to its CTA: the step's counters as of the barrier, read
@@ -240,11 +242,9 @@ __global__ void __launch_bounds__(NT, 4) k_query(const JoinArgs *__restrict__ cf
             copy_words<NT>(&args_s[(t + 1) & 1], cfgs + (t - t0 + 2));
             copy_words<NT>(&ins_s[(t + 1) & 1], &st[1].in);
         }
-        const LongTable lt = long_table(in_s.S, long_room(in_s.S_words, t), t, R, &st->nlong);
+        const LongTable lt = long_table(in_s.S, in_s.S_rows, t, R, &st->nlong);
         int32_t *const out = in_s.out;
-        uint64_t cap = in_s.out_bytes / (4ull * (uint64_t)(t + 1));
-        if (in_s.row_cap && in_s.row_cap < cap) cap = in_s.row_cap;
-        if (in_s.count_only) cap = 0;
+        const uint64_t cap = in_s.out_rows;                   // from the host: 64-bit divisions take as long as a round trip
         if (blockIdx.x == 0 && threadIdx.x == 0) st->out_cap = cap;
         prev_cap = cap;
         // ---- short rows joined inline, long rows set aside (one pass over M)
@@ -518,12 +518,10 @@ gsi_status step_coop(const gsi_graph *g, const int32_t *M, uint64_t R, const Joi
     DStepIn &in = h.steps[1].in;
     in.M = M;
     in.out = out;
-    in.out_bytes = ~0ull;                             // the limit is in rows: as bytes a large one ("all of
-    in.row_cap = out_cap;                             // them") would wrap to a small one
+    in.out_rows = out_cap;
     in.S = reinterpret_cast<uint64_t *>(d + head + memo);
-    in.S_words = scratch / 8;
+    in.S_rows = long_room(scratch / 8, s.t);
     in.t = s.t;
-    in.count_only = out_cap == 0;
     h.steps[0].count = R;
     if (give_up) {
         h.ctl.bar = BAR_FAIL;

@@ -88,12 +88,6 @@ __host__ __device__ __forceinline__ unsigned long_fails(unsigned long long old, 
            ((old >> rbits) + slots >= 1ull << (64 - rbits) ? LONG_NEVER : 0u);
 }
 
-// Rows that the long-row table of step t holds in a scratch region of S_words
-// 8-byte words.
-__host__ __device__ inline uint64_t long_room(uint64_t S_words, int t) {
-    return S_words > 8 ? (S_words - 8) * 8 / (4ull * (uint64_t)t + 16ull) : 0;
-}
-
 // The long-row table of step t, whose input has R rows, with room for `room`
 // rows in the scratch region S: F, rows, bound records.
 __device__ __forceinline__ LongTable long_table(uint64_t *S, uint64_t room, int t, uint64_t R, unsigned long long *ctr) {

@@ -7,7 +7,7 @@
 // wait on an allocator (cudaMalloc can synchronise the device, and a
 // stream-ordered pool can still have to grow); a process under a strict
 // device-memory quota where an allocation in the middle of a request could
-// fail.  For them this entry point runs the same kernels as gsi_join_step, but
+// fail.  For them this entry point runs the host-sized step (join.cu), but
 // every scratch buffer (the row-bound scan, its block sums and per-row bounds,
 // the tile partition and the survivor counter) lives in one file-scope __device__ array of fixed
 // size.  The caller still provides the input table, the candidate bitmap and

@@ -498,12 +498,11 @@ gsi_status Exec::run_device(uint64_t arena_bytes, bool *overflow, bool *larger_h
         DStepIn &h = hs[t].in;
         h.M = reg[(t - 1) & 1];
         h.out = reg[t & 1];
-        h.out_bytes = t_bytes;
-        const bool last = t == k - 1;
-        h.row_cap = last ? row_cap : 0;
-        h.count_only = last ? count_only : 0;
+        h.out_rows = t_bytes / (4ull * (uint64_t)(t + 1));
+        if (t == k - 1 && row_cap) h.out_rows = std::min(h.out_rows, row_cap);
+        if (t == k - 1 && count_only) h.out_rows = 0;
         h.S = S;
-        h.S_words = s_bytes / 8;
+        h.S_rows = long_room(s_bytes / 8, t);
         h.t = t;
     }
     rc = GSI_OK;
