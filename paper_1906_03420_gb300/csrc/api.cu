@@ -428,9 +428,7 @@ gsi_status gsi_memory_trim(int32_t device, uint64_t *bytes) {
     GSI_API_BEGIN
     if (bytes) *bytes = 0;
     GSI_TRY(prepare_device(device));
-    const cudaStream_t st = library_stream(device);
-    const uint64_t n = block_trim(device, st);
-    GSI_CUDA_TRY(cudaStreamSynchronize(st));
+    const uint64_t n = block_trim(device, true);
     if (bytes) *bytes = n;
     return GSI_OK;
     GSI_API_END

@@ -10,6 +10,7 @@ struct KeptBlock {
     void *p;
     uint64_t bytes;
     cudaEvent_t done;                // null: idle
+    cudaStream_t st;                 // where it was recorded
     uint64_t turn;                   // requests before it was given back
 };
 struct BlockCache {
@@ -21,6 +22,7 @@ struct BlockCache {
     // that is in a copy to pageable memory, until that copy's stream gets there
     cudaEvent_t spare[KEPT_MOST];
     int nspare = 0;
+    cudaStream_t out = nullptr;      // blocks go back to the pool here, behind their last use and nothing else
 };
 
 BlockCache &block_cache(int dev) {   // never destroyed: results may outlive static objects
@@ -46,14 +48,31 @@ void block_remove(BlockCache &c, int i) {
 }
 
 // Gives kept block i back to the pool, behind its last use.
-void block_release(BlockCache &c, int i, cudaStream_t st) {
+void block_release(BlockCache &c, int i) {
     const KeptBlock b = c.kept[i];
+    if (!c.out && cudaStreamCreateWithFlags(&c.out, cudaStreamNonBlocking) != cudaSuccess) c.out = nullptr;
     if (b.done) {
-        cudaStreamWaitEvent(st, b.done, 0);
+        cudaStreamWaitEvent(c.out, b.done, 0);
         c.spare[c.nspare++] = b.done;
     }
-    cudaFreeAsync(b.p, st);
+    cudaFreeAsync(b.p, c.out);
     block_remove(c, i);
+}
+
+// Whether the work on a kept block has ended.
+bool block_idle(BlockCache &c, KeptBlock &k) {
+    if (!k.done) return true;
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;    // a query is no part of anyone's capture
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    const cudaError_t e = cudaEventQuery(k.done);
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    c.spare[c.nspare++] = k.done;
+    k.done = nullptr;
+    return true;
 }
 
 }  // namespace
@@ -62,7 +81,11 @@ cudaError_t device_alloc(void **p, size_t bytes, cudaStream_t st) {
     cudaError_t e = cudaMallocAsync(p, bytes, st);
     int dev = 0;
     if (e != cudaErrorMemoryAllocation || cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return e;
-    if (!block_trim(dev, st)) return e;
+    if (!block_trim(dev, false)) return e;
+    (void)cudaGetLastError();
+    e = cudaMallocAsync(p, bytes, st);
+    if (e != cudaErrorMemoryAllocation) return e;
+    block_trim(dev, true);                            // not all of it had arrived
     (void)cudaGetLastError();
     return cudaMallocAsync(p, bytes, st);
 }
@@ -72,10 +95,12 @@ cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, Block *b) {
         BlockCache &c = block_cache(dev);
         std::lock_guard<std::mutex> lk(c.mu);
         ++c.turn;
+        const cudaStream_t own = library_stream(dev);
         int at = -1;
         for (int i = 0; i < c.n; ++i) {
-            const KeptBlock &k = c.kept[i];
+            KeptBlock &k = c.kept[i];
             if (k.bytes < bytes || k.bytes - bytes > bytes / 2) continue;
+            if (!block_idle(c, k) && k.st != st && k.st != own) continue;
             const KeptBlock *best = at < 0 ? nullptr : &c.kept[at];
             if (!best || (best->done && !k.done) || (!best->done == !k.done && k.bytes < best->bytes)) at = i;
         }
@@ -97,9 +122,9 @@ cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, Block *b) {
             if (c.kept[i].bytes < bytes && bytes - c.kept[i].bytes <= c.kept[i].bytes / 2 &&
                 (less < 0 || c.kept[i].bytes > c.kept[less].bytes))
                 less = i;
-        if (less >= 0) block_release(c, less, st);
+        if (less >= 0) block_release(c, less);
         while (old < c.n && c.turn - c.kept[old].turn > KEPT_TURNS) ++old;
-        while (old-- > 0) block_release(c, 0, st);
+        while (old-- > 0) block_release(c, 0);
     }
     b->bytes = bytes;
     return device_alloc(&b->p, bytes, st);
@@ -111,9 +136,9 @@ void block_put(int dev, Block b, cudaStream_t st, bool idle) {
         BlockCache &c = block_cache(dev);
         std::lock_guard<std::mutex> lk(c.mu);
         if (c.users > 0 && b.bytes <= most) {
-            while (c.n == KEPT_MOST || c.bytes + b.bytes > most) block_release(c, 0, st);
+            while (c.n == KEPT_MOST || c.bytes + b.bytes > most) block_release(c, 0);
             const cudaEvent_t done = idle ? nullptr : take_event(c, st);
-            c.kept[c.n++] = {b.p, b.bytes, done, c.turn};
+            c.kept[c.n++] = {b.p, b.bytes, done, st, c.turn};
             c.bytes += b.bytes;
             return;
         }
@@ -121,12 +146,18 @@ void block_put(int dev, Block b, cudaStream_t st, bool idle) {
     cudaFreeAsync(b.p, st);
 }
 
-uint64_t block_trim(int dev, cudaStream_t st) {
+uint64_t block_trim(int dev, bool wait) {
     if (dev < 0 || dev >= 64) return 0;
     BlockCache &c = block_cache(dev);
-    std::lock_guard<std::mutex> lk(c.mu);
-    const uint64_t bytes = c.bytes;
-    while (c.n) block_release(c, 0, st);
+    uint64_t bytes = 0;
+    cudaStream_t out = nullptr;
+    {
+        std::lock_guard<std::mutex> lk(c.mu);
+        bytes = c.bytes;
+        while (c.n) block_release(c, 0);
+        out = c.out;
+    }
+    if (wait && out) cudaStreamSynchronize(out);
     return bytes;
 }
 
@@ -136,7 +167,7 @@ void block_users(int dev, int change) {
     std::lock_guard<std::mutex> lk(c.mu);
     c.users += change;
     if (c.users) return;
-    while (c.n) block_release(c, 0, nullptr);
+    while (c.n) block_release(c, 0);
     while (c.nspare) cudaEventDestroy(c.spare[--c.nspare]);
 }
 

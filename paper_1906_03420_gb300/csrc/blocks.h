@@ -9,6 +9,8 @@
 
 namespace gsi {
 
+// The library's own stream on a device (null: none).
+cudaStream_t library_stream(int dev);
 // Total memory of a device (looked up once per device).
 uint64_t device_total_mem(int dev);
 
@@ -24,15 +26,20 @@ cudaError_t device_alloc(T **p, size_t bytes, cudaStream_t st) { return device_a
 // new memory (four queries with rows took 14 to 25 ms instead of 2).
 //
 // Any thread and stream may take a block that another gave back: `idle` says
-// that the stream had completed, otherwise an event orders the two.  A call
-// takes the smallest kept block that holds what it asks for and is at most half
-// as large again, an idle one first: calls whose budgets differ a little share
-// blocks, and none ties up twice what it asked for.  A request that finds none
-// gives back to the pool one that is a little too small, as the new block will
-// serve in its place, and those that KEPT_TURNS requests have passed over: there
-// they can be cut for other sizes.  At most KEPT_MOST blocks and a quarter of
-// the device's memory are kept, none under BLOCK_MIN, and none at all without a
-// graph on the device.
+// that the stream had completed, otherwise an event orders the two.  A block
+// whose event has not come yet is only taken on the stream that it was given
+// back on, or from the library's own stream, where nothing waits for a caller's
+// work: a request never waits for what another caller has put on a stream since,
+// as one of the pool does not.
+//
+// A call takes the smallest kept block that holds what it asks for and is at
+// most half as large again, an idle one first: calls whose budgets differ a
+// little share blocks, and none ties up twice what it asked for.  A request that
+// finds none gives back to the pool one that is a little too small, as the new
+// block will serve in its place, and those that KEPT_TURNS requests have passed
+// over: there they can be cut for other sizes.  At most KEPT_MOST blocks and a
+// quarter of the device's memory are kept, none under BLOCK_MIN, and none at all
+// without a graph on the device.
 constexpr uint64_t BLOCK_MIN = 64ull << 20;
 constexpr int KEPT_MOST = 64;
 constexpr uint64_t KEPT_TURNS = 256;
@@ -42,8 +49,9 @@ struct Block {
 };
 cudaError_t block_get(int dev, uint64_t bytes, cudaStream_t st, Block *b);
 void block_put(int dev, Block b, cudaStream_t st, bool idle);
-// Gives every kept block back to the pool, behind the work on `st`; their bytes.
-uint64_t block_trim(int dev, cudaStream_t st);
+// Gives every kept block back to the pool, behind its last use (wait: returns
+// when they have arrived); their bytes.
+uint64_t block_trim(int dev, bool wait);
 // A graph was made on the device (+1) or destroyed (-1, with the device idle).
 void block_users(int dev, int change);
 

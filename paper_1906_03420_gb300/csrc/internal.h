@@ -45,9 +45,6 @@ struct gsi_graph {
 
 namespace gsi {
 
-// The library's own stream on a device (null: none).
-cudaStream_t library_stream(int dev);
-
 // ------------------------------------------------------------------ sort
 // Ascending, stable LSD radix sort of n keys over their bits [lo, hi).  keys
 // and tmp hold n keys each; *sorted is the one that the result ends in.

@@ -22,6 +22,7 @@
 using Clock = std::map<cudaStream_t, long>;
 static std::map<cudaStream_t, Clock> known;       // what each stream is ordered behind, itself included
 static Clock host;                                // what the host has waited for
+static Clock ended;                               // what has ended on the device
 static std::map<void *, std::pair<cudaStream_t, long>> used;
 static std::map<void *, size_t> live;             // allocated, in bytes
 static std::map<void *, size_t> pool;             // freed, in bytes
@@ -35,14 +36,18 @@ static void merge(Clock &a, const Clock &b) {
 static bool behind(cudaStream_t s, void *p) {
     if (!used.count(p)) return true;
     const auto u = used[p];
-    return known[s][u.first] >= u.second || host[u.first] >= u.second;
+    return known[s][u.first] >= u.second || host[u.first] >= u.second || ended[u.first] >= u.second;
 }
 static void use(cudaStream_t s, void *p) {
     CHECK(live.count(p));
     CHECK(behind(s, p));
     used[p] = {s, ++known[s][s]};
 }
-static void wait_host(cudaStream_t s) { merge(host, known[s]); }
+static void end(cudaStream_t s) { merge(ended, known[s]); }
+static void wait_host(cudaStream_t s) {
+    end(s);
+    merge(host, known[s]);
+}
 
 extern "C" {
 cudaError_t cudaMallocAsync(void **p, size_t n, cudaStream_t) {
@@ -84,6 +89,26 @@ cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned) {
     ++waits;
     return cudaSuccess;
 }
+cudaError_t cudaEventQuery(cudaEvent_t e) {
+    CHECK(events.count(e));
+    for (auto &x : events[e])
+        if (ended[x.first] < x.second && host[x.first] < x.second) return cudaErrorNotReady;
+    return cudaSuccess;
+}
+cudaError_t cudaThreadExchangeStreamCaptureMode(enum cudaStreamCaptureMode *m) {
+    static cudaStreamCaptureMode now = cudaStreamCaptureModeGlobal;
+    std::swap(now, *m);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+    *s = reinterpret_cast<cudaStream_t>(1000);
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    merge(ended, known[s]);
+    merge(host, known[s]);
+    return cudaSuccess;
+}
 cudaError_t cudaDeviceSynchronize(void) {
     for (auto &k : known) merge(host, k.second);
     return cudaSuccess;
@@ -92,6 +117,7 @@ cudaError_t cudaDeviceSynchronize(void) {
 
 namespace gsi {
 uint64_t device_total_mem(int) { return total; }
+cudaStream_t library_stream(int) { return reinterpret_cast<cudaStream_t>(9); }
 }
 
 using namespace gsi;
@@ -103,11 +129,11 @@ static Block get(cudaStream_t s, uint64_t bytes) {
     CHECK(block_get(0, bytes, s, &b) == cudaSuccess && b.bytes >= bytes && live[b.p] == b.bytes);
     return b;
 }
-// A block that stream 1 gave back with work on it.
-static void *from_stream_1(uint64_t bytes) {
-    const Block b = get(S(1), bytes);
-    use(S(1), b.p);
-    block_put(0, b, S(1), false);
+// A block that a stream (the library's, unless said otherwise) gave back with work on it.
+static void *given_back(uint64_t bytes, cudaStream_t s = S(9)) {
+    const Block b = get(s, bytes);
+    use(s, b.p);
+    block_put(0, b, s, false);
     return b.p;
 }
 
@@ -115,8 +141,10 @@ int main(int, char **argv) {
     const std::string what = argv[1];
     Block a, b, c;
     block_users(0, 1);
-    if (what == "abandoned set") {                // its stream waits for stream 1, but nobody has waited for it
-        void *p = from_stream_1(GB);
+    // first, sets that end with work on stream 2, be it a wait for the library's stream: stream 3 asks next, and may not have
+    // the block before that work has ended
+    if (what == "abandoned set") {
+        void *p = given_back(GB);
         {
             BlockSet set(0, S(2));
             CHECK(set.get(GB, &a) == cudaSuccess && a.p == p);
@@ -124,18 +152,24 @@ int main(int, char **argv) {
             CHECK(set.get(GB, &b) != cudaSuccess);
         }
         deny = 0;
-        use(S(3), get(S(3), GB).p);
+        b = get(S(3), GB);
+        CHECK(b.p != p);
+        use(S(3), b.p);
+        end(S(9));
+        end(S(2));
+        use(S(3), (c = get(S(3), GB)).p);
+        CHECK(c.p == p);
     } else if (what == "failed wait") {
-        from_stream_1(GB);
+        void *p = given_back(GB);
         {
             BlockSet set(0, S(2));
-            CHECK(set.get(GB, &a) == cudaSuccess);
+            CHECK(set.get(GB, &a) == cudaSuccess && a.p == p);
             use(S(2), a.p);
             CHECK(!set.waited(cudaErrorUnknown) && set.busy());
         }
-        b = get(S(3), GB);
-        CHECK(b.p == a.p);
-        use(S(3), b.p);
+        use(S(3), (b = get(S(3), GB)).p);
+        CHECK(b.p != p);
+        use(S(2), get(S(2), GB).p);
     } else if (what == "work after the wait") {
         {
             BlockSet set(0, S(2));
@@ -146,9 +180,8 @@ int main(int, char **argv) {
             set.enqueued();
             use(S(2), a.p);
         }
-        b = get(S(3), GB);
-        CHECK(b.p == a.p);
-        use(S(3), b.p);
+        use(S(3), (b = get(S(3), GB)).p);
+        CHECK(b.p != a.p);
     } else if (what == "second attempt") {        // a retry takes blocks of an attempt that was waited for
         {
             BlockSet set(0, S(2));
@@ -162,9 +195,31 @@ int main(int, char **argv) {
             CHECK(set.get(GB, &b) == cudaSuccess && b.p == a.p);
             use(S(2), b.p);                       // and ends without a wait
         }
-        b = get(S(3), GB);
-        CHECK(b.p == a.p);
-        use(S(3), b.p);
+        use(S(3), (b = get(S(3), GB)).p);
+        CHECK(b.p != a.p);
+    } else if (what == "another stream's work") {  // a block is not waited for, be it the only one, but on its own stream
+        void *p = given_back(GB, S(1));
+        const size_t before = waits;
+        a = get(S(2), GB);
+        CHECK(a.p != p && waits == before);
+        b = get(S(1), GB);
+        CHECK(b.p == p);
+        use(S(1), p);
+        block_put(0, b, S(1), false);
+        end(S(1));                                // it has ended: anyone's
+        CHECK(get(S(2), GB).p == p);
+        use(S(2), p);
+    } else if (what == "the library's stream") {  // nothing is held up there: its blocks are waited for
+        void *p = given_back(GB);
+        a = get(S(2), GB);
+        CHECK(a.p == p);
+        use(S(2), p);
+    } else if (what == "given back to the pool") {   // behind its last use, without making the caller's stream wait for it
+        given_back(GB, S(1));
+        given_back(3 * GB, S(1));
+        a = get(S(2), GB);                        // neither is taken
+        CHECK(block_trim(0, false) == 4 * GB && live.size() == 1);
+        CHECK(known[S(2)][S(1)] == 0 && known[S(9)][S(1)] == 0);
     } else if (what == "waited for") {            // no event between the two
         {
             BlockSet set(0, S(2));
@@ -199,11 +254,11 @@ int main(int, char **argv) {
         for (Block &k : x) block_put(0, k, S(1), true);
         CHECK(get(S(1), 3 * GB).p == x[2].p && get(S(1), 3 * GB).p == x[0].p && get(S(1), 3 * GB).p == x[1].p);
     } else if (what == "idle first") {            // a larger idle block goes before one with work on it
-        a = get(S(1), GB);
-        b = get(S(1), GB + 64 * MB);
-        block_put(0, b, S(1), true);
-        use(S(1), a.p);
-        block_put(0, a, S(1), false);
+        a = get(S(9), GB);
+        b = get(S(9), GB + 64 * MB);
+        block_put(0, b, S(9), true);
+        use(S(9), a.p);
+        block_put(0, a, S(9), false);
         const size_t before = waits;
         CHECK(get(S(2), GB).p == b.p && waits == before);
         c = get(S(2), GB);
@@ -252,28 +307,29 @@ int main(int, char **argv) {
         CHECK(live.empty());
     } else if (what == "out of memory") {         // any failed allocation gives the kept blocks back and tries again
         total = 8 * GB;
-        from_stream_1(GB);
-        from_stream_1(GB + GB / 8);
+        given_back(GB);
+        given_back(GB + GB / 8);
         void *p = nullptr;
         CHECK(device_alloc(&p, 7 * GB, S(2)) == cudaSuccess && live.size() == 1);
         CHECK(device_alloc(&p, 2 * GB, S(2)) == cudaErrorMemoryAllocation);
     } else if (what == "trim") {
-        from_stream_1(GB);
+        given_back(GB);
         a = get(S(2), 5 * GB);
         block_put(0, a, S(2), true);
-        CHECK(block_trim(0, S(3)) == 6 * GB && live.empty() && block_trim(0, S(3)) == 0);
+        CHECK(block_trim(0, true) == 6 * GB && live.empty() && block_trim(0, true) == 0);
     } else if (what == "events") {                // made for the first blocks only, and never more than there are blocks
         for (int i = 0; i < 300; ++i) {
             Block x[3];
             for (Block &k : x) use(S(1 + i % 3), (k = get(S(1 + i % 3), GB)).p);
             for (Block &k : x) block_put(0, k, S(1 + i % 3), false);
-            if (i % 100 == 99) block_trim(0, S(4));
+            end(S(1 + i % 3));
+            if (i % 100 == 99) block_trim(0, false);
         }
         CHECK(events.size() == 3 && created == 3);
     } else if (what == "last graph") {            // nothing is kept without one; a result that outlives it frees its block
         block_users(0, 1);
         a = get(S(1), GB);
-        from_stream_1(GB);
+        given_back(GB);
         wait_host(S(1));                          // a graph goes with the device idle
         block_users(0, -1);
         CHECK(live.size() == 2);

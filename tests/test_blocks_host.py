@@ -21,7 +21,8 @@ def program(tmp_path_factory):
     return exe
 
 
-@pytest.mark.parametrize("case", ["abandoned set", "failed wait", "work after the wait", "second attempt", "waited for",
+@pytest.mark.parametrize("case", ["abandoned set", "failed wait", "work after the wait", "second attempt", "another stream's work",
+                                  "the library's stream", "given back to the pool", "waited for",
                                   "taken block", "near size", "smallest that fits", "idle first", "changing budgets",
                                   "passed over", "a quarter of the memory", "number of blocks", "small ones", "out of memory",
                                   "trim", "events", "last graph"])

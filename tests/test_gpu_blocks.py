@@ -89,3 +89,30 @@ def test_trim_gives_back_what_is_kept_and_only_that(pkg):
     assert G.query(PATH, mem_budget=1 << 30, count_only=True).count == 60 * 59 * 58
     G.close()
     assert pkg.memory_trim() == 0                     # nothing is kept without a graph
+
+
+def test_a_query_does_not_wait_for_another_streams_work(pkg):
+    """A result goes back while a host function holds up its stream. A query of the same size on another stream goes on."""
+    import ctypes
+    import torch
+    g = complete(60)
+    G = pkg.Graph(g.vlab, g.src, g.dst, g.elab)
+    held_up, other = torch.cuda.Stream(), torch.cuda.Stream()
+    pkg.memory_trim()
+    results = [G.query(PATH, stream=held_up, mem_budget=1 << 30) for _ in range(3)]
+    pkg.memory_trim()                                 # nothing is kept but what these give back
+    free, began, count = threading.Event(), threading.Event(), []
+    hold = ctypes.CFUNCTYPE(None, ctypes.c_void_p)(lambda _: (began.set(), free.wait(60)) and None)
+    assert ctypes.CDLL("libcudart.so.13").cudaLaunchHostFunc(ctypes.c_void_p(held_up.cuda_stream), hold, None) == 0
+    began.wait(10)
+    for r in results:
+        r.close()
+    t = threading.Thread(target=lambda: count.append(G.query(PATH, stream=other, mem_budget=1 << 30, count_only=True).count))
+    t.start()
+    t.join(10)
+    went_on = not t.is_alive()
+    free.set()
+    t.join(60)
+    assert went_on and count == [60 * 59 * 58]
+    torch.cuda.synchronize()
+    G.close()
